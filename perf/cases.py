@@ -217,7 +217,7 @@ def prepare(case, seed):
                 F2 = F - G
                 jobs.append(B.lin_job([B.mat(F2), B.mat(F), B.mat(G)], [1, -1, 1],
                                       W.proof_seed(seed, layer, proj, "U" + name)))
-        return _planned(kind, B.LinPlan(jobs), B.vl_lin_proof, len(jobs))
+        return _planned(kind, B.LinPlan(jobs), B.vl_lin_proof, jobs)
     if kind == "lookups":
         jobs, seq, hidden = [], case["seq"], case["hidden"]
         for layer, proj, rank in _projections(case):
@@ -231,7 +231,7 @@ def prepare(case, seed):
                 z, shift = tables[name]()
                 jobs.append(B.lookup_job(B.mat(_remainder(z, shift)), 0, shift,
                                          W.proof_seed(seed, layer, proj, "R" + name)))
-        return _planned(kind, B.LookupPlan(jobs), B.vl_lookup_proof, len(jobs))
+        return _planned(kind, B.LookupPlan(jobs), B.vl_lookup_proof, jobs)
     if kind == "claims":
         jobs = []
         for layer, proj, rank in _projections(case):
@@ -262,9 +262,10 @@ def _with(engine, seg):
     return o
 
 
-def _planned(kind, plan, proof, count):
+def _planned(kind, plan, proof, jobs):
     need = plan.workspace_bytes()
-    st = _State(kind=kind, plan=plan, ws=_buffer(need), need=need, out=_buffer(_size(proof) * count))
+    # the jobs keep the operands alive: the plan holds their addresses only
+    st = _State(kind=kind, jobs=jobs, plan=plan, ws=_buffer(need), need=need, out=_buffer(_size(proof) * len(jobs)))
     st.release = plan.destroy
     return st
 
