@@ -69,16 +69,154 @@ VL_HD bool fr_eq(const Fr& a, const Fr& b) {
   return o == 0;
 }
 
-// t - r if t >= r else t  (t < 2^256 given as 8 limbs plus an overflow limb hi).
-VL_HD void cond_sub_r(uint32_t t[8], uint32_t hi) {
-  uint32_t d[8];
-  uint64_t borrow = 0;
+#if defined(__CUDA_ARCH__)
+// Device arithmetic on carry chains (PTX add.cc / mad.cc).  The C forms below
+// (64-bit temporaries, used on the host) spend about three ALU instructions
+// per limb on carries; with the flag kept in the condition code a limb costs
+// one instruction, and a product's mad.lo.cc / madc.hi.cc pair on an aligned
+// pair of words one wide multiply-add.  Measured on a GB300 (152 x 8 CTAs of
+// 256 threads): additions 354 -> 832 G/s, subtractions 425 -> 868 G/s,
+// Montgomery products 45.5 -> 63.9 G/s (of 78.7 G/s if the wide multiply-adds
+// of a textbook product were all that ran).
+
+// d = a + b mod 2^256.
+__device__ __forceinline__ void add8(uint32_t (&d)[8], const uint32_t (&a)[8], const uint32_t (&b)[8]) {
+  asm("add.cc.u32 %0, %8, %16; addc.cc.u32 %1, %9, %17; addc.cc.u32 %2, %10, %18; addc.cc.u32 %3, %11, %19;\n\t"
+      "addc.cc.u32 %4, %12, %20; addc.cc.u32 %5, %13, %21; addc.cc.u32 %6, %14, %22; addc.u32 %7, %15, %23;"
+      : "=&r"(d[0]), "=&r"(d[1]), "=&r"(d[2]), "=&r"(d[3]), "=&r"(d[4]), "=&r"(d[5]), "=&r"(d[6]), "=&r"(d[7])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(a[4]), "r"(a[5]), "r"(a[6]), "r"(a[7]), "r"(b[0]), "r"(b[1]),
+        "r"(b[2]), "r"(b[3]), "r"(b[4]), "r"(b[5]), "r"(b[6]), "r"(b[7]));
+}
+
+// d = a - b mod 2^256; returns 0xffffffff if it wrapped, else 0.
+__device__ __forceinline__ uint32_t sub8(uint32_t (&d)[8], const uint32_t (&a)[8], const uint32_t (&b)[8]) {
+  uint32_t w;
+  asm("sub.cc.u32 %0, %9, %17; subc.cc.u32 %1, %10, %18; subc.cc.u32 %2, %11, %19; subc.cc.u32 %3, %12, %20;\n\t"
+      "subc.cc.u32 %4, %13, %21; subc.cc.u32 %5, %14, %22; subc.cc.u32 %6, %15, %23; subc.cc.u32 %7, %16, %24;\n\t"
+      "subc.u32 %8, 0, 0;"
+      : "=&r"(d[0]), "=&r"(d[1]), "=&r"(d[2]), "=&r"(d[3]), "=&r"(d[4]), "=&r"(d[5]), "=&r"(d[6]), "=&r"(d[7]),
+        "=&r"(w)
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(a[4]), "r"(a[5]), "r"(a[6]), "r"(a[7]), "r"(b[0]), "r"(b[1]),
+        "r"(b[2]), "r"(b[3]), "r"(b[4]), "r"(b[5]), "r"(b[6]), "r"(b[7]));
+  return w;
+}
+
+// A running product or reduction is kept as two arrays, value = e + 2^32 o:
+// e[2i], e[2i+1] and o[2i], o[2i+1] are the aligned word pairs that wide
+// multiply-adds by the even and the odd limbs of the other factor land on.
+
+// o += a_odd b, e += a_even b (first row: e, o overwritten).
+__device__ __forceinline__ void mul_row0(uint32_t (&e)[8], uint32_t (&o)[8], const uint32_t (&a)[8], uint32_t b) {
+  asm("mul.lo.u32 %0, %8, %12; mul.hi.u32 %1, %8, %12; mul.lo.u32 %2, %9, %12; mul.hi.u32 %3, %9, %12;\n\t"
+      "mul.lo.u32 %4, %10, %12; mul.hi.u32 %5, %10, %12; mul.lo.u32 %6, %11, %12; mul.hi.u32 %7, %11, %12;"
+      : "=&r"(e[0]), "=&r"(e[1]), "=&r"(e[2]), "=&r"(e[3]), "=&r"(e[4]), "=&r"(e[5]), "=&r"(e[6]), "=&r"(e[7])
+      : "r"(a[0]), "r"(a[2]), "r"(a[4]), "r"(a[6]), "r"(b));
+  asm("mul.lo.u32 %0, %8, %12; mul.hi.u32 %1, %8, %12; mul.lo.u32 %2, %9, %12; mul.hi.u32 %3, %9, %12;\n\t"
+      "mul.lo.u32 %4, %10, %12; mul.hi.u32 %5, %10, %12; mul.lo.u32 %6, %11, %12; mul.hi.u32 %7, %11, %12;"
+      : "=&r"(o[0]), "=&r"(o[1]), "=&r"(o[2]), "=&r"(o[3]), "=&r"(o[4]), "=&r"(o[5]), "=&r"(o[6]), "=&r"(o[7])
+      : "r"(a[1]), "r"(a[3]), "r"(a[5]), "r"(a[7]), "r"(b));
+}
+
+// Add m r with m = -e[0] (r = 1 mod 2^32, so n' = -1), which makes e[0] zero.
+// r's lowest limb is 1: its product with m is an addition.
+__device__ __forceinline__ void redc_row(uint32_t (&e)[8], uint32_t (&o)[8]) {
+  const uint32_t m = 0u - e[0];
+  asm("mad.lo.cc.u32 %0, %8, %9, %0; madc.hi.cc.u32 %1, %8, %9, %1; madc.lo.cc.u32 %2, %8, %10, %2;\n\t"
+      "madc.hi.cc.u32 %3, %8, %10, %3; madc.lo.cc.u32 %4, %8, %11, %4; madc.hi.cc.u32 %5, %8, %11, %5;\n\t"
+      "madc.lo.cc.u32 %6, %8, %12, %6; madc.hi.u32 %7, %8, %12, %7;"
+      : "+&r"(o[0]), "+&r"(o[1]), "+&r"(o[2]), "+&r"(o[3]), "+&r"(o[4]), "+&r"(o[5]), "+&r"(o[6]), "+&r"(o[7])
+      : "r"(m), "r"(r_limb(1)), "r"(r_limb(3)), "r"(r_limb(5)), "r"(r_limb(7)));
+  asm("add.cc.u32 %0, %0, %9; addc.cc.u32 %1, %1, 0; madc.lo.cc.u32 %2, %9, %10, %2;\n\t"
+      "madc.hi.cc.u32 %3, %9, %10, %3; madc.lo.cc.u32 %4, %9, %11, %4; madc.hi.cc.u32 %5, %9, %11, %5;\n\t"
+      "madc.lo.cc.u32 %6, %9, %12, %6; madc.hi.cc.u32 %7, %9, %12, %7; addc.u32 %8, %8, 0;"
+      : "+&r"(e[0]), "+&r"(e[1]), "+&r"(e[2]), "+&r"(e[3]), "+&r"(e[4]), "+&r"(e[5]), "+&r"(e[6]), "+&r"(e[7]), "+&r"(o[7])
+      : "r"(m), "r"(r_limb(2)), "r"(r_limb(4)), "r"(r_limb(6)));
+}
+
+// Drop the zero word e[0] (the value moves down by 2^32: o becomes the even
+// array with e[1] added at its bottom, e[2..7] the odd one) and add a b.
+__device__ __forceinline__ void mul_row(uint32_t (&e)[8], uint32_t (&o)[8], const uint32_t (&a)[8], uint32_t b) {
+  uint32_t n[8];
+  asm("add.cc.u32 %8, %8, %9; madc.lo.cc.u32 %0, %16, %20, %10; madc.hi.cc.u32 %1, %16, %20, %11;\n\t"
+      "madc.lo.cc.u32 %2, %17, %20, %12; madc.hi.cc.u32 %3, %17, %20, %13; madc.lo.cc.u32 %4, %18, %20, %14;\n\t"
+      "madc.hi.cc.u32 %5, %18, %20, %15; madc.lo.cc.u32 %6, %19, %20, 0; madc.hi.u32 %7, %19, %20, 0;"
+      : "=&r"(n[0]), "=&r"(n[1]), "=&r"(n[2]), "=&r"(n[3]), "=&r"(n[4]), "=&r"(n[5]), "=&r"(n[6]), "=&r"(n[7]),
+        "+&r"(o[0])
+      : "r"(e[1]), "r"(e[2]), "r"(e[3]), "r"(e[4]), "r"(e[5]), "r"(e[6]), "r"(e[7]), "r"(a[1]), "r"(a[3]), "r"(a[5]),
+        "r"(a[7]), "r"(b));
+  asm("mad.lo.cc.u32 %0, %9, %13, %0; madc.hi.cc.u32 %1, %9, %13, %1; madc.lo.cc.u32 %2, %10, %13, %2;\n\t"
+      "madc.hi.cc.u32 %3, %10, %13, %3; madc.lo.cc.u32 %4, %11, %13, %4; madc.hi.cc.u32 %5, %11, %13, %5;\n\t"
+      "madc.lo.cc.u32 %6, %12, %13, %6; madc.hi.cc.u32 %7, %12, %13, %7; addc.u32 %8, %8, 0;"
+      : "+&r"(o[0]), "+&r"(o[1]), "+&r"(o[2]), "+&r"(o[3]), "+&r"(o[4]), "+&r"(o[5]), "+&r"(o[6]), "+&r"(o[7]), "+&r"(n[7])
+      : "r"(a[0]), "r"(a[2]), "r"(a[4]), "r"(a[6]), "r"(b));
 #pragma unroll
+  for (int j = 0; j < 8; j++) {
+    e[j] = o[j];
+    o[j] = n[j];
+  }
+}
+
+// Drop the zero word e[0] and run the next reduction row: the carry of the
+// drop goes straight into the row's odd chain.
+__device__ __forceinline__ void redc_next(uint32_t (&e)[8], uint32_t (&o)[8]) {
+  uint32_t n[8], m;
+  asm("add.cc.u32 %8, %8, %10; sub.u32 %9, 0, %8; madc.lo.cc.u32 %0, %9, %17, %11;\n\t"
+      "madc.hi.cc.u32 %1, %9, %17, %12; madc.lo.cc.u32 %2, %9, %18, %13; madc.hi.cc.u32 %3, %9, %18, %14;\n\t"
+      "madc.lo.cc.u32 %4, %9, %19, %15; madc.hi.cc.u32 %5, %9, %19, %16; madc.lo.cc.u32 %6, %9, %20, 0;\n\t"
+      "madc.hi.u32 %7, %9, %20, 0;"
+      : "=&r"(n[0]), "=&r"(n[1]), "=&r"(n[2]), "=&r"(n[3]), "=&r"(n[4]), "=&r"(n[5]), "=&r"(n[6]), "=&r"(n[7]),
+        "+&r"(o[0]), "=&r"(m)
+      : "r"(e[1]), "r"(e[2]), "r"(e[3]), "r"(e[4]), "r"(e[5]), "r"(e[6]), "r"(e[7]), "r"(r_limb(1)), "r"(r_limb(3)),
+        "r"(r_limb(5)), "r"(r_limb(7)));
+  asm("add.cc.u32 %0, %0, %9; addc.cc.u32 %1, %1, 0; madc.lo.cc.u32 %2, %9, %10, %2;\n\t"
+      "madc.hi.cc.u32 %3, %9, %10, %3; madc.lo.cc.u32 %4, %9, %11, %4; madc.hi.cc.u32 %5, %9, %11, %5;\n\t"
+      "madc.lo.cc.u32 %6, %9, %12, %6; madc.hi.cc.u32 %7, %9, %12, %7; addc.u32 %8, %8, 0;"
+      : "+&r"(o[0]), "+&r"(o[1]), "+&r"(o[2]), "+&r"(o[3]), "+&r"(o[4]), "+&r"(o[5]), "+&r"(o[6]), "+&r"(o[7]), "+&r"(n[7])
+      : "r"(m), "r"(r_limb(2)), "r"(r_limb(4)), "r"(r_limb(6)));
+#pragma unroll
+  for (int j = 0; j < 8; j++) {
+    e[j] = o[j];
+    o[j] = n[j];
+  }
+}
+
+// o + e / 2^32 for e[0] = 0 (a value below 2^256).
+__device__ __forceinline__ Fr join_rows(const uint32_t (&e)[8], const uint32_t (&o)[8]) {
+  const uint32_t s[8] = {e[1], e[2], e[3], e[4], e[5], e[6], e[7], 0u};
+  Fr x;
+  add8(x.v, o, s);
+  return x;
+}
+
+// (t + m r) / 2^256 for the m that makes it whole, t < 2^256: in [0, r].
+__device__ __forceinline__ Fr redc_low(const uint32_t (&t)[8]) {
+  uint32_t e[8], o[8];
+#pragma unroll
+  for (int j = 0; j < 8; j++) {
+    e[j] = t[j];
+    o[j] = 0;
+  }
+  redc_row(e, o);
+#pragma unroll
+  for (int i = 1; i < 8; i++) redc_next(e, o);
+  return join_rows(e, o);
+}
+#endif
+
+// t - r if t >= r else t  (t < 2^256 given as 8 limbs plus an overflow limb hi).
+VL_HD void cond_sub_r(uint32_t (&t)[8], uint32_t hi) {
+  uint32_t d[8];
+#if defined(__CUDA_ARCH__)
+  const uint32_t r[8] = {r_limb(0), r_limb(1), r_limb(2), r_limb(3), r_limb(4), r_limb(5), r_limb(6), r_limb(7)};
+  const uint32_t borrow = sub8(d, t, r);
+#else
+  uint64_t borrow = 0;
   for (int i = 0; i < 8; i++) {
     uint64_t x = (uint64_t)t[i] - r_limb(i) - borrow;
     d[i] = (uint32_t)x;
     borrow = (x >> 63) & 1;
   }
+#endif
   // t >= r iff no borrow out of the 256-bit subtraction, or hi is set.
   bool take = (hi != 0) || (borrow == 0);
 #pragma unroll
@@ -97,21 +235,31 @@ VL_HD bool lt_r(const Fr& a) {
 
 VL_HD Fr fr_add(const Fr& a, const Fr& b) {
   Fr s;
+#if defined(__CUDA_ARCH__)
+  add8(s.v, a.v, b.v);  // below 2r < 2^256: no carry out
+  cond_sub_r(s.v, 0);
+#else
   uint64_t c = 0;
-#pragma unroll
   for (int i = 0; i < 8; i++) {
     c += (uint64_t)a.v[i] + b.v[i];
     s.v[i] = (uint32_t)c;
     c >>= 32;
   }
   cond_sub_r(s.v, (uint32_t)c);
+#endif
   return s;
 }
 
 VL_HD Fr fr_sub(const Fr& a, const Fr& b) {
   Fr d;
+#if defined(__CUDA_ARCH__)
+  // Add r back when the subtraction wrapped.
+  const uint32_t w = sub8(d.v, a.v, b.v);
+  const uint32_t rw[8] = {r_limb(0) & w, r_limb(1) & w, r_limb(2) & w, r_limb(3) & w,
+                          r_limb(4) & w, r_limb(5) & w, r_limb(6) & w, r_limb(7) & w};
+  add8(d.v, d.v, rw);
+#else
   uint64_t borrow = 0;
-#pragma unroll
   for (int i = 0; i < 8; i++) {
     uint64_t x = (uint64_t)a.v[i] - b.v[i] - borrow;
     d.v[i] = (uint32_t)x;
@@ -120,28 +268,40 @@ VL_HD Fr fr_sub(const Fr& a, const Fr& b) {
   // Add r back when the subtraction wrapped.
   uint32_t mask = borrow ? 0xffffffffu : 0u;
   uint64_t c = 0;
-#pragma unroll
   for (int i = 0; i < 8; i++) {
     c += (uint64_t)d.v[i] + (r_limb(i) & mask);
     d.v[i] = (uint32_t)c;
     c >>= 32;
   }
+#endif
   return d;
 }
 
 VL_HD Fr fr_neg(const Fr& a) { return fr_sub(fr_zero(), a); }
 VL_HD Fr fr_dbl(const Fr& a) { return fr_add(a, a); }
 
-// Montgomery product a.b.R^-1 mod r (CIOS, 32-bit limbs).  Inputs a < 2^256,
-// b < r; the output is reduced (< r).
+// Montgomery product a.b.R^-1 mod r (row by row, one reduction row after each
+// row of products).  Inputs a < 2^256, b < r; the output is reduced (< r).
 VL_HD Fr mont_mul(const Fr& a, const Fr& b) {
+#if defined(__CUDA_ARCH__)
+  // The rows run over a's limbs: a row adds b a_i < r 2^32 and m r < r 2^32 to
+  // a value below 2r, which fits the nine words for any a < 2^256.
+  uint32_t e[8], o[8];
+  mul_row0(e, o, b.v, a.v[0]);
+  redc_row(e, o);
+#pragma unroll
+  for (int i = 1; i < 8; i++) {
+    mul_row(e, o, b.v, a.v[i]);
+    redc_row(e, o);
+  }
+  Fr out = join_rows(e, o);  // below 2r: a b / 2^256 < r, m r / 2^256 < r
+  cond_sub_r(out.v, 0);
+  return out;
+#else
   uint32_t t[10];
-#pragma unroll
   for (int j = 0; j < 10; j++) t[j] = 0;
-#pragma unroll
   for (int i = 0; i < 8; i++) {
     uint64_t c = 0;
-#pragma unroll
     for (int j = 0; j < 8; j++) {
       c += (uint64_t)a.v[j] * b.v[i] + t[j];
       t[j] = (uint32_t)c;
@@ -152,7 +312,6 @@ VL_HD Fr mont_mul(const Fr& a, const Fr& b) {
     t[9] = (uint32_t)(c >> 32);
     uint32_t m = t[0] * NPRIME;
     c = ((uint64_t)m * r_limb(0) + t[0]) >> 32;
-#pragma unroll
     for (int j = 1; j < 8; j++) {
       c += (uint64_t)m * r_limb(j) + t[j];
       t[j - 1] = (uint32_t)c;
@@ -163,22 +322,53 @@ VL_HD Fr mont_mul(const Fr& a, const Fr& b) {
     t[8] = t[9] + (uint32_t)(c >> 32);
   }
   Fr out;
-#pragma unroll
   for (int j = 0; j < 8; j++) out.v[j] = t[j];
   cond_sub_r(out.v, t[8]);
   return out;
+#endif
 }
 
 VL_HD Fr to_mont(const Fr& a) { return mont_mul(a, fr_r2()); }
-VL_HD Fr from_mont(const Fr& a) { return mont_mul(a, fr_small(1)); }
+VL_HD Fr from_mont(const Fr& a) {
+#if defined(__CUDA_ARCH__)
+  Fr x = redc_low(a.v);  // the product by 1: only the reduction rows
+  cond_sub_r(x.v, 0);
+  return x;
+#else
+  return mont_mul(a, fr_small(1));
+#endif
+}
 
 // Montgomery reduction of a wide value V = sum_l acc[l] . 2^(32 l) given as
 // eight unsigned 64-bit column sums: returns V . R^-1 mod r (reduced).
 // V < 2^289, so the REDC result is below 2r before the final subtraction.
 VL_HD Fr redc_columns(const uint64_t acc[8]) {
+#if defined(__CUDA_ARCH__)
+  // t = V's ten limbs: the words of the columns are added on one carry chain.
+  uint32_t w[16], t[8], top[8];
+#pragma unroll
+  for (int l = 0; l < 8; l++) {
+    w[2 * l] = (uint32_t)acc[l];
+    w[2 * l + 1] = (uint32_t)(acc[l] >> 32);
+  }
+  t[0] = w[0];
+  asm("add.cc.u32 %0, %9, %10; addc.cc.u32 %1, %11, %12; addc.cc.u32 %2, %13, %14; addc.cc.u32 %3, %15, %16;\n\t"
+      "addc.cc.u32 %4, %17, %18; addc.cc.u32 %5, %19, %20; addc.cc.u32 %6, %21, %22; addc.cc.u32 %7, %23, 0;\n\t"
+      "addc.u32 %8, 0, 0;"
+      : "=&r"(t[1]), "=&r"(t[2]), "=&r"(t[3]), "=&r"(t[4]), "=&r"(t[5]), "=&r"(t[6]), "=&r"(t[7]), "=&r"(top[0]),
+        "=&r"(top[1])
+      : "r"(w[1]), "r"(w[2]), "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7]), "r"(w[8]), "r"(w[9]), "r"(w[10]),
+        "r"(w[11]), "r"(w[12]), "r"(w[13]), "r"(w[14]), "r"(w[15]));
+#pragma unroll
+  for (int j = 2; j < 8; j++) top[j] = 0;
+  // V / 2^256 = (low 256 bits) / 2^256 (Montgomery, at most r) + the top limbs (below 2^33)
+  Fr out = redc_low(t);
+  add8(out.v, out.v, top);
+  cond_sub_r(out.v, 0);
+  return out;
+#else
   uint32_t t[18];
   uint64_t carry = 0;
-#pragma unroll
   for (int l = 0; l < 8; l++) {
     uint64_t s = (acc[l] & 0xffffffffull) + carry;
     t[l] = (uint32_t)s;
@@ -186,19 +376,15 @@ VL_HD Fr redc_columns(const uint64_t acc[8]) {
   }
   t[8] = (uint32_t)carry;
   t[9] = (uint32_t)(carry >> 32);
-#pragma unroll
   for (int j = 10; j < 18; j++) t[j] = 0;
-#pragma unroll
   for (int i = 0; i < 8; i++) {
     uint32_t m = t[i] * NPRIME;
     uint64_t c = 0;
-#pragma unroll
     for (int j = 0; j < 8; j++) {
       c += (uint64_t)m * r_limb(j) + t[i + j];
       t[i + j] = (uint32_t)c;
       c >>= 32;
     }
-#pragma unroll
     for (int j = i + 8; j < 18; j++) {
       c += t[j];
       t[j] = (uint32_t)c;
@@ -206,10 +392,10 @@ VL_HD Fr redc_columns(const uint64_t acc[8]) {
     }
   }
   Fr out;
-#pragma unroll
   for (int j = 0; j < 8; j++) out.v[j] = t[8 + j];
   cond_sub_r(out.v, t[16]);
   return out;
+#endif
 }
 
 // Reduce a 512-bit little-endian value (lo + hi.2^256) mod r; canonical out.

@@ -16,7 +16,7 @@ static __device__ __noinline__ Fr mont_mul_ni(Fr a, Fr b) { return mont_mul(a, b
 static __device__ __noinline__ Fr redc_columns_ni(U64x8 acc) { return redc_columns(acc.v); }
 
 __device__ __forceinline__ Fr to_mont_ni(const Fr& a) { return mont_mul_ni(a, fr_r2()); }
-__device__ __forceinline__ Fr from_mont_ni(const Fr& a) { return mont_mul_ni(a, fr_small(1)); }
+static __device__ __noinline__ Fr from_mont_ni(Fr a) { return from_mont(a); }  // the reduction rows alone
 
 // (lo + hi . 2^256) mod r, canonical (hi . 2^256 = mont_mul(hi, R^2)).
 __device__ __forceinline__ Fr reduce_512_ni(const Fr& lo, const Fr& hi) {
