@@ -32,7 +32,7 @@
 #include "common.cuh"
 #include "fr_dev.cuh"
 #include "reduce.cuh"
-#include "transcript.cuh"
+#include "transcript_dev.cuh"
 
 struct vl_plan;
 
@@ -66,45 +66,60 @@ struct ChainDev {
   const vl_proof* out1;     // stage-1 proofs of this chain
   const vl_proof* out3;     // stage-3 proofs
   Fr e[4];                  // remainder evaluations (canonical)
-  uint8_t S1[32], S3[32];
+  alignas(4) uint8_t S1[32], S3[32];
 };
 
-__device__ void member_start(uint8_t out[32], const uint8_t S[32], uint32_t p) {
-  Sha256 h;
-  h.init();
-  h.update(S, 32);
-  h.byte('M');
-  h.u32le(p);
-  h.finish(out);
+// Member start SHA256(S || 'M' || p u32le), as the member's 32 state bytes.
+__device__ void member_start(uint8_t* out, const uint32_t* S, uint32_t p) {
+  uint32_t d[8];
+  dev_squeeze_block(S, 'M', p, 2, d);
+  store_digest_bytes(out, d);
 }
 
+constexpr int CH_START_THREADS = 256;
+
 // Transcript start, the stage-1 points, the stage-1 member starts.
-__global__ void chain_start_kernel(ChainDev* chains) {
+__global__ void __launch_bounds__(CH_START_THREADS) chain_start_kernel(ChainDev* chains) {
   ChainDev& C = chains[blockIdx.x];
-  __shared__ uint8_t S0[32];
+  __shared__ uint32_t S0[8], S1[8];
+  __shared__ Fr half[2 * 8 * GIVEN_VARS];
+  __shared__ __align__(16) uint8_t msg[320];
   const int tid = threadIdx.x;
-  if (tid == 0) {
-    const uint8_t dom[25] = {'v', 'e', 'r', 'i', 'l', 'o', 'r', 'a', '-', 'g', 'b', '3', '0',
-                             '0', '/', 'z', 'k', 'c', 'h', 'a', 'i', 'n', '/', 'v', '1'};
-    Sha256 h;
-    h.init();
-    h.update(dom, 25);
-    h.u32le((uint32_t)C.seed);
-    h.u32le((uint32_t)(C.seed >> 32));
+  if (tid < 32) {
+    WarpMsg h(msg);
+    h.bytes("verilora-gb300/zkchain/v1", 25);
+    h.u64le(C.seed);
     h.u32le((uint32_t)C.n);
     h.u32le((uint32_t)C.d);
     h.u32le((uint32_t)C.k);
     h.u32le((uint32_t)C.r);
-    h.update(&C.binds[0][0], 7 * 32);
-    h.finish(S0);
+    h.bytes(&C.binds[0][0], 7 * 32);
+    uint32_t d[8];
+    h.hash(d);
+    store_digest(S0, d);
   }
   __syncthreads();
   // coordinates: u_Y, v_Y, u_dX, v_dX, u_dA, v_dA, u_dB, v_dB
   const int sz[8] = {C.ln, C.lk, C.ln, C.ld, C.ld, C.lr, C.lr, C.lk};
   int total = 0;
   for (int i = 0; i < 8; i++) total += sz[i];
+  // one thread per half of a challenge (REDC(lo . R^2), REDC(hi . R^3): the
+  // challenge in Montgomery form is their sum) and one for the closing update
+  for (int e = tid; e <= 2 * total; e += blockDim.x) {
+    uint32_t d[8];
+    if (e == 2 * total) {
+      dev_squeeze_block(S0, 'p', (uint32_t)total, 2, d);
+#pragma unroll
+      for (int i = 0; i < 8; i++) S1[i] = d[i];
+      store_digest_bytes(C.S1, d);
+    } else {
+      dev_squeeze_block(S0, 'p', (uint32_t)(e >> 1), e & 1, d);
+      half[e] = mont_mul_ni(digest_le(d), (e & 1) ? fr_r3() : fr_r2());
+    }
+  }
+  __syncthreads();
   for (int t = tid; t < total; t += blockDim.x) {
-    const Fr x = to_mont_ni(ts_challenge(S0, 'p', (uint32_t)t));
+    const Fr x = fr_add(half[2 * t], half[2 * t + 1]);
     int sl = 0, o = t;
     while (o >= sz[sl]) o -= sz[sl++];
     // slice -> members: the u or v of the members proved at that point
@@ -119,16 +134,7 @@ __global__ void chain_start_kernel(ChainDev* chains) {
       default: C.g1[5].v[o] = x; break;
     }
   }
-  __syncthreads();
-  if (tid == 0) {
-    uint8_t S[32];
-    memcpy(S, S0, 32);
-    ts_squeeze_done(S, 'p', (uint32_t)total);
-    memcpy(C.S1, S, 32);
-    memcpy(S0, S, 32);
-  }
-  __syncthreads();
-  if (tid < NS1) member_start(C.g1[tid].state, S0, (uint32_t)tid);
+  if (tid < NS1) member_start(C.g1[tid].state, S1, (uint32_t)tid);
 }
 
 // Points of the four claims on H (p1, p2) and dH (q1, q2): x over the row
@@ -175,19 +181,25 @@ __global__ void chain_eval_kernel(ChainDev* chains) {
 // Bind the stage-1 proofs and the evaluations; the stage-3 starts and points.
 __global__ void chain_link_kernel(ChainDev* chains) {
   ChainDev& C = chains[blockIdx.x];
-  __shared__ uint8_t S3[32];
+  __shared__ uint32_t S3[8];
+  __shared__ __align__(16) uint8_t msg[256];
   const int tid = threadIdx.x;
-  if (tid == 0) {
-    uint8_t S[32];
-    Sha256 h;
-    h.init();
-    h.update(C.S1, 32);
-    h.byte('L');
-    for (int p = 0; p < NS1; p++) h.update(C.out1[p].state, 32);
-    h.finish(S);
-    ts_absorb_fr(S, 'e', C.e, 4);
-    memcpy(C.S3, S, 32);
-    memcpy(S3, S, 32);
+  if (tid < 32) {
+    uint32_t d[8];
+    WarpMsg l(msg);
+    l.bytes(C.S1, 32);
+    l.byte('L');
+    for (int p = 0; p < NS1; p++) l.bytes(C.out1[p].state, 32);
+    l.hash(d);
+    store_digest(S3, d);
+    __syncwarp();
+    WarpMsg e(msg);
+    e.state(S3);
+    e.byte('e');
+    e.bytes(C.e, 4 * 32);
+    e.hash(d);
+    store_digest(S3, d);
+    if (tid == 0) store_digest_bytes(C.S3, d);
   }
   __syncthreads();
   if (tid < NS3) member_start(C.g3[tid].state, S3, (uint32_t)(NS1 + tid));
@@ -213,15 +225,17 @@ __global__ void chain_finish_kernel(ChainDev* chains, vl_chain_proof* out) {
     const vl_proof* src = p < NS1 ? C.out1 + p : C.out3 + (p - NS1);
     reinterpret_cast<uint32_t*>(&P.sub[p])[w] = reinterpret_cast<const uint32_t*>(src)[w];
   }
-  if (tid == 0) {
-    uint8_t S[32];
-    Sha256 h;
-    h.init();
-    h.update(C.S3, 32);
+  if (tid < 32) {
+    __shared__ __align__(16) uint8_t msg[192];
+    uint32_t S[8];
+    WarpMsg h(msg);
+    h.bytes(C.S3, 32);
     h.byte('Z');
-    for (int p = 0; p < NS3; p++) h.update(C.out3[p].state, 32);
-    h.finish(S);
-    memcpy(P.state, S, 32);
+    for (int p = 0; p < NS3; p++) h.bytes(C.out3[p].state, 32);
+    h.hash(S);
+    if (tid == 0) store_digest_bytes(P.state, S);
+  }
+  if (tid == 0) {
     P.n = C.n; P.d = C.d; P.k = C.k; P.r = C.r;
     P.reserved = 0;
     int st = VL_OK;
@@ -399,7 +413,7 @@ int chain_run(ChainBatch* B, uint8_t* ws, size_t bytes, vl_chain_proof* out, cud
   plan_set_points(B->s3, giv3, r3);
   cudaError_t ce = cudaMemcpyAsync(dcd, cd.data(), sizeof(ChainDev) * nc, cudaMemcpyHostToDevice, st);
   if (ce == cudaSuccess) {
-    chain_start_kernel<<<nc, 128, 0, st>>>(dcd);
+    chain_start_kernel<<<nc, CH_START_THREADS, 0, st>>>(dcd);
     ce = cudaGetLastError();
   }
   if (ce != cudaSuccess) return cuda_err(ce, "chain_start_kernel");

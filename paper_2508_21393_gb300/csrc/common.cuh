@@ -19,7 +19,7 @@ enum : int32_t { MODE_COLSUM = 0, MODE_ROWDOT = 1 };
 
 // Per-proof mutable state (device, in the workspace).
 struct ProofScratch {
-  uint8_t state[32];  // transcript state after the u, v squeezes (then after each round)
+  alignas(4) uint8_t state[32];  // transcript state after the u, v squeezes (then after each round)
   Fr corrA;           // 2^15 . sum E_u  (Montgomery), int16 offset correction
   Fr corrB;           // 2^15 . sum E_v
   int32_t status;
@@ -79,7 +79,7 @@ struct DevProof {
 // entries), v (d2 entries) in Montgomery form.
 static constexpr int GIVEN_VARS = 16;  // log2 of VL_MAX_REDUCE
 struct GivenPoint {
-  uint8_t state[32];
+  alignas(4) uint8_t state[32];
   Fr u[GIVEN_VARS];
   Fr v[GIVEN_VARS];
 };

@@ -29,7 +29,21 @@ __device__ __forceinline__ Fr bt_level0(const DevProof& P, int side, int w) {
   return P.fdirB ? P.fB[w] : load_acc_fr(P.accB, w, P.scr->corrB);
 }
 
-__device__ __forceinline__ void bt_bytes(uint8_t out[32], const Fr& canonical) { fr_to_le_bytes(canonical, out); }
+// The 32 serialised bytes of a canonical element as big-endian words Y[at..at + 8).
+template <int N>
+__device__ __forceinline__ void bt_words(uint32_t (&Y)[N], int at, const Fr& canonical) {
+#pragma unroll
+  for (int l = 0; l < 8; l++) Y[at + l] = bswap32(canonical.v[l]);
+}
+
+// Tree node `i` (32 bytes, 16-byte aligned) as big-endian words, and back.
+template <int N>
+__device__ __forceinline__ void bt_load_node(const uint8_t* tree, int i, uint32_t (&Y)[N], int at) {
+  const uint4* p = reinterpret_cast<const uint4*>(tree + (size_t)i * 32);
+  const uint4 a = p[0], b = p[1];
+  Y[at] = bswap32(a.x), Y[at + 1] = bswap32(a.y), Y[at + 2] = bswap32(a.z), Y[at + 3] = bswap32(a.w);
+  Y[at + 4] = bswap32(b.x), Y[at + 5] = bswap32(b.y), Y[at + 6] = bswap32(b.z), Y[at + 7] = bswap32(b.w);
+}
 
 // One block per product.
 __global__ void __launch_bounds__(BT_THREADS) bt_claims_kernel(const DevProof* dp, BtState* B) {
@@ -44,14 +58,13 @@ __global__ void __launch_bounds__(BT_THREADS) bt_claims_kernel(const DevProof* d
     B->c[i] = acc[0];
     const Fr c = from_mont_ni(acc[0]);
     for (int l = 0; l < 8; l++) B->c_out[i].limb[l] = c.v[l];
-    uint8_t cb[32];
-    bt_bytes(cb, c);
-    Sha256 h;
-    h.init();
-    h.byte(0);
-    h.update(P.scr->state, 32);
-    h.update(cb, 32);
-    h.finish(B->tree + (size_t)(B->P2 + i) * 32);
+    uint32_t Y[16], node[8];  // leaf: 0x00 || S_i || c_i
+    const uint32_t* st = reinterpret_cast<const uint32_t*>(P.scr->state);
+#pragma unroll
+    for (int l = 0; l < 8; l++) Y[l] = bswap32(st[l]);
+    bt_words(Y, 8, c);
+    dev_hash_tagged<16>(0u, Y, node);
+    store_digest_bytes(B->tree + (size_t)(B->P2 + i) * 32, node);
     if (P.scr->status != VL_OK) atomicExch(&B->status, P.scr->status);
   }
 }
@@ -64,8 +77,13 @@ __device__ void bt_tree(BtState* B) {
     for (int b = 0; b < 32; b++) t[(size_t)(B->P2 + i) * 32 + b] = 0;
   __syncthreads();
   for (int lvl = B->P2 >> 1; lvl >= 1; lvl >>= 1) {
-    for (int j = lvl + threadIdx.x; j < 2 * lvl; j += blockDim.x)
-      merkle_node(t + (size_t)j * 32, t + (size_t)(2 * j) * 32, t + (size_t)(2 * j + 1) * 32);
+    for (int j = lvl + threadIdx.x; j < 2 * lvl; j += blockDim.x) {
+      uint32_t Y[16], node[8];  // 0x01 || left || right
+      bt_load_node(t, 2 * j, Y, 0);
+      bt_load_node(t, 2 * j + 1, Y, 8);
+      dev_hash_tagged<16>(1u, Y, node);
+      store_digest_bytes(t + (size_t)j * 32, node);
+    }
     __syncthreads();
   }
 }
@@ -77,11 +95,16 @@ __global__ void __launch_bounds__(BT_THREADS) bt_start_kernel(BtState* B) {
   __shared__ Fr ch[1];
   __shared__ Fr red[BT_THREADS / 32];
   bt_tree(B);
-  if (threadIdx.x == 0) {
-    uint8_t b[32];
-    ts_start_batch(b, B->seed, (uint32_t)B->K, B->tree + 32);
-    for (int i = 0; i < 8; i++)
-      S0[i] = ((uint32_t)b[4 * i] << 24) | ((uint32_t)b[4 * i + 1] << 16) | ((uint32_t)b[4 * i + 2] << 8) | b[4 * i + 3];
+  if (threadIdx.x < 32) {
+    __shared__ __align__(16) uint8_t msg[128];
+    WarpMsg h(msg);  // the message of ts_start_batch
+    h.bytes("verilora-gb300/zkbatch/v1", 25);
+    h.u64le(B->seed);
+    h.u32le((uint32_t)B->K);
+    h.bytes(B->tree + 32, 32);
+    uint32_t d[8];
+    h.hash(d);
+    store_digest(S0, d);
   }
   __syncthreads();
   squeeze_dev(S0, LBL_P, 1, ch, S1, dig);
@@ -212,35 +235,26 @@ __global__ void __launch_bounds__(32) bt_final_kernel(const DevProof* dp, BtStat
     B->a_out[i].limb[l] = ac.v[l];
     B->b_out[i].limb[l] = bc.v[l];
   }
-  uint8_t ab[32], bb[32];
-  bt_bytes(ab, ac);
-  bt_bytes(bb, bc);
-  Sha256 h;
-  h.init();
-  h.byte(0);
-  h.u32le((uint32_t)i);
-  h.update(ab, 32);
-  h.update(bb, 32);
-  h.finish(B->tree + (size_t)(B->P2 + i) * 32);
+  uint32_t Y[17], node[8];  // leaf: 0x00 || i u32le || a_i || b_i
+  Y[0] = bswap32((uint32_t)i);
+  bt_words(Y, 1, ac);
+  bt_words(Y, 9, bc);
+  dev_hash_tagged<17>(0u, Y, node);
+  store_digest_bytes(B->tree + (size_t)(B->P2 + i) * 32, node);
 }
 
 // One block: the root of the final values, absorb 'f', the proof.
 __global__ void __launch_bounds__(BT_THREADS) bt_close_kernel(BtState* B, int k) {
   bt_tree(B);
-  if (threadIdx.x != 0) return;
-  uint8_t S[32];
-  for (int i = 0; i < 32; i++) S[i] = (uint8_t)(B->St[i >> 2] >> (24 - 8 * (i & 3)));
-  Sha256 h;
-  h.init();
-  h.update(S, 32);
-  h.byte(LBL_F);
-  h.update(B->tree + 32, 32);
-  h.finish(S);
   vl_batch_proof* out = B->out;
-  for (int i = 0; i < 32; i++) out->state[i] = S[i];
-  for (int t = B->d1; t < VL_MAX_ROUNDS; t++)
-    for (int q = 0; q < 3; q++)
-      for (int l = 0; l < 8; l++) out->g[t][q].limb[l] = 0u;
+  for (int i = threadIdx.x; i < (VL_MAX_ROUNDS - B->d1) * 24; i += blockDim.x)
+    out->g[B->d1 + i / 24][(i / 8) % 3].limb[i & 7] = 0u;
+  if (threadIdx.x != 0) return;
+  uint32_t S[8], Y[8];
+  for (int i = 0; i < 8; i++) S[i] = B->St[i];
+  bt_load_node(B->tree, 1, Y, 0);
+  dev_absorb_words<8>(S, LBL_F, Y);
+  store_digest_bytes(out->state, S);
   out->K = B->K;
   out->k = k;
   out->d1 = B->d1;

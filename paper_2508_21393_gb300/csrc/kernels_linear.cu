@@ -24,23 +24,6 @@ namespace {
 
 constexpr uint8_t LBL_X = 'x', LBL_Y = 'y', LBL_E = 'e';
 constexpr int LIN_THREADS = 256;
-constexpr int LIN_FAC_THREADS = LIN_THREADS - 32;  // the last warp computes the correction
-
-// Factor entry j of one side (lo entries first): a product of eq factors,
-// starting from 1 in double-Montgomery (lo of the reduced side) or
-// Montgomery form (everything else).
-__device__ Fr lin_factor(const Fr* x, int d, int j, bool lo_double, bool* is_lo, int* idx) {
-  const int s = (d + 1) >> 1, dh = d - s, nlo = 1 << s;
-  *is_lo = j < nlo;
-  const int jj = *is_lo ? j : j - nlo, nv = *is_lo ? s : dh, base = *is_lo ? dh : 0;
-  *idx = jj;
-  Fr acc = (*is_lo && lo_double) ? fr_r2() : fr_r1();
-  for (int t = 0; t < nv; t++) {
-    const Fr& xt = x[base + t];
-    acc = mont_mul_ni(acc, ((jj >> (nv - 1 - t)) & 1) ? xt : fr_sub(fr_r1(), xt));
-  }
-  return acc;
-}
 
 // One block per proof.
 __global__ void __launch_bounds__(LIN_THREADS) lin_start_kernel(LinDev* Ls) {
@@ -48,34 +31,34 @@ __global__ void __launch_bounds__(LIN_THREADS) lin_start_kernel(LinDev* Ls) {
   __shared__ uint32_t S0[8], S1[8], S2[8];
   __shared__ uint32_t dig[2 * MAX_VARS + 1][8];
   __shared__ Fr xs[MAX_VARS], ys[MAX_VARS];
+  __shared__ __align__(16) Fr sub[128];  // factor tables; before them the statement's message (at most 17 blocks)
+  static_assert(sizeof(sub) >= 64 * ((23 + 20 + 64 * VL_LIN_MAX + 9 + 63) / 64), "message buffer");
   const int tid = threadIdx.x;
-  if (tid == 0) {
-    uint8_t b[32];
-    ts_start_linear(b, L->seed, (uint32_t)L->rows, (uint32_t)L->cols, L->nmats, L->coeffs, L->binds);
-    for (int i = 0; i < 8; i++)
-      S0[i] = ((uint32_t)b[4 * i] << 24) | ((uint32_t)b[4 * i + 1] << 16) | ((uint32_t)b[4 * i + 2] << 8) | b[4 * i + 3];
+  if (tid < 32) {
+    WarpMsg h(sub);  // the message of ts_start_linear
+    h.bytes("verilora-gb300/zklin/v1", 23);
+    h.u64le(L->seed);
+    h.u32le((uint32_t)L->rows);
+    h.u32le((uint32_t)L->cols);
+    h.u32le((uint32_t)L->nmats);
+    h.bytes(L->coeffs, 32 * L->nmats);
+    h.bytes(L->binds, 32 * L->nmats);
+    uint32_t d[8];
+    h.hash(d);
+    store_digest(S0, d);
   }
   __syncthreads();
   squeeze_dev(S0, LBL_X, L->d0, xs, S1, dig);
   squeeze_dev(S1, LBL_Y, L->d1, ys, S2, dig);
   if (tid < 8) L->S[tid] = S2[tid];
   const bool rr = L->red_rows != 0;
-  if (tid < LIN_FAC_THREADS) {
-    // Both sides' factor tables in one loop: [x lo | x hi | y lo | y hi].
-    const int sx = (L->d0 + 1) >> 1, sy = (L->d1 + 1) >> 1;
-    const int nx = (1 << sx) + ((L->rows + (1 << sx) - 1) >> sx);
-    const int ny = (1 << sy) + ((L->cols + (1 << sy) - 1) >> sy);
-    for (int j = tid; j < nx + ny; j += LIN_FAC_THREADS) {
-      const bool xside = j < nx;
-      bool is_lo;
-      int idx;
-      const Fr v = xside ? lin_factor(xs, L->d0, j, rr, &is_lo, &idx) : lin_factor(ys, L->d1, j - nx, !rr, &is_lo, &idx);
-      L->fac[(xside ? 0 : 2 * EQ_FAC) + (is_lo ? 0 : EQ_FAC) + idx] = v;
-    }
-  } else if (tid == LIN_FAC_THREADS) {
+  eq_factors(xs, L->d0, L->rows, rr, ys, L->d1, L->cols, !rr, L->fac, sub);
+  if (tid < 32) {
     const Fr sum = rr ? eq_prefix_sum(xs, L->d0, L->rows) : eq_prefix_sum(ys, L->d1, L->cols);
-    L->corr = mont_mul_ni(sum, to_mont_ni(fr_small(1u << 15)));
-    L->scr->status = VL_OK;
+    if (tid == 0) {
+      L->corr = mont_mul_ni(sum, to_mont_ni(fr_small(1u << 15)));
+      L->scr->status = VL_OK;
+    }
   }
 }
 
@@ -221,6 +204,7 @@ __global__ void __launch_bounds__(LIN_THREADS) lin_dot_kernel(LinDev* Ls) {
 __global__ void __launch_bounds__(LIN_THREADS) lin_finish_kernel(const LinDev* Ls, vl_lin_proof* outs) {
   __shared__ Fr red[LIN_THREADS / 32];
   __shared__ Fr ev[VL_LIN_MAX];
+  __shared__ __align__(16) uint8_t msg[64 * ((33 + 32 * VL_LIN_MAX + 9 + 63) / 64)];
   const LinDev* L = Ls + blockIdx.x;
   vl_lin_proof* out = outs + blockIdx.x;
   const int tid = threadIdx.x, nm = L->nmats;
@@ -233,17 +217,22 @@ __global__ void __launch_bounds__(LIN_THREADS) lin_finish_kernel(const LinDev* L
     if (tid == 0) ev[q] = from_mont_ni(acc[0]);
   }
   __syncthreads();
-  if (tid == 0) {
-    uint8_t S[32];
-    for (int i = 0; i < 32; i++) S[i] = (uint8_t)(L->S[i >> 2] >> (24 - 8 * (i & 3)));
-    ts_absorb_fr(S, LBL_E, ev, nm);
-    out->rows = L->rows;
-    out->cols = L->cols;
-    out->d0 = L->d0;
-    out->d1 = L->d1;
-    out->nmats = nm;
-    out->status = L->scr->status;
-    for (int i = 0; i < 32; i++) out->state[i] = S[i];
+  if (tid < 32) {
+    WarpMsg h(msg);  // absorb 'e'
+    h.state(L->S);
+    h.byte(LBL_E);
+    h.bytes(ev, 32 * nm);
+    uint32_t S[8];
+    h.hash(S);
+    if (tid == 0) {
+      out->rows = L->rows;
+      out->cols = L->cols;
+      out->d0 = L->d0;
+      out->d1 = L->d1;
+      out->nmats = nm;
+      out->status = L->scr->status;
+      store_digest_bytes(out->state, S);
+    }
   }
   for (int i = tid; i < VL_LIN_MAX * 8; i += blockDim.x)
     out->evals[i >> 3].limb[i & 7] = (i >> 3) < nm ? ev[i >> 3].v[i & 7] : 0u;

@@ -37,15 +37,22 @@ namespace {
 __global__ void __launch_bounds__(LK_THREADS) lk_start_kernel(LkDev* Ls) {
   LkDev* L = Ls + blockIdx.x;
   __shared__ uint32_t S0[8], S1[8], S2[8], S3[8];
-  __shared__ uint32_t dig[2 * LK_MAX_L + 1][8];
+  __shared__ __align__(16) uint32_t dig[2 * LK_MAX_L + 1][8];
   __shared__ Fr ch[LK_MAX_L];
   __shared__ Fr beta_sh, alpha_sh;
   const int tid = threadIdx.x;
-  if (tid == 0) {
-    uint8_t b[32];
-    ts_start_lookup(b, L->seed, (uint32_t)L->n, (uint32_t)L->L, (uint32_t)L->log2_n, L->t0, L->bind);
-    for (int i = 0; i < 8; i++)
-      S0[i] = ((uint32_t)b[4 * i] << 24) | ((uint32_t)b[4 * i + 1] << 16) | ((uint32_t)b[4 * i + 2] << 8) | b[4 * i + 3];
+  if (tid < 32) {
+    WarpMsg h(dig);  // the message of ts_start_lookup
+    h.bytes("verilora-gb300/zklookup/v1", 26);
+    h.u64le(L->seed);
+    h.u32le((uint32_t)L->n);
+    h.u32le((uint32_t)L->L);
+    h.u32le((uint32_t)L->log2_n);
+    h.u64le((uint64_t)L->t0);
+    h.bytes(L->bind, 32);
+    uint32_t d[8];
+    h.hash(d);
+    store_digest(S0, d);
   }
   __syncthreads();
   squeeze_dev(S0, LBL_BETA, 1, ch, S1, dig);

@@ -140,8 +140,9 @@ __device__ static void squeeze_dev(const uint32_t* Sw, uint32_t label, int count
 // Transcript start and the squeezes of u, v into shared memory, or, for a
 // proof with a given point, the given start state and point; the state after
 // them goes to P.scr->state.  Block-wide.
+// msg: 192 bytes of scratch.
 __device__ static void start_or_given(const DevProof& P, uint32_t* S0, uint32_t* S1, uint32_t* S2,
-                                      uint32_t (*dig)[8], Fr* u, Fr* v) {
+                                      uint32_t (*dig)[8], Fr* u, Fr* v, void* msg) {
   const int tid = threadIdx.x;
   if (P.given) {
     for (int i = tid; i < P.d0 + P.d2; i += blockDim.x) {
@@ -152,14 +153,25 @@ __device__ static void start_or_given(const DevProof& P, uint32_t* S0, uint32_t*
     __syncthreads();
     return;
   }
-  if (tid == 0) {
-    uint8_t b[32];
-    if (P.member1 > 0)
-      ts_start_member(b, P.seed, (uint32_t)P.nmembers, (uint32_t)(P.member1 - 1), P.m, P.k, P.n, P.tp, P.tq, P.binds);
-    else
-      ts_start(b, P.seed, P.m, P.k, P.n, P.tp, P.tq, P.binds);
-    for (int i = 0; i < 8; i++)
-      S0[i] = ((uint32_t)b[4 * i] << 24) | ((uint32_t)b[4 * i + 1] << 16) | ((uint32_t)b[4 * i + 2] << 8) | b[4 * i + 3];
+  if (tid < 32) {
+    // the message of ts_start (a product of a batch: of ts_start_member)
+    WarpMsg h(msg);
+    if (P.member1 > 0) h.bytes("verilora-gb300/zkbatch/v1/member", 32);
+    else h.bytes("verilora-gb300/zkmat/v1", 23);
+    h.u64le(P.seed);
+    if (P.member1 > 0) {
+      h.u32le((uint32_t)P.nmembers);
+      h.u32le((uint32_t)(P.member1 - 1));
+    }
+    h.u32le((uint32_t)P.m);
+    h.u32le((uint32_t)P.k);
+    h.u32le((uint32_t)P.n);
+    h.byte((uint32_t)(P.tp & 1));
+    h.byte((uint32_t)(P.tq & 1));
+    h.bytes(P.binds, 96);
+    uint32_t d[8];
+    h.hash(d);
+    store_digest(S0, d);
   }
   __syncthreads();
   squeeze_dev(S0, LBL_U, P.d0, u, S1, dig);
@@ -184,7 +196,7 @@ static __device__ void prologue_block(const DevProof& P, uint8_t* smem) {
   Fr* red = hi + MAX_HALF;
   const int tid = threadIdx.x;
 
-  start_or_given(P, S0, S1, S2, dig, u, v);
+  start_or_given(P, S0, S1, S2, dig, u, v, v + MAX_VARS);
 
   Fr ca = build_eq(u, P.d0, P.m, P.tabA, P.eqA, P.eqA_soa, P.soa_pitchA, P.w8A, lo, hi, red);
   __syncthreads();
@@ -197,22 +209,50 @@ static __device__ void prologue_block(const DevProof& P, uint8_t* smem) {
   __syncthreads();
 }
 
-// Factor tables of one side into global memory: lo[j] (2^s entries,
-// double-Montgomery) and hi[j] (ceil(size / 2^s) entries, Montgomery), with
-// E[i] = hi[i >> s] . lo[i mod 2^s] and s = ceil(d / 2).  Block-wide.
-__device__ static void eq_factors(const Fr* x, int d, int size, Fr* lo, Fr* hi) {
+// Factor tables of the eq tables of two sides x (dx variables) and y (dy),
+// block-wide: side q's table is E[i] = hi[i >> s] . lo[i mod 2^s] with s =
+// ceil(d / 2), lo over the last s variables (2^s entries), hi over the others
+// (ceil(size / 2^s) entries); all in Montgomery form but lo of a side with
+// `dbl` set, which is in double-Montgomery form.  Written to fac + 2 q EQ_FAC
+// (lo) and EQ_FAC further (hi).  Each block of at most 8 variables is split
+// once more into two of at most 4: 8 small tables of at most 16 entries, one
+// entry per thread (four products on a thread's chain), then one product per
+// factor entry, instead of one chain of up to eight products per entry.
+// sub: 128 entries of shared memory.
+__device__ static void eq_factors(const Fr* x, int dx, int sizex, bool dblx, const Fr* y, int dy, int sizey, bool dbly,
+                                  Fr* fac, Fr* sub) {
   const int tid = threadIdx.x;
-  const int s = (d + 1) >> 1, dh = d - s;
-  const int nlo = 1 << s, nhi = (size + nlo - 1) >> s;
-  for (int j = tid; j < nlo + nhi; j += blockDim.x) {
-    const bool is_lo = j < nlo;
-    const int jj = is_lo ? j : j - nlo, nv = is_lo ? s : dh, base = is_lo ? dh : 0;
-    Fr acc = is_lo ? fr_r2() : fr_r1();
-    for (int t = 0; t < nv; t++) {
-      const Fr& xt = x[base + t];
-      acc = mont_mul_ni(acc, ((jj >> (nv - 1 - t)) & 1) ? xt : fr_sub(fr_r1(), xt));
+  for (int e = tid; e < 128; e += blockDim.x) {
+    const int q = e >> 4, j = e & 15;  // q: side, hi block, low half
+    const bool second = q & 4;
+    const int d = second ? dy : dx, s = (d + 1) >> 1;
+    const int nv = (q & 2) ? d - s : s, base = (q & 2) ? 0 : d - s;
+    const int nl = nv >> 1, n = (q & 1) ? nl : nv - nl, v0 = base + ((q & 1) ? nv - nl : 0);
+    if (j < (1 << n)) {
+      const Fr* z = second ? y : x;
+      Fr acc = fr_r1();
+      for (int t = 0; t < n; t++) {
+        const Fr& xt = z[v0 + t];
+        const Fr f = ((j >> (n - 1 - t)) & 1) ? xt : fr_sub(fr_r1(), xt);
+        acc = t == 0 ? f : mont_mul_ni(acc, f);
+      }
+      // double-Montgomery: one factor of R more, on the low block's high half
+      if ((q & 3) == 0 && (second ? dbly : dblx)) acc = to_mont_ni(acc);
+      sub[e] = acc;
     }
-    (is_lo ? lo : hi)[jj] = acc;
+  }
+  __syncthreads();
+  const int sx = (dx + 1) >> 1, sy = (dy + 1) >> 1;
+  const int lx = 1 << sx, hx = (sizex + lx - 1) >> sx, ly = 1 << sy, hy = (sizey + ly - 1) >> sy;
+  for (int e = tid; e < lx + hx + ly + hy; e += blockDim.x) {
+    const bool second = e >= lx + hx;
+    const int e2 = second ? e - (lx + hx) : e, nlo = second ? ly : lx;
+    const bool hi = e2 >= nlo;
+    const int j = hi ? e2 - nlo : e2, d = second ? dy : dx, s = second ? sy : sx;
+    const int nl = (hi ? d - s : s) >> 1;
+    const Fr* tab = sub + 64 * second + 32 * hi;
+    fac[(second ? 2 * EQ_FAC : 0) + (hi ? EQ_FAC : 0) + j] =
+        nl ? mont_mul_ni(tab[j >> nl], tab[16 + (j & ((1 << nl) - 1))]) : tab[j];
   }
 }
 
@@ -220,17 +260,28 @@ __device__ static void eq_factors(const Fr* x, int d, int size, Fr* lo, Fr* hi) 
 // exactly when, at the first bit (from the top) where i and size differ, i
 // has 0 and size has 1; the bits below are free and their eq factors sum to
 // 1.  So the sum runs over the 1-bits t of size: prod of the factors of size's
-// bits above t, times (1 - x_t).  O(d) products, one thread.
+// bits above t, times (1 - x_t).  By one warp: lane t holds variable t, the
+// products above it by a scan (five products deep instead of 2 d); every lane
+// returns the sum.
 __device__ static Fr eq_prefix_sum(const Fr* x, int d, int size) {
   if (size >= (1 << d)) return fr_r1();  // the whole cube: sum 1
-  Fr sum = fr_zero(), pre = fr_r1();
-  for (int t = 0; t < d; t++) {
-    const int b = (size >> (d - 1 - t)) & 1;
-    const Fr one_minus = fr_sub(fr_r1(), x[t]);
-    if (b) sum = fr_add(sum, mont_mul_ni(pre, one_minus));
-    pre = mont_mul_ni(pre, b ? x[t] : one_minus);
+  const int lane = threadIdx.x & 31;
+  const bool in = lane < d, one = in && ((size >> (d - 1 - lane)) & 1);
+  const Fr xt = in ? x[lane] : fr_zero(), om = fr_sub(fr_r1(), xt);
+  Fr pre = in ? (one ? xt : om) : fr_r1();
+  for (int off = 1; off < d; off <<= 1) {  // inclusive products
+    Fr up;
+#pragma unroll
+    for (int l = 0; l < 8; l++) up.v[l] = __shfl_up_sync(0xffffffffu, pre.v[l], off);
+    const Fr p = mont_mul_ni(pre, up);
+    if (lane >= off) pre = p;
   }
-  return sum;
+  Fr above;
+#pragma unroll
+  for (int l = 0; l < 8; l++) above.v[l] = __shfl_up_sync(0xffffffffu, pre.v[l], 1);
+  if (lane == 0) above = fr_r1();
+  const Fr term = mont_mul_ni(above, om);
+  return warp_sum_fr(one ? term : fr_zero());
 }
 
 // First launch of the prologue, one proof per block (any multiple of 32
@@ -245,16 +296,17 @@ static __device__ void transcript_block(const DevProof& P, uint8_t* smem) {
   Fr* u = reinterpret_cast<Fr*>(smem + 128 + 2 * MAX_VARS * 32);
   Fr* v = u + MAX_VARS;
   const int tid = threadIdx.x;
-  start_or_given(P, S0, S1, S2, dig, u, v);
-  eq_factors(u, P.d0, P.m, P.fac, P.fac + EQ_FAC);
-  eq_factors(v, P.d2, P.n, P.fac + 2 * EQ_FAC, P.fac + 3 * EQ_FAC);
-  if (tid == 0 || tid == 32) {
-    const bool a = tid == 0;
+  start_or_given(P, S0, S1, S2, dig, u, v, v + MAX_VARS);
+  eq_factors(u, P.d0, P.m, true, v, P.d2, P.n, true, P.fac, v + MAX_VARS);
+  if (tid < 64) {
+    const bool a = tid < 32;
     const Fr sum = a ? eq_prefix_sum(u, P.d0, P.m) : eq_prefix_sum(v, P.d2, P.n);
-    // sum . R times 2^15 . R, reduced once: 2^15 . sum (Montgomery)
-    const Fr corr = mont_mul_ni(sum, to_mont_ni(fr_small(1u << 15)));
-    const bool i16 = (a ? P.dtypeA : P.dtypeB) == VL_I16;
-    (a ? P.scr->corrA : P.scr->corrB) = i16 ? corr : fr_zero();
+    if ((tid & 31) == 0) {
+      // sum . R times 2^15 . R, reduced once: 2^15 . sum (Montgomery)
+      const Fr corr = mont_mul_ni(sum, to_mont_ni(fr_small(1u << 15)));
+      const bool i16 = (a ? P.dtypeA : P.dtypeB) == VL_I16;
+      (a ? P.scr->corrA : P.scr->corrB) = i16 ? corr : fr_zero();
+    }
   }
   if (tid == 0) P.scr->status = VL_OK;
   __syncthreads();

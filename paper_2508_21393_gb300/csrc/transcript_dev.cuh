@@ -141,4 +141,122 @@ __device__ __forceinline__ Fr digest_le(const uint32_t d[8]) {
   return x;
 }
 
+// SHA256(tag byte || Y_0 || ... || Y_{N-1}) for big-endian words Y, one thread.
+template <int N>
+__device__ __forceinline__ void dev_hash_tagged(uint32_t tag, const uint32_t (&Y)[N], uint32_t (&out)[8]) {
+  constexpr int LEN = 1 + 4 * N;
+  constexpr int NB = (LEN + 9 + 63) / 64;
+  sha256_iv(out);
+#pragma unroll
+  for (int b = 0; b < NB; b++) {
+    uint32_t m[16];
+#pragma unroll
+    for (int i = 0; i < 16; i++) {
+      const int gi = 16 * b + i;
+      uint32_t w = 0;
+      if (gi < N) w = __funnelshift_r(Y[gi < N ? gi : 0], gi == 0 ? tag : Y[gi > 0 && gi < N ? gi - 1 : 0], 8);
+      else if (gi == N) w = (Y[N - 1] << 24) | 0x00800000u;
+      if (gi == 16 * NB - 1) w = (uint32_t)LEN * 8u;
+      m[i] = w;
+    }
+    sha256_block(out, m);
+  }
+}
+
+// S <- SHA256(S || label || Y_0 || ... || Y_{N-1}) for big-endian words Y, one thread.
+template <int N>
+__device__ __forceinline__ void dev_absorb_words(uint32_t (&S)[8], uint32_t label, const uint32_t (&Y)[N]) {
+  constexpr int LEN = 33 + 4 * N;
+  constexpr int NB = (LEN + 9 + 63) / 64;
+  uint32_t st[8];
+  sha256_iv(st);
+#pragma unroll
+  for (int b = 0; b < NB; b++) {
+    uint32_t m[16];
+#pragma unroll
+    for (int i = 0; i < 16; i++) {
+      const int gi = 16 * b + i, q = gi - 8;
+      uint32_t w = 0;
+      if (gi < 8) w = S[gi < 8 ? gi : 0];
+      else if (q < N) w = __funnelshift_r(Y[q >= 0 && q < N ? q : 0], q == 0 ? label : Y[q > 0 && q < N ? q - 1 : 0], 8);
+      else if (q == N) w = (Y[N - 1] << 24) | 0x00800000u;
+      if (gi == 16 * NB - 1) w = (uint32_t)LEN * 8u;
+      m[i] = w;
+    }
+    sha256_block(st, m);
+  }
+#pragma unroll
+  for (int i = 0; i < 8; i++) S[i] = st[i];
+}
+
+__device__ __forceinline__ uint32_t bswap32(uint32_t x) { return __byte_perm(x, 0, 0x0123); }
+
+// A message whose layout is known only at run time (transcript starts, long
+// absorbs): the lanes of one warp write its bytes to shared memory, then
+// every lane runs the compressions on the same words (one warp instruction
+// either way), so the digest ends in every lane's registers.  One thread feeding
+// a byte-wise hash with its buffer in local memory took several times as long:
+// with both sides' eq factors formed from small tables, a lone 64 x 128 x 64
+// proof went from 278 to 256 us, the 256 update proofs of a 7B step from 382 to
+// 303 us and four chained 7B projections from 1014 to 787 us.
+// `buf`: 16-byte aligned shared memory of at least 64 ceil((bytes + 9) / 64).
+struct WarpMsg {
+  uint8_t* buf;
+  int len;
+  __device__ explicit WarpMsg(void* shared) : buf(static_cast<uint8_t*>(shared)), len(0) {}
+  __device__ void bytes(const void* src, int n) {
+    for (int i = threadIdx.x & 31; i < n; i += 32) buf[len + i] = static_cast<const uint8_t*>(src)[i];
+    len += n;
+  }
+  __device__ void byte(uint32_t x) {
+    if ((threadIdx.x & 31) == 0) buf[len] = (uint8_t)x;
+    len += 1;
+  }
+  __device__ void u32le(uint32_t x) {
+    const int lane = threadIdx.x & 31;
+    if (lane < 4) buf[len + lane] = (uint8_t)(x >> (8 * lane));
+    len += 4;
+  }
+  __device__ void u64le(uint64_t x) {
+    u32le((uint32_t)x);
+    u32le((uint32_t)(x >> 32));
+  }
+  // a transcript state (eight big-endian words, in memory)
+  __device__ void state(const uint32_t* S) {
+    const int lane = threadIdx.x & 31;
+    buf[len + lane] = (uint8_t)(S[lane >> 2] >> (24 - 8 * (lane & 3)));
+    len += 32;
+  }
+  // The digest (big-endian words); the buffer may be reused afterwards.
+  __device__ void hash(uint32_t (&out)[8]) {
+    const int end = (len + 9 + 63) / 64 * 64;
+    for (int i = len + (int)(threadIdx.x & 31); i < end; i += 32)
+      buf[i] = i == len ? 0x80 : i >= end - 4 ? (uint8_t)((uint32_t)(len * 8) >> (8 * (end - 1 - i))) : 0;
+    __syncwarp();
+    sha256_iv(out);
+    for (int b = 0; b < end; b += 64) {
+      uint32_t m[16];
+#pragma unroll
+      for (int q = 0; q < 4; q++) {
+        const uint4 v = reinterpret_cast<const uint4*>(buf + b)[q];
+        m[4 * q] = bswap32(v.x), m[4 * q + 1] = bswap32(v.y), m[4 * q + 2] = bswap32(v.z), m[4 * q + 3] = bswap32(v.w);
+      }
+      sha256_block(out, m);
+    }
+    __syncwarp();
+  }
+};
+// Lane 0 stores a digest that every lane holds.
+__device__ __forceinline__ void store_digest(uint32_t* dst, const uint32_t (&d)[8]) {
+  if ((threadIdx.x & 31) == 0) {
+#pragma unroll
+    for (int i = 0; i < 8; i++) dst[i] = d[i];
+  }
+}
+// The same as 32 bytes (16-byte aligned).
+__device__ __forceinline__ void store_digest_bytes(uint8_t* dst, const uint32_t (&d)[8]) {
+#pragma unroll
+  for (int i = 0; i < 8; i++) reinterpret_cast<uint32_t*>(dst)[i] = bswap32(d[i]);
+}
+
 }  // namespace vl
