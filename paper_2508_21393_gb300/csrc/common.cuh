@@ -25,6 +25,7 @@ struct ProofScratch {
   int32_t status;
   int32_t pad[7];
   Fr r;               // batched rounds: the latest challenge (Montgomery)
+  Fr claim;           // batched rounds: the running claim (canonical)
 };
 
 // Batched rounds (one launch per round over all proofs): the pairs of one
@@ -108,7 +109,7 @@ struct StepItem {
 };
 // Dynamic shared memory of the prologue and rounds block functions.
 static constexpr int PRO_SMEM = 18816;
-static constexpr int RND_SMEM = 1792;
+static constexpr int RND_SMEM = 20736;
 // Prologue items run this many proofs ahead of their fold tiles in the queue.
 static constexpr int STEP_LOOKAHEAD = 256;
 

@@ -23,7 +23,8 @@
 
 namespace vl {
 
-struct Fr {
+// 16-byte aligned: elements move as two 16-byte loads or stores.
+struct alignas(16) Fr {
   uint32_t v[8];
 };
 
@@ -69,7 +70,7 @@ VL_HD bool fr_eq(const Fr& a, const Fr& b) {
   return o == 0;
 }
 
-#if defined(__CUDA_ARCH__)
+#if defined(__CUDACC__)
 // Device arithmetic on carry chains (PTX add.cc / mad.cc).  The C forms below
 // (64-bit temporaries, used on the host) spend about three ALU instructions
 // per limb on carries; with the flag kept in the condition code a limb costs
@@ -188,6 +189,39 @@ __device__ __forceinline__ Fr join_rows(const uint32_t (&e)[8], const uint32_t (
   return x;
 }
 
+// w += a b for a 17-limb accumulator (512-bit products, unreduced; up to 2^34
+// of them): half a Montgomery product's multiply-adds.  A sum of products
+// is reduced once at its end (wide_redc).
+__device__ __forceinline__ void wide_mac(uint32_t (&w)[17], const Fr& a, const Fr& b) {
+  uint32_t e[8], o[8];
+  asm("mul.lo.u32 %0, %8, %12; mul.hi.u32 %1, %8, %12; mul.lo.u32 %2, %9, %12; mul.hi.u32 %3, %9, %12;\n\t"
+      "mul.lo.u32 %4, %10, %12; mul.hi.u32 %5, %10, %12; mul.lo.u32 %6, %11, %12; mul.hi.u32 %7, %11, %12;"
+      : "=&r"(o[0]), "=&r"(o[1]), "=&r"(o[2]), "=&r"(o[3]), "=&r"(o[4]), "=&r"(o[5]), "=&r"(o[6]), "=&r"(o[7])
+      : "r"(a.v[1]), "r"(a.v[3]), "r"(a.v[5]), "r"(a.v[7]), "r"(b.v[0]));
+#pragma unroll
+  for (int j = 0; j < 8; j++) e[j] = w[j];
+  asm("mad.lo.cc.u32 %0, %9, %13, %0; madc.hi.cc.u32 %1, %9, %13, %1; madc.lo.cc.u32 %2, %10, %13, %2;\n\t"
+      "madc.hi.cc.u32 %3, %10, %13, %3; madc.lo.cc.u32 %4, %11, %13, %4; madc.hi.cc.u32 %5, %11, %13, %5;\n\t"
+      "madc.lo.cc.u32 %6, %12, %13, %6; madc.hi.cc.u32 %7, %12, %13, %7; addc.u32 %8, %8, 0;"
+      : "+&r"(e[0]), "+&r"(e[1]), "+&r"(e[2]), "+&r"(e[3]), "+&r"(e[4]), "+&r"(e[5]), "+&r"(e[6]), "+&r"(e[7]),
+        "+&r"(o[7])
+      : "r"(a.v[0]), "r"(a.v[2]), "r"(a.v[4]), "r"(a.v[6]), "r"(b.v[0]));
+  w[0] = e[0];
+#pragma unroll
+  for (int i = 1; i < 8; i++) {
+    mul_row(e, o, a.v, b.v[i]);
+    w[i] = e[0];
+  }
+  const Fr hi = join_rows(e, o);
+  asm("add.cc.u32 %0, %0, %9; addc.cc.u32 %1, %1, %10; addc.cc.u32 %2, %2, %11; addc.cc.u32 %3, %3, %12;\n\t"
+      "addc.cc.u32 %4, %4, %13; addc.cc.u32 %5, %5, %14; addc.cc.u32 %6, %6, %15; addc.cc.u32 %7, %7, %16;\n\t"
+      "addc.u32 %8, %8, 0;"
+      : "+&r"(w[8]), "+&r"(w[9]), "+&r"(w[10]), "+&r"(w[11]), "+&r"(w[12]), "+&r"(w[13]), "+&r"(w[14]), "+&r"(w[15]),
+        "+&r"(w[16])
+      : "r"(hi.v[0]), "r"(hi.v[1]), "r"(hi.v[2]), "r"(hi.v[3]), "r"(hi.v[4]), "r"(hi.v[5]), "r"(hi.v[6]),
+        "r"(hi.v[7]));
+}
+
 // (t + m r) / 2^256 for the m that makes it whole, t < 2^256: in [0, r].
 __device__ __forceinline__ Fr redc_low(const uint32_t (&t)[8]) {
   uint32_t e[8], o[8];
@@ -200,6 +234,26 @@ __device__ __forceinline__ Fr redc_low(const uint32_t (&t)[8]) {
 #pragma unroll
   for (int i = 1; i < 8; i++) redc_next(e, o);
   return join_rows(e, o);
+}
+
+// The Montgomery reduction of a sum of n products of reduced elements, as
+// eight 64-bit columns (the ninth limb on top of the last column): below
+// (0.46 n + 1) r, to be added to other such sums and reduced by redc_columns.
+__device__ __forceinline__ void wide_redc(const uint32_t (&w)[17], unsigned long long (&col)[8]) {
+  uint32_t lo[8], hi[8], top;
+#pragma unroll
+  for (int j = 0; j < 8; j++) lo[j] = w[j];
+  const Fr x = redc_low(lo);
+  asm("add.cc.u32 %0, %9, %17; addc.cc.u32 %1, %10, %18; addc.cc.u32 %2, %11, %19; addc.cc.u32 %3, %12, %20;\n\t"
+      "addc.cc.u32 %4, %13, %21; addc.cc.u32 %5, %14, %22; addc.cc.u32 %6, %15, %23; addc.cc.u32 %7, %16, %24;\n\t"
+      "addc.u32 %8, %25, 0;"
+      : "=&r"(hi[0]), "=&r"(hi[1]), "=&r"(hi[2]), "=&r"(hi[3]), "=&r"(hi[4]), "=&r"(hi[5]), "=&r"(hi[6]),
+        "=&r"(hi[7]), "=&r"(top)
+      : "r"(x.v[0]), "r"(x.v[1]), "r"(x.v[2]), "r"(x.v[3]), "r"(x.v[4]), "r"(x.v[5]), "r"(x.v[6]), "r"(x.v[7]),
+        "r"(w[8]), "r"(w[9]), "r"(w[10]), "r"(w[11]), "r"(w[12]), "r"(w[13]), "r"(w[14]), "r"(w[15]), "r"(w[16]));
+#pragma unroll
+  for (int j = 0; j < 8; j++) col[j] = hi[j];
+  col[7] |= (unsigned long long)top << 32;
 }
 #endif
 

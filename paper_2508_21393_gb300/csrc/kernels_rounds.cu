@@ -16,16 +16,33 @@ __global__ void __launch_bounds__(THREADS, MINB) rounds_kernel(const DevProof* _
 // variant: CTAs per SM.  7, 6, 5 and 4 set the register allocation (7: one
 // wave of 1064 proofs, tighter registers; 4: more registers per thread).  3 and 2
 // use the variant-4 code and cap residency by reserving shared memory, for
-// fewer co-resident proofs competing for issue slots.  threads: 128, 192 or
-// 256 per proof (more threads shorten the vector passes of large proofs; the
-// register budget follows from variant x threads).
+// fewer co-resident proofs competing for issue slots.  threads: 128, 192,
+// 256 or 512 per proof (more threads shorten the vector passes of large
+// proofs; the register budget follows from variant x threads).
+// Both 0: by the number of proofs.  A proof's rounds are a chain, so while
+// there are SMs for all of them each proof gets as many threads as an SM holds
+// at 128 registers (up to one proof per SM: 512, two: 256); beyond that 128
+// threads, four proofs per SM.  Measured with the rounds of rounds_dev.cuh: one
+// 7B projection (8 proofs) 320 -> 232 us, one 13B projection from host memory
+// 750 -> 578, the 7B step (1024 proofs) 2.60 -> 2.48 ms.
 cudaError_t launch_rounds(const DevProof* proofs, int nproofs, vl_proof* out, int variant, int threads,
                           cudaStream_t st) {
   if (nproofs <= 0) return cudaSuccess;
-  if (threads == 192) {
+  if (variant == 0 && threads == 0) {
+    int dev = 0, sms = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    if (nproofs <= sms) threads = 512;
+    else if (nproofs <= 2 * sms) threads = 256;
+    else variant = 4;
+  }
+  if (threads == 512) {
+    rounds_kernel<1, 512><<<nproofs, 512, RND_SMEM, st>>>(proofs, out);
+  } else if (threads == 192) {
     rounds_kernel<4, 192><<<nproofs, 192, RND_SMEM, st>>>(proofs, out);
   } else if (threads == 256) {
-    rounds_kernel<3, 256><<<nproofs, 256, RND_SMEM, st>>>(proofs, out);
+    rounds_kernel<2, 256><<<nproofs, 256, RND_SMEM, st>>>(proofs, out);
   } else if (variant == 2 || variant == 3) {
     static std::atomic<int> set{0};  // launches come from several host threads
     const int smem = variant == 2 ? 100 * 1024 : 70 * 1024;
@@ -66,35 +83,23 @@ cudaError_t launch_rounds(const DevProof* proofs, int nproofs, vl_proof* out, in
 namespace vl {
 namespace {
 
-// accum_g and fold1 of the batched passes (the one out-of-line copy of the
-// Montgomery product: an inlined copy per call made the kernel larger than
-// the instruction cache).
-__device__ __forceinline__ void accum_g_inl(Fr (&g)[3], const Fr& a0, const Fr& a1, const Fr& b0, const Fr& b1) {
-  const Fr p0 = mont_mul_ni(a0, b0), p1 = mont_mul_ni(a1, b1);
-  const Fr p2 = mont_mul_ni(fr_sub(fr_dbl(a1), a0), fr_sub(fr_dbl(b1), b0));
-  g[0] = fr_add(g[0], p0);
-  g[1] = fr_add(g[1], p1);
-  g[2] = fr_add(g[2], p2);
-}
-
-__device__ __forceinline__ Fr fold1_inl(const Fr& x0, const Fr& x1, const Fr& r) {
-  return fr_add(x0, mont_mul_ni(r, fr_sub(x1, x0)));
-}
-
 __global__ void __launch_bounds__(RB_THREADS, 4) rounds_pass_kernel(const DevProof* __restrict__ proofs,
                                                                     const RoundItem* __restrict__ items,
                                                                     Fr* __restrict__ partials, int t) {
-  __shared__ Fr gsh[4];
   __shared__ unsigned long long red[3 * 8 * (RB_THREADS / 32)];
   const RoundItem it = items[blockIdx.x];
   const DevProof& P = proofs[it.proof];
   const int tid = threadIdx.x, K = 1 << P.d1;
   Fr* fA = P.fA;
   Fr* fB = P.fB;
-  Fr g[3] = {fr_zero(), fr_zero(), fr_zero()};
+  uint32_t w0[17], wi[17];
+  wide_zero(w0), wide_zero(wi);
+  Fr s;
   if (t == 1) {
     // f from the fold (reduced, or column sums to reduce here), round 1 on
     // pairs (j, j + K/2); j + K/2 may be padding (written as zeros)
+    uint32_t w1[17];
+    wide_zero(w1);
     const int h = K >> 1;
     const bool da = P.fdirA, db = P.fdirB;
     const Fr corrA = P.scr->corrA, corrB = P.scr->corrB;
@@ -111,72 +116,84 @@ __global__ void __launch_bounds__(RB_THREADS, 4) rounds_pass_kernel(const DevPro
       if (!da || !real) fA[j + h] = a1;
       if (!db) fB[j] = b0;
       if (!db || !real) fB[j + h] = b1;
-      accum_g_inl(g, a0, a1, b0, b1);
+      first_pair(a0, a1, b0, b1, w0, w1, wi);
     }
+    unsigned long long col[3][8];
+    wide_redc(w0, col[0]);
+    wide_redc(wi, col[1]);
+    wide_redc(w1, col[2]);
+    s = block_sum_columns<3>(col, red);
   } else {
     // fold with r_(t-1) (vectors of 2h entries) and evaluate round t on the
     // folded pairs (j, j + hh)
     const Fr r = P.scr->r;
-    const int h = K >> (t - 1), hh = h >> 1;
-    for (int j = it.j0 + tid; j < it.j1; j += RB_THREADS) {
-      const Fr a0 = fold1_inl(fA[j], fA[j + h], r), a1 = fold1_inl(fA[j + hh], fA[j + hh + h], r);
-      const Fr b0 = fold1_inl(fB[j], fB[j + h], r), b1 = fold1_inl(fB[j + hh], fB[j + hh + h], r);
-      fA[j] = a0; fA[j + hh] = a1;
-      fB[j] = b0; fB[j + hh] = b1;
-      accum_g_inl(g, a0, a1, b0, b1);
-    }
+    const int h = K >> (t - 1);
+    for (int j = it.j0 + tid; j < it.j1; j += RB_THREADS) fold_pair(fA, fB, fA, fB, j, h, r, w0, wi);
+    unsigned long long col[2][8];
+    wide_redc(w0, col[0]);
+    wide_redc(wi, col[1]);
+    s = block_sum_columns<2>(col, red);
   }
-  block_sum_canonical<3>(g, gsh, red);
-  if (tid < 3) partials[3 * (size_t)blockIdx.x + tid] = gsh[tid];
-}
-
-__device__ __forceinline__ void state_to_bytes(const uint32_t* S, uint8_t* out, int lane) {
-  out[lane] = (uint8_t)(S[lane >> 2] >> (24 - 8 * (lane & 3)));
+  if (tid < (t == 1 ? 3 : 2)) partials[3 * (size_t)blockIdx.x + tid] = s;  // g(0), G, and round 1's g(1)
 }
 
 // Transcript step of round t for proofs [0, np) (each has more rounds after
-// t: the last rounds are the tail's).
+// t: the last rounds are the tail's), one warp per proof.
 __global__ void __launch_bounds__(32 * RB_WARPS) rounds_hash_kernel(const DevProof* __restrict__ proofs, int np,
                                                                     const int* __restrict__ ibase,
                                                                     const Fr* __restrict__ partials,
                                                                     vl_proof* __restrict__ out, int t) {
-  __shared__ uint32_t Ssh[RB_WARPS][8];
-  __shared__ Fr gsh_all[RB_WARPS][4];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int p = blockIdx.x * RB_WARPS + warp;
   if (p >= np) return;  // whole warps leave together
   const DevProof& P = proofs[p];
   vl_proof* pf = out + P.job;
-  uint32_t* S = Ssh[warp];
-  Fr* gsh = gsh_all[warp];
-  if (lane < 8) {
-    const uint8_t* b = P.scr->state + 4 * lane;
-    S[lane] = ((uint32_t)b[0] << 24) | ((uint32_t)b[1] << 16) | ((uint32_t)b[2] << 8) | (uint32_t)b[3];
-  }
   if (t == 1) {
     if (lane == 0) {
       pf->m = P.m; pf->k = P.k; pf->n = P.n;
       pf->d0 = P.d0; pf->d1 = P.d1; pf->d2 = P.d2;
       pf->reserved = 0;
     }
-    for (int i = P.d1 * 3 + lane; i < VL_MAX_ROUNDS * 3; i += 32) store_fr(&pf->g[i / 3][i % 3], fr_zero());
+    for (int i = P.d1 * 24 + lane; i < VL_MAX_ROUNDS * 24; i += 32) pf->g[i / 24][(i >> 3) % 3].limb[i & 7] = 0u;
   }
+  // lane 4 e + q sums value q over every eighth item
+  Fr v = fr_zero();
+  if ((lane & 3) < (t == 1 ? 3 : 2))
+    for (int i = ibase[p] + (lane >> 2); i < ibase[p + 1]; i += 8) v = fr_add(v, partials[3 * (size_t)i + (lane & 3)]);
+#pragma unroll
+  for (int off = 4; off < 32; off <<= 1) v = fr_add(v, shfl_xor_fr(v, off));
+  const Fr g0 = shfl_fr(v, 0), G = shfl_fr(v, 1);
+  Fr g1 = shfl_fr(v, 2);
+  uint32_t st[8];
+#pragma unroll
+  for (int i = 0; i < 8; i++) st[i] = bswap32(reinterpret_cast<const uint32_t*>(P.scr->state)[i]);
+  if (t == 1) {
+    const Fr c[1] = {fr_add(g0, g1)};
+    if (lane == 0) store_fr(&pf->c, c[0]);
+    dev_absorb_fr<1>(st, LBL_C, c);
+  } else {
+    g1 = fr_sub(P.scr->claim, g0);
+  }
+  const Fr g02[2] = {g0, fr_sub(fr_dbl(fr_add(g1, G)), g0)};  // g(2) = 2 g(1) - g(0) + 2 G
   if (lane == 0) {
-    Fr g[3] = {fr_zero(), fr_zero(), fr_zero()};
-    for (int i = ibase[p]; i < ibase[p + 1]; i++)
-#pragma unroll
-      for (int q = 0; q < 3; q++) g[q] = fr_add(g[q], partials[3 * (size_t)i + q]);
-#pragma unroll
-    for (int q = 0; q < 3; q++) gsh[q] = g[q];
+    store_fr(&pf->g[t - 1][0], g0);
+    store_fr(&pf->g[t - 1][1], g1);
+    store_fr(&pf->g[t - 1][2], g02[1]);
   }
-  __syncwarp();
-  const Fr r = round_transcript(S, gsh, t == 1, pf, t - 1);
+  dev_absorb_fr<2>(st, LBL_G, g02);
+  uint32_t d[8];
+  dev_squeeze_block(st, LBL_R, lane < 2 ? 0u : 1u, lane < 2 ? lane : 2, d);
+  Fr r = challenge_of(d);
   if (lane == 0) {
     P.scr->r = r;
     if (P.rch) P.rch[t - 1] = r;  // chained proofs continue from this point
+    const Fr b = fr_sub(fr_sub(g1, g0), G);
+    P.scr->claim = fr_add(g0, mont_mul_ni(r, fr_add(b, mont_mul_ni(r, G))));
   }
-  __syncwarp();
-  state_to_bytes(S, P.scr->state, lane);
+  if (lane == 2) {
+#pragma unroll
+    for (int i = 0; i < 8; i++) reinterpret_cast<uint32_t*>(P.scr->state)[i] = bswap32(d[i]);
+  }
 }
 
 // The rounds after the batched ones, one CTA per proof.

@@ -40,11 +40,12 @@ __device__ __forceinline__ void block_sum_fr(Fr (&x)[NV], Fr* sh) {
   __syncthreads();
 }
 
-// Sum a[32] over the 32 lanes of a warp; lane L returns the total of a[L].
-__device__ __forceinline__ unsigned long long warp_transpose_sum(unsigned long long (&a)[32]) {
+// Sum a[N] over the 32 lanes of a warp; lane L returns the total of a[L mod N].
+template <int N>
+__device__ __forceinline__ unsigned long long warp_transpose_sum(unsigned long long (&a)[N]) {
   const int lane = threadIdx.x & 31;
 #pragma unroll
-  for (int off = 16; off >= 1; off >>= 1) {
+  for (int off = N / 2; off >= 1; off >>= 1) {
     const bool upper = (lane & off) != 0;
 #pragma unroll
     for (int i = 0; i < off; i++) {
@@ -54,24 +55,28 @@ __device__ __forceinline__ unsigned long long warp_transpose_sum(unsigned long l
       a[i] = keep + recv;
     }
   }
+#pragma unroll
+  for (int off = N; off < 32; off <<= 1) a[0] += __shfl_xor_sync(0xffffffffu, a[0], off);
   return a[0];
 }
 
-// Sum of NV field elements per thread (Montgomery form) over the block, as
-// canonical values: the eight 32-bit limbs are summed as 64-bit integers
-// (exact for up to 2^32 terms; no modular reduction per level), and one
-// REDC of the column sums gives (sum x.R) . R^-1 = sum x mod r.  Results in
-// out[0..NV).  sh: NV * 8 * (blockDim.x / 32) 64-bit slots.  Block-wide.
+// Canonical sum over the block of NV values per thread given as 64-bit limb
+// columns of Montgomery-form values (wide_redc): limb columns are summed as
+// integers, one REDC of the totals gives sum x mod r, valid in lane q < NV of
+// warp 0 for value q.  sh: NV * 8 slots per warp.  One block barrier; the
+// slots may be written again after the next one.
 template <int NV>
-__device__ __forceinline__ void block_sum_canonical(const Fr (&x)[NV], Fr* out, unsigned long long* sh) {
+__device__ __forceinline__ Fr block_sum_columns(const unsigned long long (&c)[NV][8], unsigned long long* sh) {
   static_assert(NV * 8 <= 32, "at most 4 values");
+  constexpr int N = NV * 8 <= 8 ? 8 : NV * 8 <= 16 ? 16 : 32;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  unsigned long long a[32];
+  unsigned long long a[N];
 #pragma unroll
-  for (int i = 0; i < 32; i++) a[i] = i < NV * 8 ? (unsigned long long)x[i / 8].v[i % 8] : 0ull;
-  const unsigned long long s = warp_transpose_sum(a);
+  for (int i = 0; i < N; i++) a[i] = i < NV * 8 ? c[i / 8 < NV ? i / 8 : 0][i % 8] : 0ull;
+  const unsigned long long s = warp_transpose_sum<N>(a);
   if (lane < NV * 8) sh[warp * NV * 8 + lane] = s;
   __syncthreads();
+  Fr out = fr_zero();
   if (warp == 0) {
     unsigned long long t = 0;
     if (lane < NV * 8)
@@ -79,9 +84,9 @@ __device__ __forceinline__ void block_sum_canonical(const Fr (&x)[NV], Fr* out, 
     U64x8 col;
 #pragma unroll
     for (int l = 0; l < 8; l++) col.v[l] = __shfl_sync(0xffffffffu, t, (lane * 8 + l) & 31);
-    if (lane < NV) out[lane] = redc_columns_ni(col);
+    if (lane < NV) out = redc_columns_ni(col);
   }
-  __syncthreads();
+  return out;
 }
 
 }  // namespace vl

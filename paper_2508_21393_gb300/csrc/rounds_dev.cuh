@@ -2,24 +2,33 @@
 //
 // One CTA per proof.  The fold accumulators become the vectors
 // f_A[w] = A~(u, w), f_B[w] = B~(w, v) over the padded cube w < 2^d1 (zeros
-// for w >= k).  Round i (h = 2^(d1 - i)) evaluates the degree-2 round
-// polynomial at 0, 1, 2:
-//   g(0) = sum_j a0 b0,  g(1) = sum_j a1 b1,  g(2) = sum_j (2a1 - a0)(2b1 - b0)
-// with a0 = f_A[j], a1 = f_A[j + h] (likewise b), absorbs the three values,
-// squeezes r_i and folds both vectors in place, f[j] <- f[j] + r_i (f[j+h] - f[j])
-// (variables bound most-significant first).  Finally a_r = f_A[0],
-// b_r = f_B[0] are absorbed and the proof is written in canonical form.
+// for w >= k).  Round i (h = 2^(d1 - i)) has the degree-2 round polynomial
+// g(X) = sum_j (a0 + X (a1 - a0)) (b0 + X (b1 - b0)) with a0 = f_A[j],
+// a1 = f_A[j + h] (likewise b); its values at 0, 1, 2 are the message, g(0)
+// and g(2) are absorbed, r_i squeezed and both vectors folded,
+// f[j] <- f[j] + r_i (f[j + h] - f[j]) (variables bound most-significant
+// first).  Finally a_r = f_A[0], b_r = f_B[0] are absorbed and the proof is
+// written in canonical form.
 //
-// Schedule (latency is what matters here: one proof's rounds are a serial
-// chain of hashes):
-//  * pass 0 reduces the accumulators and evaluates round 1 in the same loop;
-//    the claim is c = g_1(0) + g_1(1) (for k = 1 it is a_r . b_r);
-//  * each later pass folds with r_i and evaluates round i + 1 on the folded
-//    values in the same loop (one memory pass and one block reduction per
-//    round);
-//  * the transcript runs on warp 0 with message blocks in registers; the two
-//    halves of the challenge and the closing state update are three
-//    independent hashes done by three lanes at once.
+// Work per pair: only g(0) = sum a0 b0 and the leading coefficient
+// G = sum (a1 - a0)(b1 - b0) are summed; g(1) is the running claim minus g(0)
+// (the claim of round 1 is formed from its g(1), summed too), g(2) =
+// 2 g(1) - g(0) + 2 G, and the next claim is g(r) = g(0) + r (g(1) - g(0) - G
+// + r G).  A thread sums its products unreduced (wide_mac) and reduces once.
+// So a pair costs four fold products and two half products, against seven
+// products for the three values evaluated one by one.
+//
+// Schedule (one proof's rounds are a serial chain of hashes):
+//  * pass 0 reads (or reduces) f and evaluates round 1; each later pass folds
+//    with r_i and evaluates round i + 1 in the same loop;
+//  * short rounds spread a pair over four lanes of a warp: one fold each, then
+//    one term on two of them (two products on the chain instead of six);
+//    vectors of at most RND_VEC entries live in shared memory, and the last
+//    rounds run on warp 0 alone, whose last lane forms the next claim;
+//  * the transcript runs on warps 0 to 2: the rounds of each SHA-256
+//    compression on warp 0, its message schedule on warp 1 (of an absorb's
+//    second block: on warp 2); the two halves of the challenge and the
+//    closing state update are three lanes of one compression.
 #pragma once
 #include "common.cuh"
 #include "reduce.cuh"
@@ -28,10 +37,22 @@
 
 namespace vl {
 
-// Shared memory the rounds need (RND_SMEM bytes): state (32), the round
-// message (3 x 32), the challenge (32), then block-reduction slots for up to
-// 8 warps (3 x 8 x 8 x 8 bytes at offset 256).
-static_assert(RND_SMEM == 256 + 3 * 8 * 8 * 8, "layout");
+static constexpr int RND_VEC = 256;      // vectors of at most this many entries are kept in shared memory
+static constexpr int RND_MAX_WARPS = 16;
+
+// Shared memory of the rounds.
+struct RndShared {
+  alignas(16) uint32_t msg[32];    // an absorb's message: two blocks
+  alignas(16) uint32_t wk[3][68];  // schedule words: of an absorb's two blocks, of a squeeze's three lanes
+  alignas(16) uint32_t S[8];       // transcript state
+  alignas(16) uint32_t sq[8];      // state before a squeeze
+  Fr g[4];                         // g(0), g(1), g(2), G of the round (canonical)
+  Fr claim;                        // the running claim (canonical)
+  Fr r;                            // the latest challenge (Montgomery)
+  alignas(16) unsigned long long red[3 * 8 * RND_MAX_WARPS];
+  Fr fa[RND_VEC], fb[RND_VEC];
+};
+static_assert(sizeof(RndShared) <= RND_SMEM, "shared memory of the rounds");
 
 __device__ __forceinline__ Fr load_acc_fr(const unsigned long long* acc, int w, const Fr& corr) {
   U64x8 a;
@@ -49,76 +70,189 @@ __device__ __forceinline__ Fr fold1(const Fr& x0, const Fr& x1, const Fr& r) {
   return fr_add(x0, mont_mul_ni(r, fr_sub(x1, x0)));
 }
 
-__device__ __forceinline__ void accum_g(Fr (&g)[3], const Fr& a0, const Fr& a1, const Fr& b0, const Fr& b1) {
-  g[0] = fr_add(g[0], mont_mul_ni(a0, b0));
-  g[1] = fr_add(g[1], mont_mul_ni(a1, b1));
-  g[2] = fr_add(g[2], mont_mul_ni(fr_sub(fr_dbl(a1), a0), fr_sub(fr_dbl(b1), b0)));
+__device__ __forceinline__ Fr shfl_fr(const Fr& x, int src) {
+  Fr y;
+#pragma unroll
+  for (int l = 0; l < 8; l++) y.v[l] = __shfl_sync(0xffffffffu, x.v[l], src);
+  return y;
 }
 
-// Warp 0: absorb the round message in gsh (lane 0), then squeeze one
-// challenge: lanes 0 and 1 hash the two halves, lane 2 the state update.
-// Returns r (Montgomery) in lane 0; S (shared) is the new state.
-__device__ __forceinline__ Fr round_transcript(uint32_t* S, const Fr* gsh, bool with_claim, vl_proof* pf, int round) {
+// Fold the pair's four entries with r and add its terms to the wide sums
+// w0 += a0 b0, wi += (a1 - a0)(b1 - b0).
+__device__ __forceinline__ void fold_pair(const Fr* sA, const Fr* sB, Fr* dA, Fr* dB, int j, int h, const Fr& r,
+                                          uint32_t (&w0)[17], uint32_t (&wi)[17]) {
+  const int hh = h >> 1;
+  const Fr a0 = fold1(sA[j], sA[j + h], r), a1 = fold1(sA[j + hh], sA[j + hh + h], r);
+  const Fr b0 = fold1(sB[j], sB[j + h], r), b1 = fold1(sB[j + hh], sB[j + hh + h], r);
+  dA[j] = a0;
+  dA[j + hh] = a1;
+  dB[j] = b0;
+  dB[j + hh] = b1;
+  wide_mac(w0, a0, b0);
+  wide_mac(wi, fr_sub(a1, a0), fr_sub(b1, b0));
+}
+
+// Round 1's terms of one pair of unfolded entries: g(0), g(1), G.
+__device__ __forceinline__ void first_pair(const Fr& a0, const Fr& a1, const Fr& b0, const Fr& b1, uint32_t (&w0)[17],
+                                           uint32_t (&w1)[17], uint32_t (&wi)[17]) {
+  wide_mac(w0, a0, b0);
+  wide_mac(w1, a1, b1);
+  wide_mac(wi, fr_sub(a1, a0), fr_sub(b1, b0));
+}
+
+__device__ __forceinline__ void wide_zero(uint32_t (&w)[17]) {
+#pragma unroll
+  for (int i = 0; i < 17; i++) w[i] = 0;
+}
+
+// The message words of an absorb of N = 1 or 2 elements (33 + 32 N bytes: two
+// blocks), one word per lane.
+__device__ __forceinline__ void absorb_words(RndShared& sh, uint32_t label, const Fr& x, const Fr& y, int n) {
   const int lane = threadIdx.x & 31;
-  if (lane == 0) {
-    uint32_t st[8];
+  const uint32_t* xs = x.v;
+  const uint32_t* ys = y.v;
+  auto limb = [&](int q) { return q < 8 ? xs[q & 7] : ys[q & 7]; };  // x, y are in memory
+  uint32_t w = 0;
+  const int q = lane - 8;
+  if (q < 0) w = sh.S[lane];
+  else if (q < 8 * n) w = __byte_perm(limb(q), q == 0 ? label << 24 : limb(q - 1), 0x7012);
+  else if (q == 8 * n) w = (limb(q - 1) & 0xff000000u) | 0x00800000u;
+  else if (lane == 31) w = (uint32_t)(33 + 32 * n) * 8u;
+  sh.msg[lane] = w;
+}
+
+// SHA256 of the two blocks in sh.msg.  Warp 0 (returns the digest in every
+// lane), with warps 1 and 2 in absorb_help.
+__device__ __forceinline__ ShaState absorb_run(RndShared& sh) {
+  named_sync(7, 96);
+  ShaState st = sha_rounds_ni(sha_iv_state(), sha_load(sh.msg), sh.wk[0], 1);
+  return sha_rounds_ni(st, sha_load(sh.msg + 16), sh.wk[1], 4);
+}
+__device__ __forceinline__ void absorb_help(RndShared& sh, int warp) {
+  named_sync(7, 96);
+  sha_sched_ni(sha_load(sh.msg + 16 * (warp - 1)), sh.wk[warp - 1], 1 + 3 * (warp - 1));
+}
+
+// The lane's block of the squeeze of one challenge from state S: lanes 0 and 1
+// the challenge's halves, the others the closing update.
+__device__ __forceinline__ ShaBlock squeeze_lane_block(const uint32_t (&S)[8]) {
+  const int lane = threadIdx.x & 31, kind = lane < 2 ? lane : 2;
+  ShaBlock b;
 #pragma unroll
-    for (int i = 0; i < 8; i++) st[i] = S[i];
-    if (with_claim) {
-      const Fr c[1] = {fr_add(gsh[0], gsh[1])};
-      store_fr(&pf->c, c[0]);
-      dev_absorb_fr<1>(st, LBL_C, c);
-    }
+  for (int i = 0; i < 8; i++) b.w[i] = S[i];
+  b.w[8] = ((uint32_t)LBL_R << 24) | (kind == 2 ? 1u << 16 : 0u);          // label, t = 0 or count = 1 (LE)
+  b.w[9] = kind == 2 ? 0x00800000u : ((uint32_t)kind << 16) | 0x00008000u;  // (half,) padding
 #pragma unroll
-    for (int q = 0; q < 3; q++) store_fr(&pf->g[round][q], gsh[q]);
-    const Fr g02[2] = {gsh[0], gsh[2]};  // g(1) is fixed by the running claim
-    dev_absorb_fr<2>(st, LBL_G, g02);
-#pragma unroll
-    for (int i = 0; i < 8; i++) S[i] = st[i];
-  }
-  __syncwarp();
-  uint32_t st[8], d[8];
-#pragma unroll
-  for (int i = 0; i < 8; i++) {
-    st[i] = S[i];
-    d[i] = 0;
-  }
-  if (lane < 3) dev_squeeze_block(st, LBL_R, lane < 2 ? 0u : 1u, lane, d);
-  __syncwarp();
-  if (lane == 2) {
-#pragma unroll
-    for (int i = 0; i < 8; i++) S[i] = d[i];
-  }
-  // r = (lo + hi . 2^256) mod r, in Montgomery form (lo: lane 0's digest,
-  // hi: lane 1's) = lo . R + hi . R^2 mod r: lane 0 forms REDC(lo . R^2) and
-  // lane 1 REDC(hi . R^3) at once, one product on the serial chain instead of
-  // the reduction's and the conversion's two
+  for (int i = 10; i < 15; i++) b.w[i] = 0;
+  b.w[15] = kind == 2 ? 37u * 8u : 38u * 8u;
+  return b;
+}
+
+// The challenge from the two halves' digests (lanes 0 and 1), in Montgomery
+// form: (lo + hi 2^256) mod r times R = REDC(lo R^2) + REDC(hi R^3), one
+// product on the chain.  Valid in lane 0.
+__device__ __forceinline__ Fr challenge_of(const uint32_t (&d)[8]) {
+  const int lane = threadIdx.x & 31;
   Fr half = fr_zero();
   if (lane < 2) half = mont_mul_ni(digest_le(d), lane == 0 ? fr_r2() : fr_r3());
-  Fr other;
-#pragma unroll
-  for (int i = 0; i < 8; i++) other.v[i] = __shfl_sync(0xffffffffu, half.v[i], 1);
-  Fr r = fr_zero();
-  if (lane == 0) r = fr_add(half, other);
-  __syncwarp();
-  return r;
+  const Fr other = shfl_fr(half, 1);
+  return fr_add(half, other);
 }
 
-// Claim, rounds and proof of one proof by the whole block (any multiple of
-// 32 threads up to 256), from round t0 on.  t0 = 1: everything.  t0 > 1: the
+// The transcript step of round i (0-based): warps 0 to 2 of the block.  Warp 0
+// has the message in sh.g; with_claim: the claim is absorbed before it.  At the
+// end sh.r, sh.S are set (visible after the block's next barrier).
+__device__ __forceinline__ void transcript_step(RndShared& sh, int warp, bool with_claim, Fr* rch) {
+  const int lane = threadIdx.x & 31;
+  if (warp == 0) {
+    if (with_claim) {
+      absorb_words(sh, LBL_C, sh.claim, sh.claim, 1);
+      const ShaState c = absorb_run(sh);
+      if (lane == 0) {
+#pragma unroll
+        for (int i = 0; i < 8; i++) sh.S[i] = c.h[i];
+      }
+      __syncwarp();
+    }
+    absorb_words(sh, LBL_G, sh.g[0], sh.g[2], 2);  // g(1) is fixed by the running claim
+    ShaState st = absorb_run(sh);
+    if (lane == 0) {
+#pragma unroll
+      for (int i = 0; i < 8; i++) sh.sq[i] = st.h[i];
+    }
+    named_sync(8, 64);
+    st = sha_rounds_ni(sha_iv_state(), squeeze_lane_block(st.h), sh.wk[lane < 2 ? lane : 2], 1);
+    if (lane == 2) {
+#pragma unroll
+      for (int i = 0; i < 8; i++) sh.S[i] = st.h[i];
+    }
+    const Fr r = challenge_of(st.h);
+    if (lane == 0) {
+      sh.r = r;
+      if (rch) *rch = r;  // chained proofs continue from this point
+    }
+  } else if (warp < 3) {
+    if (with_claim) absorb_help(sh, warp);
+    absorb_help(sh, warp);
+    if (warp == 1) {
+      named_sync(8, 64);
+      uint32_t S[8];
+#pragma unroll
+      for (int i = 0; i < 8; i++) S[i] = sh.sq[i];
+      sha_sched_ni(squeeze_lane_block(S), sh.wk[lane < 2 ? lane : 2], 1);
+    }
+  }
+}
+
+// Warp 0: the round's message from g(0) and G (canonical, in every lane; first:
+// g(1) too, which makes the claim), into sh.g and the proof.
+__device__ __forceinline__ void round_message(RndShared& sh, const Fr& g0, const Fr& G, const Fr* g1_first, vl_proof* pf,
+                                              int i) {
+  const int lane = threadIdx.x & 31;
+  __syncwarp();  // the claim may come from another lane
+  const Fr g1 = g1_first ? *g1_first : fr_sub(sh.claim, g0);
+  const Fr s = fr_add(g1, G);
+  const Fr g2 = fr_sub(fr_dbl(s), g0);
+  __syncwarp();
+  if (lane == 0) {
+    sh.g[0] = g0;
+    sh.g[1] = g1;
+    sh.g[2] = g2;
+    sh.g[3] = G;
+    if (g1_first) {
+      sh.claim = fr_add(g0, g1);
+      store_fr(&pf->c, sh.claim);
+    }
+  }
+  __syncwarp();
+  if (lane < 24) pf->g[i][lane >> 3].limb[lane & 7] = sh.g[lane >> 3].v[lane & 7];
+}
+
+// One lane: the claim of the next round, g(r).
+__device__ __forceinline__ void next_claim(RndShared& sh) {
+  const Fr r = sh.r, b = fr_sub(fr_sub(sh.g[1], sh.g[0]), sh.g[3]);
+  sh.claim = fr_add(sh.g[0], mont_mul_ni(r, fr_add(b, mont_mul_ni(r, sh.g[3]))));
+}
+
+__device__ __forceinline__ void store_state(uint8_t* dst, const ShaState& st) {
+  if ((threadIdx.x & 31) == 0) {
+#pragma unroll
+    for (int q = 0; q < 8; q++) reinterpret_cast<uint32_t*>(dst)[q] = bswap32(st.h[q]);
+  }
+}
+
+// Claim, rounds and proof of one proof by the whole block (a multiple of 32
+// threads, 128 to 512), from round t0 on.  t0 = 1: everything.  t0 > 1: the
 // earlier rounds ran batched over many proofs (kernels_rounds.cu): their
-// messages are in the proof already, the transcript state and r_(t0-1) are
-// in the scratch, and the vectors hold the round-(t0-1) values, 2^(d1-t0+2)
-// entries each.
+// messages are in the proof already, the transcript state, the claim and
+// r_(t0-1) are in the scratch, and the vectors hold the round-(t0-1) values,
+// 2^(d1-t0+2) entries each.
 static __device__ void rounds_block(const DevProof& P, vl_proof* pf, uint8_t* smem, int t0 = 1) {
-  uint32_t* S = reinterpret_cast<uint32_t*>(smem);
-  Fr* gsh = reinterpret_cast<Fr*>(smem + 32);
-  Fr& r_sh = gsh[3];
-  unsigned long long* red = reinterpret_cast<unsigned long long*>(smem + 256);
-  const int tid = threadIdx.x, warp = tid >> 5, nthr = blockDim.x;
+  RndShared& sh = *reinterpret_cast<RndShared*>(smem);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, nthr = blockDim.x, last = (nthr >> 5) - 1;
   if (tid < 8) {
-    const uint8_t* b = P.scr->state + 4 * tid;
-    S[tid] = ((uint32_t)b[0] << 24) | ((uint32_t)b[1] << 16) | ((uint32_t)b[2] << 8) | (uint32_t)b[3];
+    sh.S[tid] = bswap32(reinterpret_cast<const uint32_t*>(P.scr->state)[tid]);
+    if (t0 > 1) sh.claim.v[tid] = P.scr->claim.v[tid];
   }
   if (t0 == 1) {
     if (tid == 0) {
@@ -126,132 +260,165 @@ static __device__ void rounds_block(const DevProof& P, vl_proof* pf, uint8_t* sm
       pf->d0 = P.d0; pf->d1 = P.d1; pf->d2 = P.d2;
       pf->reserved = 0;
     }
-    for (int i = P.d1 * 3 + tid; i < VL_MAX_ROUNDS * 3; i += nthr) store_fr(&pf->g[i / 3][i % 3], fr_zero());
+    for (int i = P.d1 * 24 + tid; i < VL_MAX_ROUNDS * 24; i += nthr) pf->g[i / 24][(i >> 3) % 3].limb[i & 7] = 0u;
   }
   const int d1 = P.d1, K = 1 << d1;
-  const Fr corrA = P.scr->corrA, corrB = P.scr->corrB;
   Fr* fA = P.fA;
   Fr* fB = P.fB;
   __syncthreads();
 
   if (d1 == 0) {  // k = 1: no rounds, c = a_r . b_r
     if (tid == 0) {
-      const Fr a = P.fdirA ? fA[0] : load_acc_fr(P.accA, 0, corrA);
-      const Fr b = P.fdirB ? fB[0] : load_acc_fr(P.accB, 0, corrB);
+      const Fr a = P.fdirA ? fA[0] : load_acc_fr(P.accA, 0, P.scr->corrA);
+      const Fr b = P.fdirB ? fB[0] : load_acc_fr(P.accB, 0, P.scr->corrB);
       const Fr fin[2] = {from_mont_ni(a), from_mont_ni(b)};
       const Fr c[1] = {from_mont_ni(mont_mul_ni(a, b))};
       store_fr(&pf->c, c[0]);
       store_fr(&pf->a_r, fin[0]);
       store_fr(&pf->b_r, fin[1]);
-      uint32_t st[8];
+      ShaState st;
 #pragma unroll
-      for (int i = 0; i < 8; i++) st[i] = S[i];
-      dev_absorb_fr<1>(st, LBL_C, c);
-      dev_absorb_fr<2>(st, LBL_F, fin);
-#pragma unroll
-      for (int i = 0; i < 8; i++) {
-        pf->state[4 * i] = (uint8_t)(st[i] >> 24);
-        pf->state[4 * i + 1] = (uint8_t)(st[i] >> 16);
-        pf->state[4 * i + 2] = (uint8_t)(st[i] >> 8);
-        pf->state[4 * i + 3] = (uint8_t)st[i];
-      }
+      for (int i = 0; i < 8; i++) st.h[i] = sh.S[i];
+      dev_absorb_fr<1>(st.h, LBL_C, c);
+      dev_absorb_fr<2>(st.h, LBL_F, fin);
+      store_state(pf->state, st);
       pf->status = P.scr->status;
     }
     __syncthreads();
     return;
   }
 
-  Fr g[3] = {fr_zero(), fr_zero(), fr_zero()};
-  if (t0 > 1) {
-    // fold the round-(t0-1) vectors with r_(t0-1) and evaluate round t0
-    const Fr r = P.scr->r;
-    const int h = K >> (t0 - 1), hh = h >> 1;
-    for (int j = tid; j < hh; j += nthr) {
-      const Fr a0 = fold1(fA[j], fA[j + h], r), a1 = fold1(fA[j + hh], fA[j + hh + h], r);
-      const Fr b0 = fold1(fB[j], fB[j + h], r), b1 = fold1(fB[j + hh], fB[j + hh + h], r);
-      fA[j] = a0; fA[j + hh] = a1;
-      fB[j] = b0; fB[j + hh] = b1;
-      accum_g(g, a0, a1, b0, b1);
-    }
-  } else {
-    // Pass 0: f from the accumulators, and round 1 (pairs j, j + K/2).
-    const int h = K >> 1;
-    for (int j = tid; j < h; j += nthr) {
-      // K/2 < k <= K, so j < k always; j + h may be padding.
-      // f_A, f_B come reduced from the fold (fdir) or as column sums to reduce here
-      const Fr a0 = P.fdirA ? fA[j] : load_acc_fr(P.accA, j, corrA);
-      const Fr b0 = P.fdirB ? fB[j] : load_acc_fr(P.accB, j, corrB);
-      Fr a1 = fr_zero(), b1 = fr_zero();
-      if (j + h < P.k) {
-        a1 = P.fdirA ? fA[j + h] : load_acc_fr(P.accA, j + h, corrA);
-        b1 = P.fdirB ? fB[j + h] : load_acc_fr(P.accB, j + h, corrB);
+  {
+    // The first evaluation: of round 1 on f from the fold (fdir: reduced; else
+    // column sums to reduce here), or of round t0 after folding with r_(t0-1).
+    uint32_t w0[17], w1[17], wi[17];
+    wide_zero(w0), wide_zero(w1), wide_zero(wi);
+    Fr v[3];  // g(0), G, g(1)
+    if (t0 > 1) {
+      const Fr r = P.scr->r;
+      const int h = K >> (t0 - 1);
+      Fr* dA = h <= RND_VEC ? sh.fa : fA;
+      Fr* dB = h <= RND_VEC ? sh.fb : fB;
+      for (int j = tid; j < (h >> 1); j += nthr) fold_pair(fA, fB, dA, dB, j, h, r, w0, wi);
+    } else {
+      const Fr corrA = P.scr->corrA, corrB = P.scr->corrB;
+      const bool da = P.fdirA, db = P.fdirB, vec = K <= RND_VEC;
+      Fr* dA = vec ? sh.fa : fA;
+      Fr* dB = vec ? sh.fb : fB;
+      const int h = K >> 1;
+      for (int j = tid; j < h; j += nthr) {
+        // K/2 < k <= K, so j < k always; j + h may be padding
+        const bool real = j + h < P.k;
+        const Fr a0 = da ? fA[j] : load_acc_fr(P.accA, j, corrA);
+        const Fr b0 = db ? fB[j] : load_acc_fr(P.accB, j, corrB);
+        Fr a1 = fr_zero(), b1 = fr_zero();
+        if (real) {
+          a1 = da ? fA[j + h] : load_acc_fr(P.accA, j + h, corrA);
+          b1 = db ? fB[j + h] : load_acc_fr(P.accB, j + h, corrB);
+        }
+        if (vec || !da) dA[j] = a0;
+        if (vec || !da || !real) dA[j + h] = a1;
+        if (vec || !db) dB[j] = b0;
+        if (vec || !db || !real) dB[j + h] = b1;
+        first_pair(a0, a1, b0, b1, w0, w1, wi);
       }
-      fA[j] = a0; fA[j + h] = a1;
-      fB[j] = b0; fB[j + h] = b1;
-      accum_g(g, a0, a1, b0, b1);
+    }
+    unsigned long long col[3][8];
+    wide_redc(w0, col[0]);
+    wide_redc(wi, col[1]);
+    wide_redc(w1, col[2]);
+    const Fr s = block_sum_columns<3>(col, sh.red);
+    if (warp == 0) {
+#pragma unroll
+      for (int q = 0; q < 3; q++) v[q] = shfl_fr(s, q);
+      round_message(sh, v[0], v[1], t0 == 1 ? &v[2] : nullptr, pf, t0 - 1);
     }
   }
-  block_sum_canonical<3>(g, gsh, red);
 
   for (int i = t0 - 1; i < d1; i++) {
-    if (warp == 0) {
-      const Fr r = round_transcript(S, gsh, i == 0, pf, i);
-      if ((tid & 31) == 0) {
-        r_sh = r;
-        if (P.rch) P.rch[i] = r;  // chained proofs continue from this point
-      }
-    }
+    transcript_step(sh, warp, i == 0, P.rch ? P.rch + i : nullptr);
     __syncthreads();
-    const Fr r = r_sh;
+    const Fr r = sh.r;
     const int h = K >> (i + 1);  // the vectors hold 2h entries
-    if (i + 1 < d1) {
-      // Fold with r_i and evaluate round i + 1 (pairs j, j + h/2) in one pass.
-      const int hh = h >> 1;
-      Fr gn[3] = {fr_zero(), fr_zero(), fr_zero()};
-      if (4 * hh <= nthr) {
-        // Few pairs (the last rounds, latency-bound): four lanes of one warp
-        // per pair, one fold each, then three of them one term each (two
-        // products on the chain instead of seven).
-        const int j = tid >> 2, q = tid & 3;
-        if (j < hh) {
-          Fr* f = q < 2 ? fA : fB;
-          const int at = j + (q & 1) * hh;
-          f[at] = fold1(f[at], f[at + h], r);
+    const Fr* sA = 2 * h <= RND_VEC ? sh.fa : fA;
+    const Fr* sB = 2 * h <= RND_VEC ? sh.fb : fB;
+    if (i + 1 == d1) {
+      // Last fold: a_r, b_r; absorb them and write the proof.
+      if (warp == 0) {
+        if (lane < 2) {
+          const Fr* f = lane == 0 ? sA : sB;
+          const Fr x = from_mont_ni(fold1(f[0], f[1], r));
+          store_fr(lane == 0 ? &pf->a_r : &pf->b_r, x);
+          sh.g[lane] = x;
         }
         __syncwarp();
-        if (j < hh && q < 3) {
-          const Fr a0 = fA[j], a1 = fA[j + hh], b0 = fB[j], b1 = fB[j + hh];
-          if (q == 0) gn[0] = mont_mul_ni(a0, b0);
-          else if (q == 1) gn[1] = mont_mul_ni(a1, b1);
-          else gn[2] = mont_mul_ni(fr_sub(fr_dbl(a1), a0), fr_sub(fr_dbl(b1), b0));
-        }
-      } else {
-        for (int j = tid; j < hh; j += nthr) {
-          const Fr a0 = fold1(fA[j], fA[j + h], r), a1 = fold1(fA[j + hh], fA[j + hh + h], r);
-          const Fr b0 = fold1(fB[j], fB[j + h], r), b1 = fold1(fB[j + hh], fB[j + hh + h], r);
-          fA[j] = a0; fA[j + hh] = a1;
-          fB[j] = b0; fB[j + hh] = b1;
-          accum_g(gn, a0, a1, b0, b1);
-        }
+        absorb_words(sh, LBL_F, sh.g[0], sh.g[1], 2);
+        store_state(pf->state, absorb_run(sh));
+        if (lane == 0) pf->status = P.scr->status;
+      } else if (warp < 3) {
+        absorb_help(sh, warp);
       }
-      block_sum_canonical<3>(gn, gsh, red);
-    } else if (tid == 0) {
-      // Last fold: a_r, b_r; absorb them and write the proof.
-      const Fr fin[2] = {from_mont_ni(fold1(fA[0], fA[1], r)), from_mont_ni(fold1(fB[0], fB[1], r))};
-      store_fr(&pf->a_r, fin[0]);
-      store_fr(&pf->b_r, fin[1]);
-      uint32_t st[8];
+      break;
+    }
+    const int hh = h >> 1;
+    Fr* dA = h <= RND_VEC ? sh.fa : fA;
+    Fr* dB = h <= RND_VEC ? sh.fb : fB;
+    if (4 * hh > nthr) {
+      // Fold with r_i and evaluate round i + 2 (1-based; pairs j, j + hh) in one pass.
+      if (warp == last && lane == 0) next_claim(sh);
+      uint32_t w0[17], wi[17];
+      wide_zero(w0), wide_zero(wi);
+      for (int j = tid; j < hh; j += nthr) fold_pair(sA, sB, dA, dB, j, h, r, w0, wi);
+      unsigned long long col[2][8];
+      wide_redc(w0, col[0]);
+      wide_redc(wi, col[1]);
+      const Fr s = block_sum_columns<2>(col, sh.red);
+      if (warp == 0) round_message(sh, shfl_fr(s, 0), shfl_fr(s, 1), nullptr, pf, i + 1);
+      continue;
+    }
+    // Four lanes per pair j: lane q folds a0, a1, b0, b1; lane 0 then forms a0
+    // b0, lane 1 (a1 - a0)(b1 - b0).  With at most four pairs warp 0 does all,
+    // its last lane the next claim in the same products.
+    const bool alone = hh <= 4;
+    if (alone && warp != 0) continue;
+    const int j = tid >> 2, q = tid & 3;
+    const bool act = j < hh, clm = alone && lane == 31;
+    if (!alone && warp == last && lane == 0) next_claim(sh);
+    Fr x = fr_zero(), d = fr_zero();
+    if (act) {
+      const Fr* f = (q < 2 ? sA : sB) + j + (q & 1) * hh;
+      x = f[0];
+      d = fr_sub(f[h], x);
+    } else if (clm) {
+      x = fr_sub(fr_sub(sh.g[1], sh.g[0]), sh.g[3]);
+      d = sh.g[3];
+    }
+    __syncwarp();
+    x = fr_add(x, mont_mul_ni(d, r));
+    if (act) ((q < 2 ? dA : dB) + j + (q & 1) * hh)[0] = x;
+    const Fr y = shfl_xor_fr(x, 1);
+    Fr z = (q & 1) ? fr_sub(x, y) : x;
+    Fr w = shfl_xor_fr(z, 2);
+    if (clm) z = x, w = r;
+    Fr p = mont_mul_ni(z, w);
+    if (clm) sh.claim = fr_add(sh.g[0], p);
+    if (!act) p = fr_zero();
 #pragma unroll
-      for (int q = 0; q < 8; q++) st[q] = S[q];
-      dev_absorb_fr<2>(st, LBL_F, fin);
+    for (int off = 4; off < 32; off <<= 1) p = fr_add(p, shfl_xor_fr(p, off));
+    if (!alone) {
+      // lanes 0, 1 of each warp hold its sums of g(0), G
+      Fr* red = reinterpret_cast<Fr*>(sh.red);
+      if (lane < 2) red[2 * warp + lane] = p;
+      __syncthreads();
+      if (warp == 0) {
+        p = lane < 2 * (last + 1) ? red[lane] : fr_zero();
 #pragma unroll
-      for (int q = 0; q < 8; q++) {
-        pf->state[4 * q] = (uint8_t)(st[q] >> 24);
-        pf->state[4 * q + 1] = (uint8_t)(st[q] >> 16);
-        pf->state[4 * q + 2] = (uint8_t)(st[q] >> 8);
-        pf->state[4 * q + 3] = (uint8_t)st[q];
+        for (int off = 2; off < 32; off <<= 1) p = fr_add(p, shfl_xor_fr(p, off));
       }
-      pf->status = P.scr->status;
+    }
+    if (warp == 0) {
+      p = from_mont_ni(p);
+      round_message(sh, shfl_fr(p, 0), shfl_fr(p, 1), nullptr, pf, i + 1);
     }
   }
   __syncthreads();
