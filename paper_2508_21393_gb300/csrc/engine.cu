@@ -232,8 +232,8 @@ void add_fold_task(vl_plan* p, const vl_mat& M, int32_t mode, int proof, int sid
   if (tc_eligible(p, M)) {
     // Tensor-core tiles: 128 lines by at most TC_SEG reduced entries.
     t.bulk = 2;
-    t.box_w = mode == MODE_ROWDOT ? TC_KP : TC_M;  // row dots: 64 entries x 128 lines (128B-swizzled), two per stage
-    t.box_h = mode == MODE_ROWDOT ? TC_M : TC_KS;  // column sums: 128 lines x 128 entries (no swizzle)
+    t.box_w = 64;  // row dots: 64 entries x 128 lines, column sums: 64 lines x 128 entries; two per stage
+    t.box_h = mode == MODE_ROWDOT ? TC_M : TC_KS;
     p->tasks.push_back(t);
     tabs |= TAB_BYTES;
     const int lines = mode == MODE_COLSUM ? t.cols : t.rows, red = mode == MODE_COLSUM ? t.rows : t.cols;
@@ -716,10 +716,7 @@ bool encode_task_map(const FoldTask& t, CUtensorMap* map) {
              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// TMA descriptor of a tensor-core task's stored matrix: uint16 boxes of 64
-// columns (128 bytes, 128-byte swizzle) by 128 rows for row dots, 128 columns
-// by 128 rows (no swizzle: rows of 256 contiguous bytes stream better) for
-// column sums; out-of-range entries read as zero.
+// TMA descriptor of a tensor-core task's stored matrix.
 bool encode_tc_map(const FoldTask& t, CUtensorMap* map) {
   return vl::encode_tc_operand(t.mat, t.rows, t.cols, t.ld, t.mode, map);
 }
@@ -1355,22 +1352,19 @@ extern "C" int32_t vl_prove_matmul_noalloc(const vl_mat* P, const vl_mat* Q, con
 namespace vl {
 
 // TMA descriptor of an int16 operand of the tensor-core fold: uint16 boxes of
-// 64 columns (128 bytes, 128-byte swizzle) by 128 rows for row dots, 128
-// columns by 128 rows (no swizzle: rows of 256 contiguous bytes stream
-// better) for column sums; out-of-range entries read as zero.  False unless
-// the base is 16-byte aligned and rows are a multiple of 16 bytes apart.
+// 64 columns (128 bytes, 128-byte swizzle) by 128 rows (row dots: lines,
+// column sums: entries); out-of-range entries read as zero.  False unless the
+// base is 16-byte aligned and rows are a multiple of 16 bytes apart.
 bool encode_tc_operand(const void* base, int64_t rows, int64_t cols, int64_t ld, int32_t mode, void* out) {
   if ((reinterpret_cast<uintptr_t>(base) & 15) || (ld & 7)) return false;
   PFN_cuTensorMapEncodeTiled_v12000 enc = tensor_map_encoder();
   if (!enc) return false;
   const cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
   const cuuint64_t strides[1] = {(cuuint64_t)ld * 2};
-  const cuuint32_t box[2] = {(cuuint32_t)(mode == MODE_ROWDOT ? TC_KP : TC_M),
-                             (cuuint32_t)(mode == MODE_ROWDOT ? TC_M : TC_KS)};
+  const cuuint32_t box[2] = {64, (cuuint32_t)(mode == MODE_ROWDOT ? TC_M : TC_KS)};
   const cuuint32_t estr[2] = {1, 1};
   return enc(static_cast<CUtensorMap*>(out), CU_TENSOR_MAP_DATA_TYPE_UINT16, 2, const_cast<void*>(base), dims,
-             strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-             mode == MODE_ROWDOT ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE,
+             strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
              CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 

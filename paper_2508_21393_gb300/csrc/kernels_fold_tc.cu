@@ -27,8 +27,8 @@
 // mbarriers:
 // A pipeline stage is 128 lines x 128 entries: one accumulation period.
 //   warp 0       producer: per stage the operand (row dots: two boxes of 64
-//                entries x 128 lines, 128B-swizzled; column sums: one box of
-//                128 lines x 128 entries) into one of TC_NR shared-memory
+//                entries x 128 lines; column sums: two boxes of 64 lines x
+//                128 entries; 128B-swizzled) into one of TC_NR shared-memory
 //                slots, and the stage's 8 KB of fp16 weight bytes into one of
 //                TC_NW slots
 //   warps 1, 18-20  MMA issuers (warp 1 also owns TMEM, 512 columns): a
@@ -39,9 +39,9 @@
 //                MMA of constants (accumulator := 2^23) before the operand is
 //                converted, then 8 MMAs (K = 16) with A read from TMEM and B
 //                (weights) from shared memory
-//   warps 2-9    converters: one thread per (line, half of the stage's 128
-//                entries) reads its entries from the box, forms the fp16
-//                lo/hi operand rows and stores them to TMEM (one of TC_NC
+//   warps 2-9    converters: a warp takes 32 lines x half of the stage's 128
+//                entries from the boxes with ldmatrix, forms the fp16 lo/hi
+//                operand fragments and stores them to TMEM (one of TC_NC
 //                operand buffers) with tcgen05.st
 //   warps 10-17  drainers: accumulator buffer -> per-line digit sums (two
 //                groups of four warps, one warp per TMEM lane quarter, one
@@ -156,14 +156,32 @@ __device__ __forceinline__ void tmem_ld1(uint32_t taddr, uint32_t (&r)[32]) {
 }
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
-// 16 consecutive columns of this warp's lane quarter from r[0..15].
-__device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t (&r)[16]) {
+// 32 consecutive columns of 16 lanes (taddr: the first lane) from r[0..15]:
+// registers 2i, 2i + 1 hold, for columns 4i + lane % 4, TMEM lanes lane / 4 and
+// 8 + lane / 4 -- the fragment layout of ldmatrix.
+__device__ __forceinline__ void tmem_st_frag(uint32_t taddr, const uint32_t (&r)[16]) {
   asm volatile(
-      "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};" ::"r"(
+      "tcgen05.st.sync.aligned.16x128b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};" ::"r"(
           taddr),
       "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]),
       "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
       : "memory");
+}
+// Four 8 x 8 matrices of 16-bit entries (lane l gives the address of row l % 8
+// of matrix l / 8): r[i] is row lane / 4, entries 2 (lane % 4) and the next, of
+// matrix i, or of its transpose.
+template <bool TRANS>
+__device__ __forceinline__ void ldmatrix4(uint32_t addr, uint32_t* r) {
+  if (TRANS)
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"(addr)
+                 : "memory");
+  else
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"(addr)
+                 : "memory");
 }
 __device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
@@ -423,6 +441,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
               tma_load_2d(raw + 16384, T.tmap, kk + TC_KP, T.w0, bars.raw_full(slot));
             } else {
               tma_load_2d(raw, T.tmap, T.w0, kk, bars.raw_full(slot));
+              tma_load_2d(raw + 16384, T.tmap, T.w0 + 64, kk, bars.raw_full(slot));
             }
           }
           // the stage's weights once their slot is free (stage s - TC_NW's
@@ -501,10 +520,20 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     }
   } else if (warp < 2 + TC_CONV_WARPS) {
     // ---------------------------------------------------------------- converters
-    // Thread = line m (its TMEM lane) x half kh of the stage's 128 entries.
+    // Warp = 32 lines (its TMEM lane quarter) x half kh of the stage's 128
+    // entries, 16 lines x 64 entries at a time.  Both box layouts come out of
+    // ldmatrix as the same fragments (a register = two consecutive entries of
+    // one line), which is also a TMEM store shape: per entry a column sum needs
+    // no more instructions than a row dot.  (One 16-bit load per entry and a
+    // permute per pair, the lines of a column-sum box being 2 bytes apart: 7B
+    // step 2.48 ms against 2.31, 13B step 6.93 against 6.36.)
     const int quarter = warp & 3, kh = (warp - 2) >> 2;  // entries [64 kh, 64 kh + 64) of each stage
-    const int m = 32 * quarter + lane;
     const uint32_t tq = tmem + ((uint32_t)(32 * quarter) << 16) + ACONV_COL + 32 * kh;
+    const int l7 = lane & 7, lm = (lane >> 3) & 1, lk = lane >> 4;  // row in its matrix; matrix: line half, entry half
+    // row dots, box kh [128 lines][64 entries], 16-byte chunk j of line m at j ^ (m % 8)
+    const uint32_t row_base = 16384 * kh + (32 * quarter + 8 * lm + l7) * 128;
+    // column sums, box quarter / 2 [128 entries][64 lines], chunk j of entry k at j ^ (k % 8)
+    const uint32_t col_base = 16384 * (quarter >> 1) + (64 * kh + 8 * lk + l7) * 128;
     int ends = 0;
     for (int s = 0;; s++) {
       const int slot = s % TC_NR, c = s % TC_NC;
@@ -520,27 +549,18 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
       }
       const int tl = h.tile;
       if (tl >= 0) {
-        const uint8_t* raw = sm + SM_RAW + slot * 32768;
+        const uint32_t raw = base + SM_RAW + slot * 32768;
 #pragma unroll
-        for (int j2 = 0; j2 < 2; j2++) {  // 32 entries at a time: e0 = 64 kh + 32 j2
-          uint32_t w[16];  // entry pairs (e0 + 2i, e0 + 2i + 1) of line m
+        for (int hl = 0; hl < 2; hl++) {  // lines 16 hl .. 16 hl + 15 of the quarter
+          uint32_t w[16];                 // entry pairs, as fragments
           if (h.mode == MODE_ROWDOT) {
-            // box kh [128 lines][64 entries]: chunk j of line m at 16 (j ^ (m % 8))
+            const uint32_t a = raw + row_base + 16 * 128 * hl;
 #pragma unroll
-            for (int j = 0; j < 4; j++) {
-              const uint4 v = *reinterpret_cast<const uint4*>(raw + 16384 * kh + m * 128 +
-                                                              (((4 * j2 + j) ^ (m & 7)) << 4));
-              w[4 * j] = v.x; w[4 * j + 1] = v.y; w[4 * j + 2] = v.z; w[4 * j + 3] = v.w;
-            }
+            for (int g = 0; g < 4; g++) ldmatrix4<false>(a + (((2 * g + lk) ^ l7) << 4), w + 4 * g);
           } else {
-            // box [128 entries][128 lines], no swizzle: line m of entry k at 256 k + 2 m
-            const uint8_t* col = raw + 2 * m + (64 * kh + 32 * j2) * 256;
+            const uint32_t a = raw + col_base + (((4 * (quarter & 1) + 2 * hl + lm) ^ l7) << 4);
 #pragma unroll
-            for (int i = 0; i < 16; i++) {
-              const uint32_t a = *reinterpret_cast<const uint16_t*>(col + (2 * i) * 256);
-              const uint32_t b = *reinterpret_cast<const uint16_t*>(col + (2 * i + 1) * 256);
-              w[i] = __byte_perm(a, b, 0x5410);
-            }
+            for (int g = 0; g < 4; g++) ldmatrix4<true>(a + 16 * 128 * g, w + 4 * g);
           }
           uint32_t lo[16], hi[16];
 #pragma unroll
@@ -549,8 +569,9 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
             lo[i] = bytes_f16x2(t, 0x4240);
             hi[i] = bytes_f16x2(t, 0x4341);
           }
-          tmem_st16(tq + 128 * c + 16 * j2, lo);
-          tmem_st16(tq + 128 * c + 64 + 16 * j2, hi);
+          const uint32_t dst = tq + ((uint32_t)(16 * hl) << 16) + 128 * c;
+          tmem_st_frag(dst, lo);
+          tmem_st_frag(dst + 64, hi);
         }
         tmem_wait_st();
       }
