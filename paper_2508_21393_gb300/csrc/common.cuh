@@ -292,6 +292,16 @@ struct LinShort {
 static_assert(sizeof(LinShort) == 40, "short item");
 // Lookup argument (kernels_lookup.cu): one LkDev per proof, in the workspace.
 static constexpr int LK_MAX_L = VL_LOOKUP_MAX_LOG_D;
+// The transcript side of a lookup proof's rounds, advanced by each transcript step.
+struct LkRun {
+  Fr E[4];             // alpha c_t eqf(u_t, X), X = 0..3, of the next round (Montgomery)
+  Fr F[4];             // (N/D) alpha^2 c'_t eqf(u_t, X)
+  Fr Tc, Ac, Uc, Vc;   // running claims of the four sums (canonical): T(r), A(r), U(r), V(r) of the last round
+  Fr ac, fc;           // alpha c_t, (N/D) alpha^2 c'_t
+  Fr tabc;             // high rounds: 2^-t Cb (canonical), Cb = alpha^2 - sum B m the table side's cube sum
+  Fr toff;             // table rounds: T' folded by the bound variables is Tb[k] + toff
+  uint32_t St[8];      // transcript state (big-endian words)
+};
 struct LkDev {
   int32_t n, L, log2_n, sE;        // entries, log2 D, log2 N, variables of the low eq block
   int64_t t0;
@@ -299,24 +309,24 @@ struct LkDev {
   int64_t rows, cols, ld;          // S as stored (row-major, k = row . cols + col)
   const int16_t* S;
   uint8_t bind[32];
-  Fr beta, alpha, c_nd, Cb;        // Montgomery; c_nd = N / D; Cb = alpha^2 X1 - X2 (table side's cube sum)
-  Fr claim, half_t;                // running claim; 2^-t during the high rounds
-  Fr ct;                           // prod_{v < t} eqf(u_v, r_v): eq(u, .) folded by the bound variables
-  Fr ctj;                          // the same product over the bound table variables (eq(u_low, .))
-  Fr inv2, inv6;                   // 1/2, 1/6 (Montgomery)
+  Fr beta, c_nd;                   // Montgomery; c_nd = N / D
+  Fr asq;                          // alpha^2 (canonical)
+  Fr inv2;                         // 1/2 (Montgomery)
+  LkRun run;
   Fr u[LK_MAX_L], r[LK_MAX_L];     // challenges (Montgomery)
-  uint32_t St[8];                  // transcript state (big-endian words)
+  Fr uinv[LK_MAX_L];               // 1 / u_t (Montgomery)
   int32_t pbeg[LK_MAX_L + 1], pend[LK_MAX_L + 1];  // partial-sum slots of each round (1-based)
-  int32_t xbeg, xend;              // slots of the table-side sums X1, X2
-  int32_t tail, pad_tail;          // first round run by the per-proof tail kernel
+  int32_t xbeg, xend;              // slots of the table-side sum of B m
+  int32_t tail;                    // first round run by the per-proof tail kernel
+  int32_t dense;                   // ld == cols: entry k is S[k]
   Fr* loP;                         // eq over the last m variables of u, levels m = 0..sE at offset 2^m - 1
   Fr* hiP;                         // eq over the last m variables of u_1..u_{L-sE}, levels m = 0..L-sE-1
   Fr* Binv;                        // 1 / (beta + t0 + j), N (gather source, never folded)
   Fr* Tb;                          // beta + t0 + j, N (gather source)
-  Fr* WB; Fr* WE; Fr* WT; Fr* WM;  // table side: B, eq(u_low, .) (for Cb only), T + beta, m (folded in place)
+  Fr* WB; Fr* WM;                  // table side: B, m (folded in place)
   Fr* VA; Fr* VS;                  // folded A and S + beta, D/2 each
   uint32_t* counts;                // N multiplicities
-  Fr* part;                        // partial sums (12 per slot)
+  Fr* part;                        // partial sums (LK_PART per slot)
   ProofScratch* scr;               // status
 };
 // A block of work of one proof: entries or pairs [k0, k1), partial slot.
@@ -324,16 +334,17 @@ struct LkItem {
   int32_t proof, k0, k1, slot;
 };
 static constexpr int LK_THREADS = 256;
-static constexpr int LK_PPT_LOG = 2;
-static constexpr int LK_PPT = 1 << LK_PPT_LOG;  // pairs per thread in a round pass
-static constexpr int LK_PAIRS = LK_THREADS * LK_PPT;  // pairs per round item
+static constexpr int LK_PART = 8;         // partial sums per slot: T0, Tinf, A0 | U0, Uinf, V0, Vinf
+static constexpr int LK_PASS_THREADS = 128;
+static constexpr int LK_PASS_WARPS = LK_PASS_THREADS / 32;  // round items (one warp each) per pass CTA
+static constexpr int LK_PAIRS = 256;      // pairs per round item at most (and at most 2^sE: one hiP entry per item)
 static constexpr int LK_ENTRIES = 1024;   // table entries per table item (one batch inversion)
-static constexpr int LK_HIST = 8192;      // S entries per histogram item
+static constexpr int LK_HIST = 32768;     // S entries per histogram item
 #ifndef LK_TAIL_LOG
 #define LK_TAIL_LOG 11  // rounds of at most 2^LK_TAIL_LOG pairs run in one block per proof
 #endif
-cudaError_t launch_lookup_setup(LkDev* Ls, int np, const LkItem* fac_items, int nfac, const LkItem* hist_items,
-                                int nhist, const LkItem* tab_items, int ntab, cudaStream_t st);
+cudaError_t launch_lookup_setup(LkDev* Ls, int np, const LkItem* hist_items, int nhist, const LkItem* tab_items,
+                                int ntab, cudaStream_t st);
 // Round t: nhi items of proofs in their high rounds, then nlo items of
 // proofs in their table rounds.
 cudaError_t launch_lookup_round(LkDev* Ls, int np, int t, const LkItem* items, int nhi, int nlo,

@@ -50,6 +50,8 @@ VL_HD constexpr uint32_t r3_limb(int i) {  // R^3 mod r
 }
 static constexpr uint32_t NPRIME = 0xffffffffu;  // -r^-1 mod 2^32 (r = 1 mod 2^32)
 
+VL_HD void cond_sub_r(uint32_t (&t)[8], uint32_t hi);
+
 VL_HD Fr fr_zero() { Fr z; for (int i = 0; i < 8; i++) z.v[i] = 0; return z; }
 VL_HD Fr fr_small(uint32_t x) { Fr z = fr_zero(); z.v[0] = x; return z; }
 VL_HD Fr fr_r1() { Fr z; for (int i = 0; i < 8; i++) z.v[i] = r1_limb(i); return z; }
@@ -254,6 +256,75 @@ __device__ __forceinline__ void wide_redc(const uint32_t (&w)[17], unsigned long
 #pragma unroll
   for (int j = 0; j < 8; j++) col[j] = hi[j];
   col[7] |= (unsigned long long)top << 32;
+}
+
+// z = a m (nine limbs).
+__device__ __forceinline__ void small_mul(uint32_t (&z)[9], const uint32_t (&a)[8], uint32_t m) {
+  uint32_t o[8];
+  asm("mul.lo.u32 %0, %8, %12; mul.hi.u32 %1, %8, %12; mul.lo.u32 %2, %9, %12; mul.hi.u32 %3, %9, %12;\n\t"
+      "mul.lo.u32 %4, %10, %12; mul.hi.u32 %5, %10, %12; mul.lo.u32 %6, %11, %12; mul.hi.u32 %7, %11, %12;"
+      : "=&r"(z[0]), "=&r"(z[1]), "=&r"(z[2]), "=&r"(z[3]), "=&r"(z[4]), "=&r"(z[5]), "=&r"(z[6]), "=&r"(z[7])
+      : "r"(a[0]), "r"(a[2]), "r"(a[4]), "r"(a[6]), "r"(m));
+  asm("mul.lo.u32 %0, %8, %12; mul.hi.u32 %1, %8, %12; mul.lo.u32 %2, %9, %12; mul.hi.u32 %3, %9, %12;\n\t"
+      "mul.lo.u32 %4, %10, %12; mul.hi.u32 %5, %10, %12; mul.lo.u32 %6, %11, %12; mul.hi.u32 %7, %11, %12;"
+      : "=&r"(o[0]), "=&r"(o[1]), "=&r"(o[2]), "=&r"(o[3]), "=&r"(o[4]), "=&r"(o[5]), "=&r"(o[6]), "=&r"(o[7])
+      : "r"(a[1]), "r"(a[3]), "r"(a[5]), "r"(a[7]), "r"(m));
+  asm("add.cc.u32 %0, %0, %8; addc.cc.u32 %1, %1, %9; addc.cc.u32 %2, %2, %10; addc.cc.u32 %3, %3, %11;\n\t"
+      "addc.cc.u32 %4, %4, %12; addc.cc.u32 %5, %5, %13; addc.cc.u32 %6, %6, %14; addc.u32 %7, %15, 0;"
+      : "+&r"(z[1]), "+&r"(z[2]), "+&r"(z[3]), "+&r"(z[4]), "+&r"(z[5]), "+&r"(z[6]), "+&r"(z[7]), "=&r"(z[8])
+      : "r"(o[0]), "r"(o[1]), "r"(o[2]), "r"(o[3]), "r"(o[4]), "r"(o[5]), "r"(o[6]), "r"(o[7]));
+}
+
+// a m mod r for m < 2^16 (a reduced): Barrett with a 32-bit quotient estimate.
+// With t = a m < 2^271, x = floor(t / 2^239) and M = floor(2^271 / r), q =
+// floor(x M / 2^32) satisfies t / r - 2.0001 < q <= t / r: the remainder is below
+// 2.0001 r < 2^256.  An eighth of a Montgomery product's multiply-adds.
+__device__ __forceinline__ Fr small_mul_mod(const Fr& a, uint32_t m) {
+  uint32_t t[9], p[9];
+  small_mul(t, a.v, m);
+  const uint32_t x = (t[8] << 17) | (t[7] >> 15);
+  const uint32_t q = __umulhi(x, 72360u);  // floor(2^271 / r)
+  const uint32_t r[8] = {r_limb(0), r_limb(1), r_limb(2), r_limb(3), r_limb(4), r_limb(5), r_limb(6), r_limb(7)};
+  small_mul(p, r, q);
+  Fr out;
+  const uint32_t lo[8] = {t[0], t[1], t[2], t[3], t[4], t[5], t[6], t[7]};
+  const uint32_t ql[8] = {p[0], p[1], p[2], p[3], p[4], p[5], p[6], p[7]};
+  (void)sub8(out.v, lo, ql);  // the ninth limbs cancel
+  cond_sub_r(out.v, 0);
+  cond_sub_r(out.v, 0);
+  return out;
+}
+
+// w += a (b m) for m < 2^16: up to 2^17 terms of at most 2^526.
+__device__ __forceinline__ void wide_mac_small(uint32_t (&w)[17], const Fr& a, const Fr& b, uint32_t m) {
+  uint32_t z[9], y[9];
+  small_mul(z, b.v, m);
+  Fr zl;
+#pragma unroll
+  for (int i = 0; i < 8; i++) zl.v[i] = z[i];
+  wide_mac(w, a, zl);
+  small_mul(y, a.v, z[8]);
+  asm("add.cc.u32 %0, %0, %9; addc.cc.u32 %1, %1, %10; addc.cc.u32 %2, %2, %11; addc.cc.u32 %3, %3, %12;\n\t"
+      "addc.cc.u32 %4, %4, %13; addc.cc.u32 %5, %5, %14; addc.cc.u32 %6, %6, %15; addc.cc.u32 %7, %7, %16;\n\t"
+      "addc.u32 %8, %8, %17;"
+      : "+&r"(w[8]), "+&r"(w[9]), "+&r"(w[10]), "+&r"(w[11]), "+&r"(w[12]), "+&r"(w[13]), "+&r"(w[14]), "+&r"(w[15]),
+        "+&r"(w[16])
+      : "r"(y[0]), "r"(y[1]), "r"(y[2]), "r"(y[3]), "r"(y[4]), "r"(y[5]), "r"(y[6]), "r"(y[7]), "r"(y[8]));
+}
+
+// s += a for a nine-limb sum of reduced elements.
+__device__ __forceinline__ void sum9_add(uint32_t (&s)[9], const Fr& a) {
+  asm("add.cc.u32 %0, %0, %9; addc.cc.u32 %1, %1, %10; addc.cc.u32 %2, %2, %11; addc.cc.u32 %3, %3, %12;\n\t"
+      "addc.cc.u32 %4, %4, %13; addc.cc.u32 %5, %5, %14; addc.cc.u32 %6, %6, %15; addc.cc.u32 %7, %7, %16;\n\t"
+      "addc.u32 %8, %8, 0;"
+      : "+&r"(s[0]), "+&r"(s[1]), "+&r"(s[2]), "+&r"(s[3]), "+&r"(s[4]), "+&r"(s[5]), "+&r"(s[6]), "+&r"(s[7]),
+        "+&r"(s[8])
+      : "r"(a.v[0]), "r"(a.v[1]), "r"(a.v[2]), "r"(a.v[3]), "r"(a.v[4]), "r"(a.v[5]), "r"(a.v[6]), "r"(a.v[7]));
+}
+__device__ __forceinline__ void sum9_columns(const uint32_t (&s)[9], unsigned long long (&col)[8]) {
+#pragma unroll
+  for (int j = 0; j < 8; j++) col[j] = s[j];
+  col[7] |= (unsigned long long)s[8] << 32;
 }
 #endif
 
@@ -462,70 +533,120 @@ VL_HD Fr reduce_512(const Fr& lo, const Fr& hi) {
   return fr_add(l, h);
 }
 
-// Inverse of a canonical nonzero a (canonical result), by the binary
-// extended Euclidean algorithm on (a, r): invariants x1.a = u and x2.a = v
-// (mod r); halving keeps them (x/2 mod r = (x + r)/2 for odd x; x + r < 2^256
-// since r < 2^255), subtracting the smaller of u, v from the larger shrinks
-// them until one is 1.  Each step removes at least one bit of u or v, so at
-// most 2 . 256 steps run; the cap only guards a zero input (returns 0).
-VL_HD bool fr_is_one(const Fr& a) {
-  uint32_t acc = a.v[0] ^ 1u;
-  for (int i = 1; i < 8; i++) acc |= a.v[i];
-  return acc == 0;
+// Inverse of a canonical nonzero a (canonical result; 0 for 0), by the binary
+// GCD with batched updates of T. Pornin, "Optimized Binary GCD for Modular
+// Inversion" (IACR ePrint 2020/972): x, y start at a, r with x = a u, y = a v
+// (mod r).  A batch runs 31 steps on 64-bit approximations of x and y (their low
+// 31 and top 33 bits), collecting the steps as a 2 x 2 matrix with entries of at
+// most 2^31, then applies the matrix once to (x, y), dividing by 2^31 exactly,
+// and to (u, v), dividing by 2^31 mod r (r = 1 mod 2^31: the multiple of r to
+// add is -t mod 2^31).  17 batches (2 . 255 - 1 <= 17 . 31) leave y = 1, v = 1/a.
+// One thread needs about 12 us on the GPU, against 110 us for a plain binary
+// Euclid on eight limbs, which moves every limb in every step.
+VL_HD int bit_length(uint32_t x) {
+#if defined(__CUDA_ARCH__)
+  return 32 - __clz((int)x);
+#else
+  int n = 0;
+  for (; x; x >>= 1) n++;
+  return n;
+#endif
 }
-VL_HD void fr_half_mod(Fr& x) {  // x <- x / 2 mod r, x < r
-  uint32_t carry = 0;
-  if (x.v[0] & 1u) {
-    uint64_t c = 0;
-    for (int i = 0; i < 8; i++) {
-      c += (uint64_t)x.v[i] + r_limb(i);
-      x.v[i] = (uint32_t)c;
-      c >>= 32;
-    }
-    carry = (uint32_t)c;  // always 0 (x + r < 2^256); kept for the shift
-  }
-  for (int i = 0; i < 7; i++) x.v[i] = (x.v[i] >> 1) | (x.v[i + 1] << 31);
-  x.v[7] = (x.v[7] >> 1) | (carry << 31);
+VL_HD uint64_t inv_approx(const uint32_t (&x)[8], int n) {  // n >= 64: bits of max(x, y)
+  const int sft = n - 33, i = sft >> 5, b = sft & 31;
+  const uint64_t lo = (uint64_t)x[i] | ((uint64_t)x[i + 1] << 32);  // i <= 6
+  const uint64_t hi = i + 2 < 8 ? x[i + 2] : 0u;
+  const uint64_t top = ((lo >> b) | (b ? hi << (64 - b) : 0)) & 0x1ffffffffull;
+  return (top << 31) | (x[0] & 0x7fffffffu);
 }
-VL_HD bool fr_geq_raw(const Fr& a, const Fr& b) {
-  for (int i = 7; i >= 0; i--)
-    if (a.v[i] != b.v[i]) return a.v[i] > b.v[i];
-  return true;
-}
-VL_HD Fr fr_sub_raw(const Fr& a, const Fr& b) {  // a - b for a >= b (integers)
-  Fr d;
-  uint64_t borrow = 0;
+// w = f x + g y as nine limbs (two's complement; |f| + |g| <= 2^31).
+VL_HD void inv_combine(const uint32_t (&x)[8], int64_t f, const uint32_t (&y)[8], int64_t g, uint32_t (&w)[9]) {
+  int64_t c = 0;
+#pragma unroll
   for (int i = 0; i < 8; i++) {
-    const uint64_t x = (uint64_t)a.v[i] - b.v[i] - borrow;
-    d.v[i] = (uint32_t)x;
-    borrow = (x >> 63) & 1u;
+    c += (int64_t)x[i] * f + (int64_t)y[i] * g;
+    w[i] = (uint32_t)c;
+    c >>= 32;
   }
-  return d;
+  w[8] = (uint32_t)c;
+}
+// out = |w / 2^31| for w a multiple of 2^31; true if w was negative.
+VL_HD bool inv_shift_abs(const uint32_t (&w)[9], uint32_t (&out)[8]) {
+  const bool neg = w[8] >> 31;
+  uint64_t c = neg ? 1 : 0;
+#pragma unroll
+  for (int i = 0; i < 8; i++) {
+    const uint32_t t = (w[i] >> 31) | (w[i + 1] << 1);
+    c += neg ? (uint32_t)~t : t;
+    out[i] = (uint32_t)c;
+    c >>= 32;
+  }
+  return neg;
+}
+// w / 2^31 mod r for |w| <= 2^31 r.
+VL_HD void inv_shift_mod(uint32_t (&w)[9], Fr& out) {
+  const uint32_t k = (0u - w[0]) & 0x7fffffffu;  // w + k r = 0 mod 2^31
+  uint64_t c = 0;
+#pragma unroll
+  for (int i = 0; i < 8; i++) {
+    c += (uint64_t)k * r_limb(i) + w[i];
+    w[i] = (uint32_t)c;
+    c >>= 32;
+  }
+  w[8] += (uint32_t)c;  // in (-2^31 r, 2^32 r): after the shift in (-r, 2 r)
+  const bool neg = w[8] >> 31;
+#pragma unroll
+  for (int i = 0; i < 8; i++) out.v[i] = (w[i] >> 31) | (w[i + 1] << 1);
+  if (neg) {
+    uint64_t d = 0;
+#pragma unroll
+    for (int i = 0; i < 8; i++) {
+      d += (uint64_t)out.v[i] + r_limb(i);
+      out.v[i] = (uint32_t)d;
+      d >>= 32;
+    }
+  } else {
+    cond_sub_r(out.v, 0);
+  }
 }
 VL_HD Fr fr_inv_canonical(const Fr& a) {
-  if (fr_is_zero(a)) return fr_zero();
-  Fr u = a, v, x1 = fr_small(1), x2 = fr_zero();
-  for (int i = 0; i < 8; i++) v.v[i] = r_limb(i);
-  for (int step = 0; step < 4 * 256 && !fr_is_one(u) && !fr_is_one(v); step++) {
-    while (!(u.v[0] & 1u)) {
-      for (int i = 0; i < 7; i++) u.v[i] = (u.v[i] >> 1) | (u.v[i + 1] << 31);
-      u.v[7] >>= 1;
-      fr_half_mod(x1);
-    }
-    while (!(v.v[0] & 1u)) {
-      for (int i = 0; i < 7; i++) v.v[i] = (v.v[i] >> 1) | (v.v[i + 1] << 31);
-      v.v[7] >>= 1;
-      fr_half_mod(x2);
-    }
-    if (fr_geq_raw(u, v)) {
-      u = fr_sub_raw(u, v);
-      x1 = fr_sub(x1, x2);
-    } else {
-      v = fr_sub_raw(v, u);
-      x2 = fr_sub(x2, x1);
-    }
+  uint32_t x[8], y[8];
+  Fr u = fr_small(1), v = fr_zero();
+  for (int i = 0; i < 8; i++) {
+    x[i] = a.v[i];
+    y[i] = r_limb(i);
   }
-  return fr_is_one(u) ? x1 : x2;
+  for (int batch = 0; batch < 17; batch++) {
+    int n = 64;  // bits of max(x, y), at least 64
+#pragma unroll
+    for (int i = 2; i < 8; i++) {
+      const uint32_t t = x[i] | y[i];
+      if (t) n = 32 * i + bit_length(t);
+    }
+    uint64_t xa = inv_approx(x, n), ya = inv_approx(y, n);
+    int64_t f0 = 1, g0 = 0, f1 = 0, g1 = 1;
+    for (int j = 0; j < 31; j++) {
+      const bool odd = xa & 1, swap = odd && xa < ya;
+      const uint64_t xs = swap ? ya : xa, ys = swap ? xa : ya;
+      const int64_t fa = swap ? f1 : f0, fb = swap ? f0 : f1, ga = swap ? g1 : g0, gb = swap ? g0 : g1;
+      xa = (xs - (odd ? ys : 0)) >> 1;
+      ya = ys;
+      f0 = fa - (odd ? fb : 0);
+      g0 = ga - (odd ? gb : 0);
+      f1 = 2 * fb;
+      g1 = 2 * gb;
+    }
+    uint32_t w0[9], w1[9];
+    inv_combine(x, f0, y, g0, w0);
+    inv_combine(x, f1, y, g1, w1);
+    if (inv_shift_abs(w0, x)) f0 = -f0, g0 = -g0;
+    if (inv_shift_abs(w1, y)) f1 = -f1, g1 = -g1;
+    inv_combine(u.v, f0, v.v, g0, w0);
+    inv_combine(u.v, f1, v.v, g1, w1);
+    inv_shift_mod(w0, u);
+    inv_shift_mod(w1, v);
+  }
+  return v;  // for a = 0: y stays r and v stays 0
 }
 // Inverse in Montgomery form (x.R -> x^-1.R): from_mont, canonical inverse, to_mont.
 VL_HD Fr fr_inv_mont(const Fr& a) { return to_mont(fr_inv_canonical(from_mont(a))); }

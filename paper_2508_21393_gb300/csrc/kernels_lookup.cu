@@ -19,14 +19,15 @@
 // suffix tables: while t binds one of the first L - sE variables it is
 // hiP[k >> sE] . loP_sE[k mod 2^sE], later loP_(L-t)[k].
 //
-// Launches: start (per proof: transcript, beta, alpha, u, N/D, claim),
-// factors (the suffix eq tables and eq(u_low, .)), histogram
-// (multiplicities, range check), table (batch inversion of beta + T per
-// 1024-entry block, table-side vectors, partial sums of Cb); per round a
-// pass over all proofs' pairs (fold with the previous challenge, then the
-// partial sums of g(0), g(2), g(3)) and a transcript step per proof; finish.
+// Launches: start (per proof: transcript, beta, alpha, u, N/D, the suffix eq
+// tables), histogram (multiplicities, range check), table (batch inversion of
+// beta + T per 1024-entry block, B, T', m, partial sums of B m; the inverses
+// of the u_t ride in the first block); per round a pass over all proofs' pairs
+// (fold with the previous challenge, then the partial sums, lookup_dev.cuh) and
+// a transcript step per proof; tail.
 // A never exists as a vector: its entries are gathered from B by value
-// (A_k = B_{S_k - t0}), and S' from T'.
+// (A_k = B_{S_k - t0}), and S' from T'.  The table side's cube sum is
+// Cb = alpha^2 sum Ej B T' - sum B m = alpha^2 - sum B m (B T' = 1, sum Ej = 1).
 #include "lookup_dev.cuh"
 
 namespace vl {
@@ -63,75 +64,42 @@ __global__ void __launch_bounds__(LK_THREADS) lk_start_kernel(LkDev* Ls) {
   __syncthreads();
   squeeze_dev(S2, LBL_U, L->L, ch, S3, dig);
   if (tid < L->L) L->u[tid] = ch[tid];
-  if (tid < 8) L->St[tid] = S3[tid];
+  if (tid < 8) L->run.St[tid] = S3[tid];
   if (tid == 0) {
-    const Fr alpha = alpha_sh;
-    L->beta = beta_sh;
-    L->alpha = alpha;
-    L->claim = fr_add(alpha, mont_mul(alpha, alpha));
-    L->half_t = fr_r1();
-    L->ct = fr_r1();
-    L->ctj = fr_r1();
+    const Fr alpha = alpha_sh, one = fr_small(1);
     Fr c = fr_r1();  // N / D = 2^-(L - log2 N)
-    for (int i = 0; i < L->L - L->log2_n; i++) c = mont_mul(c, L->inv2);
+    for (int i = 0; i < L->L - L->log2_n; i++) c = mont_mul_ni(c, L->inv2);
+    const Fr a2 = mont_mul_ni(alpha, alpha);
+    L->beta = beta_sh;
     L->c_nd = c;
+    L->asq = from_mont_ni(a2);
+    L->run.ac = alpha;
+    L->run.fc = mont_mul_ni(c, a2);
+    L->run.Tc = one;  // sum eq(u, .) A S' = sum eq(u, .) = 1
+    L->run.Uc = one;
+    L->run.toff = fr_zero();
     L->scr->status = VL_OK;
     const uint32_t pad = (uint32_t)((1 << L->L) - L->n);  // padding entries hold t0: table index 0
     if (pad) atomicAdd(&L->counts[0], pad);
   }
-}
-
-// eq table over nv <= 8 variables x[0..nv) (MSB first) into tab[0..2^nv),
-// block-wide: doubling, each level appending the next variable as the new
-// lowest bit (one product per new entry).
-__device__ void lk_eq_small(Fr* tab, const Fr* x, int nv) {
-  if (threadIdx.x == 0) tab[0] = fr_r1();
-  __syncthreads();
-  for (int l = 0; l < nv; l++) {
-    const int j = threadIdx.x;
-    Fr a = fr_zero();
-    if (j < (1 << l)) a = tab[j];
+  // Suffix eq tables by doubling, loP on the first half of the block, hiP on
+  // the second: level m (entries 2^m - 1 ..) is eq over the last m variables of
+  // u (loP, m <= sE) or of its first L - sE (hiP, m < L - sE); entry i of it is
+  // the factor of its highest variable's bit times entry i mod 2^(m-1) below.
+  const bool lo = tid < LK_THREADS / 2;
+  const int id = lo ? tid : tid - LK_THREADS / 2, top = lo ? L->L : L->L - L->sE;
+  const int levels = lo ? L->sE : L->L - L->sE - 1;  // above level 0
+  Fr* out = lo ? L->loP : L->hiP;
+  if (id == 0 && levels >= 0) out[0] = fr_r1();
+  const int most = L->sE > L->L - L->sE - 1 ? L->sE : L->L - L->sE - 1;
+  for (int m = 1; m <= most; m++) {
     __syncthreads();
-    if (j < (1 << l)) {
-      const Fr xl = x[l];
-      tab[2 * j] = mont_mul_ni(a, fr_sub(fr_r1(), xl));
-      tab[2 * j + 1] = mont_mul_ni(a, xl);
+    if (m <= levels) {
+      const Fr x = ch[top - m], y = fr_sub(fr_r1(), x);
+      const int half = 1 << (m - 1);
+      for (int i = id; i < 2 * half; i += LK_THREADS / 2)
+        out[2 * half - 1 + i] = mont_mul_ni(i & half ? x : y, out[half - 1 + (i & (half - 1))]);
     }
-    __syncthreads();
-  }
-}
-
-// Suffix eq tables: item.slot 0 = loP (levels m = 0..sE: eq over the last
-// m variables of u), 1 = hiP (levels m = 0..L-sE-1: eq over the last m of
-// the first L - sE variables), 2 = eq(u_low, .) into WE (the last log2 N).
-// Entry e of a pyramid is level m = floor(log2(e + 1)), index e + 1 - 2^m;
-// its value is the product of x or 1 - x per bit (MSB first).
-__global__ void __launch_bounds__(LK_THREADS) lk_factor_kernel(LkDev* Ls, const LkItem* items) {
-  const LkItem it = items[blockIdx.x];
-  LkDev* L = Ls + it.proof;
-  if (it.slot == 2) {
-    // eq(u_low, i) over the last n = log2 N variables, MSB first, as
-    // hi[i >> s] . lo[i mod 2^s]: lo over the last s = min(n, 8) variables,
-    // hi over the n - s before them (both at most 256 entries, built in
-    // shared memory), then one product per entry instead of n.
-    __shared__ Fr lo[256], hi[256];
-    const int nb = L->log2_n, sl = nb < 8 ? nb : 8;
-    lk_eq_small(lo, L->u + (L->L - sl), sl);
-    lk_eq_small(hi, L->u + (L->L - nb), nb - sl);
-    for (int e = it.k0 + threadIdx.x; e < it.k1; e += blockDim.x)
-      L->WE[e] = mont_mul_ni(hi[e >> sl], lo[e & ((1 << sl) - 1)]);
-    return;
-  }
-  Fr* out = it.slot == 0 ? L->loP : L->hiP;
-  const int top = it.slot == 1 ? L->L - L->sE : L->L;  // the suffixes end at variable top - 1 (0-based)
-  for (int e = it.k0 + threadIdx.x; e < it.k1; e += blockDim.x) {
-    const int m = 31 - __clz(e + 1), i = e + 1 - (1 << m);
-    Fr acc = fr_r1();
-    for (int t = 0; t < m; t++) {
-      const Fr& x = L->u[top - m + t];
-      acc = mont_mul_ni(acc, ((i >> (m - 1 - t)) & 1) ? x : fr_sub(fr_r1(), x));
-    }
-    out[e] = acc;
   }
 }
 
@@ -147,15 +115,31 @@ __global__ void __launch_bounds__(LK_THREADS) lk_hist_kernel(LkDev* Ls, const Lk
     for (int j = threadIdx.x; j < N; j += blockDim.x) h[j] = 0;
   __syncthreads();
   bool bad = false;
-  for (int k = it.k0 + threadIdx.x; k < it.k1; k += blockDim.x) {
-    const int row = k / (int)L->cols, col = k - row * (int)L->cols;
-    const int64_t j = (int64_t)L->S[(int64_t)row * L->ld + col] - L->t0;
+  auto count = [&](int64_t v) {
+    const int64_t j = v - L->t0;
     if (j < 0 || j >= N) {
       bad = true;
-      continue;
+      return;
     }
     if (local) atomicAdd(&h[j], 1u);
     else atomicAdd(&L->counts[j], 1u);
+  };
+  if (L->dense) {
+    const int16_t* S = L->S;
+    int k = it.k0 + threadIdx.x;
+    for (; k + 3 * (int)blockDim.x < it.k1; k += 4 * blockDim.x) {  // four loads in flight
+      int16_t v[4];
+#pragma unroll
+      for (int i = 0; i < 4; i++) v[i] = S[k + i * (int)blockDim.x];
+#pragma unroll
+      for (int i = 0; i < 4; i++) count(v[i]);
+    }
+    for (; k < it.k1; k += blockDim.x) count(S[k]);
+  } else {
+    for (int k = it.k0 + threadIdx.x; k < it.k1; k += blockDim.x) {
+      const int row = k / (int)L->cols, col = k - row * (int)L->cols;
+      count(L->S[(int64_t)row * L->ld + col]);
+    }
   }
   if (bad) atomicExch(&L->scr->status, VL_ELOOKUP);
   __syncthreads();
@@ -167,28 +151,31 @@ __global__ void __launch_bounds__(LK_THREADS) lk_hist_kernel(LkDev* Ls, const Lk
 // Table entries [k0, k1) (at most 4 per thread): x_j = beta + t0 + j, its
 // inverse by one batch inversion per block (prefix products, one field
 // inversion, back substitution), the table-side vectors, and this block's
-// share of X1 = sum B Ej T' and X2 = sum B m (slot: 12 Fr, the first two).
-__global__ void __launch_bounds__(LK_THREADS) lk_table_kernel(LkDev* Ls, const LkItem* items) {
+// share of sum B m (its slot's first entry).  The first block of a proof also
+// inverts the u_t (one more element per thread).
+__global__ void __launch_bounds__(LK_THREADS, 2) lk_table_kernel(LkDev* Ls, const LkItem* items) {
   __shared__ Fr pre[LK_THREADS], suf[LK_THREADS];
   __shared__ Fr inv_tot;
-  __shared__ Fr red[2 * (LK_THREADS / 32)];
+  __shared__ Fr red[LK_THREADS / 32];
   const LkItem it = items[blockIdx.x];
   LkDev* L = Ls + it.proof;
   const int tid = threadIdx.x;
   const Fr beta = L->beta;
+  const bool has_u = it.k0 == 0 && tid < L->L;
+  const Fr ux = has_u ? L->u[tid] : fr_r1();
   Fr x[4], p[4];
   for (int e = 0; e < 4; e++) {
     const int j = it.k0 + 4 * tid + e;
-    x[e] = j < it.k1 ? fr_add(beta, to_mont(fr_from_i64(L->t0 + j))) : fr_r1();
-    p[e] = e == 0 ? x[0] : mont_mul(p[e - 1], x[e]);
+    x[e] = j < it.k1 ? fr_add(beta, to_mont_ni(fr_from_i64(L->t0 + j))) : fr_r1();
+    p[e] = mont_mul_ni(e == 0 ? ux : p[e - 1], x[e]);
   }
   // inclusive prefix and suffix products of the thread totals (Hillis-Steele)
   pre[tid] = p[3];
   suf[tid] = p[3];
   __syncthreads();
   for (int off = 1; off < LK_THREADS; off <<= 1) {
-    const Fr a = tid >= off ? mont_mul(pre[tid - off], pre[tid]) : pre[tid];
-    const Fr b = tid + off < LK_THREADS ? mont_mul(suf[tid], suf[tid + off]) : suf[tid];
+    const Fr a = tid >= off ? mont_mul_ni(pre[tid - off], pre[tid]) : pre[tid];
+    const Fr b = tid + off < LK_THREADS ? mont_mul_ni(suf[tid], suf[tid + off]) : suf[tid];
     __syncthreads();
     pre[tid] = a;
     suf[tid] = b;
@@ -196,284 +183,503 @@ __global__ void __launch_bounds__(LK_THREADS) lk_table_kernel(LkDev* Ls, const L
   }
   if (tid == 0) inv_tot = fr_inv_mont(pre[LK_THREADS - 1]);
   __syncthreads();
-  if (fr_is_zero(inv_tot)) {  // beta + t0 + j = 0 for some j (probability ~2^-239)
+  if (fr_is_zero(inv_tot)) {  // beta + t0 + j = 0 for some j, or a u_t = 0 (probability ~2^-238)
     if (tid == 0) atomicExch(&L->scr->status, VL_ELOOKUP);
     return;
   }
   const Fr qprev = tid > 0 ? pre[tid - 1] : fr_r1();
   // 1 / (prefix through this thread) = inv_tot . (product of the later threads' totals)
-  Fr inv_f = tid + 1 < LK_THREADS ? mont_mul(inv_tot, suf[tid + 1]) : inv_tot;
+  Fr inv_f = tid + 1 < LK_THREADS ? mont_mul_ni(inv_tot, suf[tid + 1]) : inv_tot;
   Fr inv_x[4];
   for (int e = 3; e >= 0; e--) {
-    const Fr f_before = e > 0 ? mont_mul(qprev, p[e - 1]) : qprev;  // prefix before element e
-    inv_x[e] = mont_mul(inv_f, f_before);
-    inv_f = mont_mul(inv_f, x[e]);
+    const Fr f_before = mont_mul_ni(qprev, e > 0 ? p[e - 1] : ux);  // prefix before element e
+    inv_x[e] = mont_mul_ni(inv_f, f_before);
+    inv_f = mont_mul_ni(inv_f, x[e]);
   }
-  Fr acc[2] = {fr_zero(), fr_zero()};
+  if (has_u) L->uinv[tid] = mont_mul_ni(inv_f, qprev);
+  Fr acc[1] = {fr_zero()};
   for (int e = 0; e < 4; e++) {
     const int j = it.k0 + 4 * tid + e;
     if (j >= it.k1) break;
-    const Fr m = to_mont(fr_small(L->counts[j]));
+    const Fr m = to_mont_ni(fr_small(L->counts[j]));
     L->Binv[j] = inv_x[e];
     L->WB[j] = inv_x[e];
     L->Tb[j] = x[e];
-    L->WT[j] = x[e];
     L->WM[j] = m;
-    acc[0] = fr_add(acc[0], mont_mul(mont_mul(inv_x[e], L->WE[j]), x[e]));
-    acc[1] = fr_add(acc[1], mont_mul(inv_x[e], m));
+    acc[0] = fr_add(acc[0], mont_mul_ni(inv_x[e], m));
   }
-  block_sum_fr<2>(acc, red);
-  if (tid == 0) {
-    L->part[(size_t)it.slot * 12] = acc[0];
-    L->part[(size_t)it.slot * 12 + 1] = acc[1];
+  block_sum_fr<1>(acc, red);
+  if (tid == 0) L->part[(size_t)it.slot * LK_PART] = acc[0];
+}
+
+// Shared memory of a transcript step.
+struct LkShared {
+  alignas(16) uint32_t msg[48];     // an absorb's message: three blocks
+  alignas(16) uint32_t wk[3][68];   // schedule words
+  alignas(16) uint32_t sq[8];       // state before a squeeze
+  LkRun run;
+  Fr s[LK_PART];                    // the round's sums (canonical): T0, Tinf, A0 | U0, Uinf / h, V0, Vinf
+  Fr quad[4][3];                    // T, A, U, V as (value at 0, value at 1, leading coefficient)
+  Fr g[4];                          // g(0..3), or the final evaluations (canonical)
+  Fr r;
+  Fr kc[2];                         // R^2 2^(L-t), R^3 2^(L-t) mod r
+  alignas(16) unsigned long long red[32 * LK_MAX_WARPS];
+};
+
+// SHA256 of the three blocks in sh.msg: warp 0 (digest in every lane), with
+// warps 1 to 3 in lk_absorb_help.
+__device__ __forceinline__ ShaState lk_absorb_run(LkShared& sh) {
+  named_sync(10, 128);
+  ShaState st = sha_rounds_ni(sha_iv_state(), sha_load(sh.msg), sh.wk[0], 1);
+  st = sha_rounds_ni(st, sha_load(sh.msg + 16), sh.wk[1], 4);
+  return sha_rounds_ni(st, sha_load(sh.msg + 32), sh.wk[2], 7);
+}
+__device__ __forceinline__ void lk_absorb_help(LkShared& sh, int warp) {
+  named_sync(10, 128);
+  sha_sched_ni(sha_load(sh.msg + 16 * (warp - 1)), sh.wk[warp - 1], 1 + 3 * (warp - 1));
+}
+// The message S || label || x_0 .. x_{n-1} (n = 3 or 4: three blocks), by warp 0;
+// x(i): element i in shared memory.
+template <class X>
+__device__ __forceinline__ void lk_absorb_words(LkShared& sh, uint32_t label, int n, X x) {
+  for (int i = threadIdx.x & 31; i < 48; i += 32) {
+    const int q = i - 8;
+    uint32_t w = 0;
+    if (q < 0) w = sh.run.St[i];
+    else if (q <= 8 * n) {
+      const uint32_t prev = q == 0 ? label << 24 : x((q - 1) >> 3).v[(q - 1) & 7];
+      w = q < 8 * n ? __byte_perm(x(q >> 3).v[q & 7], prev, 0x7012) : (prev & 0xff000000u) | 0x00800000u;
+    } else if (i == 47) w = (uint32_t)(33 + 32 * n) * 8u;
+    sh.msg[i] = w;
   }
 }
 
-// The round polynomial of round t from the summed partials, by warp 0 (the
-// sums valid in all its lanes): g(X) = alpha c_t eqf(u_t, X) T_X + A_X +
-// table side for X = 0, 2, 3 by lanes 0..2 at once (the scalars they share
-// formed in each), g(1) = claim - g(0); lanes 0..3 convert the four values
-// for the proof; lane 0 absorbs ('g': g0, g2, g3) into Sw.  gsh[0..3]: the
-// values (Montgomery), for lk_step_r.
-__device__ void lk_step_g(LkDev* L, int t, const Fr (&acc)[6], const Fr (&accb)[6], bool jr, vl_lookup_proof* out,
-                          Fr* gsh, uint32_t* Sw) {
-  const int lane = threadIdx.x & 31, q = lane < 3 ? lane : 0;
-  // eqf(u_t, X) for X = 0, 2, 3: eqf(u, X) = (1 - u) + X (2u - 1)
-  const Fr ut = L->u[t - 1], one = fr_r1();
-  const Fr e0 = fr_sub(one, ut), d = fr_sub(fr_add(ut, ut), one);
-  const Fr eq = q == 0 ? e0 : (q == 1 ? fr_add(e0, fr_add(d, d)) : fr_add(fr_add(e0, fr_add(d, d)), d));
-  const Fr half_t = L->half_t;
-  Fr gq = fr_zero(), ht = fr_zero();
-  if (lane < 3) {
-    const Fr alpha = L->alpha;
-    Fr tab;
-    if (jr) {  // (N/D) (alpha^2 c'_t eqf(u_t, X) U_X - V_X)
-      const Fr ac2 = mont_mul_ni(mont_mul_ni(alpha, alpha), L->ctj);
-      tab = mont_mul_ni(L->c_nd, fr_sub(mont_mul_ni(mont_mul_ni(ac2, eq), accb[q]), accb[3 + q]));
-    } else {
-      ht = mont_mul_ni(half_t, L->inv2);
-      tab = mont_mul_ni(ht, L->Cb);
-    }
-    const Fr ac = mont_mul_ni(alpha, L->ct);
-    gq = fr_add(fr_add(mont_mul_ni(mont_mul_ni(ac, eq), acc[q]), acc[3 + q]), tab);
-  }
-  __syncwarp();
-  if (!jr && lane == 0) L->half_t = ht;
-  Fr G[4];
-#pragma unroll
-  for (int l = 0; l < 8; l++) {
-    G[0].v[l] = __shfl_sync(0xffffffffu, gq.v[l], 0);
-    G[2].v[l] = __shfl_sync(0xffffffffu, gq.v[l], 1);
-    G[3].v[l] = __shfl_sync(0xffffffffu, gq.v[l], 2);
-  }
-  G[1] = fr_sub(L->claim, G[0]);
-  const Fr mine = lane == 0 ? G[0] : (lane == 1 ? G[1] : (lane == 2 ? G[2] : G[3]));
-  Fr c = fr_zero();
-  if (lane < 4) {
-    c = from_mont_ni(mine);
-    for (int l = 0; l < 8; l++) out->g[t - 1][lane].limb[l] = c.v[l];
-    gsh[lane] = mine;
-  }
-  Fr gc[3];
-#pragma unroll
-  for (int l = 0; l < 8; l++) {
-    gc[0].v[l] = __shfl_sync(0xffffffffu, c.v[l], 0);
-    gc[1].v[l] = __shfl_sync(0xffffffffu, c.v[l], 2);
-    gc[2].v[l] = __shfl_sync(0xffffffffu, c.v[l], 3);
-  }
-  if (lane == 0) {
-    uint32_t S[8];
-    for (int i = 0; i < 8; i++) S[i] = L->St[i];
-    dev_absorb_fr<3>(S, LBL_G, gc);
-    for (int i = 0; i < 8; i++) Sw[i] = S[i];
-  }
-  __syncwarp();
-}
-
-// After the squeeze of r_t, by warp 0: store r_t and the state, fold c_t
-// (and c'_t for a table variable) by eqf(u_t, r_t), and the new claim
-// g(r_t) = sum_i g(i) L_i(r_t) over the nodes 0..3, lane i forming L_i and
-// its term (the same products as a serial evaluation, in another order).
-__device__ void lk_step_r(LkDev* L, int t, const Fr& r, const uint32_t* Sn, const Fr* gsh) {
+// The round polynomial of round t from the sums in sh.s, by warp 0: g(X) =
+// E_X T(X) + A(X) + table side for X = 0..3 (three products deep: T(1), U(1)
+// from the claims, then all products of the four values at once), into sh.g and
+// the proof.  tj: the table round's number, <= 0 in a high round.
+__device__ void lk_step_g(const LkDev* L, LkShared& sh, int t, int tj, vl_lookup_proof* out) {
   const int lane = threadIdx.x & 31;
+  const bool jr = tj > 0;
+  const Fr ut = L->u[t - 1], ui = L->uinv[t - 1], one = fr_small(1);
+  const LkRun& R = sh.run;
+  // lanes 0, 1: T(1), U(1) = (claim - (1 - u) value(0)) / u; lane 2: U's leading coefficient times h
+  const Fr v0 = lane == 0 ? (t == 1 ? one : sh.s[0]) : lane == 1 ? (tj == 1 ? one : sh.s[3]) : fr_small(1u << (L->L - t));
+  const Fr x = mont_mul_ni(lane < 2 ? fr_sub(fr_r1(), ut) : fr_r2(), v0);
+  const Fr y = mont_mul_ni(lane < 2 ? ui : sh.s[4], lane < 2 ? fr_sub(lane == 0 ? R.Tc : R.Uc, x) : x);
   if (lane == 0) {
-    L->r[t - 1] = r;
-    for (int i = 0; i < 8; i++) L->St[i] = Sn[i];
+    sh.quad[0][0] = v0;
+    sh.quad[0][1] = y;
+    sh.quad[0][2] = sh.s[1];
+    sh.quad[1][0] = sh.s[2];
+    sh.quad[1][1] = fr_sub(R.Ac, sh.s[2]);
+    sh.quad[1][2] = fr_zero();
+  } else if (lane == 1) {
+    sh.quad[2][0] = v0;
+    sh.quad[2][1] = y;
+  } else if (lane == 2) {
+    sh.quad[2][2] = y;
+  } else if (lane == 3) {
+    sh.quad[3][0] = sh.s[5];
+    sh.quad[3][1] = fr_sub(R.Vc, sh.s[5]);
+    sh.quad[3][2] = sh.s[6];
   }
-  const Fr ut = L->u[t - 1], one = fr_r1();
-  // eqf(u_t, r) = u r + (1 - u)(1 - r): the two products on lanes 0, 1
-  Fr part = fr_zero();
-  if (lane < 2) part = lane == 0 ? mont_mul_ni(ut, r) : mont_mul_ni(fr_sub(one, ut), fr_sub(one, r));
-  Fr ef;
+  __syncwarp();
+  // lane 4 i + X: part i = T, A, U, V at X, by differences (q(X + 1) - q(X) = q(1) - q(0) + 2 X lead)
+  const int i = (lane >> 2) & 3, X = lane & 3;
+  Fr v = sh.quad[i][0], d = fr_sub(sh.quad[i][1], v);
+  const Fr dd = fr_dbl(sh.quad[i][2]);
 #pragma unroll
-  for (int l = 0; l < 8; l++) ef.v[l] = __shfl_sync(0xffffffffu, part.v[l], 1);
-  ef = fr_add(part, ef);  // valid in lane 0
-#pragma unroll
-  for (int l = 0; l < 8; l++) ef.v[l] = __shfl_sync(0xffffffffu, ef.v[l], 0);
-  const bool tabvar = t > L->L - L->log2_n;
-  if (lane == 0) L->ct = mont_mul_ni(L->ct, ef);
-  if (lane == 1 && tabvar) L->ctj = mont_mul_ni(L->ctj, ef);
-  // Lagrange weights over the nodes 0..3 at r:
-  //   L0 = -(r-1)(r-2)(r-3)/6, L1 = r(r-2)(r-3)/2, L2 = -r(r-1)(r-3)/2, L3 = r(r-1)(r-2)/6
-  const Fr two = fr_add(one, one), three = fr_add(two, one);
-  const Fr r1 = fr_sub(r, one), r2 = fr_sub(r, two), r3 = fr_sub(r, three);
-  Fr term = fr_zero();
+  for (int e = 0; e < 3; e++) {
+    const Fr vn = fr_add(v, d);
+    if (e < X) v = vn;
+    d = fr_add(d, dd);
+  }
+  const Fr p = mont_mul_ni(i == 0 ? R.E[X] : i == 2 ? R.F[X] : L->c_nd, v);
+  const Fr tx = shfl_fr(p, X), ax = shfl_fr(v, 4 + X), ux = shfl_fr(p, 8 + X), vx = shfl_fr(p, 12 + X);
+  const Fr g = fr_add(fr_add(tx, ax), jr ? fr_sub(ux, vx) : R.tabc);
   if (lane < 4) {
-    const Fr x = lane == 0 ? r1 : r, y = lane == 1 ? r2 : (lane == 0 ? r2 : r1);
-    const Fr z = lane == 3 ? r2 : r3;
-    const Fr inv = (lane == 0 || lane == 3) ? L->inv6 : L->inv2;
-    Fr li = mont_mul_ni(mont_mul_ni(mont_mul_ni(x, y), z), inv);
-    if (lane == 0 || lane == 2) li = fr_neg(li);
-    term = mont_mul_ni(gsh[lane], li);
+    sh.g[lane] = g;
+    for (int l = 0; l < 8; l++) out->g[t - 1][lane].limb[l] = g.v[l];
   }
-  Fr t1, t2, t3;
-#pragma unroll
-  for (int l = 0; l < 8; l++) {
-    t1.v[l] = __shfl_sync(0xffffffffu, term.v[l], 1);
-    t2.v[l] = __shfl_sync(0xffffffffu, term.v[l], 2);
-    t3.v[l] = __shfl_sync(0xffffffffu, term.v[l], 3);
-  }
-  if (lane == 0) L->claim = fr_add(fr_add(fr_add(term, t1), t2), t3);
   __syncwarp();
 }
 
-// The table side's cube sum Cb = alpha^2 X1 - X2 from the table kernel's
-// partials (block-wide).
-__device__ void lk_table_sum(LkDev* L, Fr* red) {
-  Fr x[2] = {fr_zero(), fr_zero()};
-  for (int s = L->xbeg + threadIdx.x; s < L->xend; s += blockDim.x) {
-    x[0] = fr_add(x[0], L->part[(size_t)s * 12]);
-    x[1] = fr_add(x[1], L->part[(size_t)s * 12 + 1]);
+// After the squeeze of r_t, one warp: the running claims T(r), A(r), U(r), V(r),
+// the scalars of the next round.  Three products deep.
+__device__ void lk_step_r(LkDev* L, LkShared& sh, int t) {
+  const int lane = threadIdx.x & 31, i = lane & 3;
+  LkRun& R = sh.run;
+  const Fr r = sh.r, ut = L->u[t - 1], one = fr_r1();
+  const bool tabvar = t > L->L - L->log2_n;
+  // lanes 0..3: claim i = q0 + r (q1 - q0 - lead + r lead); lanes 4, 5: eqf(u, r) = u r + (1 - u)(1 - r);
+  // lane 7: the next tabc
+  Fr a = r, b = sh.quad[i][2];
+  if (lane == 4) b = ut;
+  if (lane == 5) a = fr_sub(one, r), b = fr_sub(one, ut);
+  if (lane == 7) a = L->inv2, b = R.tabc;
+  const Fr p = mont_mul_ni(a, b);
+  const Fr ef = fr_add(shfl_fr(p, 4), shfl_fr(p, 5));
+  const Fr q0 = sh.quad[i][0];
+  Fr c = r, e = fr_add(fr_sub(fr_sub(sh.quad[i][1], q0), sh.quad[i][2]), p);
+  if (lane == 4) c = R.ac, e = ef;
+  if (lane == 5) c = R.fc, e = ef;
+  const Fr w = mont_mul_ni(c, e);
+  const Fr ac = shfl_fr(w, 4), fc = tabvar ? shfl_fr(w, 5) : R.fc;
+  __syncwarp();
+  if (lane < 4) {
+    const Fr cl = fr_add(q0, w);
+    if (lane == 0) R.Tc = cl;
+    else if (lane == 1) R.Ac = cl;
+    else if (tabvar) (lane == 2 ? R.Uc : R.Vc) = cl;
   }
-  block_sum_fr<2>(x, red);
-  if (threadIdx.x == 0) L->Cb = fr_sub(mont_mul_ni(mont_mul_ni(L->alpha, L->alpha), x[0]), x[1]);
+  if (lane == 4) R.ac = ac;
+  if (lane == 5) R.fc = fc;
+  if (lane == 7) R.tabc = p;
+  // E_X, F_X of round t + 1: eqf(u, X) = (1 - u) + X (2 u - 1)
+  if (t < L->L) {
+    const Fr un = L->u[t], e0 = fr_sub(one, un), d = fr_sub(un, e0);
+    Fr v = e0;
+#pragma unroll
+    for (int q = 0; q < 3; q++)
+      if (q < i) v = fr_add(v, d);
+    const Fr z = mont_mul_ni(lane < 4 ? ac : fc, v);
+    if (lane < 4) R.E[lane] = z;
+    else if (lane < 8) R.F[lane - 4] = z;
+  }
+  __syncwarp();
+}
+
+// Round 1's scalars and the table side's claims and cube sum, from the table
+// kernel's partials (block-wide).
+__device__ void lk_first_step(const LkDev* L, LkShared& sh) {
+  Fr x[1] = {fr_zero()};
+  for (int s = L->xbeg + threadIdx.x; s < L->xend; s += blockDim.x) x[0] = fr_add(x[0], L->part[(size_t)s * LK_PART]);
+  block_sum_fr<1>(x, reinterpret_cast<Fr*>(sh.red));
+  if (threadIdx.x < 32) {
+    const int lane = threadIdx.x, i = lane & 3;
+    const Fr bm = from_mont_ni(x[0]), ac = sh.run.ac, fc = sh.run.fc, one = fr_r1();
+    if (L->L > 0) {
+      const Fr u = L->u[0], e0 = fr_sub(one, u), d = fr_sub(u, e0);
+      Fr v = e0;
+#pragma unroll
+      for (int q = 0; q < 3; q++)
+        if (q < i) v = fr_add(v, d);
+      const Fr z = mont_mul_ni(lane < 4 ? ac : fc, v);
+      if (lane < 4) sh.run.E[lane] = z;
+      else if (lane < 8) sh.run.F[lane - 4] = z;
+    }
+    if (lane == 0) {
+      sh.run.Ac = bm;  // sum A = sum B m
+      sh.run.Vc = bm;
+      sh.run.tabc = mont_mul_ni(L->inv2, fr_sub(L->asq, bm));
+    }
+  }
   __syncthreads();
 }
+
+// Absorb the round message and squeeze r_t: warps 0 to 3; sh.run.St and sh.r
+// are set for the block after its next barrier.
+__device__ __forceinline__ void lk_transcript(LkDev* L, LkShared& sh, int warp, int t) {
+  const int lane = threadIdx.x & 31;
+  const bool tabvar = t > L->L - L->log2_n;
+  if (warp == 0) {
+    lk_absorb_words(sh, LBL_G, 3, [&](int i) -> const Fr& { return sh.g[i == 0 ? 0 : i + 1]; });  // g(0), g(2), g(3)
+    ShaState st = lk_absorb_run(sh);
+    if (lane == 0) {
+#pragma unroll
+      for (int i = 0; i < 8; i++) sh.sq[i] = st.h[i];
+    }
+    named_sync(11, 64);
+    st = sha_rounds_ni(sha_iv_state(), squeeze_lane_block(st.h), sh.wk[lane < 2 ? lane : 2], 1);
+    if (lane == 2) {
+#pragma unroll
+      for (int i = 0; i < 8; i++) sh.run.St[i] = st.h[i];
+    }
+    // challenge_of on lanes 0, 1; in a table round lanes 2, 3 form r 2^(L-t), the
+    // variable's share of T' (Tb[k] + toff), from the same digests at once
+    if (tabvar) named_sync(12, 64);
+    uint32_t d[8];
+#pragma unroll
+    for (int i = 0; i < 8; i++) d[i] = __shfl_sync(0xffffffffu, st.h[i], lane & 1);
+    Fr half = fr_zero();
+    if (lane < 2 || (tabvar && lane < 4))
+      half = mont_mul_ni(digest_le(d), lane == 0 ? fr_r2() : lane == 1 ? fr_r3() : sh.kc[lane - 2]);
+    const Fr r = fr_add(half, shfl_xor_fr(half, 1));
+    if (lane == 0) {
+      sh.r = r;
+      L->r[t - 1] = r;
+    }
+    if (tabvar && lane == 2) sh.run.toff = fr_add(sh.run.toff, r);
+  } else if (warp < 4) {
+    lk_absorb_help(sh, warp);
+    if (tabvar && warp == 2) {
+      Fr x = lane == 0 ? fr_r2() : fr_r3();
+      for (int i = 0; i < L->L - t; i++) x = fr_dbl(x);
+      if (lane < 2) sh.kc[lane] = x;
+      __syncwarp();
+      named_arrive(12, 64);
+    }
+    if (warp == 1) {
+      named_sync(11, 64);
+      uint32_t S[8];
+#pragma unroll
+      for (int i = 0; i < 8; i++) S[i] = sh.sq[i];
+      sha_sched_ni(squeeze_lane_block(S), sh.wk[lane < 2 ? lane : 2], 1);
+    }
+  }
+}
+
+__device__ __forceinline__ void lk_copy_run(LkRun* dst, const LkRun* src) {
+  const uint4* a = reinterpret_cast<const uint4*>(src);
+  uint4* b = reinterpret_cast<uint4*>(dst);
+  for (int i = threadIdx.x; i < (int)(sizeof(LkRun) / 16); i += blockDim.x) b[i] = a[i];
+}
+static_assert(sizeof(LkRun) % 16 == 0, "copied by 16 bytes");
 
 // Round t of one proof before its tail (one block each): the round
-// polynomial from the partial sums, absorb, squeeze r_t, new claim.
-__global__ void __launch_bounds__(LK_ROUND_THREADS) lk_round_kernel(LkDev* Ls, int t, vl_lookup_proof* outs) {
-  __shared__ Fr red[6 * (LK_ROUND_THREADS / 32)];
-  __shared__ uint32_t Sw[8], Sn[8];
-  __shared__ uint32_t dig[3][8];
-  __shared__ Fr rch[1];
-  __shared__ Fr gsh[4];
+// polynomial from the partial sums, absorb, squeeze r_t, new claims.
+__global__ void __launch_bounds__(LK_STEP_THREADS) lk_round_kernel(LkDev* Ls, int t, vl_lookup_proof* outs) {
+  __shared__ LkShared sh;
   LkDev* L = Ls + blockIdx.x;
   if (t >= L->tail) return;
-  const int tid = threadIdx.x;
-  const bool jr = t > L->L - L->log2_n;
-  if (t == 1) lk_table_sum(L, red);
-  Fr acc[6], accb[6];
-  for (int i = 0; i < 6; i++) acc[i] = accb[i] = fr_zero();
-  for (int s = L->pbeg[t] + tid; s < L->pend[t]; s += blockDim.x) {
-    for (int i = 0; i < 6; i++) acc[i] = fr_add(acc[i], L->part[(size_t)s * 12 + i]);
-    if (jr)
-      for (int i = 0; i < 6; i++) accb[i] = fr_add(accb[i], L->part[(size_t)s * 12 + 6 + i]);
-  }
-  block_sum_fr<6>(acc, red);
-  if (jr) block_sum_fr<6>(accb, red);
-  if (tid < 32) lk_step_g(L, t, acc, accb, jr, outs + blockIdx.x, gsh, Sw);
+  const int tid = threadIdx.x, warp = tid >> 5;
+  const int tj = t - (L->L - L->log2_n);
+  lk_copy_run(&sh.run, &L->run);
   __syncthreads();
-  squeeze_dev(Sw, LBL_R, 1, rch, Sn, dig);
-  if (tid < 32) lk_step_r(L, t, rch[0], Sn, gsh);
+  if (t == 1) lk_first_step(L, sh);
+  // the items' partial sums (Montgomery): threads stride over the slots
+  Fr acc[3], accb[4];
+  for (int i = 0; i < 3; i++) acc[i] = fr_zero();
+  for (int i = 0; i < 4; i++) accb[i] = fr_zero();
+  for (int s = L->pbeg[t] + tid; s < L->pend[t]; s += blockDim.x) {
+    const Fr* p = L->part + (size_t)s * LK_PART;
+    for (int i = 0; i < 3; i++) acc[i] = fr_add(acc[i], p[i]);
+    if (tj > 0)
+      for (int i = 0; i < 4; i++) accb[i] = fr_add(accb[i], p[3 + i]);
+  }
+  unsigned long long col[4][8];
+  {
+    unsigned long long c3[3][8];
+    for (int i = 0; i < 3; i++)
+      for (int l = 0; l < 8; l++) c3[i][l] = acc[i].v[l];
+    const Fr x = block_sum_columns<3>(c3, sh.red);
+    if (tid < 3) sh.s[tid] = x;
+  }
+  if (tj > 0) {
+    for (int i = 0; i < 4; i++)
+      for (int l = 0; l < 8; l++) col[i][l] = accb[i].v[l];
+    const Fr x = block_sum_columns<4>(col, sh.red + 32 * (LK_STEP_THREADS / 32));
+    if (tid < 4) sh.s[3 + tid] = x;
+  }
+  __syncwarp();
+  if (warp == 0) lk_step_g(L, sh, t, tj, outs + blockIdx.x);
+  lk_transcript(L, sh, warp, t);
+  __syncthreads();
+  if (warp == 0) lk_step_r(L, sh, t);
+  __syncthreads();
+  lk_copy_run(&L->run, &sh.run);
 }
 
 // The final evaluations (the last pair folded with r_L), absorb 'f', the
-// proof (thread 0; the other threads zero the unused rounds first).
-__device__ void lk_finish(LkDev* L, vl_lookup_proof* out) {
+// proof.  Warps 0 to 3.
+__device__ void lk_finish(LkDev* L, LkShared& sh, vl_lookup_proof* out) {
   for (int i = threadIdx.x; i < (VL_LOOKUP_MAX_LOG_D - L->L) * 32; i += blockDim.x)  // unused rounds
     out->g[L->L + i / 32][(i / 8) & 3].limb[i & 7] = 0u;
-  if (threadIdx.x != 0) return;
-  Fr a, s, b, m;
-  const int Lp = L->L;
-  if (Lp == 0) {
-    lk_level0(*L, 0, a, s);
-  } else if (Lp == 1) {
-    Fr a1, s1;
-    lk_level0(*L, 0, a, s);
-    lk_level0(*L, 1, a1, s1);
-    a = lk_fold(a, a1, L->r[0]);
-    s = lk_fold(s, s1, L->r[0]);
-  } else {
-    a = lk_fold(L->VA[0], L->VA[1], L->r[Lp - 1]);
-    s = lk_fold(L->VS[0], L->VS[1], L->r[Lp - 1]);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, Lp = L->L;
+  if (warp > 0) {
+    if (warp < 4) lk_absorb_help(sh, warp);
+    return;
   }
-  if (L->log2_n == 0) {
-    b = L->WB[0];
-    m = L->WM[0];
-  } else {
-    b = lk_fold(L->WB[0], L->WB[1], L->r[Lp - 1]);
-    m = lk_fold(L->WM[0], L->WM[1], L->r[Lp - 1]);
+  if (lane < 4) {  // a, s, b, m
+    Fr x0, x1 = fr_zero();
+    const bool fold = lane < 2 ? Lp > 0 : L->log2_n > 0;
+    if (lane < 2) {
+      if (Lp <= 1) {
+        const Fr* tab = lane == 0 ? L->Binv : L->Tb;
+        x0 = tab[lk_table_index(*L, 0)];
+        if (fold) x1 = tab[lk_table_index(*L, 1)];
+      } else {
+        const Fr* v = lane == 0 ? L->VA : L->VS;
+        x0 = v[0], x1 = v[1];
+      }
+    } else {
+      const Fr* v = lane == 2 ? L->WB : L->WM;
+      x0 = v[0];
+      if (fold) x1 = v[1];
+    }
+    if (fold) x0 = lk_fold(x0, x1, L->r[Lp - 1]);
+    if (lane == 1) x0 = fr_sub(x0, L->beta);
+    x0 = from_mont_ni(x0);
+    sh.g[lane] = x0;
+    vl_fr* dst = lane == 0 ? &out->a_r : lane == 1 ? &out->s_r : lane == 2 ? &out->b_r : &out->m_r;
+    for (int l = 0; l < 8; l++) dst->limb[l] = x0.v[l];
   }
-  s = fr_sub(s, L->beta);
-  const Fr fin[4] = {from_mont_ni(a), from_mont_ni(s), from_mont_ni(b), from_mont_ni(m)};
-  uint32_t S[8];
-  for (int i = 0; i < 8; i++) S[i] = L->St[i];
-  dev_absorb_fr<4>(S, LBL_F, fin);
-  out->n = L->n;
-  out->log2_d = Lp;
-  out->log2_n = L->log2_n;
-  out->t0 = L->t0;
-  for (int l = 0; l < 8; l++) {
-    out->a_r.limb[l] = fin[0].v[l];
-    out->s_r.limb[l] = fin[1].v[l];
-    out->b_r.limb[l] = fin[2].v[l];
-    out->m_r.limb[l] = fin[3].v[l];
+  __syncwarp();
+  lk_absorb_words(sh, LBL_F, 4, [&](int i) -> const Fr& { return sh.g[i]; });
+  const ShaState st = lk_absorb_run(sh);
+  if (lane == 0) {
+    store_state(out->state, st);
+    out->n = L->n;
+    out->log2_d = Lp;
+    out->log2_n = L->log2_n;
+    out->t0 = L->t0;
+    out->status = L->scr->status;
   }
-  for (int i = 0; i < 32; i++) out->state[i] = (uint8_t)(S[i >> 2] >> (24 - 8 * (i & 3)));
-  out->status = L->scr->status;
 }
 
 // One block per proof: its rounds from L->tail on (at most 2^LK_TAIL_LOG
 // pairs each), each a pass over the pairs, a block reduction and the
 // transcript step in this block, then the final evaluations and the proof.
-#ifndef LK_TAIL_MINB
-#define LK_TAIL_MINB 4  // resident tail CTAs per SM the register budget allows
-#endif
-__global__ void __launch_bounds__(LK_TAIL_THREADS, LK_TAIL_MINB) lk_tail_kernel(LkDev* Ls, vl_lookup_proof* outs) {
-  __shared__ Fr red[6 * (LK_TAIL_THREADS / 32)];
-  __shared__ uint32_t Sw[8], Sn[8];
-  __shared__ uint32_t dig[3][8];
-  __shared__ Fr rch[1];
-  __shared__ Fr gsh[4];
+// In a table round the first half of the warps take the A side's pairs, the
+// second half the table side's.  Short rounds spread a pair over four lanes
+// (one fold each, then one product and one product by f).  The last warp forms
+// the claims and scalars of the next round beside its share of a pass.
+template <int THREADS, int MINB>
+__global__ void __launch_bounds__(THREADS, MINB) lk_tail_kernel(LkDev* Ls, vl_lookup_proof* outs) {
+  __shared__ LkShared sh;
   LkDev* L = Ls + blockIdx.x;
   vl_lookup_proof* out = outs + blockIdx.x;
-  const int tid = threadIdx.x;
-  if (L->tail == 1 && L->L >= 1) lk_table_sum(L, red);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  constexpr int NW = THREADS / 32;
+  lk_copy_run(&sh.run, &L->run);
+  __syncthreads();
+  if (L->tail == 1 && L->L >= 1) lk_first_step(L, sh);
   for (int t = L->tail; t <= L->L; t++) {
     const int h = 1 << (L->L - t);
-    const bool jr = t > L->L - L->log2_n;
     const int tj = t - (L->L - L->log2_n);
+    const bool jr = tj > 0;
+    if (t > L->tail && warp == NW - 1) lk_step_r(L, sh, t - 1);
     const LkEq q(L, t);
-    Fr acc[6], accb[6];
-    for (int i = 0; i < 6; i++) acc[i] = accb[i] = fr_zero();
-    for (int k = tid; k < h; k += blockDim.x) {
-      Fr f = q.f_tab[k & q.f_mask];
-      if (q.high) f = mont_mul_ni(f, q.hi_tab[k >> L->sE]);
-      if (t == 1) lk_pair_a<0>(L, t, k, h, f, acc);
-      else if (t == 2) lk_pair_a<1>(L, t, k, h, f, acc);
-      else lk_pair_a<2>(L, t, k, h, f, acc);
-      if (jr) lk_pair_b(L, t, tj, k, h, f, accb);
+    const int na = jr ? NW / 2 : NW;  // warps of the A side
+    const bool sideb = warp >= na;
+    const int id = sideb ? tid - 32 * na : tid, nid = 32 * (sideb ? NW - na : na);
+    if (4 * h > nid) {
+      unsigned long long a[32];
+#pragma unroll
+      for (int i = 0; i < 32; i++) a[i] = 0;
+      if (!sideb) {
+        LkSumA s;
+        s.zero();
+#pragma unroll 1
+        for (int k = id; k < h; k += nid) {
+          Fr f = q.f_tab[k & q.f_mask];
+          if (q.high) f = mont_mul_ni(f, q.hi_tab[k >> L->sE]);
+          if (t == 1) lk_pair_a<0>(L, t, k, h, f, s);
+          else if (t == 2) lk_pair_a<1>(L, t, k, h, f, s);
+          else lk_pair_a<2>(L, t, k, h, f, s);
+        }
+        unsigned long long col[3][8];
+        s.columns(col);
+#pragma unroll
+        for (int i = 0; i < 24; i++) a[i] = col[i / 8][i % 8];
+      } else {
+        const Fr toff = sh.run.toff;
+        LkSumB s;
+        s.zero();
+#pragma unroll 1
+        for (int k = id; k < h; k += nid) {
+          Fr f = q.f_tab[k & q.f_mask];
+          if (q.high) f = mont_mul_ni(f, q.hi_tab[k >> L->sE]);
+          lk_pair_b(L, t, tj, k, h, f, toff, s);
+        }
+        unsigned long long col[4][8];
+        s.columns(col);
+#pragma unroll
+        for (int i = 0; i < 32; i++) a[i] = col[i / 8][i % 8];
+      }
+      sh.red[32 * warp + lane] = warp_transpose_sum<32>(a);
+      __syncthreads();
+      if (warp == 0) {
+        unsigned long long ta = 0, tb = 0;
+        for (int w = 0; w < na; w++) ta += sh.red[32 * w + lane];
+        for (int w = na; w < NW; w++) tb += sh.red[32 * w + lane];
+        U64x8 col;
+#pragma unroll
+        for (int l = 0; l < 8; l++) {
+          const int src = 8 * (lane & 3) + l;
+          const unsigned long long ca = __shfl_sync(0xffffffffu, ta, src), cb = __shfl_sync(0xffffffffu, tb, src);
+          col.v[l] = lane < 4 ? ca : cb;
+        }
+        const Fr x = redc_columns_ni(col);
+        if (lane < 3) sh.s[lane] = x;
+        else if (lane >= 4 && lane < 8) sh.s[lane - 1] = x;
+      }
+    } else {
+      const int j = id >> 2, qd = id & 3, at = j + (qd & 1) * h;
+      const bool act = j < h;
+      Fr x = fr_zero(), x1 = fr_zero(), f = fr_zero(), u0 = fr_zero();
+      bool fold = false;
+      Fr* dst = nullptr;
+      if (act) {
+        f = q.f_tab[j & q.f_mask];
+        if (q.high) f = mont_mul_ni(f, q.hi_tab[j >> L->sE]);
+        if (!sideb && t <= 2) {
+          const Fr* tab = qd < 2 ? L->Binv : L->Tb;
+          x = tab[lk_table_index(*L, at)];
+          fold = t == 2;
+          if (fold) x1 = tab[lk_table_index(*L, at + 2 * h)];
+          if (fold) dst = qd < 2 ? L->VA : L->VS;
+        } else {
+          Fr* v = sideb ? (qd < 2 ? L->WB : L->WM) : (qd < 2 ? L->VA : L->VS);
+          x = v[at];
+          fold = !sideb || tj > 1;
+          if (fold) x1 = v[at + 2 * h], dst = v;
+        }
+        if (sideb) u0 = fr_add(L->Tb[j], sh.run.toff);
+      }
+      __syncwarp();
+      if (t > 1 && (!sideb || tj > 1)) {
+        const Fr fx = fr_add(x, mont_mul_ni(L->r[t - 2], fr_sub(x1, x)));
+        if (fold) x = fx;
+      }
+      if (dst) dst[at] = x;
+      const Fr y = shfl_xor_fr(x, 1);
+      const Fr z = (qd & 1) ? fr_sub(x, y) : x;  // A: a0, da, s0, ds; table: b0, db, m0, dm
+      Fr w = shfl_xor_fr(z, 2);
+      const Fr a0 = w;
+      if (sideb && qd == 0) w = u0;
+      if (sideb && qd == 1) w = f;
+      Fr p = mont_mul_ni(z, w);
+      const Fr pf = mont_mul_ni(p, f);
+      if (sideb ? qd == 0 : qd < 2) p = pf;
+      if (!sideb && qd == 2) p = a0;
+      if (!act || (!sideb && qd == 3)) p = fr_zero();
+#pragma unroll
+      for (int off = 4; off < 32; off <<= 1) p = fr_add(p, shfl_xor_fr(p, off));
+      Fr* red = reinterpret_cast<Fr*>(sh.red);
+      if (lane < 4) red[4 * warp + lane] = p;
+      __syncthreads();
+      if (warp == 0) {
+        Fr va = fr_zero(), vb = fr_zero();
+        for (int w2 = lane >> 2; w2 < NW; w2 += 8) {
+          const Fr v = red[4 * w2 + qd];
+          if (w2 < na) va = fr_add(va, v);
+          else vb = fr_add(vb, v);
+        }
+#pragma unroll
+        for (int off = 4; off < 32; off <<= 1) {
+          va = fr_add(va, shfl_xor_fr(va, off));
+          if (jr) vb = fr_add(vb, shfl_xor_fr(vb, off));
+        }
+        const Fr v = from_mont_ni(lane < 4 ? va : vb);
+        if (lane < 3) sh.s[lane] = v;
+        else if (lane >= 4 && lane < 8) sh.s[lane - 1] = v;
+      }
     }
-    if (t == 1) lk_mode0_sums(acc);
-    if (jr && tj == 1) lk_mode0_sums(accb);
-    block_sum_fr<6>(acc, red);
-    if (jr) block_sum_fr<6>(accb, red);
-    if (tid < 32) lk_step_g(L, t, acc, accb, jr, out, gsh, Sw);
-    __syncthreads();
-    squeeze_dev(Sw, LBL_R, 1, rch, Sn, dig);
-    if (tid < 32) lk_step_r(L, t, rch[0], Sn, gsh);
+    __syncwarp();
+    if (warp == 0) lk_step_g(L, sh, t, tj, out);
+    lk_transcript(L, sh, warp, t);
     __syncthreads();  // r_t and the folded vectors are visible to the next round
   }
-  lk_finish(L, out);
+  lk_finish(L, sh, out);
 }
 
 }  // namespace
 
-cudaError_t launch_lookup_setup(LkDev* Ls, int np, const LkItem* fac_items, int nfac, const LkItem* hist_items,
-                                int nhist, const LkItem* tab_items, int ntab, cudaStream_t st) {
+cudaError_t launch_lookup_setup(LkDev* Ls, int np, const LkItem* hist_items, int nhist, const LkItem* tab_items,
+                                int ntab, cudaStream_t st) {
   lk_start_kernel<<<np, LK_THREADS, 0, st>>>(Ls);
-  if (nfac) lk_factor_kernel<<<nfac, LK_THREADS, 0, st>>>(Ls, fac_items);
   if (nhist) lk_hist_kernel<<<nhist, LK_THREADS, 0, st>>>(Ls, hist_items);
   if (ntab) lk_table_kernel<<<ntab, LK_THREADS, 0, st>>>(Ls, tab_items);
   return cudaGetLastError();
@@ -483,12 +689,21 @@ cudaError_t launch_lookup_round(LkDev* Ls, int np, int t, const LkItem* items, i
                                 vl_lookup_proof* out, cudaStream_t st) {
   const cudaError_t e = launch_lookup_passes(Ls, t, items, nhi, nlo, st);
   if (e != cudaSuccess) return e;
-  lk_round_kernel<<<np, LK_ROUND_THREADS, 0, st>>>(Ls, t, out);
+  lk_round_kernel<<<np, LK_STEP_THREADS, 0, st>>>(Ls, t, out);
   return cudaGetLastError();
 }
 
+// A proof's tail is a chain of rounds: with an SM for every proof it runs on 512
+// threads, else on 128, four proofs per SM (one lookup of 512 x 16 remainders
+// 0.98 -> 0.44 ms, the 512 of a 7B step 8.86 -> 4.42 ms with the other changes
+// described in lookup_dev.cuh).
 cudaError_t launch_lookup_finish(LkDev* Ls, int np, vl_lookup_proof* out, cudaStream_t st) {
-  lk_tail_kernel<<<np, LK_TAIL_THREADS, 0, st>>>(Ls, out);
+  int dev = 0, sms = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e != cudaSuccess) return e;
+  if (np <= sms) lk_tail_kernel<512, 1><<<np, 512, 0, st>>>(Ls, out);
+  else lk_tail_kernel<128, 4><<<np, 128, 0, st>>>(Ls, out);
   return cudaGetLastError();
 }
 

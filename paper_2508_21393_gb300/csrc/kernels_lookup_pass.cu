@@ -1,63 +1,63 @@
 // Lookup-argument sumcheck: the batched round passes (the rounds of every
-// proof before its tail), one kernel instance per side set and round mode.
-// Kept apart from kernels_lookup.cu so the two compile in parallel.
+// proof before its tail).  Kept apart from kernels_lookup.cu so the two compile
+// in parallel.
 #include "lookup_dev.cuh"
 
 namespace vl {
 
 namespace {
 
-// Round t over pairs [k0, k1) of one proof (the rounds before the proof's
-// tail): the partial sums of lk_pair_a (and lk_pair_b in table rounds, JR)
-// into the item's slot.  Warp w of the block takes the 32 LK_PPT pairs from
-// k0 + 32 LK_PPT w, lanes strided by one (coalesced loads).  In a high round
-// with 2^sE >= 32 LK_PPT the warp's pairs lie in one block of 2^sE pairs, so
-// the block's hiP factor multiplies each lane's sums once; with smaller
-// blocks it multiplies every pair's eq factor.
-#ifndef LK_PASS_MINB
-#define LK_PASS_MINB 2  // resident CTAs per SM the register budget of the passes allows
-#endif
+// Column sums over the warp's lanes of NV values, reduced: lane q < NV returns
+// value q in Montgomery form, value q < nf multiplied by hf (Montgomery).
+template <int NV>
+__device__ __forceinline__ Fr lk_warp_sum(const unsigned long long (&c)[NV][8], int nf, const Fr* hf) {
+  const int lane = threadIdx.x & 31;
+  unsigned long long a[32];
+#pragma unroll
+  for (int i = 0; i < 32; i++) a[i] = i < NV * 8 ? c[i / 8 < NV ? i / 8 : 0][i % 8] : 0ull;
+  const unsigned long long t = warp_transpose_sum<32>(a);
+  U64x8 col;
+#pragma unroll
+  for (int l = 0; l < 8; l++) col.v[l] = __shfl_sync(0xffffffffu, t, (lane * 8 + l) & 31);
+  Fr x = redc_columns_ni(col);  // canonical
+  if (hf && lane < nf) x = mont_mul_ni(x, *hf);
+  return to_mont_ni(x);
+}
+
+// Round t, one warp per item (pairs [k0, k1) of one proof, lanes strided by
+// one: coalesced loads): the item's partial sums into its slot.  The item's
+// pairs lie in one block of 2^sE pairs (LK_PAIRS, 2^sE), so a high round's hiP
+// factor multiplies the item's sums once.
 template <bool JR, int MODE>
-__global__ void __launch_bounds__(LK_THREADS, LK_PASS_MINB) lk_pass_kernel(LkDev* Ls, int t, const LkItem* items) {
-  __shared__ Fr red[6 * (LK_THREADS / 32)];
-  const LkItem it = items[blockIdx.x];
+__global__ void __launch_bounds__(LK_PASS_THREADS, 4) lk_pass_kernel(LkDev* Ls, int t, const LkItem* items, int n) {
+  const int i = blockIdx.x * LK_PASS_WARPS + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (i >= n) return;  // whole warps leave together
+  const LkItem it = items[i];
   LkDev* L = Ls + it.proof;
   const int h = 1 << (L->L - t);
-  const int tj = t - (L->L - L->log2_n);  // table round number (1-based) when JR
   const LkEq q(L, t);
-  const bool lane_factor = q.high && L->sE >= LK_PPT_LOG + 5;  // the warp's pairs share one hiP entry
-  const int kw = it.k0 + (threadIdx.x >> 5) * (32 * LK_PPT);
-  Fr acc[6];
-#pragma unroll
-  for (int i = 0; i < 6; i++) acc[i] = fr_zero();
-  Fr accb[6];
-  if constexpr (JR) {
-#pragma unroll
-    for (int i = 0; i < 6; i++) accb[i] = fr_zero();
-  }
+  const Fr* hf = q.high ? q.hi_tab + (it.k0 >> L->sE) : nullptr;
+  {
+    LkSumA s;
+    s.zero();
 #pragma unroll 1
-  for (int k = kw + (threadIdx.x & 31); k < min(it.k1, kw + 32 * LK_PPT); k += 32) {
-    Fr f = q.f_tab[k & q.f_mask];
-    if (q.high && !lane_factor) f = mont_mul_ni(f, q.hi_tab[k >> L->sE]);
-    lk_pair_a<MODE>(L, t, k, h, f, acc);
-    if constexpr (JR) lk_pair_b(L, t, tj, k, h, f, accb);
+    for (int k = it.k0 + lane; k < it.k1; k += 32) lk_pair_a<MODE>(L, t, k, h, q.f_tab[k & q.f_mask], s);
+    unsigned long long col[3][8];
+    s.columns(col);
+    const Fr x = lk_warp_sum<3>(col, 2, hf);
+    if (lane < 3) L->part[(size_t)it.slot * LK_PART + lane] = x;
   }
-  if constexpr (MODE == 0) lk_mode0_sums(acc);
-  if constexpr (JR)
-    if (tj == 1) lk_mode0_sums(accb);
-  if (lane_factor && kw < it.k1) {  // the eq factor over the remaining high variables
-    const Fr hf = q.hi_tab[kw >> L->sE];
-    for (int i = 0; i < 3; i++) acc[i] = mont_mul_ni(acc[i], hf);
-    if constexpr (JR)
-      for (int i = 0; i < 3; i++) accb[i] = mont_mul_ni(accb[i], hf);
-  }
-  block_sum_fr<6>(acc, red);
-  if (threadIdx.x == 0)
-    for (int i = 0; i < 6; i++) L->part[(size_t)it.slot * 12 + i] = acc[i];
   if constexpr (JR) {
-    block_sum_fr<6>(accb, red);
-    if (threadIdx.x == 0)
-      for (int i = 0; i < 6; i++) L->part[(size_t)it.slot * 12 + 6 + i] = accb[i];
+    const int tj = t - (L->L - L->log2_n);  // table round number (1-based)
+    const Fr toff = L->run.toff;
+    LkSumB s;
+    s.zero();
+#pragma unroll 1
+    for (int k = it.k0 + lane; k < it.k1; k += 32) lk_pair_b(L, t, tj, k, h, q.f_tab[k & q.f_mask], toff, s);
+    unsigned long long col[4][8];
+    s.columns(col);
+    const Fr x = lk_warp_sum<4>(col, 2, hf);
+    if (lane < 4) L->part[(size_t)it.slot * LK_PART + 3 + lane] = x;
   }
 }
 
@@ -66,15 +66,16 @@ __global__ void __launch_bounds__(LK_THREADS, LK_PASS_MINB) lk_pass_kernel(LkDev
 // Round t's passes: nhi items of proofs in their high rounds, then nlo items
 // of proofs in their table rounds.
 cudaError_t launch_lookup_passes(LkDev* Ls, int t, const LkItem* items, int nhi, int nlo, cudaStream_t st) {
+  const int ghi = (nhi + LK_PASS_WARPS - 1) / LK_PASS_WARPS, glo = (nlo + LK_PASS_WARPS - 1) / LK_PASS_WARPS;
   if (nhi) {
-    if (t == 1) lk_pass_kernel<false, 0><<<nhi, LK_THREADS, 0, st>>>(Ls, t, items);
-    else if (t == 2) lk_pass_kernel<false, 1><<<nhi, LK_THREADS, 0, st>>>(Ls, t, items);
-    else lk_pass_kernel<false, 2><<<nhi, LK_THREADS, 0, st>>>(Ls, t, items);
+    if (t == 1) lk_pass_kernel<false, 0><<<ghi, LK_PASS_THREADS, 0, st>>>(Ls, t, items, nhi);
+    else if (t == 2) lk_pass_kernel<false, 1><<<ghi, LK_PASS_THREADS, 0, st>>>(Ls, t, items, nhi);
+    else lk_pass_kernel<false, 2><<<ghi, LK_PASS_THREADS, 0, st>>>(Ls, t, items, nhi);
   }
   if (nlo) {
-    if (t == 1) lk_pass_kernel<true, 0><<<nlo, LK_THREADS, 0, st>>>(Ls, t, items + nhi);
-    else if (t == 2) lk_pass_kernel<true, 1><<<nlo, LK_THREADS, 0, st>>>(Ls, t, items + nhi);
-    else lk_pass_kernel<true, 2><<<nlo, LK_THREADS, 0, st>>>(Ls, t, items + nhi);
+    if (t == 1) lk_pass_kernel<true, 0><<<glo, LK_PASS_THREADS, 0, st>>>(Ls, t, items + nhi, nlo);
+    else if (t == 2) lk_pass_kernel<true, 1><<<glo, LK_PASS_THREADS, 0, st>>>(Ls, t, items + nhi, nlo);
+    else lk_pass_kernel<true, 2><<<glo, LK_PASS_THREADS, 0, st>>>(Ls, t, items + nhi, nlo);
   }
   return cudaGetLastError();
 }

@@ -45,7 +45,7 @@ int check_job(const vl_lookup_job& J) {
 }
 
 struct LkBufs {
-  size_t lop = 0, hip = 0, binv = 0, tb = 0, wb = 0, we = 0, wt = 0, wm = 0, va = 0, vs = 0, counts = 0, stage = 0;
+  size_t lop = 0, hip = 0, binv = 0, tb = 0, wb = 0, wm = 0, va = 0, vs = 0, counts = 0, stage = 0;
 };
 
 int cuda_fail(const char* where, cudaError_t e) {
@@ -62,9 +62,9 @@ struct vl_lookup_plan {
   int np = 0, maxL = 0, nslots = 0, nrounds = 0;
   std::vector<LkDev> Ls;  // statements; device pointers filled at bind time
   std::vector<LkBufs> buf;
-  std::vector<LkItem> fac, hist, tab, rounds;
+  std::vector<LkItem> hist, tab, rounds;
   std::vector<int> roff, nhi, nlo;  // round t: items [roff[t], roff[t] + nhi[t] + nlo[t])
-  size_t off_L = 0, off_scr = 0, off_fac = 0, off_hist = 0, off_tab = 0, off_rounds = 0, off_part = 0,
+  size_t off_L = 0, off_scr = 0, off_hist = 0, off_tab = 0, off_rounds = 0, off_part = 0,
          off_out = 0, off_counts = 0, counts_bytes = 0, total = 0;
   uint8_t* bound_ws = nullptr;
   int device = -1;
@@ -89,7 +89,7 @@ int lk_build(vl_lookup_plan* P, const vl_lookup_job* jobs, int32_t njobs) {
   P->np = njobs;
   P->Ls.assign(njobs, LkDev{});
   P->buf.assign(njobs, LkBufs{});
-  const Fr inv2 = to_mont(fr_inv_canonical(fr_small(2))), inv6 = to_mont(fr_inv_canonical(fr_small(6)));
+  const Fr inv2 = to_mont(fr_inv_canonical(fr_small(2)));
   int slot = 0;
   for (int i = 0; i < njobs; i++) {
     const vl_lookup_job& J = jobs[i];
@@ -107,16 +107,11 @@ int lk_build(vl_lookup_plan* P, const vl_lookup_job* jobs, int32_t njobs) {
     L.ld = J.S.space == VL_HOST ? J.S.cols : J.S.ld;  // host operands are staged densely
     std::memcpy(L.bind, J.bind, 32);
     L.inv2 = inv2;
-    L.inv6 = inv6;
+    L.dense = L.ld == L.cols ? 1 : 0;
     L.tail = std::max(1, L.L - LK_TAIL_LOG);  // rounds with h = 2^(L-t) <= 2^LK_TAIL_LOG pairs
     if (L.L == 0) L.tail = 1;
     P->maxL = std::max(P->maxL, L.L);
     const int N = 1 << L.log2_n;
-    // suffix eq tables (loP: levels 0..sE; hiP: levels 0..L-sE-1) and eq(u_low, .)
-    const int sizes[3] = {(2 << L.sE) - 1, (1 << (L.L - L.sE)) - 1, N};
-    for (int w = 0; w < 3; w++)
-      for (int k0 = 0; k0 < sizes[w]; k0 += LK_THREADS * 4)
-        P->fac.push_back(LkItem{i, k0, std::min(sizes[w], k0 + LK_THREADS * 4), w});
     for (int k0 = 0; k0 < L.n; k0 += LK_HIST) P->hist.push_back(LkItem{i, k0, std::min(L.n, k0 + LK_HIST), 0});
     L.xbeg = slot;
     for (int k0 = 0; k0 < N; k0 += LK_ENTRIES) P->tab.push_back(LkItem{i, k0, std::min(N, k0 + LK_ENTRIES), slot++});
@@ -136,8 +131,9 @@ int lk_build(vl_lookup_plan* P, const vl_lookup_job* jobs, int32_t njobs) {
         if (jr != (pass == 1)) continue;
         const int h = 1 << (L.L - t);
         L.pbeg[t] = slot;
-        for (int k0 = 0; k0 < h; k0 += LK_PAIRS) {
-          P->rounds.push_back(LkItem{i, k0, std::min(h, k0 + LK_PAIRS), slot++});
+        const int pairs = std::min(LK_PAIRS, 1 << L.sE);
+        for (int k0 = 0; k0 < h; k0 += pairs) {
+          P->rounds.push_back(LkItem{i, k0, std::min(h, k0 + pairs), slot++});
           (pass ? P->nlo : P->nhi)[t]++;
         }
         L.pend[t] = slot;
@@ -155,11 +151,10 @@ int lk_build(vl_lookup_plan* P, const vl_lookup_job* jobs, int32_t njobs) {
   };
   P->off_L = take(sizeof(LkDev) * njobs);
   P->off_scr = take(sizeof(ProofScratch) * njobs);
-  P->off_fac = take(sizeof(LkItem) * P->fac.size());
   P->off_hist = take(sizeof(LkItem) * P->hist.size());
   P->off_tab = take(sizeof(LkItem) * P->tab.size());
   P->off_rounds = take(sizeof(LkItem) * P->rounds.size());
-  P->off_part = take(sizeof(Fr) * 12 * (size_t)std::max(1, P->nslots));
+  P->off_part = take(sizeof(Fr) * LK_PART * (size_t)std::max(1, P->nslots));
   P->off_out = take(sizeof(vl_lookup_proof) * njobs);
   // multiplicities of every proof in one region (one clear per run)
   size_t cnt = 0;
@@ -178,8 +173,6 @@ int lk_build(vl_lookup_plan* P, const vl_lookup_job* jobs, int32_t njobs) {
     b.binv = take(sizeof(Fr) * N);
     b.tb = take(sizeof(Fr) * N);
     b.wb = take(sizeof(Fr) * N);
-    b.we = take(sizeof(Fr) * N);
-    b.wt = take(sizeof(Fr) * N);
     b.wm = take(sizeof(Fr) * N);
     b.va = take(sizeof(Fr) * half);
     b.vs = take(sizeof(Fr) * half);
@@ -201,8 +194,6 @@ int lk_bind(vl_lookup_plan* P, uint8_t* ws, cudaStream_t st) {
     L.Binv = reinterpret_cast<Fr*>(ws + b.binv);
     L.Tb = reinterpret_cast<Fr*>(ws + b.tb);
     L.WB = reinterpret_cast<Fr*>(ws + b.wb);
-    L.WE = reinterpret_cast<Fr*>(ws + b.we);
-    L.WT = reinterpret_cast<Fr*>(ws + b.wt);
     L.WM = reinterpret_cast<Fr*>(ws + b.wm);
     L.VA = reinterpret_cast<Fr*>(ws + b.va);
     L.VS = reinterpret_cast<Fr*>(ws + b.vs);
@@ -215,7 +206,6 @@ int lk_bind(vl_lookup_plan* P, uint8_t* ws, cudaStream_t st) {
     if (ce == cudaSuccess && bytes) ce = cudaMemcpyAsync(ws + off, src, bytes, cudaMemcpyHostToDevice, st);
   };
   up(P->off_L, P->Ls.data(), sizeof(LkDev) * P->np);
-  up(P->off_fac, P->fac.data(), sizeof(LkItem) * P->fac.size());
   up(P->off_hist, P->hist.data(), sizeof(LkItem) * P->hist.size());
   up(P->off_tab, P->tab.data(), sizeof(LkItem) * P->tab.size());
   up(P->off_rounds, P->rounds.data(), sizeof(LkItem) * P->rounds.size());
@@ -288,8 +278,8 @@ extern "C" int32_t vl_lookup_plan_run(vl_lookup_plan* P, void* workspace, size_t
   auto items = [&](size_t off) { return reinterpret_cast<const LkItem*>(ws + off); };
   if (ce == cudaSuccess) ce = cudaEventRecord(P->ev[0], st);
   if (ce == cudaSuccess)
-    ce = launch_lookup_setup(dL, P->np, items(P->off_fac), (int)P->fac.size(), items(P->off_hist),
-                             (int)P->hist.size(), items(P->off_tab), (int)P->tab.size(), st);
+    ce = launch_lookup_setup(dL, P->np, items(P->off_hist), (int)P->hist.size(), items(P->off_tab),
+                             (int)P->tab.size(), st);
   if (ce == cudaSuccess) ce = cudaEventRecord(P->ev[1], st);
   for (int t = 1; t <= P->nrounds && ce == cudaSuccess; t++)
     ce = launch_lookup_round(dL, P->np, t, items(P->off_rounds) + P->roff[t], P->nhi[t], P->nlo[t], dout, st);
