@@ -357,20 +357,23 @@ cudaError_t launch_lookup_passes(LkDev* Ls, int t, const LkItem* items, int nhi,
 struct BtState {
   int32_t K, d1, status, P2;       // products, rounds, status, leaves of the Merkle trees (2^t >= K)
   uint64_t seed;
-  Fr rho, claim, inv2;             // Montgomery
-  Fr r[VL_MAX_ROUNDS];
+  int32_t ticket, pad;             // CTAs of the running pass that are done
+  Fr claim;                        // running claim (canonical)
+  Fr r[VL_MAX_ROUNDS];             // challenges (Montgomery)
   uint32_t St[8];                  // batch transcript state (big-endian words)
   int32_t pbeg[VL_MAX_ROUNDS + 1], pend[VL_MAX_ROUNDS + 1];  // partial-sum slots of each round
-  Fr* w;                           // rho^i
-  Fr* c;                           // claims (Montgomery)
+  Fr* w;                           // rho^i (Montgomery)
+  Fr* c;                           // per product (canonical): claim, round 1's g(0) and leading coefficient
   uint8_t* tree;                   // 2 P2 nodes of 32 bytes (leaves at [P2, 2 P2), root at 1)
-  Fr* part;                        // partial sums, 2 per slot (g(0), g(2))
+  Fr* part;                        // partial sums, 2 per slot (weighted g(0), leading coefficient; canonical)
   vl_fr* c_out;                    // canonical outputs: claims, a_i, b_i
   vl_fr* a_out;
   vl_fr* b_out;
   vl_batch_proof* out;
 };
+// Claims (one CTA per product), then the batch start with round 1.
 cudaError_t launch_batch_claims(const DevProof* dp, int np, BtState* B, cudaStream_t st);
+// Round t >= 2.
 cudaError_t launch_batch_round(const DevProof* dp, BtState* B, int t, const LkItem* items, int nitems,
                                cudaStream_t st);
 cudaError_t launch_batch_finish(const DevProof* dp, int np, BtState* B, int k, cudaStream_t st);

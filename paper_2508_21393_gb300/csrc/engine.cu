@@ -1391,7 +1391,7 @@ struct BatchLayout {
          off_aout = 0, off_bout = 0, off_proof = 0, total = 0;
 };
 
-constexpr int BT_PAIRS = 1024;
+constexpr int BT_PAIRS = 256;  // pairs per pass CTA: one per thread
 
 int batch_layout(const vl_job* jobs, int32_t njobs, BatchLayout* L) {
   if (!jobs || njobs < 1 || njobs > 65535) return VL_EINVAL;
@@ -1413,6 +1413,7 @@ int batch_layout(const vl_job* jobs, int32_t njobs, BatchLayout* L) {
   L->roff.assign(L->d1 + 2, 0);
   for (int t = 1; t <= L->d1; t++) {
     L->roff[t] = (int)L->items.size();
+    if (t == 1) continue;  // round 1 is evaluated with the claims
     const int h = 1 << (L->d1 - t);
     for (int s = 0; s < njobs; s++)
       for (int k0 = 0; k0 < h; k0 += BT_PAIRS)
@@ -1427,7 +1428,7 @@ int batch_layout(const vl_job* jobs, int32_t njobs, BatchLayout* L) {
   };
   L->off_state = take(sizeof(BtState));
   L->off_w = take(sizeof(Fr) * njobs);
-  L->off_c = take(sizeof(Fr) * njobs);
+  L->off_c = take(sizeof(Fr) * 3 * (size_t)njobs);
   L->off_tree = take(64 * (size_t)L->P2);
   L->off_part = take(sizeof(Fr) * 2 * std::max<size_t>(1, L->items.size()));
   L->off_items = take(sizeof(LkItem) * std::max<size_t>(1, L->items.size()));
@@ -1481,7 +1482,6 @@ extern "C" int32_t vl_claims_plan_create(const vl_job* jobs, int32_t njobs, uint
   S.status = VL_OK;
   S.P2 = C->L.P2;
   S.seed = seed;
-  S.inv2 = to_mont(fr_inv_canonical(fr_small(2)));
   for (int t = 1; t <= C->L.d1; t++) {
     S.pbeg[t] = C->L.roff[t];
     S.pend[t] = C->L.roff[t + 1];
@@ -1548,7 +1548,7 @@ extern "C" int32_t vl_claims_plan_run(vl_claims_plan* C, void* workspace, size_t
   if (ce == cudaSuccess) ce = launch_fold_tc(dc, (int)p->tc_tiles.size(), dp, wait_ns(p), st);
   if (ce == cudaSuccess) ce = launch_fold(dt, dl, (int)p->tiles.size(), dp, p->fold_smem, wait_ns(p), st);
   if (ce == cudaSuccess) ce = launch_batch_claims(dp, np, dS, st);
-  for (int t = 1; t <= L.d1 && ce == cudaSuccess; t++)
+  for (int t = 2; t <= L.d1 && ce == cudaSuccess; t++)
     ce = launch_batch_round(dp, dS, t, di + L.roff[t], L.roff[t + 1] - L.roff[t], st);
   if (ce == cudaSuccess) ce = launch_batch_finish(dp, np, dS, L.k, st);
   const cudaMemcpyKind kind = out_space == VL_HOST ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice;

@@ -3,13 +3,16 @@
 //
 // The products' prologues (member transcripts, eq tables) and folds are the
 // single-proof kernels; then:
-//   claims  (one CTA per product): c_i = sum_w f_A[w] f_B[w], its Merkle leaf
+//   claims  (one CTA per product): c_i = sum_w f_A[w] f_B[w] and round 1's terms
+//           of the product from the same loop, the Merkle leaf
 //           SHA256(0x00 || S_i || c_i);
 //   start   (one CTA): the Merkle root, the batch transcript start, rho, the
-//           weights rho^i, the combined claim sum_i rho^i c_i;
-//   rounds  per variable: a pass over every product's pairs (fold with the
-//           previous challenge, then rho^i-weighted sums of g(0), g(2)) and
-//           one CTA for the transcript step (g(1) = claim - g(0));
+//           weights rho^i, the combined claim sum_i rho^i c_i, round 1's
+//           transcript step;
+//   rounds  t >= 2, one launch each: every product's pairs (fold with the
+//           previous challenge, then rho^i-weighted sums of g(0) and the leading
+//           coefficient, see rounds_dev.cuh); the CTA that finishes last runs
+//           the transcript step (g(1) = claim - g(0));
 //   finish  (one CTA per product) a_i, b_i and their leaves; (one CTA) the
 //           root, absorb 'f', the proof.
 #include "prologue_dev.cuh"
@@ -45,27 +48,47 @@ __device__ __forceinline__ void bt_load_node(const uint8_t* tree, int i, uint32_
   Y[at + 4] = bswap32(b.x), Y[at + 5] = bswap32(b.y), Y[at + 6] = bswap32(b.z), Y[at + 7] = bswap32(b.w);
 }
 
-// One block per product.
+// One block per product: the claim, round 1's g(0) and leading coefficient;
+// f_A, f_B left reduced in their vectors (zeros past k) for the later rounds.
 __global__ void __launch_bounds__(BT_THREADS) bt_claims_kernel(const DevProof* dp, BtState* B) {
-  __shared__ Fr red[BT_THREADS / 32];
+  __shared__ unsigned long long red[3 * 8 * (BT_THREADS / 32)];
   const DevProof& P = dp[blockIdx.x];
-  const int i = P.member1 - 1;
-  Fr acc[1] = {fr_zero()};
-  for (int w = threadIdx.x; w < P.k; w += blockDim.x)
-    acc[0] = fr_add(acc[0], mont_mul_ni(bt_level0(P, 0, w), bt_level0(P, 1, w)));
-  block_sum_fr<1>(acc, red);
-  if (threadIdx.x == 0) {
-    B->c[i] = acc[0];
-    const Fr c = from_mont_ni(acc[0]);
-    for (int l = 0; l < 8; l++) B->c_out[i].limb[l] = c.v[l];
+  const int i = P.member1 - 1, K = 1 << P.d1, h = K >> 1;
+  uint32_t w0[17], w1[17], wi[17];
+  wide_zero(w0), wide_zero(w1), wide_zero(wi);
+  for (int j = threadIdx.x; j < max(h, 1); j += blockDim.x) {
+    const Fr a0 = bt_level0(P, 0, j), b0 = bt_level0(P, 1, j);
+    if (h == 0) {  // k = 1: no rounds
+      P.fA[0] = a0, P.fB[0] = b0;
+      wide_mac(w0, a0, b0);
+      break;
+    }
+    const Fr a1 = bt_level0(P, 0, j + h), b1 = bt_level0(P, 1, j + h);
+    P.fA[j] = a0, P.fA[j + h] = a1;
+    P.fB[j] = b0, P.fB[j + h] = b1;
+    first_pair(a0, a1, b0, b1, w0, w1, wi);
+  }
+  unsigned long long col[3][8];
+  wide_redc(w0, col[0]);
+  wide_redc(w1, col[1]);
+  wide_redc(wi, col[2]);
+  const Fr s = block_sum_columns<3>(col, red);
+  if (threadIdx.x < 32) {
+    const Fr g0 = shfl_fr(s, 0), g1 = shfl_fr(s, 1), G = shfl_fr(s, 2), c = fr_add(g0, g1);
     uint32_t Y[16], node[8];  // leaf: 0x00 || S_i || c_i
     const uint32_t* st = reinterpret_cast<const uint32_t*>(P.scr->state);
 #pragma unroll
     for (int l = 0; l < 8; l++) Y[l] = bswap32(st[l]);
     bt_words(Y, 8, c);
     dev_hash_tagged<16>(0u, Y, node);
-    store_digest_bytes(B->tree + (size_t)(B->P2 + i) * 32, node);
-    if (P.scr->status != VL_OK) atomicExch(&B->status, P.scr->status);
+    if (threadIdx.x == 0) {
+      B->c[3 * (size_t)i] = c;
+      B->c[3 * (size_t)i + 1] = g0;
+      B->c[3 * (size_t)i + 2] = G;
+      store_fr(&B->c_out[i], c);
+      store_digest_bytes(B->tree + (size_t)(B->P2 + i) * 32, node);
+      if (P.scr->status != VL_OK) atomicExch(&B->status, P.scr->status);
+    }
   }
 }
 
@@ -88,12 +111,41 @@ __device__ void bt_tree(BtState* B) {
   }
 }
 
-// One block: batch start, rho, weights, combined claim.
+// Round t's transcript step by the whole block (at least 4 warps) from g(0)
+// and the leading coefficient G (canonical, valid in warp 0): message, absorb,
+// squeeze r_t, the next claim.
+__device__ void bt_step(BtState* B, RndShared& sh, int t, const Fr& g0, const Fr& G) {
+  const int tid = threadIdx.x, warp = tid >> 5;
+  if (tid < 8) sh.S[tid] = B->St[tid];
+  if (tid == 0) sh.claim = B->claim;
+  __syncthreads();
+  if (warp == 0) {
+    const Fr g1 = fr_sub(sh.claim, g0), g2 = fr_sub(fr_dbl(fr_add(g1, G)), g0);
+    if (tid == 0) {
+      sh.g[0] = g0;
+      sh.g[1] = g1;
+      sh.g[2] = g2;
+      sh.g[3] = G;
+    }
+    __syncwarp();
+    if (tid < 24) B->out->g[t - 1][tid >> 3].limb[tid & 7] = sh.g[tid >> 3].v[tid & 7];
+  }
+  transcript_step(sh, warp, false, &B->r[t - 1]);
+  __syncthreads();
+  if (tid < 8) B->St[tid] = sh.S[tid];
+  if (tid == 0) {
+    next_claim(sh);
+    B->claim = sh.claim;
+  }
+}
+
+// One block: batch start, rho, weights, combined claim, round 1.
 __global__ void __launch_bounds__(BT_THREADS) bt_start_kernel(BtState* B) {
+  __shared__ RndShared sh;
   __shared__ uint32_t S0[8], S1[8];
   __shared__ uint32_t dig[3][8];
   __shared__ Fr ch[1];
-  __shared__ Fr red[BT_THREADS / 32];
+  __shared__ Fr red[3 * (BT_THREADS / 32)];
   bt_tree(B);
   if (threadIdx.x < 32) {
     __shared__ __align__(16) uint8_t msg[128];
@@ -109,7 +161,7 @@ __global__ void __launch_bounds__(BT_THREADS) bt_start_kernel(BtState* B) {
   __syncthreads();
   squeeze_dev(S0, LBL_P, 1, ch, S1, dig);
   const Fr rho = ch[0];
-  Fr acc[1] = {fr_zero()};
+  Fr acc[3] = {fr_zero(), fr_zero(), fr_zero()};  // claim, g(0), G
   for (int i = threadIdx.x; i < B->K; i += blockDim.x) {
     Fr w = fr_r1(), base = rho;  // rho^i by squaring
     for (int e = i; e; e >>= 1) {
@@ -117,130 +169,111 @@ __global__ void __launch_bounds__(BT_THREADS) bt_start_kernel(BtState* B) {
       base = mont_mul_ni(base, base);
     }
     B->w[i] = w;
-    acc[0] = fr_add(acc[0], mont_mul_ni(w, B->c[i]));
+    for (int q = 0; q < 3; q++) acc[q] = fr_add(acc[q], mont_mul_ni(w, B->c[3 * (size_t)i + q]));
   }
-  block_sum_fr<1>(acc, red);
-  if (threadIdx.x == 0) {
-    B->rho = rho;
-    B->claim = acc[0];
-    for (int i = 0; i < 8; i++) B->St[i] = S1[i];
-  }
+  block_sum_fr<3>(acc, red);
+  if (threadIdx.x == 0) B->claim = acc[0];
+  if (threadIdx.x < 8) B->St[threadIdx.x] = S1[threadIdx.x];
+  __syncthreads();
+  if (B->d1 > 0) bt_step(B, sh, 1, acc[1], acc[2]);
 }
 
-// Round t over pairs [k0, k1) of one product (item.proof = its DevProof
-// index): fold with r_{t-1} (the first round reads the unfolded vectors, the
-// second folds them into fA/fB, later rounds fold in place), then the
-// rho^i-weighted sums of a0 b0 and (2a1 - a0)(2b1 - b0).
-__global__ void __launch_bounds__(BT_THREADS) bt_pass_kernel(const DevProof* dp, BtState* B, int t,
-                                                              const LkItem* items) {
-  __shared__ Fr red[2 * (BT_THREADS / 32)];
+// Round t >= 2 over pairs [k0, k1) of one product per CTA (item.proof = its
+// DevProof index): fold with r_{t-1} in place, then the rho^i-weighted sums of
+// a0 b0 and (a1 - a0)(b1 - b0).  Short rounds take four lanes per pair.  The CTA
+// that finishes last adds the partial sums and runs the transcript step (a
+// launch of its own per round cost 30 us, most of it launch and one thread's
+// serial hashes and products).
+__global__ void __launch_bounds__(BT_THREADS) bt_round_kernel(const DevProof* dp, BtState* B, int t,
+                                                               const LkItem* items) {
+  __shared__ RndShared sh;
+  __shared__ bool last;
   const LkItem it = items[blockIdx.x];
   const DevProof& P = dp[it.proof];
-  const int h = 1 << (B->d1 - t);
-  Fr acc[2] = {fr_zero(), fr_zero()};
-  for (int j = it.k0 + threadIdx.x; j < it.k1; j += blockDim.x) {
-    Fr a0, a1, b0, b1;
-    if (t == 1) {
-      a0 = bt_level0(P, 0, j), a1 = bt_level0(P, 0, j + h);
-      b0 = bt_level0(P, 1, j), b1 = bt_level0(P, 1, j + h);
-    } else if (t == 2) {
-      const Fr r = B->r[0];
-      a0 = fold1(bt_level0(P, 0, j), bt_level0(P, 0, j + 2 * h), r);
-      a1 = fold1(bt_level0(P, 0, j + h), bt_level0(P, 0, j + 3 * h), r);
-      b0 = fold1(bt_level0(P, 1, j), bt_level0(P, 1, j + 2 * h), r);
-      b1 = fold1(bt_level0(P, 1, j + h), bt_level0(P, 1, j + 3 * h), r);
-      P.fA[j] = a0, P.fA[j + h] = a1, P.fB[j] = b0, P.fB[j + h] = b1;
-    } else {
-      const Fr r = B->r[t - 2];
-      a0 = fold1(P.fA[j], P.fA[j + 2 * h], r);
-      a1 = fold1(P.fA[j + h], P.fA[j + 3 * h], r);
-      b0 = fold1(P.fB[j], P.fB[j + 2 * h], r);
-      b1 = fold1(P.fB[j + h], P.fB[j + 3 * h], r);
-      P.fA[j] = a0, P.fA[j + h] = a1, P.fB[j] = b0, P.fB[j + h] = b1;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, hh = 1 << (B->d1 - t), h = 2 * hh;
+  const Fr r = B->r[t - 2];
+  Fr s = fr_zero();
+  if (4 * hh <= BT_THREADS) {
+    const int j = tid >> 2, q = tid & 3;
+    const bool act = j < hh;
+    Fr* f = (q < 2 ? P.fA : P.fB) + j + (q & 1) * hh;
+    Fr x = fr_zero(), d = fr_zero();
+    if (act) {
+      x = f[0];
+      d = fr_sub(f[h], x);
     }
-    acc[0] = fr_add(acc[0], mont_mul_ni(a0, b0));
-    acc[1] = fr_add(acc[1], mont_mul_ni(fr_sub(fr_dbl(a1), a0), fr_sub(fr_dbl(b1), b0)));
-  }
-  block_sum_fr<2>(acc, red);
-  if (threadIdx.x == 0) {
-    const Fr w = B->w[P.member1 - 1];
-    B->part[(size_t)it.slot * 2] = mont_mul_ni(w, acc[0]);
-    B->part[(size_t)it.slot * 2 + 1] = mont_mul_ni(w, acc[1]);
-  }
-}
-
-// One block: round t's polynomial from the partial sums, its values in the
-// proof, absorb, squeeze r_t, new claim.
-__global__ void __launch_bounds__(BT_THREADS) bt_round_kernel(BtState* B, int t) {
-  __shared__ Fr red[2 * (BT_THREADS / 32)];
-  __shared__ uint32_t Sw[8], Sn[8];
-  __shared__ uint32_t dig[3][8];
-  __shared__ Fr ch[1];
-  __shared__ Fr gsh[3];
-  Fr acc[2] = {fr_zero(), fr_zero()};
-  for (int s = B->pbeg[t] + threadIdx.x; s < B->pend[t]; s += blockDim.x) {
-    acc[0] = fr_add(acc[0], B->part[(size_t)s * 2]);
-    acc[1] = fr_add(acc[1], B->part[(size_t)s * 2 + 1]);
-  }
-  block_sum_fr<2>(acc, red);
-  if (threadIdx.x == 0) {
-    const Fr g[3] = {acc[0], fr_sub(B->claim, acc[0]), acc[1]};
-    Fr gc[3];
-    for (int q = 0; q < 3; q++) {
-      gsh[q] = g[q];
-      gc[q] = from_mont_ni(g[q]);
-      for (int l = 0; l < 8; l++) B->out->g[t - 1][q].limb[l] = gc[q].v[l];
+    __syncwarp();
+    Fr p = quad_terms(x, d, r, false);
+    if (act) f[0] = x;
+    else p = fr_zero();
+    Fr* red = reinterpret_cast<Fr*>(sh.red);
+#pragma unroll
+    for (int off = 4; off < 32; off <<= 1) p = fr_add(p, shfl_xor_fr(p, off));
+    if (lane < 2) red[2 * warp + lane] = p;
+    __syncthreads();
+    if (warp == 0) {
+      p = lane < 2 * (BT_THREADS / 32) ? red[lane] : fr_zero();
+#pragma unroll
+      for (int off = 2; off < 32; off <<= 1) p = fr_add(p, shfl_xor_fr(p, off));
+      s = from_mont_ni(p);
     }
-    uint32_t S[8];
-    for (int i = 0; i < 8; i++) S[i] = B->St[i];
-    const Fr m2[2] = {gc[0], gc[2]};
-    dev_absorb_fr<2>(S, LBL_G, m2);
-    for (int i = 0; i < 8; i++) Sw[i] = S[i];
+  } else {
+    uint32_t w0[17], wi[17];
+    wide_zero(w0), wide_zero(wi);
+    for (int j = it.k0 + tid; j < it.k1; j += BT_THREADS) fold_pair(P.fA, P.fB, P.fA, P.fB, j, h, r, w0, wi);
+    unsigned long long col[2][8];
+    wide_redc(w0, col[0]);
+    wide_redc(wi, col[1]);
+    s = block_sum_columns<2>(col, sh.red);
+  }
+  if (tid < 2) {
+    B->part[(size_t)it.slot * 2 + tid] = mont_mul_ni(B->w[P.member1 - 1], s);
+    __threadfence();  // the partial sums before the ticket
   }
   __syncthreads();
-  squeeze_dev(Sw, LBL_R, 1, ch, Sn, dig);
-  if (threadIdx.x == 0) {
-    const Fr r = ch[0];
-    B->r[t - 1] = r;
-    for (int i = 0; i < 8; i++) B->St[i] = Sn[i];
-    // g(r) through (0, g0), (1, g1), (2, g2): g0 (r-1)(r-2)/2 - g1 r(r-2) + g2 r(r-1)/2
-    const Fr one = fr_r1(), two = fr_add(one, one);
-    const Fr r1 = fr_sub(r, one), r2 = fr_sub(r, two);
-    const Fr l0 = mont_mul_ni(mont_mul_ni(r1, r2), B->inv2);
-    const Fr l1 = fr_neg(mont_mul_ni(r, r2));
-    const Fr l2 = mont_mul_ni(mont_mul_ni(r, r1), B->inv2);
-    B->claim = fr_add(fr_add(mont_mul_ni(gsh[0], l0), mont_mul_ni(gsh[1], l1)), mont_mul_ni(gsh[2], l2));
+  if (tid == 0) last = atomicAdd(&B->ticket, 1) == (int)gridDim.x - 1;
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  if (tid == 0) B->ticket = 0;
+  Fr acc[2] = {fr_zero(), fr_zero()};
+  for (int i = B->pbeg[t] + tid; i < B->pend[t]; i += BT_THREADS) {
+    const uint4* p = reinterpret_cast<const uint4*>(B->part + (size_t)i * 2);
+    Fr v[2];
+#pragma unroll
+    for (int q = 0; q < 4; q++) {
+      const uint4 a = __ldcg(p + q);  // other CTAs' writes: past the L1
+      v[q >> 1].v[4 * (q & 1)] = a.x, v[q >> 1].v[4 * (q & 1) + 1] = a.y;
+      v[q >> 1].v[4 * (q & 1) + 2] = a.z, v[q >> 1].v[4 * (q & 1) + 3] = a.w;
+    }
+    acc[0] = fr_add(acc[0], v[0]);
+    acc[1] = fr_add(acc[1], v[1]);
   }
+  __syncthreads();
+  block_sum_fr<2>(acc, reinterpret_cast<Fr*>(sh.red));
+  bt_step(B, sh, t, acc[0], acc[1]);
 }
 
-// One warp per product: a_i, b_i (the last pair folded with r_d1), their
-// canonical outputs and Merkle leaf.
+// One warp per product: a_i (lane 0) and b_i (lane 1), the last pair folded with
+// r_d1, their canonical outputs and Merkle leaf.
 __global__ void __launch_bounds__(32) bt_final_kernel(const DevProof* dp, BtState* B) {
-  if (threadIdx.x != 0) return;
   const DevProof& P = dp[blockIdx.x];
-  const int i = P.member1 - 1, d1 = B->d1;
-  Fr a, b;
-  if (d1 == 0) {
-    a = bt_level0(P, 0, 0);
-    b = bt_level0(P, 1, 0);
-  } else if (d1 == 1) {
-    a = fold1(bt_level0(P, 0, 0), bt_level0(P, 0, 1), B->r[0]);
-    b = fold1(bt_level0(P, 1, 0), bt_level0(P, 1, 1), B->r[0]);
-  } else {
-    a = fold1(P.fA[0], P.fA[1], B->r[d1 - 1]);
-    b = fold1(P.fB[0], P.fB[1], B->r[d1 - 1]);
+  const int i = P.member1 - 1, d1 = B->d1, lane = threadIdx.x;
+  Fr x = fr_zero();
+  if (lane < 2) {
+    const Fr* f = lane == 0 ? P.fA : P.fB;
+    x = d1 == 0 ? f[0] : fold1(f[0], f[1], B->r[d1 - 1]);
+    x = from_mont_ni(x);
+    store_fr(lane == 0 ? &B->a_out[i] : &B->b_out[i], x);
   }
-  const Fr ac = from_mont_ni(a), bc = from_mont_ni(b);
-  for (int l = 0; l < 8; l++) {
-    B->a_out[i].limb[l] = ac.v[l];
-    B->b_out[i].limb[l] = bc.v[l];
-  }
+  __syncwarp();
+  const Fr ac = shfl_fr(x, 0), bc = shfl_fr(x, 1);
   uint32_t Y[17], node[8];  // leaf: 0x00 || i u32le || a_i || b_i
   Y[0] = bswap32((uint32_t)i);
   bt_words(Y, 1, ac);
   bt_words(Y, 9, bc);
   dev_hash_tagged<17>(0u, Y, node);
-  store_digest_bytes(B->tree + (size_t)(B->P2 + i) * 32, node);
+  if (lane == 0) store_digest_bytes(B->tree + (size_t)(B->P2 + i) * 32, node);
 }
 
 // One block: the root of the final values, absorb 'f', the proof.
@@ -271,8 +304,7 @@ cudaError_t launch_batch_claims(const DevProof* dp, int np, BtState* B, cudaStre
 
 cudaError_t launch_batch_round(const DevProof* dp, BtState* B, int t, const LkItem* items, int nitems,
                                cudaStream_t st) {
-  if (nitems) bt_pass_kernel<<<nitems, BT_THREADS, 0, st>>>(dp, B, t, items);
-  bt_round_kernel<<<1, BT_THREADS, 0, st>>>(B, t);
+  bt_round_kernel<<<nitems, BT_THREADS, 0, st>>>(dp, B, t, items);
   return cudaGetLastError();
 }
 

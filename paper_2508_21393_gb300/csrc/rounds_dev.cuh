@@ -100,6 +100,19 @@ __device__ __forceinline__ void first_pair(const Fr& a0, const Fr& a1, const Fr&
   wide_mac(wi, fr_sub(a1, a0), fr_sub(b1, b0));
 }
 
+// Four lanes of a pair: lane q (mod 4) folds x (+ d r: a0, a1, b0, b1); returned
+// are the pair's terms, a0 b0 on lane 0 and (a1 - a0)(b1 - b0) on lane 1.  A
+// lane with `clm` set forms (x + d r) r instead.
+__device__ __forceinline__ Fr quad_terms(Fr& x, const Fr& d, const Fr& r, bool clm) {
+  const int q = threadIdx.x & 3;
+  x = fr_add(x, mont_mul_ni(d, r));
+  const Fr y = shfl_xor_fr(x, 1);
+  Fr z = (q & 1) ? fr_sub(x, y) : x;
+  Fr w = shfl_xor_fr(z, 2);
+  if (clm) z = x, w = r;
+  return mont_mul_ni(z, w);
+}
+
 __device__ __forceinline__ void wide_zero(uint32_t (&w)[17]) {
 #pragma unroll
   for (int i = 0; i < 17; i++) w[i] = 0;
@@ -394,13 +407,8 @@ static __device__ void rounds_block(const DevProof& P, vl_proof* pf, uint8_t* sm
       d = sh.g[3];
     }
     __syncwarp();
-    x = fr_add(x, mont_mul_ni(d, r));
+    Fr p = quad_terms(x, d, r, clm);
     if (act) ((q < 2 ? dA : dB) + j + (q & 1) * hh)[0] = x;
-    const Fr y = shfl_xor_fr(x, 1);
-    Fr z = (q & 1) ? fr_sub(x, y) : x;
-    Fr w = shfl_xor_fr(z, 2);
-    if (clm) z = x, w = r;
-    Fr p = mont_mul_ni(z, w);
     if (clm) sh.claim = fr_add(sh.g[0], p);
     if (!act) p = fr_zero();
 #pragma unroll
