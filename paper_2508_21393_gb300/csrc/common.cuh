@@ -222,6 +222,7 @@ static constexpr int NSTAGE = 4;
 static constexpr int STAGE_BYTES = 16384;
 static constexpr int SLOT_BYTES = 24576;
 static constexpr int ROWDOT_STAGE_COLS = STAGE_BYTES / (ROWDOT_BLOCK_ROWS * 2);  // 128
+static constexpr int FOLD_TILE_TARGET = 304;  // CUDA-core fold tiles a batch is cut into at least (two per SM)
 static constexpr int FOLD_SMEM_HEAD = 128;  // mbarriers
 // Default bound on any single wait for a bulk copy (ns of %globaltimer).
 static constexpr unsigned long long FOLD_WAIT_NS = 2000000000ull;

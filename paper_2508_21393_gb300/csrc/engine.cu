@@ -259,9 +259,20 @@ void add_fold_task(vl_plan* p, const vl_mat& M, int32_t mode, int proof, int sid
   p->tasks.push_back(t);
   const size_t tiles_before = p->tiles.size();
   const bool fr = M.dtype == VL_FR_MONT;
+  // Tiles are cut smaller while the batch would leave SMs without work: two
+  // tiles per SM over all tasks, down to 32 rows (16 of a Montgomery column
+  // sum), then to 256 columns.  A lone 601 x 2057 x 1033 product with odd rows has
+  // 43 full-size tiles (435 us, 407 in 350 small ones), one of 512 x 2048 x 256
+  // Montgomery operands 32 (563 and 378 us).
+  const int64_t want = std::max<int64_t>(1, FOLD_TILE_TARGET / (2 * (int64_t)p->jobs.size()));
+  auto count = [&](int tr, int tc) { return (((int64_t)t.rows + tr - 1) / tr) * (((int64_t)t.cols + tc - 1) / tc); };
   if (mode == MODE_COLSUM) {
-    const int tc = fr ? FR_COLSUM_TILE_COLS : COLSUM_TILE_COLS;
-    const int tr = p->opts.colsum_rows > 0 ? p->opts.colsum_rows : 256;
+    int tc = fr ? FR_COLSUM_TILE_COLS : COLSUM_TILE_COLS;
+    int tr = p->opts.colsum_rows > 0 ? p->opts.colsum_rows : 256;
+    if (p->opts.colsum_rows <= 0) {
+      while (tr > (fr ? 16 : 32) && count(tr, tc) < want) tr /= 2;
+      while (tc > 256 && count(tr, tc) < want) tc /= 2;
+    }
     for (int c0 = 0; c0 < t.cols; c0 += tc)
       for (int r0 = 0; r0 < t.rows; r0 += tr) {
         FoldTile ft{};
@@ -276,12 +287,17 @@ void add_fold_task(vl_plan* p, const vl_mat& M, int32_t mode, int proof, int sid
   } else {
     int tcmax = p->opts.rowdot_cols > 0 ? p->opts.rowdot_cols : ROWDOT_TILE_COLS;
     tcmax = (tcmax + 7) & ~7;
+    int tr = ROWDOT_TILE_ROWS;
+    if (p->opts.rowdot_cols <= 0) {
+      while (tr > 32 && count(tr, tcmax) < want) tr /= 2;
+      while (tcmax > (fr ? 64 : 256) && count(tr, tcmax) < want) tcmax /= 2;
+    }
     for (int c0 = 0; c0 < t.cols; c0 += tcmax)
-      for (int r0 = 0; r0 < t.rows; r0 += ROWDOT_TILE_ROWS) {
+      for (int r0 = 0; r0 < t.rows; r0 += tr) {
         FoldTile ft{};
         ft.task = task;
         ft.r0 = r0;
-        ft.r1 = std::min<int>(t.rows, r0 + ROWDOT_TILE_ROWS);
+        ft.r1 = std::min<int>(t.rows, r0 + tr);
         ft.c0 = c0;
         ft.c1 = std::min<int>(t.cols, c0 + tcmax);
         p->tiles.push_back(ft);

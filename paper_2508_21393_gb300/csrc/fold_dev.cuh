@@ -24,10 +24,10 @@
 // (again bounded) for its own copies still in flight, and returns.  Operands
 // that are not aligned take a register-load path.
 //
-// Montgomery operands (32 bytes per entry): one Montgomery product per entry,
-// mont_mul(E.R^2, x.R) = E.x.R^2, summed mod r per thread; partial sums are
-// added limb-wise into the same 64-bit accumulators, whose REDC again gives
-// the Montgomery form.
+// Montgomery operands (32 bytes per entry): a thread sums the 512-bit products
+// (E.R^2)(x.R) unreduced (64 multiply-adds per entry) and reduces once,
+// to E.x.R^2; partial sums are added limb-wise into the same 64-bit
+// accumulators, whose REDC again gives the Montgomery form.
 #pragma once
 #include "common.cuh"
 #include "reduce.cuh"
@@ -606,15 +606,17 @@ static __device__ void colsum_fr(const FoldTask& T, const FoldTile& t, const Fr*
   const int col = tid & (G - 1), lr = tid / G;
   if (col >= ncols) return;
   const Fr* M = static_cast<const Fr*>(T.mat) + t.c0 + col;
-  Fr s = fr_zero();
-  for (int r = lr; r < nrows; r += RL) {
-    const Fr x = load_fr(M + (int64_t)(t.r0 + r) * T.ld);
-    const Fr* e = reinterpret_cast<const Fr*>(sm + 2 * r);
-    s = fr_add(s, mont_mul(x, *e));
-  }
+  uint32_t w[17];
+#pragma unroll
+  for (int i = 0; i < 17; i++) w[i] = 0;
+#pragma unroll 2
+  for (int r = lr; r < nrows; r += RL)
+    wide_mac(w, load_fr(M + (int64_t)(t.r0 + r) * T.ld), reinterpret_cast<const Fr*>(sm)[r]);
+  u64 s[8];
+  wide_redc(w, s);
   u64* dst = acc + (size_t)(t.c0 + col) * 8;
 #pragma unroll
-  for (int l = 0; l < 8; l++) red_add_u64(dst + l, s.v[l]);
+  for (int l = 0; l < 8; l++) red_add_u64(dst + l, s[l]);
 }
 
 // ROWDOT of a Montgomery matrix: 4 rows per warp, lanes over columns.
@@ -632,24 +634,30 @@ static __device__ void rowdot_fr(const FoldTask& T, const FoldTile& t, const Fr*
   const int warp = tid >> 5, lane = tid & 31;
   const int rb = t.r0 + warp * ROWDOT_ROWS_PER_WARP;
   const Fr* M = static_cast<const Fr*>(T.mat);
-  Fr s[ROWDOT_ROWS_PER_WARP];
-#pragma unroll
-  for (int rr = 0; rr < ROWDOT_ROWS_PER_WARP; rr++) s[rr] = fr_zero();
-  for (int j = lane; j < ncols; j += 32) {
-    Fr e;
-#pragma unroll
-    for (int l = 0; l < 8; l++) e.v[l] = sm[l * pitch + j];
-#pragma unroll
-    for (int rr = 0; rr < ROWDOT_ROWS_PER_WARP; rr++) {
-      const int r = rb + rr;
-      if (r < t.r1) s[rr] = fr_add(s[rr], mont_mul(load_fr(M + (int64_t)r * T.ld + t.c0 + j), e));
-    }
-  }
   u64 a[32];
 #pragma unroll
-  for (int rr = 0; rr < ROWDOT_ROWS_PER_WARP; rr++)
+  for (int r2 = 0; r2 < ROWDOT_ROWS_PER_WARP; r2 += 2) {  // two rows at a time (their wide sums in registers)
+    uint32_t w[2][17];
 #pragma unroll
-    for (int l = 0; l < 8; l++) a[rr * 8 + l] = s[rr].v[l];
+    for (int i = 0; i < 17; i++) w[0][i] = w[1][i] = 0;
+    for (int j = lane; j < ncols; j += 32) {
+      Fr e;
+#pragma unroll
+      for (int l = 0; l < 8; l++) e.v[l] = sm[l * pitch + j];
+#pragma unroll
+      for (int rr = 0; rr < 2; rr++) {
+        const int r = rb + r2 + rr;
+        if (r < t.r1) wide_mac(w[rr], load_fr(M + (int64_t)r * T.ld + t.c0 + j), e);
+      }
+    }
+#pragma unroll
+    for (int rr = 0; rr < 2; rr++) {
+      u64 c[8];
+      wide_redc(w[rr], c);
+#pragma unroll
+      for (int l = 0; l < 8; l++) a[(r2 + rr) * 8 + l] = c[l];
+    }
+  }
   const u64 tot = warp_transpose_sum(a);
   const int r = rb + (lane >> 3);
   if (r < t.r1) red_add_u64(acc + (size_t)r * 8 + (lane & 7), tot);
