@@ -170,7 +170,9 @@ struct vl_plan {
   std::vector<RoundItem> ritems;
   std::vector<int> ibase;           // per round: np_t + 1 prefix offsets into that round's items
   std::vector<int> r_item0, r_nitem, r_ib0, r_np;  // per round t (index t): first item, items, ibase start, proofs
-  size_t off_ritems = 0, off_ibase = 0, off_partials = 0;
+  size_t off_ritems = 0, off_ibase = 0, off_ritems_end = 0, off_partials = 0;
+  size_t off_tables_end = 0;
+  std::vector<uint8_t> upload;      // the packed tables while their copy may be running
   struct PerProof {
     size_t eqA, eqB, soaA, soaB, w8A, w8B, accA, accB, fA, fB, fac;
   };
@@ -440,12 +442,12 @@ int build_plan(vl_plan* p) {
   p->proofs.resize(np);
   p->pp.resize(np);
   size_t off = 0;
-  p->off_proofs = off;
-  off = align_up(off + sizeof(DevProof) * np);
   p->off_scr = off;
   off = align_up(off + sizeof(ProofScratch) * np);
   p->off_out = off;
   off = align_up(off + sizeof(vl_proof) * np);
+  p->off_proofs = off;
+  off = align_up(off + sizeof(DevProof) * np);
 
   // Proofs are laid out by k descending (their rounds take longest, so they
   // should finish first); DevProof.job maps back to the caller's order.
@@ -514,6 +516,7 @@ int build_plan(vl_plan* p) {
   off = align_up(off + sizeof(CUtensorMap) * p->tasks.size());
   p->off_items = off;
   off = align_up(off + sizeof(StepItem) * p->items.size());
+  p->off_tables_end = off;
   // step control block and accumulators: one contiguous region, zeroed each pass
   p->off_ctl = off;
   off = align_up(off + sizeof(int) * (STEP_CTL_HEAD_INTS + 2 * (size_t)np));
@@ -597,6 +600,7 @@ int build_plan(vl_plan* p) {
     off = align_up(off + sizeof(RoundItem) * std::max<size_t>(p->ritems.size(), 1));
     p->off_ibase = off;
     off = align_up(off + sizeof(int) * std::max<size_t>(p->ibase.size(), 1));
+    p->off_ritems_end = off;
     p->off_partials = off;
     off = align_up(off + 3 * sizeof(Fr) * max_items);
   }
@@ -751,8 +755,10 @@ bool encode_weight_map(const FoldTask& t, const uint32_t* soa, int pitch, CUtens
              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// Fill device pointers for this workspace and upload the descriptor tables.
-int bind_workspace(vl_plan* p, uint8_t* ws, cudaStream_t st) {
+// Fill device pointers for this workspace and upload the descriptor tables
+// (wait: until the copies are done, for callers whose plan may go, or be bound
+// again, before they next wait for the stream).
+int bind_workspace(vl_plan* p, uint8_t* ws, cudaStream_t st, bool wait = true) {
   const int np = (int)p->jobs.size();
   for (int i = 0; i < np; i++) {
     DevProof& P = p->proofs[i];
@@ -820,40 +826,33 @@ int bind_workspace(vl_plan* p, uint8_t* ws, cudaStream_t st) {
     d.corrR = direct ? (R.side ? &PR.scr->corrB : &PR.scr->corrA) : nullptr;
     d.accC = C.side ? PC.accB : PC.accA;
   }
-  cudaError_t e = cudaMemcpyAsync(ws + p->off_proofs, p->proofs.data(), sizeof(DevProof) * np,
-                                  cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess && !p->dual_tiles.empty())
-    e = cudaMemcpyAsync(ws + p->off_dual_tiles, p->dual_tiles.data(), sizeof(DualTile) * p->dual_tiles.size(),
-                        cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess && !p->tasks.empty())
-    e = cudaMemcpyAsync(ws + p->off_tasks, p->tasks.data(), sizeof(FoldTask) * p->tasks.size(),
-                        cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess && !p->tiles.empty())
-    e = cudaMemcpyAsync(ws + p->off_tiles, p->tiles.data(), sizeof(FoldTile) * p->tiles.size(),
-                        cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess && !p->tc_tiles.empty())
-    e = cudaMemcpyAsync(ws + p->off_tc_tiles, p->tc_tiles.data(), sizeof(TcTile) * p->tc_tiles.size(),
-                        cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess && !p->eq_items.empty())
-    e = cudaMemcpyAsync(ws + p->off_eq_items, p->eq_items.data(), sizeof(EqItem) * p->eq_items.size(),
-                        cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess && !p->tmaps.empty())
-    e = cudaMemcpyAsync(ws + p->off_tmaps, p->tmaps.data(), sizeof(CUtensorMap) * p->tmaps.size(),
-                        cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess && !p->etmaps.empty())
-    e = cudaMemcpyAsync(ws + p->off_etmaps, p->etmaps.data(), sizeof(CUtensorMap) * p->etmaps.size(),
-                        cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess && !p->items.empty())
-    e = cudaMemcpyAsync(ws + p->off_items, p->items.data(), sizeof(StepItem) * p->items.size(),
-                        cudaMemcpyHostToDevice, st);
+  // The tables lie in two runs of the workspace (descriptors and items, the
+  // batched rounds' items): each is packed on the host and copied at once.
+  p->upload.assign(p->off_tables_end - p->off_proofs + p->off_ritems_end - p->off_ritems, 0);
+  auto put = [&](size_t base, size_t off, const void* src, size_t bytes) {
+    if (bytes) std::memcpy(p->upload.data() + base + off, src, bytes);
+  };
+  const size_t second = p->off_tables_end - p->off_proofs;
+  auto first = [&](size_t off, const void* src, size_t bytes) { put(0, off - p->off_proofs, src, bytes); };
+  first(p->off_proofs, p->proofs.data(), sizeof(DevProof) * np);
+  first(p->off_tasks, p->tasks.data(), sizeof(FoldTask) * p->tasks.size());
+  first(p->off_tiles, p->tiles.data(), sizeof(FoldTile) * p->tiles.size());
+  first(p->off_tc_tiles, p->tc_tiles.data(), sizeof(TcTile) * p->tc_tiles.size());
+  first(p->off_eq_items, p->eq_items.data(), sizeof(EqItem) * p->eq_items.size());
+  first(p->off_dual_tiles, p->dual_tiles.data(), sizeof(DualTile) * p->dual_tiles.size());
+  first(p->off_tmaps, p->tmaps.data(), sizeof(CUtensorMap) * p->tmaps.size());
+  first(p->off_etmaps, p->etmaps.data(), sizeof(CUtensorMap) * p->etmaps.size());
+  first(p->off_items, p->items.data(), sizeof(StepItem) * p->items.size());
+  put(second, 0, p->ritems.data(), sizeof(RoundItem) * p->ritems.size());
+  put(second, p->off_ibase - p->off_ritems, p->ibase.data(), sizeof(int) * p->ibase.size());
+  cudaError_t e = cudaMemcpyAsync(ws + p->off_proofs, p->upload.data(), second, cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess && !p->ritems.empty())
-    e = cudaMemcpyAsync(ws + p->off_ritems, p->ritems.data(), sizeof(RoundItem) * p->ritems.size(),
+    e = cudaMemcpyAsync(ws + p->off_ritems, p->upload.data() + second, p->off_ritems_end - p->off_ritems,
                         cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess && !p->ibase.empty())
-    e = cudaMemcpyAsync(ws + p->off_ibase, p->ibase.data(), sizeof(int) * p->ibase.size(), cudaMemcpyHostToDevice,
-                        st);
-  // The host vectors must outlive the copies: wait for them.
-  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+  if (wait && e == cudaSuccess) {
+    e = cudaStreamSynchronize(st);
+    std::vector<uint8_t>().swap(p->upload);
+  }
   if (e == cudaSuccess && p->fold_smem > 0) e = fold_set_smem(p->fold_smem);
   if (e == cudaSuccess && !p->tc_tiles.empty()) e = fold_tc_prepare();
   if (e == cudaSuccess && !p->dual_tiles.empty()) e = fold_dual_prepare();
@@ -884,21 +883,28 @@ cudaError_t ensure_events(vl_plan* p) {
       if (e != cudaSuccess) return e;
     }
   }
-  if (!p->ring.empty()) return cudaSuccess;
-  p->ring.resize((size_t)p->ring_runs * vl_plan::NEV);
-  for (cudaEvent_t& ev : p->ring) {
-    cudaError_t e = cudaEventCreate(&ev);
-    if (e != cudaSuccess) return e;
-  }
-  for (cudaEvent_t& ev : p->cap_ev) {
-    cudaError_t e = cudaEventCreate(&ev);
-    if (e != cudaSuccess) return e;
-  }
   return cudaSuccess;
 }
 
-cudaEvent_t* slot_events(vl_plan* p, long run) {
-  return &p->ring[(size_t)(run % p->ring_runs) * vl_plan::NEV];
+// The phase-boundary events of a run of a plan that its caller may ask for
+// phase times, made when its ring slot is first used (a plan of 64 timed runs
+// would make 256 of them before its first proof).
+cudaError_t slot_events(vl_plan* p, long run, cudaEvent_t** out) {
+  if (p->ring.empty()) p->ring.assign((size_t)p->ring_runs * vl_plan::NEV, nullptr);
+  cudaEvent_t* ev = &p->ring[(size_t)(run % p->ring_runs) * vl_plan::NEV];
+  for (int q = 0; q < vl_plan::NEV; q++)
+    if (!ev[q])
+      if (cudaError_t e = cudaEventCreate(&ev[q])) return e;
+  *out = ev;
+  return cudaSuccess;
+}
+
+// The events that stand for the phase boundaries in a captured graph.
+cudaError_t capture_events(vl_plan* p) {
+  for (cudaEvent_t& ev : p->cap_ev)
+    if (!ev)
+      if (cudaError_t e = cudaEventCreate(&ev)) return e;
+  return cudaSuccess;
 }
 
 // Claims and rounds of every proof: one CTA per proof (rounds_kernel), or
@@ -928,7 +934,7 @@ int rounds_launches(const vl_plan* p) {
 }
 
 // The device part of one proving pass (graph-capturable).  `ev`: the four
-// phase-boundary events to record.
+// phase-boundary events to record, or null.
 cudaError_t enqueue_pass(vl_plan* p, uint8_t* ws, vl_proof* dout, cudaStream_t st, cudaEvent_t* ev,
                          bool capturing) {
   const DevProof* dp = reinterpret_cast<const DevProof*>(ws + p->off_proofs);
@@ -940,19 +946,20 @@ cudaError_t enqueue_pass(vl_plan* p, uint8_t* ws, vl_proof* dout, cudaStream_t s
   // Under capture, external records become event-record nodes of the graph
   // (the flag is only valid while capturing).
   const unsigned flags = capturing ? cudaEventRecordExternal : cudaEventRecordDefault;
-  cudaError_t e = cudaEventRecordWithFlags(ev[0], st, flags);
+  auto record = [&](int q) { return ev ? cudaEventRecordWithFlags(ev[q], st, flags) : cudaSuccess; };
+  cudaError_t e = record(0);
   if (persistent(p)) {
     // One launch: [0] clear, [1] the persistent step (prologues, folds and
     // rounds interleaved), [2] empty.
     int* ctl = reinterpret_cast<int*>(ws + p->off_ctl);
     const StepItem* di = reinterpret_cast<const StepItem*>(ws + p->off_items);
     if (e == cudaSuccess) e = cudaMemsetAsync(ws + p->off_ctl, 0, p->off_acc - p->off_ctl + p->acc_bytes, st);
-    if (e == cudaSuccess) e = cudaEventRecordWithFlags(ev[1], st, flags);
+    if (e == cudaSuccess) e = record(1);
     if (e == cudaSuccess)
       e = launch_step(di, (int)p->items.size(), dt, dl, dp, np, dout, ctl, p->step_grid, p->step_smem, wait_ns(p),
                       never_ready_slot(p), st);
-    if (e == cudaSuccess) e = cudaEventRecordWithFlags(ev[2], st, flags);
-    if (e == cudaSuccess) e = cudaEventRecordWithFlags(ev[3], st, flags);
+    if (e == cudaSuccess) e = record(2);
+    if (e == cudaSuccess) e = record(3);
     return e;
   }
   // Phase launches in groups: stream st folds group g while the rounds stream
@@ -965,15 +972,15 @@ cudaError_t enqueue_pass(vl_plan* p, uint8_t* ws, vl_proof* dout, cudaStream_t s
     // One group: everything in order on the caller's stream.
     if (e == cudaSuccess) e = cudaMemsetAsync(ws + p->off_ctl, 0, p->off_acc + p->acc_bytes - p->off_ctl, st);
     if (e == cudaSuccess) e = launch_prologue(dp, 0, np, de, (int)p->eq_items.size(), st);
-    if (e == cudaSuccess) e = cudaEventRecordWithFlags(ev[1], st, flags);
+    if (e == cudaSuccess) e = record(1);
     if (e == cudaSuccess)
       e = launch_fold_dual(reinterpret_cast<const DualTile*>(ws + p->off_dual_tiles), (int)p->dual_tiles.size(), dp,
                            wait_ns(p), st);
     if (e == cudaSuccess) e = launch_fold_tc(dc, (int)p->tc_tiles.size(), dp, wait_ns(p), st);
     if (e == cudaSuccess) e = launch_fold(dt, dl, (int)p->tiles.size(), dp, p->fold_smem, wait_ns(p), st);
-    if (e == cudaSuccess) e = cudaEventRecordWithFlags(ev[2], st, flags);
+    if (e == cudaSuccess) e = record(2);
     if (e == cudaSuccess) e = enqueue_rounds(p, ws, dp, dout, st);
-    if (e == cudaSuccess) e = cudaEventRecordWithFlags(ev[3], st, flags);
+    if (e == cudaSuccess) e = record(3);
     return e;
   }
   cudaStream_t rs = p->side[0], ps = p->side[1];
@@ -985,7 +992,7 @@ cudaError_t enqueue_pass(vl_plan* p, uint8_t* ws, vl_proof* dout, cudaStream_t s
   if (e == cudaSuccess) e = cudaStreamWaitEvent(rs, gev[2 * ng], 0);
   const vl_plan::Group& g0 = p->groups[0];
   if (e == cudaSuccess) e = launch_prologue(dp, g0.p0, g0.p1, de + g0.e0, g0.e1 - g0.e0, st);
-  if (e == cudaSuccess) e = cudaEventRecordWithFlags(ev[1], st, flags);
+  if (e == cudaSuccess) e = record(1);
   for (int g = 1; g < ng && e == cudaSuccess; g++) {
     const vl_plan::Group& G = p->groups[g];
     e = launch_prologue(dp, G.p0, G.p1, de + G.e0, G.e1 - G.e0, ps);
@@ -1001,12 +1008,12 @@ cudaError_t enqueue_pass(vl_plan* p, uint8_t* ws, vl_proof* dout, cudaStream_t s
     if (e == cudaSuccess) e = cudaStreamWaitEvent(rs, gev[ng + g], 0);
     if (e == cudaSuccess) e = launch_rounds(dp + G.p0, G.p1 - G.p0, dout, p->opts.rounds_variant, p->opts.rounds_threads, rs);
   }
-  if (e == cudaSuccess) e = cudaEventRecordWithFlags(ev[2], st, flags);
+  if (e == cudaSuccess) e = record(2);
   if (e == cudaSuccess) e = cudaEventRecord(gev[2 * ng + 1], rs);
   if (e == cudaSuccess) e = cudaStreamWaitEvent(st, gev[2 * ng + 1], 0);
   if (e == cudaSuccess) e = cudaEventRecord(gev[0], ps);  // join the prologue stream too
   if (e == cudaSuccess) e = cudaStreamWaitEvent(st, gev[0], 0);
-  if (e == cudaSuccess) e = cudaEventRecordWithFlags(ev[3], st, flags);
+  if (e == cudaSuccess) e = record(3);
   return e;
 }
 
@@ -1048,8 +1055,11 @@ int stage_host_operands(vl_plan* p, uint8_t* ws, cudaStream_t st) {
   return VL_OK;
 }
 
+// timed: record the phase boundaries (vl_plan_phase_ms).  keep: the plan lives
+// on after the call; a plan made for one call with host output need not wait for
+// its table uploads, since the call waits for the proofs anyway.
 int run_plan(vl_plan* p, void* workspace, size_t ws_bytes, vl_proof* out, int32_t out_space,
-             cudaStream_t st, bool graph) {
+             cudaStream_t st, bool graph, bool timed = true, bool keep = true) {
   if (!workspace || !out) return VL_EINVAL;
   if (out_space != VL_DEVICE && out_space != VL_HOST) return VL_EINVAL;
   if (ws_bytes < p->total) return VL_ENOMEM;
@@ -1060,15 +1070,17 @@ int run_plan(vl_plan* p, void* workspace, size_t ws_bytes, vl_proof* out, int32_
   if (p->bound_ws != workspace || !owns_workspace(p, workspace)) {
     // The graph holds kernel arguments into the workspace; rebuilt on change.
     if (p->bound_ws != workspace) drop_graph(p);
-    int e = bind_workspace(p, ws, st);
+    int e = bind_workspace(p, ws, st, keep || out_space != VL_HOST);
     if (e != VL_OK) return e;
     p->bound_ws = workspace;
     claim_workspace(p, workspace);
   }
   int e = stage_host_operands(p, ws, st);
   if (e != VL_OK) return e;
-  cudaEvent_t* ev = slot_events(p, p->runs);
   cudaError_t ce;
+  cudaEvent_t* ev = nullptr;
+  if ((graph || timed) && (ce = slot_events(p, p->runs, &ev)) != cudaSuccess) return cuda_status(ce, "cudaEventCreate");
+  if (graph && (ce = capture_events(p)) != cudaSuccess) return cuda_status(ce, "cudaEventCreate");
   if (graph) {
     if (p->gexec && p->bound_out != dout) drop_graph(p);
     if (!p->gexec) {
@@ -1146,7 +1158,7 @@ void plan_set_points(vl_plan* p, const std::vector<const GivenPoint*>& given, co
 }
 // Enqueue one pass (no graph), proofs to device memory in job order.
 int plan_enqueue(vl_plan* p, uint8_t* ws, size_t bytes, vl_proof* dout, cudaStream_t st) {
-  return run_plan(p, ws, bytes, dout, VL_DEVICE, st, false);
+  return run_plan(p, ws, bytes, dout, VL_DEVICE, st, false, false);
 }
 }  // namespace vl
 
@@ -1211,7 +1223,7 @@ int32_t vl_plan_phase_ms(vl_plan* plan, float* ms, int32_t max_runs, int32_t res
   const long cnt = std::min<long>(avail, max_runs);
   for (long i = 0; i < cnt; i++) {
     const long run = plan->runs - cnt + i;
-    cudaEvent_t* ev = slot_events(plan, run);
+    cudaEvent_t* ev = &plan->ring[(size_t)(run % plan->ring_runs) * vl_plan::NEV];
     if (cudaEventSynchronize(ev[3]) != cudaSuccess) return -VL_ECUDA;
     for (int q = 0; q < 3; q++)
       if (cudaEventElapsedTime(&ms[i * 3 + q], ev[q], ev[q + 1]) != cudaSuccess) return -VL_ECUDA;
@@ -1237,7 +1249,8 @@ void vl_plan_destroy(vl_plan* plan) {
     if (s2) cudaStreamDestroy(s2);
   for (cudaEvent_t ev : plan->gev)
     if (ev) cudaEventDestroy(ev);
-  for (cudaEvent_t ev : plan->ring) cudaEventDestroy(ev);
+  for (cudaEvent_t ev : plan->ring)
+    if (ev) cudaEventDestroy(ev);
   for (cudaEvent_t ev : plan->cap_ev)
     if (ev) cudaEventDestroy(ev);
   delete plan;
@@ -1249,9 +1262,11 @@ int32_t vl_prove_batch(const vl_job* jobs, int32_t njobs, void* workspace, size_
   vl_plan* p = nullptr;
   int e = make_plan(jobs, njobs, opts, &p);
   if (e != VL_OK) return e;
-  // Descriptor tables are uploaded synchronously, so the host plan can go
-  // while device work is still queued.
-  e = run_plan(p, workspace, workspace_bytes, out, out_space, static_cast<cudaStream_t>(stream), false);
+  // With device output the descriptor tables are uploaded synchronously, so the
+  // host plan can go while device work is still queued; with host output the
+  // call ends with a wait for the stream.
+  e = run_plan(p, workspace, workspace_bytes, out, out_space, static_cast<cudaStream_t>(stream), false, false, false);
+  if (e != VL_OK) (void)cudaStreamSynchronize(static_cast<cudaStream_t>(stream));  // uploads of a failed call
   vl_plan_destroy(p);
   return e;
   VL_ABI_CATCH(VL_ENOMEM)
