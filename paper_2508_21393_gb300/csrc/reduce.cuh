@@ -68,7 +68,7 @@ __device__ __forceinline__ unsigned long long warp_transpose_sum(unsigned long l
 template <int NV>
 __device__ __forceinline__ Fr block_sum_columns(const unsigned long long (&c)[NV][8], unsigned long long* sh) {
   static_assert(NV * 8 <= 32, "at most 4 values");
-  constexpr int N = NV * 8 <= 8 ? 8 : NV * 8 <= 16 ? 16 : 32;
+  constexpr int N = NV == 1 ? 8 : NV == 2 ? 16 : 32;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   unsigned long long a[N];
 #pragma unroll
