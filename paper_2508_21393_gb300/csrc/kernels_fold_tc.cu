@@ -33,8 +33,8 @@
 //                TC_NW slots
 //   warps 1, 18-20  MMA issuers (warp 1 also owns TMEM, 512 columns): a
 //                pair per stage parity, in each pair one thread for the lo
-//                and one for the hi products.  One thread issues an MMA only
-//                every ~140 cycles, whatever N, while the SM runs several
+//                and one for the hi products.  One thread issues an MMA
+//                every ~58 cycles, whatever N, while the SM runs several
 //                issuers' MMAs at once; so per stage each thread issues the
 //                MMA of constants (accumulator := 2^23) before the operand is
 //                converted, then 8 MMAs (K = 16) with A read from TMEM and B
@@ -112,6 +112,17 @@ __device__ __forceinline__ void umma_ts(uint32_t d, uint32_t a, uint64_t b, uint
       "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
       "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}" ::"r"(d),
       "r"(a), "l"(b), "r"(idesc), "r"(accumulate));
+}
+
+// One lane of a converged warp.  fold_tc_kernel's MMA issuers run under this and not under
+// "lane == 0": the instruction takes its operands from uniform registers, and
+// only an elected lane lets the compiler see that one thread is active (157
+// cycles per MMA and thread under lane == 0, 58 elected; M128 N32 K16, A in TMEM:
+// 7B step 2.31 -> 2.28 ms, 13B step 6.36 -> 6.26).
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n}" : "=r"(p));
+  return p != 0;
 }
 
 // Arrive on `bar` once every MMA this thread issued so far has completed.
@@ -480,7 +491,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     // accumulator buffer and the constant MMA (accumulator := 2^23) go ahead
     // of the wait for the converted operand; only the stage's 8 operand MMAs
     // follow it.
-    if (lane == 0) {
+    if (elect_one()) {
       const int j = warp == 1 ? 0 : warp - (TC_THREADS / 32 - (TC_ISSUERS - 1)) + 1;  // 0..3
       const uint32_t plane = j & 1;
       for (int s = j >> 1;; s += TC_PAIRS) {
