@@ -10,11 +10,15 @@
 // are two dense products (M = 128 lines w, N = 32 bytes b, K = the reduced
 // index i), and
 //     sum_i E_i p[w, i] = sum_{t=0}^{32} 2^(8t) s_t,  s_t = D_lo[w, t] + D_hi[w, t-1].
-// All operands are integers in [0, 255] (exact in fp16); a product is at most
-// 255^2, so over one 128-entry pipeline stage each of D_lo and D_hi is below
-// 255^2 . 128 < 2^23 and fp32 accumulation is exact.  Both accumulators of a
-// stage start at 2^23 (one MMA of constants each), which puts them in
-// [2^23, 2^24), where the fp32 bit pattern is 0x4B000000 + D: the drainers
+// The weights are integers in [0, 255] in fp16; the operand's bytes stand in the
+// low bits of a 16-bit word as they are, which read as fp16 is the subnormal
+// byte . 2^-24 (two logic operations and a permute convert a pair of entries; as
+// 2^10 + byte less 2^10 it took two fp16 subtractions more: 7B step 2.28 -> 2.18
+// ms, 13B step 6.26 -> 6.04).  Products are 2^-24 times integers of at most
+// 255^2, so over one 128-entry pipeline stage each of D_lo and D_hi is 2^-24 times an
+// integer below 255^2 . 128 < 2^23 and fp32 accumulation is exact.  Both accumulators
+// of a stage start at 1/2 (one MMA of constants each), which puts them in
+// [1/2, 1), where the fp32 bit pattern is 0x3F000000 + D 2^24: the drainers
 // add bit patterns as 32-bit integers, s_t += bits(D_lo[t]) +
 // bits(D_hi[t-1]) in one three-input add, and remove the offsets once per
 // tile.  At the end of a tile the 33
@@ -36,11 +40,11 @@
 //                and one for the hi products.  One thread issues an MMA
 //                every ~58 cycles, whatever N, while the SM runs several
 //                issuers' MMAs at once; so per stage each thread issues the
-//                MMA of constants (accumulator := 2^23) before the operand is
+//                MMA of constants (accumulator := 1/2) before the operand is
 //                converted, then 8 MMAs (K = 16) with A read from TMEM and B
 //                (weights) from shared memory
 //   warps 2-9    converters: a warp takes 32 lines x half of the stage's 128
-//                entries from the boxes with ldmatrix, forms the fp16 lo/hi
+//                entries from the boxes with ldmatrix, forms the lo/hi byte
 //                operand fragments and stores them to TMEM (one of TC_NC
 //                operand buffers) with tcgen05.st
 //   warps 10-17  drainers: accumulator buffer -> per-line digit sums (two
@@ -63,8 +67,8 @@ namespace {
 
 constexpr int SM_RAW = 0;                          // TC_NR x 32 KB of int16 operand
 constexpr int SM_W = SM_RAW + TC_NR * 32768;       // TC_NW x 8 KB of fp16 weight bytes
-constexpr int SM_ACONST = SM_W + TC_NW * 8192;    // 128 x 16 fp16, K-major: column 0 = 256
-constexpr int SM_BCONST = SM_ACONST + 4096;        // 16 x 32 fp16, MN-major: row 0 = 32768
+constexpr int SM_ACONST = SM_W + TC_NW * 8192;    // 128 x 16 fp16, K-major: column 0 = 1/2
+constexpr int SM_BCONST = SM_ACONST + 4096;        // 16 x 32 fp16, MN-major: row 0 = 1
 constexpr int SM_XCH = SM_BCONST + 1024;           // 128 lines x 4 u64: drainer groups' column exchange
 constexpr int SM_HDR = SM_XCH + 4096;              // TC_HR stage headers
 constexpr int SM_BAR = SM_HDR + TC_HR * 48;
@@ -196,15 +200,6 @@ __device__ __forceinline__ void ldmatrix4(uint32_t addr, uint32_t* r) {
 }
 __device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
-// Two fp16 values from bytes of t selected by `sel` (bytes 0x64 fill the
-// high halves): 0x64bb is 1024 + bb exactly, minus 1024 leaves bb.
-__device__ __forceinline__ uint32_t bytes_f16x2(uint32_t t, uint32_t sel) {
-  const uint32_t v = __byte_perm(t, 0x64646464u, sel);
-  uint32_t r;
-  asm("sub.rn.f16x2 %0, %1, %2;" : "=r"(r) : "r"(v), "r"(0x64006400u));
-  return r;
-}
-
 // try_wait with a suspend-time hint: a thread whose phase is not complete is
 // suspended in hardware (woken when the phase completes, or after ~1 us)
 // instead of polling, which would take issue slots from the working warps.
@@ -285,7 +280,7 @@ __device__ __forceinline__ void mark_timeout(const DevProof* proofs, const TcTil
 }
 
 // Add one (lo, hi) accumulator pair (lo at ta, hi at ta + 32, both started
-// at 2^23: bit patterns 0x4B000000 + D) to the digit sums s_t, t in [T0, T1]:
+// at 1/2: bit patterns 0x3F000000 + D 2^24) to the digit sums s_t, t in [T0, T1]:
 // dg[t - T0] += bits(D_lo[t]) + bits(D_hi[t - 1]) (D_lo[32] and D_hi[-1] are
 // absent).  The two digit groups read disjoint columns: [0, 15] reads lo
 // 0..15 and hi 0..14, [16, 32] reads lo 16..31 and hi 15..31.
@@ -318,11 +313,11 @@ __device__ __forceinline__ void release_acc(uint32_t acc_empty) {
 }
 
 // The offsets in a digit sum after nst stages of PAIRS accumulator pairs
-// each: 0x4B000000 per accumulator drained into it (digits 0 and 32 take one
+// each: 0x3F000000 per accumulator drained into it (digits 0 and 32 take one
 // accumulator of a pair, the others two).
 template <int PAIRS>
 __device__ __forceinline__ uint32_t digit_offset(int t, int nst) {
-  return (uint32_t)(nst * PAIRS * ((t == 0 || t == 32) ? 1 : 2)) * 0x4B000000u;
+  return (uint32_t)(nst * PAIRS * ((t == 0 || t == 32) ? 1 : 2)) * 0x3F000000u;
 }
 
 // Column sums col_j = sum_q 2^(8q) s_{4j+q} of the digits s_t, t in [T0, T1]
@@ -393,16 +388,16 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
   }
   if (warp >= 2 && warp < 2 + TC_CONV_WARPS) {
-    // Constant operands of the init MMA: A[m][0] = 256, B[0][n] = 32768, so
-    // an accumulator starts at 2^23; every other entry 0.
+    // Constant operands of the init MMA: A[m][0] = 1/2, B[0][n] = 1, so an
+    // accumulator starts at 1/2; every other entry 0.
     const int wi = tid - 64, nw = 32 * TC_CONV_WARPS;
     uint32_t* ac = reinterpret_cast<uint32_t*>(sm + SM_ACONST);
     // A K-major: entry (m, k = 0) at byte m * 16 of the first 2 KB (k < 8).
-    for (int i = wi; i < 1024; i += nw) ac[i] = (i < 512 && (i & 3) == 0) ? 0x5C00u : 0u;
+    for (int i = wi; i < 1024; i += nw) ac[i] = (i < 512 && (i & 3) == 0) ? 0x3800u : 0u;
     // B MN-major: row k = 0 is bytes [0, 16) of each 128-byte core matrix of
     // the first 512 bytes (k < 8).
     uint32_t* bc = reinterpret_cast<uint32_t*>(sm + SM_BCONST);
-    for (int i = wi; i < 256; i += nw) bc[i] = (i < 128 && (i & 31) < 4) ? 0x78007800u : 0u;
+    for (int i = wi; i < 256; i += nw) bc[i] = (i < 128 && (i & 31) < 4) ? 0x3C003C00u : 0u;
     fence_proxy_async_smem();
   }
   tc_fence_before();
@@ -488,7 +483,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     // ---------------------------------------------------------------- MMA issuers
     // Pair g takes stages g, g + TC_PAIRS, ...; in a pair one thread for the
     // lo and one for the hi products.  The waits for the weights and the
-    // accumulator buffer and the constant MMA (accumulator := 2^23) go ahead
+    // accumulator buffer and the constant MMA (accumulator := 1/2) go ahead
     // of the wait for the converted operand; only the stage's 8 operand MMAs
     // follow it.
     if (elect_one()) {
@@ -576,9 +571,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
           uint32_t lo[16], hi[16];
 #pragma unroll
           for (int i = 0; i < 16; i++) {
-            const uint32_t t = w[i] ^ 0x80008000u;  // p = x + 2^15, per entry
-            lo[i] = bytes_f16x2(t, 0x4240);
-            hi[i] = bytes_f16x2(t, 0x4341);
+            lo[i] = w[i] & 0x00ff00ffu;  // p = x + 2^15, per entry: the sign bit flips
+            hi[i] = __byte_perm(w[i], 0, 0x4341) ^ 0x00800080u;
           }
           const uint32_t dst = tq + ((uint32_t)(16 * hl) << 16) + 128 * c;
           tmem_st_frag(dst, lo);
@@ -677,7 +671,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
 //
 // One stored matrix W folded both ways in one pass (DualTile): a strip of 128
 // rows streamed in stages of 128 columns.  Each stage's 128 x 128 block is
-// loaded once (two row-dot TMA boxes), converted once into fp16 lo and hi
+// loaded once (two row-dot TMA boxes), converted once into lo and hi
 // byte planes in shared memory, and read by two MMA sets as their A operand:
 // K-major for the row dots (M = the strip's rows, K = the stage's columns),
 // MN-major for the column sums (M = the stage's columns, K = the strip's
@@ -685,7 +679,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
 // (16 bytes per row along the columns), core (rb, cb) at (16 rb + cb) x 128
 // bytes: along the columns the core stride is 128 bytes, along the rows
 // 2048.  The exactness of the byte-limb products is as in fold_tc_kernel
-// (one accumulation period per stage, accumulators preloaded with 2^23);
+// (one accumulation period per stage, accumulators preloaded with 1/2);
 // the row-dot digit sums run across the strip, the column-sum digits of a
 // stage are turned into column sums and added with red.add at once.
 // Roles: warp 0 producer; warps 1, 18, 19, 20 MMA issuers (row-dot lo, hi,
@@ -789,12 +783,12 @@ __global__ void __launch_bounds__(DU_THREADS, 1)
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
   }
   if (warp >= 2 && warp < 2 + TC_CONV_WARPS) {
-    // constant operands of the 2^23 preload, as in fold_tc_kernel
+    // constant operands of the 1/2 preload, as in fold_tc_kernel
     const int wi = tid - 64, nw = 32 * TC_CONV_WARPS;
     uint32_t* ac = reinterpret_cast<uint32_t*>(sm + DS_ACONST);
-    for (int i = wi; i < 1024; i += nw) ac[i] = (i < 512 && (i & 3) == 0) ? 0x5C00u : 0u;
+    for (int i = wi; i < 1024; i += nw) ac[i] = (i < 512 && (i & 3) == 0) ? 0x3800u : 0u;
     uint32_t* bc = reinterpret_cast<uint32_t*>(sm + DS_BCONST);
-    for (int i = wi; i < 256; i += nw) bc[i] = (i < 128 && (i & 31) < 4) ? 0x78007800u : 0u;
+    for (int i = wi; i < 256; i += nw) bc[i] = (i < 128 && (i & 31) < 4) ? 0x3C003C00u : 0u;
     fence_proxy_async_smem();
   }
   tc_fence_before();
@@ -917,7 +911,7 @@ __global__ void __launch_bounds__(DU_THREADS, 1)
         }
         tc_fence_after();
         const uint32_t d = tmem + 128 * side + 64 * a + half;
-        umma_ss(d, sdesc(base + DS_ACONST, 2048, 128), sdesc(base + DS_BCONST, 512, 128), IDESC, 0);  // := 2^23
+        umma_ss(d, sdesc(base + DS_ACONST, 2048, 128), sdesc(base + DS_BCONST, 512, 128), IDESC, 0);  // := 1/2
 #pragma unroll
         for (int ks = 0; ks < 8; ks++) {
           // K-major rows (row dots): cores 2ks, 2ks + 1 of the columns;
@@ -971,9 +965,8 @@ __global__ void __launch_bounds__(DU_THREADS, 1)
         uint32_t lo[16], hi[16];
 #pragma unroll
         for (int i = 0; i < 16; i++) {
-          const uint32_t t = w[i] ^ 0x80008000u;  // p = x + 2^15
-          lo[i] = bytes_f16x2(t, 0x4240);
-          hi[i] = bytes_f16x2(t, 0x4341);
+          lo[i] = w[i] & 0x00ff00ffu;  // p = x + 2^15
+          hi[i] = __byte_perm(w[i], 0, 0x4341) ^ 0x00800080u;
         }
 #pragma unroll
         for (int c = 0; c < 4; c++) {  // core columns 8 kh + 4 j2 + c: 8 columns, 16 bytes per plane
