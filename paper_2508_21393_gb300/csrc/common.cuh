@@ -109,7 +109,7 @@ struct StepItem {
 };
 // Dynamic shared memory of the prologue and rounds block functions.
 static constexpr int PRO_SMEM = 18816;
-static constexpr int RND_SMEM = 20736;
+static constexpr int RND_SMEM = 21760;
 // Prologue items run this many proofs ahead of their fold tiles in the queue.
 static constexpr int STEP_LOOKAHEAD = 256;
 
@@ -411,7 +411,7 @@ cudaError_t launch_rounds_pass(const DevProof* proofs, const RoundItem* items, i
 cudaError_t launch_rounds_hash(const DevProof* proofs, int nproofs, const int* ibase, const Fr* partials,
                                vl_proof* out, int t, cudaStream_t st);
 cudaError_t launch_rounds_tail(const DevProof* proofs, int nproofs, vl_proof* out, cudaStream_t st);
-cudaError_t launch_rounds(const DevProof* proofs, int nproofs, vl_proof* out, int variant, int threads,
+cudaError_t launch_rounds(const DevProof* proofs, int nproofs, vl_proof* out, int variant, int threads, int max_d1,
                           cudaStream_t st);
 cudaError_t launch_encode(const int16_t* src, int64_t rows, int64_t cols, int64_t ld, Fr* dst,
                           cudaStream_t st);

@@ -913,7 +913,7 @@ cudaError_t capture_events(vl_plan* p) {
 cudaError_t enqueue_rounds(vl_plan* p, uint8_t* ws, const DevProof* dp, vl_proof* dout, cudaStream_t st) {
   const int np = (int)p->jobs.size();
   if (p->opts.rounds_variant != 8)
-    return launch_rounds(dp, np, dout, p->opts.rounds_variant, p->opts.rounds_threads, st);
+    return launch_rounds(dp, np, dout, p->opts.rounds_variant, p->opts.rounds_threads, p->proofs[0].d1, st);
   const RoundItem* items = reinterpret_cast<const RoundItem*>(ws + p->off_ritems);
   const int* ibase = reinterpret_cast<const int*>(ws + p->off_ibase);
   Fr* partials = reinterpret_cast<Fr*>(ws + p->off_partials);
@@ -1006,7 +1006,9 @@ cudaError_t enqueue_pass(vl_plan* p, uint8_t* ws, vl_proof* dout, cudaStream_t s
     if (e == cudaSuccess) e = launch_fold(dt, dl + G.t0, G.t1 - G.t0, dp, p->fold_smem, wait_ns(p), st);
     if (e == cudaSuccess) e = cudaEventRecord(gev[ng + g], st);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(rs, gev[ng + g], 0);
-    if (e == cudaSuccess) e = launch_rounds(dp + G.p0, G.p1 - G.p0, dout, p->opts.rounds_variant, p->opts.rounds_threads, rs);
+    // (no clusters here: they would wait for whole groups of SMs beside the next group's folds)
+    if (e == cudaSuccess)
+      e = launch_rounds(dp + G.p0, G.p1 - G.p0, dout, p->opts.rounds_variant, p->opts.rounds_threads, 0, rs);
   }
   if (e == cudaSuccess) e = record(2);
   if (e == cudaSuccess) e = cudaEventRecord(gev[2 * ng + 1], rs);
@@ -1366,7 +1368,7 @@ extern "C" int32_t vl_prove_matmul_noalloc(const vl_mat* P, const vl_mat* Q, con
     const EqItem* de = reinterpret_cast<const EqItem*>(ws + p->off_eq_items);
     if (ce == cudaSuccess) ce = launch_prologue(dp, 0, 1, de, (int)p->eq_items.size(), st);
     if (ce == cudaSuccess) ce = launch_fold(dt, dl, (int)p->tiles.size(), dp, p->fold_smem, FOLD_WAIT_NS, st);
-    if (ce == cudaSuccess) ce = launch_rounds(dp, 1, dout, 0, 0, st);
+    if (ce == cudaSuccess) ce = launch_rounds(dp, 1, dout, 0, 0, p->proofs[0].d1, st);
     if (ce == cudaSuccess) ce = cudaMemcpyAsync(out, dout, sizeof(vl_proof), cudaMemcpyDeviceToHost, st);
     if (ce == cudaSuccess) ce = cudaStreamSynchronize(st);
     // A failed enqueue may leave earlier kernels of this call running on the

@@ -1,4 +1,4 @@
-// Rounds kernel: one CTA per proof (see rounds_dev.cuh).
+// Rounds kernels: one CTA or one cluster per proof (see rounds_dev.cuh).
 #include <atomic>
 
 #include "rounds_dev.cuh"
@@ -13,6 +13,14 @@ __global__ void __launch_bounds__(THREADS, MINB) rounds_kernel(const DevProof* _
   rounds_block(P, out + P.job, rnd_smem);
 }
 
+// A cluster of CTAs per proof, its first rounds over the cluster.
+__global__ void __launch_bounds__(512, 1) rounds_cluster_kernel(const DevProof* __restrict__ proofs,
+                                                                vl_proof* __restrict__ out) {
+  extern __shared__ __align__(128) uint8_t rnd_smem[];
+  const DevProof& P = proofs[blockIdx.x / cluster_size()];
+  rounds_block(P, out + P.job, rnd_smem, 1, true);
+}
+
 // variant: CTAs per SM.  7, 6, 5 and 4 set the register allocation (7: one
 // wave of 1064 proofs, tighter registers; 4: more registers per thread).  3 and 2
 // use the variant-4 code and cap residency by reserving shared memory, for
@@ -20,12 +28,15 @@ __global__ void __launch_bounds__(THREADS, MINB) rounds_kernel(const DevProof* _
 // 256 or 512 per proof (more threads shorten the vector passes of large
 // proofs; the register budget follows from variant x threads).
 // Both 0: by the number of proofs.  A proof's rounds are a chain, so while
-// there are SMs for all of them each proof gets as many threads as an SM holds
-// at 128 registers (up to one proof per SM: 512, two: 256); beyond that 128
-// threads, four proofs per SM.  Measured with the rounds of rounds_dev.cuh: one
-// 7B projection (8 proofs) 320 -> 232 us, one 13B projection from host memory
-// 750 -> 578, the 7B step (1024 proofs) 2.60 -> 2.48 ms.
-cudaError_t launch_rounds(const DevProof* proofs, int nproofs, vl_proof* out, int variant, int threads,
+// there are SMs for all of them each proof gets a cluster of 8, 4 or 2 CTAs of
+// 512 threads (max_d1: the largest of the batch; 0: no clusters), or as many
+// threads as an SM holds at 128 registers (up to one proof per SM: 512, two:
+// 256); beyond that 128 threads, four proofs per SM.  Measured, one CTA per
+// proof: one 7B projection (8 proofs) 320 -> 232 us, one 13B projection from
+// host memory 750 -> 578, the 7B step (1024 proofs) 2.60 -> 2.48 ms; with the
+// clusters: the 7B projection 230 -> 207 us (rounds 154 -> 131), the 13B one 460 ->
+// 411, a lone product of 2057 terms 294 -> 250.
+cudaError_t launch_rounds(const DevProof* proofs, int nproofs, vl_proof* out, int variant, int threads, int max_d1,
                           cudaStream_t st) {
   if (nproofs <= 0) return cudaSuccess;
   if (variant == 0 && threads == 0) {
@@ -33,6 +44,8 @@ cudaError_t launch_rounds(const DevProof* proofs, int nproofs, vl_proof* out, in
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
+    const int ctas = cluster_rounds(max_d1) > 0 ? cluster_ctas(nproofs, sms) : 1;
+    if (ctas > 1) return launch_clusters(rounds_cluster_kernel, nproofs, ctas, 512, RND_SMEM, st, proofs, out);
     if (nproofs <= sms) threads = 512;
     else if (nproofs <= 2 * sms) threads = 256;
     else variant = 4;

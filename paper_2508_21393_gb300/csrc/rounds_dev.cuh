@@ -1,6 +1,6 @@
 // Claim and sumcheck rounds of each proof (Sec. II-B; Eq. eq:zk-mle-matmul).
 //
-// One CTA per proof.  The fold accumulators become the vectors
+// One CTA per proof, or a cluster of them.  The fold accumulators become the vectors
 // f_A[w] = A~(u, w), f_B[w] = B~(w, v) over the padded cube w < 2^d1 (zeros
 // for w >= k).  Round i (h = 2^(d1 - i)) has the degree-2 round polynomial
 // g(X) = sum_j (a0 + X (a1 - a0)) (b0 + X (b1 - b0)) with a0 = f_A[j],
@@ -39,6 +39,7 @@ namespace vl {
 
 static constexpr int RND_VEC = 256;      // vectors of at most this many entries are kept in shared memory
 static constexpr int RND_MAX_WARPS = 16;
+static constexpr int RND_MAX_CTAS = 8;   // CTAs of a cluster
 
 // Shared memory of the rounds.
 struct RndShared {
@@ -51,6 +52,7 @@ struct RndShared {
   Fr r;                            // the latest challenge (Montgomery)
   alignas(16) unsigned long long red[3 * 8 * RND_MAX_WARPS];
   Fr fa[RND_VEC], fb[RND_VEC];
+  Fr part[RND_MAX_CTAS][4];        // rounds of a cluster: each CTA's g(0), G, g(1), in the first CTA
 };
 static_assert(sizeof(RndShared) <= RND_SMEM, "shared memory of the rounds");
 
@@ -254,20 +256,212 @@ __device__ __forceinline__ void store_state(uint8_t* dst, const ShaState& st) {
   }
 }
 
+// Entries j and j + h of f from the fold: reduced already (direct), or column
+// sums to reduce here; j + h may be padding (!real).  They are written to dst
+// where the vector does not hold them yet (write: always).
+__device__ __forceinline__ void first_entries(const Fr* f, bool direct, const unsigned long long* acc, const Fr& corr,
+                                              int j, int h, bool real, bool write, Fr* dst, Fr& x0, Fr& x1) {
+  x0 = direct ? f[j] : load_acc_fr(acc, j, corr);
+  x1 = fr_zero();
+  if (real) x1 = direct ? f[j + h] : load_acc_fr(acc, j + h, corr);
+  if (write || !direct) dst[j] = x0;
+  if (write || !direct || !real) dst[j + h] = x1;
+}
+
+// One pass of a pair per four lanes over hh pairs (4 hh at most the threads of
+// the calling warps): the vectors sA, sB (2h = 4 hh entries) folded with r into
+// dA, dB, and the round's terms, summed over the warp: lane 0 g(0), lane 1 G
+// (Montgomery form).  j: the thread's pair.  clm: this lane forms the next claim.
+__device__ __forceinline__ Fr quad_pass(RndShared& sh, const Fr* sA, const Fr* sB, Fr* dA, Fr* dB, int j, bool act,
+                                        int h, const Fr& r, bool clm) {
+  const int hh = h >> 1, q = threadIdx.x & 3;
+  Fr x = fr_zero(), d = fr_zero();
+  if (act) {
+    const Fr* f = (q < 2 ? sA : sB) + j + (q & 1) * hh;
+    x = f[0];
+    d = fr_sub(f[h], x);
+  } else if (clm) {
+    x = fr_sub(fr_sub(sh.g[1], sh.g[0]), sh.g[3]);
+    d = sh.g[3];
+  }
+  __syncwarp();
+  Fr p = quad_terms(x, d, r, clm);
+  if (act) ((q < 2 ? dA : dB) + j + (q & 1) * hh)[0] = x;
+  if (clm) sh.claim = fr_add(sh.g[0], p);
+  if (!act) p = fr_zero();
+#pragma unroll
+  for (int off = 4; off < 32; off <<= 1) p = fr_add(p, shfl_xor_fr(p, off));
+  return p;
+}
+
+// The block's sums of quad_pass's terms, canonical, in lanes 0 and 1 of warp 0
+// (one block barrier).
+__device__ __forceinline__ Fr quad_block_sum(RndShared& sh, Fr p, int warp, int last) {
+  const int lane = threadIdx.x & 31;
+  Fr* red = reinterpret_cast<Fr*>(sh.red);
+  if (lane < 2) red[2 * warp + lane] = p;
+  __syncthreads();
+  if (warp == 0) {
+    p = lane < 2 * (last + 1) ? red[lane] : fr_zero();
+#pragma unroll
+    for (int off = 2; off < 32; off <<= 1) p = fr_add(p, shfl_xor_fr(p, off));
+    p = from_mont_ni(p);
+  }
+  return p;
+}
+
+// ------------------------------------------------------------------ clusters
+//
+// The first rounds of one proof by a cluster of up to RND_MAX_CTAS CTAs: CTA c
+// owns the entries j with (j / 32) mod CTAs = c, so folding moves no entry
+// between CTAs while a round has at least 32 pairs per CTA.  A round costs two
+// cluster barriers: each CTA writes its sums of the round's terms into the first
+// CTA's shared memory, and the first CTA, after the transcript step, the
+// challenge into the others'.  The rounds below RND_CL_PAIRS pairs are the
+// first CTA's alone.  What bounds a lone proof's first rounds is one SM's field
+// products (4096-entry vectors: about 43 us of them, 5 on eight SMs).
+static constexpr int RND_CL_PAIRS = 32 * RND_MAX_CTAS;
+// Rounds of a proof with d1 variables that a cluster runs: those with at least
+// RND_CL_PAIRS pairs (round t has 2^(d1 - t)).
+__host__ __device__ __forceinline__ int cluster_rounds(int d1) { return d1 > 8 ? d1 - 8 : 0; }
+static_assert(RND_CL_PAIRS == 1 << 8, "cluster_rounds");
+
+// CTAs per cluster for n chains: while every CTA finds an SM of its own.
+static inline int cluster_ctas(int n, int sms) { return 8 * n <= sms ? 8 : 4 * n <= sms ? 4 : 2 * n <= sms ? 2 : 1; }
+
+// n clusters of `ctas` CTAs.
+template <class... P, class... A>
+cudaError_t launch_clusters(void (*kernel)(P...), int n, int ctas, int threads, size_t smem, cudaStream_t st, A... args) {
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = ctas;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(n * ctas);
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
+__device__ __forceinline__ uint32_t cluster_rank() {
+  uint32_t x;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(x));
+  return x;
+}
+__device__ __forceinline__ uint32_t cluster_size() {
+  uint32_t x;
+  asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(x));
+  return x;
+}
+// Every thread of the cluster arrives; what was written before is visible after.
+__device__ __forceinline__ void cluster_sync() {
+  __syncwarp();
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// Write `v` to `p` (shared memory of this CTA) in CTA `rank` of the cluster.
+__device__ __forceinline__ void st_cluster(const void* p, uint32_t rank, uint32_t v) {
+  uint32_t a;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
+  asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
+}
+
+// Rounds 1 to n = cluster_rounds(d1) >= 1 of the proof, the fold with r_n left
+// out.  The first CTA returns with sh.r = r_n and the vectors in memory as round
+// n saw them (rounds_block goes on from there); the others may leave.
+static __device__ void rounds_cluster(const DevProof& P, vl_proof* pf, RndShared& sh, int n) {
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, nthr = blockDim.x, last = (nthr >> 5) - 1;
+  const int rank = (int)cluster_rank(), C = (int)cluster_size();
+  const int K = 1 << P.d1;
+  Fr* fA = P.fA;
+  Fr* fB = P.fB;
+  const bool da = P.fdirA, db = P.fdirB;
+  cluster_sync();  // every CTA has started: its shared memory may be written
+  for (int t = 1; t <= n; t++) {
+    const int hh = K >> t, own = hh / C;  // the round's pairs, this CTA's
+    auto pair = [&](int l) { return ((l >> 5) * C + rank) * 32 + (l & 31); };
+    Fr s;
+    if (t == 1) {
+      uint32_t w0[17], w1[17], wi[17];
+      wide_zero(w0), wide_zero(w1), wide_zero(wi);
+      const Fr corrA = P.scr->corrA, corrB = P.scr->corrB;
+      for (int l = tid; l < own; l += nthr) {
+        const int j = pair(l);
+        const bool real = j + hh < P.k;
+        Fr a0, a1, b0, b1;
+        first_entries(fA, da, P.accA, corrA, j, hh, real, false, fA, a0, a1);
+        first_entries(fB, db, P.accB, corrB, j, hh, real, false, fB, b0, b1);
+        first_pair(a0, a1, b0, b1, w0, w1, wi);
+      }
+      unsigned long long col[3][8];
+      wide_redc(w0, col[0]);
+      wide_redc(wi, col[1]);
+      wide_redc(w1, col[2]);
+      s = block_sum_columns<3>(col, sh.red);
+    } else {
+      const Fr r = sh.r;
+      const int h = 2 * hh;
+      if (rank == 0 && warp == last && lane == 0) next_claim(sh);
+      if (4 * own <= nthr) {
+        const int l = tid >> 2;
+        s = quad_pass(sh, fA, fB, fA, fB, pair(l), l < own, h, r, false);
+        s = quad_block_sum(sh, s, warp, last);
+      } else {
+        uint32_t w0[17], wi[17];
+        wide_zero(w0), wide_zero(wi);
+        for (int l = tid; l < own; l += nthr) fold_pair(fA, fB, fA, fB, pair(l), h, r, w0, wi);
+        unsigned long long col[2][8];
+        wide_redc(w0, col[0]);
+        wide_redc(wi, col[1]);
+        s = block_sum_columns<2>(col, sh.red);
+      }
+    }
+    if (warp == 0 && lane < 3) {
+#pragma unroll
+      for (int q = 0; q < 8; q++) st_cluster(&sh.part[rank][lane].v[q], 0, s.v[q]);
+    }
+    cluster_sync();
+    if (rank == 0) {
+      if (warp == 0) {
+        // lane 4 c + q: value q of CTA c
+        Fr v = (lane >> 2) < C && (lane & 3) < 3 ? sh.part[lane >> 2][lane & 3] : fr_zero();
+#pragma unroll
+        for (int off = 4; off < 32; off <<= 1) v = fr_add(v, shfl_xor_fr(v, off));
+        const Fr g1 = shfl_fr(v, 2);
+        round_message(sh, shfl_fr(v, 0), shfl_fr(v, 1), t == 1 ? &g1 : nullptr, pf, t - 1);
+      }
+      transcript_step(sh, warp, t == 1, P.rch ? P.rch + (t - 1) : nullptr);
+      if (warp == 0 && t < n) {
+        __syncwarp();
+        for (int i = lane; i < 8 * (C - 1); i += 32) st_cluster(&sh.r.v[i & 7], 1 + (i >> 3), sh.r.v[i & 7]);
+      }
+    }
+    if (t < n) cluster_sync();
+  }
+  __syncthreads();
+}
+
 // Claim, rounds and proof of one proof by the whole block (a multiple of 32
-// threads, 128 to 512), from round t0 on.  t0 = 1: everything.  t0 > 1: the
-// earlier rounds ran batched over many proofs (kernels_rounds.cu): their
-// messages are in the proof already, the transcript state, the claim and
-// r_(t0-1) are in the scratch, and the vectors hold the round-(t0-1) values,
-// 2^(d1-t0+2) entries each.
-static __device__ void rounds_block(const DevProof& P, vl_proof* pf, uint8_t* smem, int t0 = 1) {
+// threads, 128 to 512), from round t0 on.  t0 = 1: everything (clustered: the
+// first cluster_rounds(d1) rounds by the cluster).  t0 > 1: the earlier rounds
+// ran batched over many proofs (kernels_rounds.cu): their messages are in the
+// proof already, the transcript state, the claim and r_(t0-1) are in the
+// scratch, and the vectors hold the round-(t0-1) values, 2^(d1-t0+2) entries each.
+static __device__ void rounds_block(const DevProof& P, vl_proof* pf, uint8_t* smem, int t0 = 1,
+                                    bool clustered = false) {
   RndShared& sh = *reinterpret_cast<RndShared*>(smem);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, nthr = blockDim.x, last = (nthr >> 5) - 1;
+  const int d1 = P.d1, K = 1 << d1;
+  const int ncl = clustered ? cluster_rounds(d1) : 0;
+  const bool lead = !clustered || cluster_rank() == 0;
+  if (!lead && ncl == 0) return;
   if (tid < 8) {
     sh.S[tid] = bswap32(reinterpret_cast<const uint32_t*>(P.scr->state)[tid]);
     if (t0 > 1) sh.claim.v[tid] = P.scr->claim.v[tid];
   }
-  if (t0 == 1) {
+  if (t0 == 1 && lead) {
     if (tid == 0) {
       pf->m = P.m; pf->k = P.k; pf->n = P.n;
       pf->d0 = P.d0; pf->d1 = P.d1; pf->d2 = P.d2;
@@ -275,7 +469,6 @@ static __device__ void rounds_block(const DevProof& P, vl_proof* pf, uint8_t* sm
     }
     for (int i = P.d1 * 24 + tid; i < VL_MAX_ROUNDS * 24; i += nthr) pf->g[i / 24][(i >> 3) % 3].limb[i & 7] = 0u;
   }
-  const int d1 = P.d1, K = 1 << d1;
   Fr* fA = P.fA;
   Fr* fB = P.fB;
   __syncthreads();
@@ -301,7 +494,10 @@ static __device__ void rounds_block(const DevProof& P, vl_proof* pf, uint8_t* sm
     return;
   }
 
-  {
+  if (ncl > 0) {
+    rounds_cluster(P, pf, sh, ncl);
+    if (!lead) return;
+  } else {
     // The first evaluation: of round 1 on f from the fold (fdir: reduced; else
     // column sums to reduce here), or of round t0 after folding with r_(t0-1).
     uint32_t w0[17], w1[17], wi[17];
@@ -322,17 +518,9 @@ static __device__ void rounds_block(const DevProof& P, vl_proof* pf, uint8_t* sm
       for (int j = tid; j < h; j += nthr) {
         // K/2 < k <= K, so j < k always; j + h may be padding
         const bool real = j + h < P.k;
-        const Fr a0 = da ? fA[j] : load_acc_fr(P.accA, j, corrA);
-        const Fr b0 = db ? fB[j] : load_acc_fr(P.accB, j, corrB);
-        Fr a1 = fr_zero(), b1 = fr_zero();
-        if (real) {
-          a1 = da ? fA[j + h] : load_acc_fr(P.accA, j + h, corrA);
-          b1 = db ? fB[j + h] : load_acc_fr(P.accB, j + h, corrB);
-        }
-        if (vec || !da) dA[j] = a0;
-        if (vec || !da || !real) dA[j + h] = a1;
-        if (vec || !db) dB[j] = b0;
-        if (vec || !db || !real) dB[j + h] = b1;
+        Fr a0, a1, b0, b1;
+        first_entries(fA, da, P.accA, corrA, j, h, real, vec, dA, a0, a1);
+        first_entries(fB, db, P.accB, corrB, j, h, real, vec, dB, b0, b1);
         first_pair(a0, a1, b0, b1, w0, w1, wi);
       }
     }
@@ -348,9 +536,11 @@ static __device__ void rounds_block(const DevProof& P, vl_proof* pf, uint8_t* sm
     }
   }
 
-  for (int i = t0 - 1; i < d1; i++) {
-    transcript_step(sh, warp, i == 0, P.rch ? P.rch + i : nullptr);
-    __syncthreads();
+  for (int i = ncl > 0 ? ncl - 1 : t0 - 1; i < d1; i++) {
+    if (i >= ncl) {
+      transcript_step(sh, warp, i == 0, P.rch ? P.rch + i : nullptr);
+      __syncthreads();
+    }
     const Fr r = sh.r;
     const int h = K >> (i + 1);  // the vectors hold 2h entries
     const Fr* sA = 2 * h <= RND_VEC ? sh.fa : fA;
@@ -394,40 +584,11 @@ static __device__ void rounds_block(const DevProof& P, vl_proof* pf, uint8_t* sm
     // its last lane the next claim in the same products.
     const bool alone = hh <= 4;
     if (alone && warp != 0) continue;
-    const int j = tid >> 2, q = tid & 3;
-    const bool act = j < hh, clm = alone && lane == 31;
+    const int j = tid >> 2;
     if (!alone && warp == last && lane == 0) next_claim(sh);
-    Fr x = fr_zero(), d = fr_zero();
-    if (act) {
-      const Fr* f = (q < 2 ? sA : sB) + j + (q & 1) * hh;
-      x = f[0];
-      d = fr_sub(f[h], x);
-    } else if (clm) {
-      x = fr_sub(fr_sub(sh.g[1], sh.g[0]), sh.g[3]);
-      d = sh.g[3];
-    }
-    __syncwarp();
-    Fr p = quad_terms(x, d, r, clm);
-    if (act) ((q < 2 ? dA : dB) + j + (q & 1) * hh)[0] = x;
-    if (clm) sh.claim = fr_add(sh.g[0], p);
-    if (!act) p = fr_zero();
-#pragma unroll
-    for (int off = 4; off < 32; off <<= 1) p = fr_add(p, shfl_xor_fr(p, off));
-    if (!alone) {
-      // lanes 0, 1 of each warp hold its sums of g(0), G
-      Fr* red = reinterpret_cast<Fr*>(sh.red);
-      if (lane < 2) red[2 * warp + lane] = p;
-      __syncthreads();
-      if (warp == 0) {
-        p = lane < 2 * (last + 1) ? red[lane] : fr_zero();
-#pragma unroll
-        for (int off = 2; off < 32; off <<= 1) p = fr_add(p, shfl_xor_fr(p, off));
-      }
-    }
-    if (warp == 0) {
-      p = from_mont_ni(p);
-      round_message(sh, shfl_fr(p, 0), shfl_fr(p, 1), nullptr, pf, i + 1);
-    }
+    Fr p = quad_pass(sh, sA, sB, dA, dB, j, j < hh, h, r, alone && j >= hh && lane == 31);
+    p = alone ? from_mont_ni(p) : quad_block_sum(sh, p, warp, last);
+    if (warp == 0) round_message(sh, shfl_fr(p, 0), shfl_fr(p, 1), nullptr, pf, i + 1);
   }
   __syncthreads();
 }
