@@ -320,11 +320,14 @@ struct LkDev {
   int32_t xbeg, xend;              // slots of the table-side sum of B m
   int32_t tail;                    // first round run by the per-proof tail kernel
   int32_t dense;                   // ld == cols: entry k is S[k]
+  int32_t round2, pad2;            // round 2 is batched and reads A from the tables UB, VB
+  Fr w4[4];                        // eq weights of (r_1, r_2): (1-r1)(1-r2), (1-r1) r2, r1 (1-r2), r1 r2
   Fr* loP;                         // eq over the last m variables of u, levels m = 0..sE at offset 2^m - 1
   Fr* hiP;                         // eq over the last m variables of u_1..u_{L-sE}, levels m = 0..L-sE-1
   Fr* Binv;                        // 1 / (beta + t0 + j), N (gather source, never folded)
   Fr* Tb;                          // beta + t0 + j, N (gather source)
   Fr* WB; Fr* WM;                  // table side: B, m (folded in place)
+  Fr* UB; Fr* VB;                  // (1 - r_1) B, r_1 B, N each (round2)
   Fr* VA; Fr* VS;                  // folded A and S + beta, D/2 each
   uint32_t* counts;                // N multiplicities
   Fr* part;                        // partial sums (LK_PART per slot)
@@ -338,18 +341,29 @@ static constexpr int LK_THREADS = 256;
 static constexpr int LK_PART = 8;         // partial sums per slot: T0, Tinf, A0 | U0, Uinf, V0, Vinf
 static constexpr int LK_PASS_THREADS = 128;
 static constexpr int LK_PASS_WARPS = LK_PASS_THREADS / 32;  // round items (one warp each) per pass CTA
-static constexpr int LK_PAIRS = 256;      // pairs per round item at most (and at most 2^sE: one hiP entry per item)
-static constexpr int LK_ENTRIES = 1024;   // table entries per table item (one batch inversion)
+static constexpr int LK_PAIRS = 512;      // pairs per round item at most (and at most 2^sE: one hiP entry per item)
+// Pairs per round item go down to LK_PAIRS_MIN (one per lane) while a round has
+// fewer items than warps fit on the GPU at a time (LK_ITEMS: 152 SMs x 16): the last
+// batched round of the 512 lookups of a 7B step 226 us at 512 pairs, 52 at 64.
+static constexpr int LK_PAIRS_MIN = 32;
+static constexpr int LK_ITEMS = 2432;
+static constexpr int LK_ENTRIES = 4096;   // table entries per table item (one batch inversion)
 static constexpr int LK_HIST = 32768;     // S entries per histogram item
-#ifndef LK_TAIL_LOG
-#define LK_TAIL_LOG 11  // rounds of at most 2^LK_TAIL_LOG pairs run in one block per proof
-#endif
+// Rounds of at most 2^LK_TAIL_LOG pairs run in one block per proof; of at most
+// 2^LK_TAIL_LOG_MANY in batches of more than LK_MANY proofs, whose tails run on
+// 128 threads each (the 512 lookups of a 7B step: tails 1107 -> 513 us, the two more
+// batched rounds 165).
+static constexpr int LK_TAIL_LOG = 11;
+static constexpr int LK_TAIL_LOG_MANY = 9;
+static constexpr int LK_MANY = 152;
 cudaError_t launch_lookup_setup(LkDev* Ls, int np, const LkItem* hist_items, int nhist, const LkItem* tab_items,
                                 int ntab, cudaStream_t st);
 // Round t: nhi items of proofs in their high rounds, then nlo items of
 // proofs in their table rounds.
 cudaError_t launch_lookup_round(LkDev* Ls, int np, int t, const LkItem* items, int nhi, int nlo,
                                 vl_lookup_proof* out, cudaStream_t st);
+// Between rounds 1 and 2: the tables UB, VB of the proofs that use them.
+cudaError_t launch_lookup_tables2(LkDev* Ls, const LkItem* tab_items, int ntab, cudaStream_t st);
 cudaError_t launch_lookup_finish(LkDev* Ls, int np, vl_lookup_proof* out, cudaStream_t st);
 cudaError_t launch_lookup_passes(LkDev* Ls, int t, const LkItem* items, int nhi, int nlo, cudaStream_t st);
 

@@ -275,15 +275,13 @@ __device__ __forceinline__ void small_mul(uint32_t (&z)[9], const uint32_t (&a)[
       : "r"(o[0]), "r"(o[1]), "r"(o[2]), "r"(o[3]), "r"(o[4]), "r"(o[5]), "r"(o[6]), "r"(o[7]));
 }
 
-// a m mod r for m < 2^16 (a reduced): Barrett with a 32-bit quotient estimate.
-// With t = a m < 2^271, x = floor(t / 2^239) and M = floor(2^271 / r), q =
-// floor(x M / 2^32) satisfies t / r - 2.0001 < q <= t / r: the remainder is below
-// 2.0001 r < 2^256.  An eighth of a Montgomery product's multiply-adds.
-__device__ __forceinline__ Fr small_mul_mod(const Fr& a, uint32_t m) {
-  uint32_t t[9], p[9];
-  small_mul(t, a.v, m);
-  const uint32_t x = (t[8] << 17) | (t[7] >> 15);
-  const uint32_t q = __umulhi(x, 72360u);  // floor(2^271 / r)
+// t mod r for t < 2^273: Barrett with a 32-bit quotient estimate.  With x =
+// floor(t / 2^241) and M = floor(2^273 / r), q = floor(x M / 2^32) satisfies
+// t / r - 2.0001 < q <= t / r: the remainder is below 2.0001 r < 2^256.
+__device__ __forceinline__ Fr small_reduce(const uint32_t (&t)[9]) {
+  uint32_t p[9];
+  const uint32_t x = (t[8] << 15) | (t[7] >> 17);
+  const uint32_t q = __umulhi(x, 289441u);
   const uint32_t r[8] = {r_limb(0), r_limb(1), r_limb(2), r_limb(3), r_limb(4), r_limb(5), r_limb(6), r_limb(7)};
   small_mul(p, r, q);
   Fr out;
@@ -293,6 +291,24 @@ __device__ __forceinline__ Fr small_mul_mod(const Fr& a, uint32_t m) {
   cond_sub_r(out.v, 0);
   cond_sub_r(out.v, 0);
   return out;
+}
+
+// a m mod r for m < 2^18 (a reduced): an eighth of a Montgomery product's
+// multiply-adds.
+__device__ __forceinline__ Fr small_mul_mod(const Fr& a, uint32_t m) {
+  uint32_t t[9];
+  small_mul(t, a.v, m);
+  return small_reduce(t);
+}
+
+// t += z (nine limbs).
+__device__ __forceinline__ void add9(uint32_t (&t)[9], const uint32_t (&z)[9]) {
+  asm("add.cc.u32 %0, %0, %9; addc.cc.u32 %1, %1, %10; addc.cc.u32 %2, %2, %11; addc.cc.u32 %3, %3, %12;\n\t"
+      "addc.cc.u32 %4, %4, %13; addc.cc.u32 %5, %5, %14; addc.cc.u32 %6, %6, %15; addc.cc.u32 %7, %7, %16;\n\t"
+      "addc.u32 %8, %8, %17;"
+      : "+&r"(t[0]), "+&r"(t[1]), "+&r"(t[2]), "+&r"(t[3]), "+&r"(t[4]), "+&r"(t[5]), "+&r"(t[6]), "+&r"(t[7]),
+        "+&r"(t[8])
+      : "r"(z[0]), "r"(z[1]), "r"(z[2]), "r"(z[3]), "r"(z[4]), "r"(z[5]), "r"(z[6]), "r"(z[7]), "r"(z[8]));
 }
 
 // w += a (b m) for m < 2^16: up to 2^17 terms of at most 2^526.

@@ -21,7 +21,7 @@
 //
 // Launches: start (per proof: transcript, beta, alpha, u, N/D, the suffix eq
 // tables), histogram (multiplicities, range check), table (batch inversion of
-// beta + T per 1024-entry block, B, T', m, partial sums of B m; the inverses
+// beta + T per 4096-entry block, B, T', m, partial sums of B m; the inverses
 // of the u_t ride in the first block); per round a pass over all proofs' pairs
 // (fold with the previous challenge, then the partial sums, lookup_dev.cuh) and
 // a transcript step per proof; tail.
@@ -148,30 +148,33 @@ __global__ void __launch_bounds__(LK_THREADS) lk_hist_kernel(LkDev* Ls, const Lk
       if (h[j]) atomicAdd(&L->counts[j], h[j]);
 }
 
-// Table entries [k0, k1) (at most 4 per thread): x_j = beta + t0 + j, its
-// inverse by one batch inversion per block (prefix products, one field
-// inversion, back substitution), the table-side vectors, and this block's
-// share of sum B m (its slot's first entry).  The first block of a proof also
-// inverts the u_t (one more element per thread).
+// Table entries [k0, k1) (at most 16 per thread, consecutive): x_j = beta + t0 +
+// j, its inverse by one batch inversion per block (the products before each entry
+// within its thread, left in Binv; scans over the threads; one field inversion;
+// back substitution, two products per entry), the table-side vectors, and this
+// block's share of sum B m (canonical, its slot's first entry).  The first
+// block of a proof also inverts the u_t (one more element per thread).  Bound
+// by products and the serial inversion: the tables of the 512 lookups of a 7B
+// step take 258 us, with 1024-entry blocks (one inversion for 1024) 456.
 __global__ void __launch_bounds__(LK_THREADS, 2) lk_table_kernel(LkDev* Ls, const LkItem* items) {
   __shared__ Fr pre[LK_THREADS], suf[LK_THREADS];
   __shared__ Fr inv_tot;
-  __shared__ Fr red[LK_THREADS / 32];
+  __shared__ unsigned long long red[8 * (LK_THREADS / 32)];
   const LkItem it = items[blockIdx.x];
   LkDev* L = Ls + it.proof;
-  const int tid = threadIdx.x;
-  const Fr beta = L->beta;
+  const int tid = threadIdx.x, E = (it.k1 - it.k0 + LK_THREADS - 1) / LK_THREADS;
+  const int j0 = it.k0 + E * tid, j1 = min(j0 + E, it.k1);
   const bool has_u = it.k0 == 0 && tid < L->L;
   const Fr ux = has_u ? L->u[tid] : fr_r1();
-  Fr x[4], p[4];
-  for (int e = 0; e < 4; e++) {
-    const int j = it.k0 + 4 * tid + e;
-    x[e] = j < it.k1 ? fr_add(beta, to_mont_ni(fr_from_i64(L->t0 + j))) : fr_r1();
-    p[e] = mont_mul_ni(e == 0 ? ux : p[e - 1], x[e]);
+  Fr x = fr_add(L->beta, to_mont_ni(fr_from_i64(L->t0 + j0))), run = ux;
+  for (int j = j0; j < j1; j++) {
+    L->Binv[j] = run;
+    run = mont_mul_ni(run, x);
+    x = fr_add(x, fr_r1());
   }
   // inclusive prefix and suffix products of the thread totals (Hillis-Steele)
-  pre[tid] = p[3];
-  suf[tid] = p[3];
+  pre[tid] = run;
+  suf[tid] = run;
   __syncthreads();
   for (int off = 1; off < LK_THREADS; off <<= 1) {
     const Fr a = tid >= off ? mont_mul_ni(pre[tid - off], pre[tid]) : pre[tid];
@@ -187,29 +190,43 @@ __global__ void __launch_bounds__(LK_THREADS, 2) lk_table_kernel(LkDev* Ls, cons
     if (tid == 0) atomicExch(&L->scr->status, VL_ELOOKUP);
     return;
   }
-  const Fr qprev = tid > 0 ? pre[tid - 1] : fr_r1();
-  // 1 / (prefix through this thread) = inv_tot . (product of the later threads' totals)
-  Fr inv_f = tid + 1 < LK_THREADS ? mont_mul_ni(inv_tot, suf[tid + 1]) : inv_tot;
-  Fr inv_x[4];
-  for (int e = 3; e >= 0; e--) {
-    const Fr f_before = mont_mul_ni(qprev, e > 0 ? p[e - 1] : ux);  // prefix before element e
-    inv_x[e] = mont_mul_ni(inv_f, f_before);
-    inv_f = mont_mul_ni(inv_f, x[e]);
+  // 1 / (this thread's total) = inv_tot . (the totals of the threads before) . (of those after)
+  Fr inv = inv_tot;
+  if (tid > 0) inv = mont_mul_ni(inv, pre[tid - 1]);
+  if (tid + 1 < LK_THREADS) inv = mont_mul_ni(inv, suf[tid + 1]);
+  unsigned long long bm[1][8];
+#pragma unroll
+  for (int l = 0; l < 8; l++) bm[0][l] = 0;
+  for (int j = j1 - 1; j >= j0; j--) {
+    x = fr_sub(x, fr_r1());
+    const Fr b = mont_mul_ni(inv, L->Binv[j]);
+    inv = mont_mul_ni(inv, x);
+    const uint32_t m = L->counts[j];
+    L->Binv[j] = b;
+    L->WB[j] = b;
+    L->Tb[j] = x;
+    L->WM[j] = to_mont_ni(fr_small(m));
+#pragma unroll
+    for (int l = 0; l < 8; l++) bm[0][l] += (unsigned long long)b.v[l] * m;  // sum m <= 2^24
   }
-  if (has_u) L->uinv[tid] = mont_mul_ni(inv_f, qprev);
-  Fr acc[1] = {fr_zero()};
-  for (int e = 0; e < 4; e++) {
-    const int j = it.k0 + 4 * tid + e;
-    if (j >= it.k1) break;
-    const Fr m = to_mont_ni(fr_small(L->counts[j]));
-    L->Binv[j] = inv_x[e];
-    L->WB[j] = inv_x[e];
-    L->Tb[j] = x[e];
-    L->WM[j] = m;
-    acc[0] = fr_add(acc[0], mont_mul_ni(inv_x[e], m));
+  if (has_u) L->uinv[tid] = inv;
+  const Fr s = block_sum_columns<1>(bm, red);
+  if (tid == 0) L->part[(size_t)it.slot * LK_PART] = s;
+}
+
+// The tables of round 2 (entries of a table item): UB = (1 - r_1) B, VB = r_1 B.
+// One product per entry (51 us for the 512 lookups of a 7B step) against two per
+// pair: with S' left to round 3, round 2's pass took 1068 us, now 892.
+__global__ void __launch_bounds__(LK_THREADS) lk_tables2_kernel(LkDev* Ls, const LkItem* items) {
+  const LkItem it = items[blockIdx.x];
+  LkDev* L = Ls + it.proof;
+  if (!L->round2) return;
+  const Fr r = L->r[0];
+  for (int j = it.k0 + threadIdx.x; j < it.k1; j += LK_THREADS) {
+    const Fr b = L->Binv[j], v = mont_mul_ni(r, b);
+    L->VB[j] = v;
+    L->UB[j] = fr_sub(b, v);
   }
-  block_sum_fr<1>(acc, red);
-  if (tid == 0) L->part[(size_t)it.slot * LK_PART] = acc[0];
 }
 
 // Shared memory of a transcript step.
@@ -257,14 +274,20 @@ __device__ __forceinline__ void lk_absorb_words(LkShared& sh, uint32_t label, in
 // The round polynomial of round t from the sums in sh.s, by warp 0: g(X) =
 // E_X T(X) + A(X) + table side for X = 0..3 (three products deep: T(1), U(1)
 // from the claims, then all products of the four values at once), into sh.g and
-// the proof.  tj: the table round's number, <= 0 in a high round.
-__device__ void lk_step_g(const LkDev* L, LkShared& sh, int t, int tj, vl_lookup_proof* out) {
+// the proof.  tj: the table round's number, <= 0 in a high round; qform: the
+// first sum is Q with T(0) = 1 - r_1 (1 - r_1) Q (round 2).
+__device__ void lk_step_g(const LkDev* L, LkShared& sh, int t, int tj, bool qform, vl_lookup_proof* out) {
   const int lane = threadIdx.x & 31;
   const bool jr = tj > 0;
   const Fr ut = L->u[t - 1], ui = L->uinv[t - 1], one = fr_small(1);
   const LkRun& R = sh.run;
+  Fr t0 = t == 1 ? one : sh.s[0];
+  if (qform) {
+    const Fr r1 = L->r[0];
+    t0 = fr_sub(one, mont_mul_ni(mont_mul_ni(r1, fr_sub(fr_r1(), r1)), t0));
+  }
   // lanes 0, 1: T(1), U(1) = (claim - (1 - u) value(0)) / u; lane 2: U's leading coefficient times h
-  const Fr v0 = lane == 0 ? (t == 1 ? one : sh.s[0]) : lane == 1 ? (tj == 1 ? one : sh.s[3]) : fr_small(1u << (L->L - t));
+  const Fr v0 = lane == 0 ? t0 : lane == 1 ? (tj == 1 ? one : sh.s[3]) : fr_small(1u << (L->L - t));
   const Fr x = mont_mul_ni(lane < 2 ? fr_sub(fr_r1(), ut) : fr_r2(), v0);
   const Fr y = mont_mul_ni(lane < 2 ? ui : sh.s[4], lane < 2 ? fr_sub(lane == 0 ? R.Tc : R.Uc, x) : x);
   if (lane == 0) {
@@ -336,6 +359,15 @@ __device__ void lk_step_r(LkDev* L, LkShared& sh, int t) {
   if (lane == 4) R.ac = ac;
   if (lane == 5) R.fc = fc;
   if (lane == 7) R.tabc = p;
+  if (t == 2) {  // the weights of round 3's S'
+    const Fr r1 = L->r[0], p11 = mont_mul_ni(r1, r);
+    if (lane == 0) {
+      L->w4[3] = p11;
+      L->w4[2] = fr_sub(r1, p11);
+      L->w4[1] = fr_sub(r, p11);
+      L->w4[0] = fr_sub(fr_sub(one, r1), fr_sub(r, p11));
+    }
+  }
   // E_X, F_X of round t + 1: eqf(u, X) = (1 - u) + X (2 u - 1)
   if (t < L->L) {
     const Fr un = L->u[t], e0 = fr_sub(one, un), d = fr_sub(un, e0);
@@ -358,7 +390,7 @@ __device__ void lk_first_step(const LkDev* L, LkShared& sh) {
   block_sum_fr<1>(x, reinterpret_cast<Fr*>(sh.red));
   if (threadIdx.x < 32) {
     const int lane = threadIdx.x, i = lane & 3;
-    const Fr bm = from_mont_ni(x[0]), ac = sh.run.ac, fc = sh.run.fc, one = fr_r1();
+    const Fr bm = x[0], ac = sh.run.ac, fc = sh.run.fc, one = fr_r1();
     if (L->L > 0) {
       const Fr u = L->u[0], e0 = fr_sub(one, u), d = fr_sub(u, e0);
       Fr v = e0;
@@ -473,7 +505,7 @@ __global__ void __launch_bounds__(LK_STEP_THREADS) lk_round_kernel(LkDev* Ls, in
     if (tid < 4) sh.s[3 + tid] = x;
   }
   __syncwarp();
-  if (warp == 0) lk_step_g(L, sh, t, tj, outs + blockIdx.x);
+  if (warp == 0) lk_step_g(L, sh, t, tj, t == 2, outs + blockIdx.x);
   lk_transcript(L, sh, warp, t);
   __syncthreads();
   if (warp == 0) lk_step_r(L, sh, t);
@@ -499,6 +531,10 @@ __device__ void lk_finish(LkDev* L, LkShared& sh, vl_lookup_proof* out) {
         const Fr* tab = lane == 0 ? L->Binv : L->Tb;
         x0 = tab[lk_table_index(*L, 0)];
         if (fold) x1 = tab[lk_table_index(*L, 1)];
+      } else if (Lp == 2 && lane == 1) {  // rounds 1 and 2 leave S' unfolded
+        const Fr r1 = L->r[0];
+        x0 = lk_fold(L->Tb[lk_table_index(*L, 0)], L->Tb[lk_table_index(*L, 2)], r1);
+        x1 = lk_fold(L->Tb[lk_table_index(*L, 1)], L->Tb[lk_table_index(*L, 3)], r1);
       } else {
         const Fr* v = lane == 0 ? L->VA : L->VS;
         x0 = v[0], x1 = v[1];
@@ -549,7 +585,15 @@ __global__ void __launch_bounds__(THREADS, MINB) lk_tail_kernel(LkDev* Ls, vl_lo
     const int h = 1 << (L->L - t);
     const int tj = t - (L->L - L->log2_n);
     const bool jr = tj > 0;
-    if (t > L->tail && warp == NW - 1) lk_step_r(L, sh, t - 1);
+    if (t > L->tail) {
+      if (t == 3) {  // round 3 needs the weights that the step leaves
+        if (warp == NW - 1) lk_step_r(L, sh, t - 1);
+        __syncthreads();
+      } else if (warp == NW - 1) {
+        lk_step_r(L, sh, t - 1);
+      }
+    }
+    const bool qform = t == 2 && 4 * h > THREADS / (t > L->L - L->log2_n ? 2 : 1);  // see the loop below
     const LkEq q(L, t);
     const int na = jr ? NW / 2 : NW;  // warps of the A side
     const bool sideb = warp >= na;
@@ -567,7 +611,8 @@ __global__ void __launch_bounds__(THREADS, MINB) lk_tail_kernel(LkDev* Ls, vl_lo
           if (q.high) f = mont_mul_ni(f, q.hi_tab[k >> L->sE]);
           if (t == 1) lk_pair_a<0>(L, t, k, h, f, s);
           else if (t == 2) lk_pair_a<1>(L, t, k, h, f, s);
-          else lk_pair_a<2>(L, t, k, h, f, s);
+          else if (t == 3) lk_pair_a<2>(L, t, k, h, f, s);
+          else lk_pair_a<3>(L, t, k, h, f, s);
         }
         unsigned long long col[3][8];
         s.columns(col);
@@ -619,7 +664,10 @@ __global__ void __launch_bounds__(THREADS, MINB) lk_tail_kernel(LkDev* Ls, vl_lo
           x = tab[lk_table_index(*L, at)];
           fold = t == 2;
           if (fold) x1 = tab[lk_table_index(*L, at + 2 * h)];
-          if (fold) dst = qd < 2 ? L->VA : L->VS;
+          if (fold && qd < 2) dst = L->VA;  // S' is formed in round 3
+        } else if (!sideb && t == 3 && qd >= 2) {
+          x = lk_s_round3(L, at, L->L - 2);
+          dst = L->VS;
         } else {
           Fr* v = sideb ? (qd < 2 ? L->WB : L->WM) : (qd < 2 ? L->VA : L->VS);
           x = v[at];
@@ -668,7 +716,7 @@ __global__ void __launch_bounds__(THREADS, MINB) lk_tail_kernel(LkDev* Ls, vl_lo
       }
     }
     __syncwarp();
-    if (warp == 0) lk_step_g(L, sh, t, tj, out);
+    if (warp == 0) lk_step_g(L, sh, t, tj, qform, out);
     lk_transcript(L, sh, warp, t);
     __syncthreads();  // r_t and the folded vectors are visible to the next round
   }
@@ -685,6 +733,11 @@ cudaError_t launch_lookup_setup(LkDev* Ls, int np, const LkItem* hist_items, int
   return cudaGetLastError();
 }
 
+cudaError_t launch_lookup_tables2(LkDev* Ls, const LkItem* tab_items, int ntab, cudaStream_t st) {
+  lk_tables2_kernel<<<ntab, LK_THREADS, 0, st>>>(Ls, tab_items);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_lookup_round(LkDev* Ls, int np, int t, const LkItem* items, int nhi, int nlo,
                                 vl_lookup_proof* out, cudaStream_t st) {
   const cudaError_t e = launch_lookup_passes(Ls, t, items, nhi, nlo, st);
@@ -695,7 +748,7 @@ cudaError_t launch_lookup_round(LkDev* Ls, int np, int t, const LkItem* items, i
 
 // A proof's tail is a chain of rounds: with an SM for every proof it runs on 512
 // threads, else on 128, four proofs per SM (one lookup of 512 x 16 remainders
-// 0.98 -> 0.44 ms, the 512 of a 7B step 8.86 -> 4.42 ms with the other changes
+// 0.98 -> 0.42 ms, the 512 of a 7B step 8.86 -> 4.13 ms with the other changes
 // described in lookup_dev.cuh).
 cudaError_t launch_lookup_finish(LkDev* Ls, int np, vl_lookup_proof* out, cudaStream_t st) {
   int dev = 0, sms = 0;

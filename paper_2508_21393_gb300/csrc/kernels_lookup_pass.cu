@@ -1,6 +1,8 @@
 // Lookup-argument sumcheck: the batched round passes (the rounds of every
 // proof before its tail).  Kept apart from kernels_lookup.cu so the two compile
 // in parallel.
+#include <type_traits>
+
 #include "lookup_dev.cuh"
 
 namespace vl {
@@ -29,7 +31,7 @@ __device__ __forceinline__ Fr lk_warp_sum(const unsigned long long (&c)[NV][8], 
 // pairs lie in one block of 2^sE pairs (LK_PAIRS, 2^sE), so a high round's hiP
 // factor multiplies the item's sums once.
 template <bool JR, int MODE>
-__global__ void __launch_bounds__(LK_PASS_THREADS, 4) lk_pass_kernel(LkDev* Ls, int t, const LkItem* items, int n) {
+__global__ void __launch_bounds__(LK_PASS_THREADS, JR ? 3 : 4) lk_pass_kernel(LkDev* Ls, int t, const LkItem* items, int n) {
   const int i = blockIdx.x * LK_PASS_WARPS + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (i >= n) return;  // whole warps leave together
   const LkItem it = items[i];
@@ -67,16 +69,15 @@ __global__ void __launch_bounds__(LK_PASS_THREADS, 4) lk_pass_kernel(LkDev* Ls, 
 // of proofs in their table rounds.
 cudaError_t launch_lookup_passes(LkDev* Ls, int t, const LkItem* items, int nhi, int nlo, cudaStream_t st) {
   const int ghi = (nhi + LK_PASS_WARPS - 1) / LK_PASS_WARPS, glo = (nlo + LK_PASS_WARPS - 1) / LK_PASS_WARPS;
-  if (nhi) {
-    if (t == 1) lk_pass_kernel<false, 0><<<ghi, LK_PASS_THREADS, 0, st>>>(Ls, t, items, nhi);
-    else if (t == 2) lk_pass_kernel<false, 1><<<ghi, LK_PASS_THREADS, 0, st>>>(Ls, t, items, nhi);
-    else lk_pass_kernel<false, 2><<<ghi, LK_PASS_THREADS, 0, st>>>(Ls, t, items, nhi);
-  }
-  if (nlo) {
-    if (t == 1) lk_pass_kernel<true, 0><<<glo, LK_PASS_THREADS, 0, st>>>(Ls, t, items + nhi, nlo);
-    else if (t == 2) lk_pass_kernel<true, 1><<<glo, LK_PASS_THREADS, 0, st>>>(Ls, t, items + nhi, nlo);
-    else lk_pass_kernel<true, 2><<<glo, LK_PASS_THREADS, 0, st>>>(Ls, t, items + nhi, nlo);
-  }
+  auto run = [&](auto jr, const LkItem* it, int n, int grid) {
+    constexpr bool JR = decltype(jr)::value;
+    if (t == 1) lk_pass_kernel<JR, 0><<<grid, LK_PASS_THREADS, 0, st>>>(Ls, t, it, n);
+    else if (t == 2) lk_pass_kernel<JR, 1><<<grid, LK_PASS_THREADS, 0, st>>>(Ls, t, it, n);
+    else if (t == 3) lk_pass_kernel<JR, 2><<<grid, LK_PASS_THREADS, 0, st>>>(Ls, t, it, n);
+    else lk_pass_kernel<JR, 3><<<grid, LK_PASS_THREADS, 0, st>>>(Ls, t, it, n);
+  };
+  if (nhi) run(std::false_type{}, items, nhi, ghi);
+  if (nlo) run(std::true_type{}, items + nhi, nlo, glo);
   return cudaGetLastError();
 }
 

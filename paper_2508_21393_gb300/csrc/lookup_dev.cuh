@@ -13,9 +13,14 @@
 // two products per pair instead of three.  What else a pair does not need:
 //  * T(0) = T(1) = 1 in round 1 and U(0) = U(1) = 1 in the first table round
 //    (A S' = B T' = 1 on unfolded entries and the eq factors sum to 1);
-//  * S' differs between table entries by a small integer: round 1's leading
-//    term f (a1 - a0)(j1 - j0) and round 2's fold of S' are products by 16-bit
-//    integers;
+//  * S' differs between table entries by a small integer, and A S' = 1: round
+//    1's leading term is f (a1 - a0)(j1 - j0); round 2 needs S' only in the
+//    difference of a pair, and its T(0) is 1 - r (1 - r) sum f (a' - a)(j' - j)
+//    over the entries a, a' that fold into a pair's first; round 3 forms S'
+//    from the four table indices and the four eq weights of (r_1, r_2): products
+//    by integers of 16 to 18 bits throughout;
+//  * round 2's folded A comes from the tables (1 - r) B, r B (two products per
+//    table entry instead of two per pair);
 //  * T'(k) = beta + t0 + k is affine in k: folded it is Tb[k] + toff, and its
 //    leading coefficient the constant h;
 //  * sums of products are reduced once per thread (wide_mac).
@@ -47,12 +52,23 @@ __device__ __forceinline__ Fr lk_fold(const Fr& x0, const Fr& x1, const Fr& r) {
   return fr_add(x0, mont_mul_ni(r, fr_sub(x1, x0)));
 }
 
-// S' at entries j0, j1 of the unfolded cube folded with r: Tb[j0] + r (j1 - j0).
-__device__ __forceinline__ Fr lk_fold_s(const LkDev* L, int j0, int j1, const Fr& r) {
-  const int d = j1 - j0;
-  const Fr z = small_mul_mod(r, (uint32_t)(d < 0 ? -d : d));
-  const Fr s = L->Tb[j0];
-  return d < 0 ? fr_sub(s, z) : fr_add(s, z);
+// a d mod r for a signed integer |d| < 2^18.
+__device__ __forceinline__ Fr lk_times(const Fr& a, int d) {
+  const Fr z = small_mul_mod(a, (uint32_t)(d < 0 ? -d : d));
+  return d < 0 ? fr_neg(z) : z;
+}
+
+// S' at entry k of the cube folded by r_1 and r_2 (2^q entries): beta + t0 +
+// sum_b w4[b] j(k + b 2^q).
+__device__ __forceinline__ Fr lk_s_round3(const LkDev* L, int k, int q) {
+  uint32_t t[9], z[9];
+  small_mul(t, L->w4[0].v, (uint32_t)lk_table_index(*L, k));
+#pragma unroll
+  for (int b = 1; b < 4; b++) {
+    small_mul(z, L->w4[b].v, (uint32_t)lk_table_index(*L, k + (b << q)));
+    add9(t, z);
+  }
+  return fr_add(L->Tb[0], small_reduce(t));
 }
 
 // Sums of one thread's pairs, A side: T(0), T(inf), A(0).
@@ -81,9 +97,10 @@ struct LkSumB {
   }
 };
 
-// One pair (k, k + h) of round t, A side: the first round reads the unfolded
-// cube, the second folds it on the fly and writes the folded vectors, later
-// rounds fold them in place (MODE 0, 1, 2).
+// One pair (k, k + h) of round t, A side.  MODE 0: round 1, from the unfolded
+// cube; 1: round 2, A folded on the fly and written, t0 summing Q = f (a' - a)(j'
+// - j) (T(0) = 1 - r (1 - r) Q); 2: round 3, A folded in place, S' formed and
+// written; 3: later rounds, both folded in place.
 template <int MODE>
 __device__ __forceinline__ void lk_pair_a(LkDev* L, int t, int k, int h, const Fr& f, LkSumA& s) {
   if constexpr (MODE == 0) {
@@ -92,24 +109,38 @@ __device__ __forceinline__ void lk_pair_a(LkDev* L, int t, int k, int h, const F
     sum9_add(s.a0, a0);
     // (a1 - a0)(s1 - s0) = (a1 - a0)(j1 - j0), both signs flipped for j1 < j0
     wide_mac_small(s.ti, f, d < 0 ? fr_sub(a0, a1) : fr_sub(a1, a0), (uint32_t)(d < 0 ? -d : d));
-  }
-  Fr a0, a1, s0, s1;
-  if constexpr (MODE == 1) {
+  } else if constexpr (MODE == 1) {
     const Fr r = L->r[0];
     const int j0 = lk_table_index(*L, k), j1 = lk_table_index(*L, k + h);
     const int j2 = lk_table_index(*L, k + 2 * h), j3 = lk_table_index(*L, k + 3 * h);
-    a0 = lk_fold(L->Binv[j0], L->Binv[j2], r);
-    a1 = lk_fold(L->Binv[j1], L->Binv[j3], r);
-    s0 = lk_fold_s(L, j0, j2, r);
-    s1 = lk_fold_s(L, j1, j3, r);
-  } else if constexpr (MODE == 2) {
+    const Fr b0 = L->Binv[j0], b2 = L->Binv[j2];
+    Fr a0, a1;
+    if (L->round2) {
+      a0 = fr_add(L->UB[j0], L->VB[j2]);
+      a1 = fr_add(L->UB[j1], L->VB[j3]);
+    } else {
+      a0 = lk_fold(b0, b2, r);
+      a1 = lk_fold(L->Binv[j1], L->Binv[j3], r);
+    }
+    L->VA[k] = a0, L->VA[k + h] = a1;
+    sum9_add(s.a0, a0);
+    const int d = j2 - j0;
+    wide_mac_small(s.t0, f, d < 0 ? fr_sub(b0, b2) : fr_sub(b2, b0), (uint32_t)(d < 0 ? -d : d));
+    // s1 - s0 = (j1 - j0) + r ((j3 - j2) - (j1 - j0))
+    const Fr ds = fr_add(lk_times(fr_r1(), j1 - j0), lk_times(r, (j3 - j2) - (j1 - j0)));
+    wide_mac(s.ti, f, mont_mul_ni(fr_sub(a1, a0), ds));
+  } else {
     const Fr r = L->r[t - 2];
-    a0 = lk_fold(L->VA[k], L->VA[k + 2 * h], r);
-    a1 = lk_fold(L->VA[k + h], L->VA[k + 3 * h], r);
-    s0 = lk_fold(L->VS[k], L->VS[k + 2 * h], r);
-    s1 = lk_fold(L->VS[k + h], L->VS[k + 3 * h], r);
-  }
-  if constexpr (MODE != 0) {
+    const Fr a0 = lk_fold(L->VA[k], L->VA[k + 2 * h], r);
+    const Fr a1 = lk_fold(L->VA[k + h], L->VA[k + 3 * h], r);
+    Fr s0, s1;
+    if constexpr (MODE == 2) {
+      s0 = lk_s_round3(L, k, L->L - 2);
+      s1 = lk_s_round3(L, k + h, L->L - 2);
+    } else {
+      s0 = lk_fold(L->VS[k], L->VS[k + 2 * h], r);
+      s1 = lk_fold(L->VS[k + h], L->VS[k + 3 * h], r);
+    }
     L->VA[k] = a0, L->VA[k + h] = a1;
     L->VS[k] = s0, L->VS[k + h] = s1;
     sum9_add(s.a0, a0);

@@ -45,7 +45,7 @@ int check_job(const vl_lookup_job& J) {
 }
 
 struct LkBufs {
-  size_t lop = 0, hip = 0, binv = 0, tb = 0, wb = 0, wm = 0, va = 0, vs = 0, counts = 0, stage = 0;
+  size_t lop = 0, hip = 0, binv = 0, tb = 0, wb = 0, wm = 0, ub = 0, vb = 0, va = 0, vs = 0, counts = 0, stage = 0;
 };
 
 int cuda_fail(const char* where, cudaError_t e) {
@@ -60,6 +60,7 @@ int cuda_fail(const char* where, cudaError_t e) {
 struct vl_lookup_plan {
   std::vector<vl_lookup_job> jobs;
   int np = 0, maxL = 0, nslots = 0, nrounds = 0;
+  bool tables2 = false;  // some proof reads round 2's A from its tables
   std::vector<LkDev> Ls;  // statements; device pointers filled at bind time
   std::vector<LkBufs> buf;
   std::vector<LkItem> hist, tab, rounds;
@@ -108,8 +109,11 @@ int lk_build(vl_lookup_plan* P, const vl_lookup_job* jobs, int32_t njobs) {
     std::memcpy(L.bind, J.bind, 32);
     L.inv2 = inv2;
     L.dense = L.ld == L.cols ? 1 : 0;
-    L.tail = std::max(1, L.L - LK_TAIL_LOG);  // rounds with h = 2^(L-t) <= 2^LK_TAIL_LOG pairs
+    L.tail = std::max(1, L.L - (njobs > LK_MANY ? LK_TAIL_LOG_MANY : LK_TAIL_LOG));  // rounds with h = 2^(L-t) pairs
     if (L.L == 0) L.tail = 1;
+    // two table products per entry against two fold products per pair of round 2
+    L.round2 = L.tail > 2 && L.L > L.log2_n + 1 ? 1 : 0;
+    P->tables2 = P->tables2 || L.round2;
     P->maxL = std::max(P->maxL, L.L);
     const int N = 1 << L.log2_n;
     for (int k0 = 0; k0 < L.n; k0 += LK_HIST) P->hist.push_back(LkItem{i, k0, std::min(L.n, k0 + LK_HIST), 0});
@@ -123,6 +127,12 @@ int lk_build(vl_lookup_plan* P, const vl_lookup_job* jobs, int32_t njobs) {
   P->nlo.assign(P->maxL + 2, 0);
   for (int t = 1; t <= P->maxL; t++) {
     P->roff[t] = (int)P->rounds.size();
+    // pairs per item: LK_PAIRS, halved while the round has too few items
+    int64_t total = 0;
+    for (const LkDev& L : P->Ls)
+      if (t < L.tail) total += int64_t(1) << (L.L - t);
+    int per = LK_PAIRS;
+    while (per > LK_PAIRS_MIN && total < (int64_t)per * LK_ITEMS) per >>= 1;
     for (int pass = 0; pass < 2; pass++)
       for (int i = 0; i < njobs; i++) {
         LkDev& L = P->Ls[i];
@@ -131,7 +141,7 @@ int lk_build(vl_lookup_plan* P, const vl_lookup_job* jobs, int32_t njobs) {
         if (jr != (pass == 1)) continue;
         const int h = 1 << (L.L - t);
         L.pbeg[t] = slot;
-        const int pairs = std::min(LK_PAIRS, 1 << L.sE);
+        const int pairs = std::min(per, 1 << L.sE);
         for (int k0 = 0; k0 < h; k0 += pairs) {
           P->rounds.push_back(LkItem{i, k0, std::min(h, k0 + pairs), slot++});
           (pass ? P->nlo : P->nhi)[t]++;
@@ -174,6 +184,10 @@ int lk_build(vl_lookup_plan* P, const vl_lookup_job* jobs, int32_t njobs) {
     b.tb = take(sizeof(Fr) * N);
     b.wb = take(sizeof(Fr) * N);
     b.wm = take(sizeof(Fr) * N);
+    if (L.round2) {
+      b.ub = take(sizeof(Fr) * N);
+      b.vb = take(sizeof(Fr) * N);
+    }
     b.va = take(sizeof(Fr) * half);
     b.vs = take(sizeof(Fr) * half);
     if (jobs[i].S.space == VL_HOST) b.stage = take(sizeof(int16_t) * (size_t)L.n);
@@ -195,6 +209,8 @@ int lk_bind(vl_lookup_plan* P, uint8_t* ws, cudaStream_t st) {
     L.Tb = reinterpret_cast<Fr*>(ws + b.tb);
     L.WB = reinterpret_cast<Fr*>(ws + b.wb);
     L.WM = reinterpret_cast<Fr*>(ws + b.wm);
+    L.UB = L.round2 ? reinterpret_cast<Fr*>(ws + b.ub) : nullptr;
+    L.VB = L.round2 ? reinterpret_cast<Fr*>(ws + b.vb) : nullptr;
     L.VA = reinterpret_cast<Fr*>(ws + b.va);
     L.VS = reinterpret_cast<Fr*>(ws + b.vs);
     L.counts = reinterpret_cast<uint32_t*>(ws + P->off_counts + b.counts);
@@ -281,8 +297,11 @@ extern "C" int32_t vl_lookup_plan_run(vl_lookup_plan* P, void* workspace, size_t
     ce = launch_lookup_setup(dL, P->np, items(P->off_hist), (int)P->hist.size(), items(P->off_tab),
                              (int)P->tab.size(), st);
   if (ce == cudaSuccess) ce = cudaEventRecord(P->ev[1], st);
-  for (int t = 1; t <= P->nrounds && ce == cudaSuccess; t++)
+  for (int t = 1; t <= P->nrounds && ce == cudaSuccess; t++) {
+    if (t == 2 && P->tables2) ce = launch_lookup_tables2(dL, items(P->off_tab), (int)P->tab.size(), st);
+    if (ce != cudaSuccess) break;
     ce = launch_lookup_round(dL, P->np, t, items(P->off_rounds) + P->roff[t], P->nhi[t], P->nlo[t], dout, st);
+  }
   if (ce == cudaSuccess) ce = cudaEventRecord(P->ev[2], st);
   if (ce == cudaSuccess) ce = launch_lookup_finish(dL, P->np, dout, st);
   if (ce == cudaSuccess) ce = cudaEventRecord(P->ev[3], st);
