@@ -349,11 +349,14 @@ static constexpr int LK_PAIRS_MIN = 32;
 static constexpr int LK_ITEMS = 2432;
 static constexpr int LK_ENTRIES = 4096;   // table entries per table item (one batch inversion)
 static constexpr int LK_HIST = 32768;     // S entries per histogram item
-// Rounds of at most 2^LK_TAIL_LOG pairs run in one block per proof; of at most
-// 2^LK_TAIL_LOG_MANY in batches of more than LK_MANY proofs, whose tails run on
-// 128 threads each (the 512 lookups of a 7B step: tails 1107 -> 513 us, the two more
-// batched rounds 165).
+// Rounds of at most 2^LK_TAIL_LOG pairs run in one launch over the proofs (the
+// tails): of at most 2^LK_TAIL_LOG_FEW in batches of up to LK_FEW proofs, for
+// which a tail has eight CTAs; of at most 2^LK_TAIL_LOG_MANY in batches of more
+// than LK_MANY proofs, whose tails run on 128 threads each (the 512 lookups of a
+// 7B step: tails 1107 -> 513 us, the two more batched rounds 165).
 static constexpr int LK_TAIL_LOG = 11;
+static constexpr int LK_TAIL_LOG_FEW = 12;
+static constexpr int LK_FEW = 19;
 static constexpr int LK_TAIL_LOG_MANY = 9;
 static constexpr int LK_MANY = 152;
 cudaError_t launch_lookup_setup(LkDev* Ls, int np, const LkItem* hist_items, int nhist, const LkItem* tab_items,

@@ -564,41 +564,52 @@ __device__ void lk_finish(LkDev* L, LkShared& sh, vl_lookup_proof* out) {
   }
 }
 
-// One block per proof: its rounds from L->tail on (at most 2^LK_TAIL_LOG
-// pairs each), each a pass over the pairs, a block reduction and the
+// One block or cluster per proof: its rounds from L->tail on, each a pass over the pairs, a block reduction and the
 // transcript step in this block, then the final evaluations and the proof.
 // In a table round the first half of the warps take the A side's pairs, the
 // second half the table side's.  Short rounds spread a pair over four lanes
 // (one fold each, then one product and one product by f).  The last warp forms
 // the claims and scalars of the next round beside its share of a pass.
-template <int THREADS, int MINB>
+// In a cluster (CL) the rounds of at least RND_CL_PAIRS pairs are spread over its
+// CTAs as in rounds_cluster (CTA c owns the entries k with (k / 32) mod CTAs = c);
+// the first CTA makes the transcript steps and, alone, the rounds after those.
+template <int THREADS, int MINB, bool CL>
 __global__ void __launch_bounds__(THREADS, MINB) lk_tail_kernel(LkDev* Ls, vl_lookup_proof* outs) {
   __shared__ LkShared sh;
-  LkDev* L = Ls + blockIdx.x;
-  vl_lookup_proof* out = outs + blockIdx.x;
+  __shared__ Fr part[CL ? RND_MAX_CTAS : 1][8];  // each CTA's sums of a spread round, in the first CTA
+  const int C = CL ? (int)cluster_size() : 1, rank = CL ? (int)cluster_rank() : 0;
+  const int proof = CL ? (int)blockIdx.x / C : (int)blockIdx.x;
+  LkDev* L = Ls + proof;
+  vl_lookup_proof* out = outs + proof;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   constexpr int NW = THREADS / 32;
   lk_copy_run(&sh.run, &L->run);
   __syncthreads();
   if (L->tail == 1 && L->L >= 1) lk_first_step(L, sh);
+  if (CL) cluster_sync();  // every CTA has started: its shared memory may be written
   for (int t = L->tail; t <= L->L; t++) {
     const int h = 1 << (L->L - t);
+    const bool spread = CL && h >= RND_CL_PAIRS;
+    if (CL && !spread && rank > 0) return;
+    const int own = spread ? h / C : h;  // this CTA's pairs
+    auto pair = [&](int l) { return spread ? ((l >> 5) * C + rank) * 32 + (l & 31) : l; };
     const int tj = t - (L->L - L->log2_n);
     const bool jr = tj > 0;
     if (t > L->tail) {
       if (t == 3) {  // round 3 needs the weights that the step leaves
-        if (warp == NW - 1) lk_step_r(L, sh, t - 1);
+        if (warp == NW - 1 && rank == 0) lk_step_r(L, sh, t - 1);
         __syncthreads();
-      } else if (warp == NW - 1) {
+        if (spread) cluster_sync();
+      } else if (warp == NW - 1 && rank == 0) {
         lk_step_r(L, sh, t - 1);
       }
     }
-    const bool qform = t == 2 && 4 * h > THREADS / (t > L->L - L->log2_n ? 2 : 1);  // see the loop below
+    const bool qform = t == 2 && 4 * own > THREADS / (t > L->L - L->log2_n ? 2 : 1);  // see the loop below
     const LkEq q(L, t);
     const int na = jr ? NW / 2 : NW;  // warps of the A side
     const bool sideb = warp >= na;
     const int id = sideb ? tid - 32 * na : tid, nid = 32 * (sideb ? NW - na : na);
-    if (4 * h > nid) {
+    if (4 * own > nid) {
       unsigned long long a[32];
 #pragma unroll
       for (int i = 0; i < 32; i++) a[i] = 0;
@@ -606,7 +617,8 @@ __global__ void __launch_bounds__(THREADS, MINB) lk_tail_kernel(LkDev* Ls, vl_lo
         LkSumA s;
         s.zero();
 #pragma unroll 1
-        for (int k = id; k < h; k += nid) {
+        for (int l = id; l < own; l += nid) {
+          const int k = pair(l);
           Fr f = q.f_tab[k & q.f_mask];
           if (q.high) f = mont_mul_ni(f, q.hi_tab[k >> L->sE]);
           if (t == 1) lk_pair_a<0>(L, t, k, h, f, s);
@@ -623,7 +635,8 @@ __global__ void __launch_bounds__(THREADS, MINB) lk_tail_kernel(LkDev* Ls, vl_lo
         LkSumB s;
         s.zero();
 #pragma unroll 1
-        for (int k = id; k < h; k += nid) {
+        for (int l = id; l < own; l += nid) {
+          const int k = pair(l);
           Fr f = q.f_tab[k & q.f_mask];
           if (q.high) f = mont_mul_ni(f, q.hi_tab[k >> L->sE]);
           lk_pair_b(L, t, tj, k, h, f, toff, s);
@@ -651,8 +664,8 @@ __global__ void __launch_bounds__(THREADS, MINB) lk_tail_kernel(LkDev* Ls, vl_lo
         else if (lane >= 4 && lane < 8) sh.s[lane - 1] = x;
       }
     } else {
-      const int j = id >> 2, qd = id & 3, at = j + (qd & 1) * h;
-      const bool act = j < h;
+      const int j = pair(id >> 2), qd = id & 3, at = j + (qd & 1) * h;
+      const bool act = (id >> 2) < own;
       Fr x = fr_zero(), x1 = fr_zero(), f = fr_zero(), u0 = fr_zero();
       bool fold = false;
       Fr* dst = nullptr;
@@ -716,11 +729,38 @@ __global__ void __launch_bounds__(THREADS, MINB) lk_tail_kernel(LkDev* Ls, vl_lo
       }
     }
     __syncwarp();
-    if (warp == 0) lk_step_g(L, sh, t, tj, qform, out);
-    lk_transcript(L, sh, warp, t);
+    if (spread) {
+      if (warp == 0 && lane < 7) {
+#pragma unroll
+        for (int l = 0; l < 8; l++) st_cluster(&part[rank][lane].v[l], 0, sh.s[lane].v[l]);
+      }
+      cluster_sync();
+      if (rank == 0 && warp == 0) {
+        // lane 8 (c mod 4) + q: value q of CTAs c, c + 4
+        const int c = lane >> 3;
+        Fr v = c < C ? part[c][lane & 7] : fr_zero();
+        if (c + 4 < C) v = fr_add(v, part[c + 4][lane & 7]);
+#pragma unroll
+        for (int off = 8; off < 32; off <<= 1) v = fr_add(v, shfl_xor_fr(v, off));
+        if (lane < 7) sh.s[lane] = v;
+        __syncwarp();
+      }
+    }
+    if (rank == 0) {
+      if (warp == 0) lk_step_g(L, sh, t, tj, qform, out);
+      lk_transcript(L, sh, warp, t);
+    }
+    if (spread && (h >> 1) >= RND_CL_PAIRS) {
+      // the other CTAs need T''s offset (r_t is in memory)
+      if (rank == 0 && warp == 0) {
+        __syncwarp();
+        for (int i = lane; i < 8 * (C - 1); i += 32) st_cluster(&sh.run.toff.v[i & 7], 1 + (i >> 3), sh.run.toff.v[i & 7]);
+      }
+      cluster_sync();
+    }
     __syncthreads();  // r_t and the folded vectors are visible to the next round
   }
-  lk_finish(L, sh, out);
+  if (rank == 0) lk_finish(L, sh, out);
 }
 
 }  // namespace
@@ -746,8 +786,9 @@ cudaError_t launch_lookup_round(LkDev* Ls, int np, int t, const LkItem* items, i
   return cudaGetLastError();
 }
 
-// A proof's tail is a chain of rounds: with an SM for every proof it runs on 512
-// threads, else on 128, four proofs per SM (one lookup of 512 x 16 remainders
+// A proof's tail is a chain of rounds: with SMs to spare it runs on a cluster of 8,
+// 4 or 2 CTAs (one lookup of 512 x 16 remainders 423 -> 355 us, its tail now from
+// 2^LK_TAIL_LOG_FEW pairs), with an SM for every proof on 512 threads, else on 128, four proofs per SM (one lookup of 512 x 16 remainders
 // 0.98 -> 0.42 ms, the 512 of a 7B step 8.86 -> 4.13 ms with the other changes
 // described in lookup_dev.cuh).
 cudaError_t launch_lookup_finish(LkDev* Ls, int np, vl_lookup_proof* out, cudaStream_t st) {
@@ -755,8 +796,10 @@ cudaError_t launch_lookup_finish(LkDev* Ls, int np, vl_lookup_proof* out, cudaSt
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return e;
-  if (np <= sms) lk_tail_kernel<512, 1><<<np, 512, 0, st>>>(Ls, out);
-  else lk_tail_kernel<128, 4><<<np, 128, 0, st>>>(Ls, out);
+  const int ctas = cluster_ctas(np, sms);
+  if (ctas > 1) return launch_clusters(lk_tail_kernel<512, 1, true>, np, ctas, 512, 0, st, Ls, out);
+  if (np <= sms) lk_tail_kernel<512, 1, false><<<np, 512, 0, st>>>(Ls, out);
+  else lk_tail_kernel<128, 4, false><<<np, 128, 0, st>>>(Ls, out);
   return cudaGetLastError();
 }
 

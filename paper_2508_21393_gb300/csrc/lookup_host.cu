@@ -109,7 +109,8 @@ int lk_build(vl_lookup_plan* P, const vl_lookup_job* jobs, int32_t njobs) {
     std::memcpy(L.bind, J.bind, 32);
     L.inv2 = inv2;
     L.dense = L.ld == L.cols ? 1 : 0;
-    L.tail = std::max(1, L.L - (njobs > LK_MANY ? LK_TAIL_LOG_MANY : LK_TAIL_LOG));  // rounds with h = 2^(L-t) pairs
+    const int tail_log = njobs > LK_MANY ? LK_TAIL_LOG_MANY : njobs > LK_FEW ? LK_TAIL_LOG : LK_TAIL_LOG_FEW;
+    L.tail = std::max(1, L.L - tail_log);  // round t has 2^(L-t) pairs
     if (L.L == 0) L.tail = 1;
     // two table products per entry against two fold products per pair of round 2
     L.round2 = L.tail > 2 && L.L > L.log2_n + 1 ? 1 : 0;
