@@ -263,34 +263,39 @@ struct LinDev {
   int32_t rows, cols, d0, d1, nmats;
   int32_t red_rows;                // 1: reduce over rows (weights E_x); 0: over columns (E_y)
   int32_t lines;                   // entries of each folded vector
-  int32_t nblk;                    // inner sums per matrix: ceil(lines / 2^s), s = ceil(d_lines / 2)
+  int32_t nblk;                    // partial sums per matrix: inner sums, ceil(lines / 2^s), s = ceil(d_lines / 2),
+                                   //   or a short reduction's items
   uint64_t seed;
   Fr coeffs[VL_LIN_MAX];           // canonical
   uint8_t binds[VL_LIN_MAX][32];
   uint32_t S[8];                   // transcript state after the squeezes (big-endian words)
   Fr corr;                         // 2^15 . sum of the reduced side's eq table (Montgomery)
+  Fr lcorr;                        // corr . sum of the lines side's eq table
   Fr* fac;                         // eq factors: [lo_x 256 | hi_x 256 | lo_y 256 | hi_y 256]; lo of the
                                    //   reduced side double-Montgomery, all others Montgomery
   uint32_t* w8;                    // reduced side's eq table as fp16 bytes (fold weights)
   Fr* f;                           // one segment per tile: nmats x lines, M_q~ folded (Montgomery)
   unsigned long long* acc;         // several segments: nmats x lines x 8 column sums
-  Fr* part;                        // nmats x nblk inner sums (Montgomery)
+  Fr* part;                        // nmats x nblk partial sums (Montgomery)
   ProofScratch* scr;               // status (the fold's DevProof points here)
-  Fr* e2;                          // short reductions: the reduced side's eq table, double-Montgomery
+  Fr* el;                          // short reductions: the lines side's eq table (Montgomery); else null
+  uint32_t* bf;                    // short reductions: the reduced side's weight bytes as MMA fragments
 };
-// Linear zkMat, short reductions (at most LIN_SHORT_MAX entries): the fold on
-// CUDA cores, one thread per line (a tensor-core stage would be mostly
-// padding).  One item per block of LIN_SHORT_LINES lines of one matrix.
+// Linear zkMat, short reductions (at most LIN_SHORT_MAX entries): a tensor-core
+// fold stage (128 entries) would be mostly padding.  One item per block of at
+// most LIN_SHORT_LINES lines of one matrix.
 static constexpr int LIN_SHORT_MAX = 128;
-static constexpr int LIN_SHORT_LINES = 256;
+static constexpr int LIN_SHORT_LINES = 1024;  // 4 tiles of 32 lines per warp (the bound of the unreduced sums)
+static constexpr int LIN_SHORT_THREADS = 256;
 struct LinShort {
   const int16_t* base;  // stored matrix (device)
   int64_t ld;           // elements between stored rows
   int32_t proof, q;     // proof, matrix of the proof
   int32_t w0, nw;       // lines [w0, w0 + nw): stored rows (ROWDOT) or columns (COLSUM)
   int32_t mode, red;    // MODE_ROWDOT / MODE_COLSUM, reduced entries per line
+  int32_t part, pad;    // partial-sum slot within the matrix
 };
-static_assert(sizeof(LinShort) == 40, "short item");
+static_assert(sizeof(LinShort) == 48, "short item");
 // Lookup argument (kernels_lookup.cu): one LkDev per proof, in the workspace.
 static constexpr int LK_MAX_L = VL_LOOKUP_MAX_LOG_D;
 // The transcript side of a lookup proof's rounds, advanced by each transcript step.
@@ -406,9 +411,12 @@ void ws_claim(const void* owner, const void* ws);
 void ws_release(const void* owner);
 // Batches: one LinDev per proof; chunks of the reduced side's eq table as
 // EqItem {proof, side (unused), i0, i1}.
-// Short-reduction folds (kernels_linear.cu): f_q of every item's lines.
-cudaError_t launch_linear_short(const LinDev* Ls, const LinShort* items, int nitems, cudaStream_t st);
+// Short reductions (kernels_linear.cu): fold and inner sums of every item, of
+// at most max_red reduced entries.
+cudaError_t linear_short_prepare();
+cudaError_t launch_linear_short(const LinDev* Ls, const LinShort* items, int nitems, int max_red, cudaStream_t st);
 cudaError_t launch_linear_start(LinDev* Ls, int nproofs, const EqItem* items, int nitems, cudaStream_t st);
+// max_nblk: inner sums per matrix of the proofs that fold on tensor cores (0: none).
 cudaError_t launch_linear_finish(LinDev* Ls, int nproofs, int max_nblk, int max_nmats, vl_lin_proof* out,
                                  cudaStream_t st);
 cudaError_t step_set_smem(int smem_bytes);

@@ -311,10 +311,9 @@ __device__ __forceinline__ void add9(uint32_t (&t)[9], const uint32_t (&z)[9]) {
       : "r"(z[0]), "r"(z[1]), "r"(z[2]), "r"(z[3]), "r"(z[4]), "r"(z[5]), "r"(z[6]), "r"(z[7]), "r"(z[8]));
 }
 
-// w += a (b m) for m < 2^16: up to 2^17 terms of at most 2^526.
-__device__ __forceinline__ void wide_mac_small(uint32_t (&w)[17], const Fr& a, const Fr& b, uint32_t m) {
-  uint32_t z[9], y[9];
-  small_mul(z, b.v, m);
+// w += a z for a nine-limb z (the caller keeps the sum below 2^544).
+__device__ __forceinline__ void wide_mac9(uint32_t (&w)[17], const Fr& a, const uint32_t (&z)[9]) {
+  uint32_t y[9];
   Fr zl;
 #pragma unroll
   for (int i = 0; i < 8; i++) zl.v[i] = z[i];
@@ -326,6 +325,13 @@ __device__ __forceinline__ void wide_mac_small(uint32_t (&w)[17], const Fr& a, c
       : "+&r"(w[8]), "+&r"(w[9]), "+&r"(w[10]), "+&r"(w[11]), "+&r"(w[12]), "+&r"(w[13]), "+&r"(w[14]), "+&r"(w[15]),
         "+&r"(w[16])
       : "r"(y[0]), "r"(y[1]), "r"(y[2]), "r"(y[3]), "r"(y[4]), "r"(y[5]), "r"(y[6]), "r"(y[7]), "r"(y[8]));
+}
+
+// w += a (b m) for m < 2^16: up to 2^17 terms of at most 2^526.
+__device__ __forceinline__ void wide_mac_small(uint32_t (&w)[17], const Fr& a, const Fr& b, uint32_t m) {
+  uint32_t z[9];
+  small_mul(z, b.v, m);
+  wide_mac9(w, a, z);
 }
 
 // s += a for a nine-limb sum of reduced elements.
@@ -480,13 +486,11 @@ VL_HD Fr from_mont(const Fr& a) {
 #endif
 }
 
-// Montgomery reduction of a wide value V = sum_l acc[l] . 2^(32 l) given as
-// eight unsigned 64-bit column sums: returns V . R^-1 mod r (reduced).
-// V < 2^289, so the REDC result is below 2r before the final subtraction.
-VL_HD Fr redc_columns(const uint64_t acc[8]) {
-#if defined(__CUDA_ARCH__)
-  // t = V's ten limbs: the words of the columns are added on one carry chain.
-  uint32_t w[16], t[8], top[8];
+#if defined(__CUDACC__)
+// The ten limbs of V = sum_l acc[l] . 2^(32 l), one carry chain over the words
+// of the columns.
+__device__ __forceinline__ void column_limbs(const uint64_t (&acc)[8], uint32_t (&t)[10]) {
+  uint32_t w[16];
 #pragma unroll
   for (int l = 0; l < 8; l++) {
     w[2 * l] = (uint32_t)acc[l];
@@ -496,12 +500,26 @@ VL_HD Fr redc_columns(const uint64_t acc[8]) {
   asm("add.cc.u32 %0, %9, %10; addc.cc.u32 %1, %11, %12; addc.cc.u32 %2, %13, %14; addc.cc.u32 %3, %15, %16;\n\t"
       "addc.cc.u32 %4, %17, %18; addc.cc.u32 %5, %19, %20; addc.cc.u32 %6, %21, %22; addc.cc.u32 %7, %23, 0;\n\t"
       "addc.u32 %8, 0, 0;"
-      : "=&r"(t[1]), "=&r"(t[2]), "=&r"(t[3]), "=&r"(t[4]), "=&r"(t[5]), "=&r"(t[6]), "=&r"(t[7]), "=&r"(top[0]),
-        "=&r"(top[1])
+      : "=&r"(t[1]), "=&r"(t[2]), "=&r"(t[3]), "=&r"(t[4]), "=&r"(t[5]), "=&r"(t[6]), "=&r"(t[7]), "=&r"(t[8]),
+        "=&r"(t[9])
       : "r"(w[1]), "r"(w[2]), "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7]), "r"(w[8]), "r"(w[9]), "r"(w[10]),
         "r"(w[11]), "r"(w[12]), "r"(w[13]), "r"(w[14]), "r"(w[15]));
+}
+#endif
+
+// Montgomery reduction of a wide value V = sum_l acc[l] . 2^(32 l) given as
+// eight unsigned 64-bit column sums: returns V . R^-1 mod r (reduced).
+// V < 2^289, so the REDC result is below 2r before the final subtraction.
+VL_HD Fr redc_columns(const uint64_t acc[8]) {
+#if defined(__CUDA_ARCH__)
+  uint32_t v[10], t[8], top[8];
+  const uint64_t c[8] = {acc[0], acc[1], acc[2], acc[3], acc[4], acc[5], acc[6], acc[7]};
+  column_limbs(c, v);
 #pragma unroll
-  for (int j = 2; j < 8; j++) top[j] = 0;
+  for (int j = 0; j < 8; j++) {
+    t[j] = v[j];
+    top[j] = j < 2 ? v[8 + j] : 0u;
+  }
   // V / 2^256 = (low 256 bits) / 2^256 (Montgomery, at most r) + the top limbs (below 2^33)
   Fr out = redc_low(t);
   add8(out.v, out.v, top);

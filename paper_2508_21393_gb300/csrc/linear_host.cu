@@ -10,7 +10,7 @@
 // partial dot products against the other dimension's eq table, and the
 // finish kernel (per proof: evaluations, absorb, proof); then one copy of the
 // proofs to the host.  Reductions of at most LIN_SHORT_MAX entries (the LoRA
-// factors' rank dimension) fold on CUDA cores instead of the tensor cores.
+// factors' rank dimension) run fold and dot products in a kernel of their own.
 #include <cuda.h>
 #include <cuda_runtime.h>
 
@@ -50,17 +50,17 @@ constexpr int LIN_MAX_JOBS = 65535;
 struct LinShape {
   int rows = 0, cols = 0, d0 = 0, d1 = 0, q = 0;
   bool red_rows = true;
-  bool shortf = false;  // reduction of at most LIN_SHORT_MAX entries: CUDA-core fold
+  bool shortf = false;  // reduction of at most LIN_SHORT_MAX entries: lin_short_kernel
   int red = 0, lines = 0, seg = 0, nsplit = 0, nblk = 0, ntiles = 0, nshort = 0;
 };
 
 // Workspace offsets of one proof's buffers.
 struct LinBufs {
-  size_t fac = 0, w8 = 0, f = 0, part = 0, e2 = 0;
+  size_t fac = 0, w8 = 0, f = 0, part = 0, el = 0, bf = 0;
 };
 
 struct LinLayout {
-  int np = 0, nmats = 0, ntiles = 0, nshort = 0, max_nblk = 1, max_q = 1;
+  int np = 0, nmats = 0, ntiles = 0, nshort = 0, max_nblk = 0, max_q = 1, max_short = 0, short_lines = LIN_SHORT_LINES;
   std::vector<LinShape> shape;
   std::vector<LinBufs> buf;
   std::vector<EqItem> items;
@@ -111,13 +111,11 @@ int lin_shape(const vl_lin_job& J, LinShape* S) {
   S->seg = ((S->red + split - 1) / split + TC_KS - 1) / TC_KS * TC_KS;
   S->nsplit = (S->red + S->seg - 1) / S->seg;
   S->ntiles = J.nmats * ntl * S->nsplit;
-  // A short reduction would fill few entries of a tensor-core stage: fold it
-  // on CUDA cores, one thread per line.
+  // A short reduction would fill few entries of a tensor-core stage.
   S->shortf = S->red <= LIN_SHORT_MAX;
   if (S->shortf) {
     S->nsplit = 1;
     S->ntiles = 0;
-    S->nshort = J.nmats * ((S->lines + LIN_SHORT_LINES - 1) / LIN_SHORT_LINES);
   }
   // inner sums of the lines side: blocks of 2^s lines, s = ceil(d / 2)
   const int dl = S->red_rows ? S->d1 : S->d0, sl = (dl + 1) >> 1;
@@ -130,18 +128,34 @@ int lin_layout(const vl_lin_job* jobs, int32_t njobs, LinLayout* L) {
   L->np = njobs;
   L->shape.resize(njobs);
   L->buf.resize(njobs);
+  int64_t short_total = 0;
   for (int i = 0; i < njobs; i++) {
     const int e = lin_shape(jobs[i], &L->shape[i]);
     if (e != VL_OK) return e;
     const LinShape& S = L->shape[i];
+    if (S.shortf) short_total += (int64_t)S.q * S.lines;
+  }
+  // Lines per short item: 1024, fewer (a tile of 32 per warp: 256) while a small
+  // batch would leave SMs without a block.
+  while (L->short_lines > LIN_SHORT_THREADS && short_total / L->short_lines < 2 * 152) L->short_lines /= 2;
+  for (int i = 0; i < njobs; i++) {
+    LinShape& S = L->shape[i];
+    if (S.shortf) {
+      S.nblk = (S.lines + L->short_lines - 1) / L->short_lines;
+      S.nshort = S.q * S.nblk;
+      L->max_short = std::max(L->max_short, S.red);
+      L->items.push_back(EqItem{i, 1, 0, S.red});
+      for (int i0 = 0; i0 < S.lines; i0 += EQ_CHUNK) L->items.push_back(EqItem{i, 0, i0, std::min(S.lines, i0 + EQ_CHUNK)});
+    } else {
+      L->max_nblk = std::max(L->max_nblk, S.nblk);
+      // chunks of the reduced side's eq table (padded to whole stages)
+      const int rend = (S.red + TC_KS - 1) / TC_KS * TC_KS;
+      for (int i0 = 0; i0 < rend; i0 += EQ_CHUNK) L->items.push_back(EqItem{i, 1, i0, std::min(rend, i0 + EQ_CHUNK)});
+    }
     L->nmats += S.q;
     L->ntiles += S.ntiles;
     L->nshort += S.nshort;
-    L->max_nblk = std::max(L->max_nblk, S.nblk);
     L->max_q = std::max(L->max_q, S.q);
-    // chunks of the reduced side's eq table (padded to whole stages)
-    const int rend = (S.red + TC_KS - 1) / TC_KS * TC_KS;
-    for (int i0 = 0; i0 < rend; i0 += EQ_CHUNK) L->items.push_back(EqItem{i, 1, i0, std::min(rend, i0 + EQ_CHUNK)});
   }
   size_t off = 0;
   auto take = [&off](size_t bytes) {
@@ -161,11 +175,15 @@ int lin_layout(const vl_lin_job* jobs, int32_t njobs, LinLayout* L) {
     const LinShape& S = L->shape[i];
     LinBufs& b = L->buf[i];
     b.fac = take(sizeof(Fr) * 4 * EQ_FAC);
-    b.w8 = take((size_t)8192 * ((S.red + TC_KS - 1) / TC_KS));
-    // f (one segment per tile) or the column-sum accumulators (several)
-    b.f = take((S.nsplit == 1 ? sizeof(Fr) : 8 * sizeof(unsigned long long)) * (size_t)S.q * S.lines);
+    if (S.shortf) {
+      b.el = take(sizeof(Fr) * (size_t)S.lines);
+      b.bf = take((size_t)1024 * ((S.red + 15) / 16));
+    } else {
+      b.w8 = take((size_t)8192 * ((S.red + TC_KS - 1) / TC_KS));
+      // f (one segment per tile) or the column-sum accumulators (several)
+      b.f = take((S.nsplit == 1 ? sizeof(Fr) : 8 * sizeof(unsigned long long)) * (size_t)S.q * S.lines);
+    }
     b.part = take(sizeof(Fr) * (size_t)S.q * S.nblk);
-    b.e2 = S.shortf ? take(sizeof(Fr) * (size_t)S.red) : 0;
   }
   L->off_stage.assign(L->nmats, 0);
   L->stage_ld.assign(L->nmats, 0);
@@ -227,11 +245,12 @@ int lin_bind(vl_lin_plan* P, uint8_t* ws, cudaStream_t st) {
     const LinBufs& b = lay.buf[i];
     LinDev& L = P->Ls[i];
     L.fac = reinterpret_cast<Fr*>(ws + b.fac);
-    L.w8 = reinterpret_cast<uint32_t*>(ws + b.w8);
-    L.f = S.nsplit == 1 ? reinterpret_cast<Fr*>(ws + b.f) : nullptr;
+    L.w8 = S.shortf ? nullptr : reinterpret_cast<uint32_t*>(ws + b.w8);
+    L.f = S.nsplit == 1 && !S.shortf ? reinterpret_cast<Fr*>(ws + b.f) : nullptr;
     L.acc = S.nsplit == 1 ? nullptr : reinterpret_cast<unsigned long long*>(ws + b.f);
     L.part = reinterpret_cast<Fr*>(ws + b.part);
-    L.e2 = S.shortf ? reinterpret_cast<Fr*>(ws + b.e2) : nullptr;
+    L.el = S.shortf ? reinterpret_cast<Fr*>(ws + b.el) : nullptr;
+    L.bf = S.shortf ? reinterpret_cast<uint32_t*>(ws + b.bf) : nullptr;
     L.scr = reinterpret_cast<ProofScratch*>(ws + lay.off_scr) + i;
     std::memset(&P->dps[i], 0, sizeof(DevProof));
     P->dps[i].scr = L.scr;  // the fold reports a timeout through this proof's status
@@ -253,16 +272,17 @@ int lin_bind(vl_lin_plan* P, uint8_t* ws, cudaStream_t st) {
       // Column sums reduce over stored rows, row dots over stored columns.
       const int32_t mode = (S.red_rows != (M.trans != 0)) ? MODE_COLSUM : MODE_ROWDOT;
       if (S.shortf) {
-        for (int w0 = 0; w0 < S.lines; w0 += LIN_SHORT_LINES) {
+        for (int w0 = 0; w0 < S.lines; w0 += lay.short_lines) {
           LinShort it{};
           it.base = static_cast<const int16_t*>(base);
           it.ld = ld;
           it.proof = i;
           it.q = q;
           it.w0 = w0;
-          it.nw = std::min(LIN_SHORT_LINES, S.lines - w0);
+          it.nw = std::min(lay.short_lines, S.lines - w0);
           it.mode = mode;
           it.red = S.red;
+          it.part = w0 / lay.short_lines;
           P->shorts.push_back(it);
         }
         continue;
@@ -307,6 +327,7 @@ int lin_bind(vl_lin_plan* P, uint8_t* ws, cudaStream_t st) {
   up(lay.off_items, lay.items.data(), sizeof(EqItem) * lay.items.size());
   if (ce == cudaSuccess) ce = cudaStreamSynchronize(st);
   if (ce == cudaSuccess) ce = fold_tc_prepare();
+  if (ce == cudaSuccess && lay.nshort > 0) ce = linear_short_prepare();
   if (ce != cudaSuccess) return cuda_fail("linear proofs: bind", ce);
   P->bound_ws = ws;
   ws_claim(P, ws);
@@ -413,7 +434,8 @@ extern "C" int32_t vl_lin_plan_run(vl_lin_plan* P, void* workspace, size_t works
     ce = launch_fold_tc(reinterpret_cast<const TcTile*>(ws + lay.off_tiles), lay.ntiles,
                         reinterpret_cast<const DevProof*>(ws + lay.off_dp), FOLD_WAIT_NS, st);
   if (ce == cudaSuccess)
-    ce = launch_linear_short(dL, reinterpret_cast<const LinShort*>(ws + lay.off_short), lay.nshort, st);
+    ce = launch_linear_short(dL, reinterpret_cast<const LinShort*>(ws + lay.off_short), lay.nshort, lay.max_short,
+                             st);
   if (ce == cudaSuccess) ce = cudaEventRecord(ev[2], st);
   if (ce == cudaSuccess) ce = launch_linear_finish(dL, lay.np, lay.max_nblk, lay.max_q, dout, st);
   if (ce == cudaSuccess) ce = cudaEventRecord(ev[3], st);
