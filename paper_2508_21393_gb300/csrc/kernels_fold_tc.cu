@@ -43,10 +43,15 @@
 //                MMA of constants (accumulator := 1/2) before the operand is
 //                converted, then 8 MMAs (K = 16) with A read from TMEM and B
 //                (weights) from shared memory
-//   warps 2-9    converters: a warp takes 32 lines x half of the stage's 128
-//                entries from the boxes with ldmatrix, forms the lo/hi byte
-//                operand fragments and stores them to TMEM (one of TC_NC
-//                operand buffers) with tcgen05.st
+//   warps 2-9    converters, two groups of four warps that take the stages in
+//                turn: a warp takes 32 lines x 128 entries from the boxes with
+//                ldmatrix, forms the lo/hi byte operand fragments and stores them
+//                to TMEM (one of TC_NC operand buffers) with tcgen05.st.  (With
+//                all eight warps on every stage, half its entries each, a stage
+//                took 1290 cycles, 690 of them conversion, the rest waits and
+//                arrivals; in turn a warp pays these every other stage: 7B step's
+//                fold 1.64 -> 1.48 ms, 13B step's 5.00 -> 4.70.  With the
+//                conversion left out the fold of the 7B step takes 1.32 ms.)
 //   warps 10-17  drainers: accumulator buffer -> per-line digit sums (two
 //                groups of four warps, one warp per TMEM lane quarter, one
 //                group digits 0-15, the other 16-32); tile epilogue
@@ -81,6 +86,10 @@ constexpr int TC_PAIRS = TC_ISSUERS / 2;
 // Pair g takes the stages s = g (mod TC_PAIRS): every operand, weight and
 // accumulator barrier (s mod TC_NC, TC_NW, TC_NA) belongs to one pair.
 static_assert(TC_NC % TC_PAIRS == 0 && TC_NW % TC_PAIRS == 0 && TC_NA % TC_PAIRS == 0, "rings per pair");
+// Converter groups of four warps; as many as pairs (an end marker each), and a
+// group's stages keep to its own slots and buffers.
+constexpr int TC_CONV_GROUPS = TC_CONV_WARPS / 4;
+static_assert(TC_CONV_GROUPS == TC_PAIRS && TC_NR % TC_CONV_GROUPS == 0, "rings per group");
 static_assert(TC_ND > TC_NW && TC_ND > TC_NC && TC_ND >= TC_NA, "stage-done ring");
 constexpr int NBAR = 2 * TC_NR + TC_NC + TC_NA + TC_NW + TC_ND + 3;
 constexpr int SM_TMEM = SM_BAR + NBAR * 8;
@@ -371,9 +380,9 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
   if (tid == 0) {
     for (int s = 0; s < TC_NR; s++) {
       mbar_init(bars.raw_full(s), 1);
-      mbar_init(bars.raw_empty(s), TC_CONV_WARPS);
+      mbar_init(bars.raw_empty(s), 4);  // a group's warps
     }
-    for (int c = 0; c < TC_NC; c++) mbar_init(bars.conv_full(c), TC_CONV_WARPS);
+    for (int c = 0; c < TC_NC; c++) mbar_init(bars.conv_full(c), 4);
     for (int a = 0; a < TC_NA; a++) mbar_init(bars.acc_empty(a), TC_DRAIN_WARPS);
     for (int w = 0; w < TC_NW; w++) mbar_init(bars.w_full(w), 1);
     for (int d = 0; d < TC_ND; d++) mbar_init(bars.done(d), 2);  // the lo and hi issuers of the stage commit
@@ -526,67 +535,72 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     }
   } else if (warp < 2 + TC_CONV_WARPS) {
     // ---------------------------------------------------------------- converters
-    // Warp = 32 lines (its TMEM lane quarter) x half kh of the stage's 128
-    // entries, 16 lines x 64 entries at a time.  Both box layouts come out of
+    // Warp = 32 lines (its TMEM lane quarter) of every TC_CONV_GROUPS-th stage, 16
+    // lines x 64 entries at a time.  Both box layouts come out of
     // ldmatrix as the same fragments (a register = two consecutive entries of
     // one line), which is also a TMEM store shape: per entry a column sum needs
     // no more instructions than a row dot.  (One 16-bit load per entry and a
     // permute per pair, the lines of a column-sum box being 2 bytes apart: 7B
     // step 2.48 ms against 2.31, 13B step 6.93 against 6.36.)
-    const int quarter = warp & 3, kh = (warp - 2) >> 2;  // entries [64 kh, 64 kh + 64) of each stage
-    const uint32_t tq = tmem + ((uint32_t)(32 * quarter) << 16) + ACONV_COL + 32 * kh;
+    const int quarter = warp & 3;
+    const uint32_t tq = tmem + ((uint32_t)(32 * quarter) << 16) + ACONV_COL;
     const int l7 = lane & 7, lm = (lane >> 3) & 1, lk = lane >> 4;  // row in its matrix; matrix: line half, entry half
     // row dots, box kh [128 lines][64 entries], 16-byte chunk j of line m at j ^ (m % 8)
-    const uint32_t row_base = 16384 * kh + (32 * quarter + 8 * lm + l7) * 128;
+    const uint32_t row_base = (32 * quarter + 8 * lm + l7) * 128;
     // column sums, box quarter / 2 [128 entries][64 lines], chunk j of entry k at j ^ (k % 8)
-    const uint32_t col_base = 16384 * (quarter >> 1) + (64 * kh + 8 * lk + l7) * 128;
-    int ends = 0;
-    for (int s = 0;; s++) {
+    const uint32_t col_base = 16384 * (quarter >> 1) + (8 * lk + l7) * 128;
+    for (int s = (warp - 2) >> 2;; s += TC_CONV_GROUPS) {
       const int slot = s % TC_NR, c = s % TC_NC;
       if (!warp_wait(bars.raw_full(slot), (s / TC_NR) & 1, wait_ns)) {
         ok = false;
         break;
       }
       const StageHdr& h = hdr[s % TC_HR];
-      if (s >= TC_NC && !warp_wait(bars.done(s - TC_NC), done_parity(s - TC_NC), wait_ns)) {
-        ok = false;
-        mark_timeout(proofs, tiles, h.tile);
-        break;
-      }
       const int tl = h.tile;
-      if (tl >= 0) {
-        const uint32_t raw = base + SM_RAW + slot * 32768;
+      const bool rowdot = h.mode == MODE_ROWDOT;
+      const uint32_t raw = base + SM_RAW + slot * 32768;
 #pragma unroll
-        for (int hl = 0; hl < 2; hl++) {  // lines 16 hl .. 16 hl + 15 of the quarter
-          uint32_t w[16];                 // entry pairs, as fragments
-          if (h.mode == MODE_ROWDOT) {
-            const uint32_t a = raw + row_base + 16 * 128 * hl;
+      for (int part = 0; part < 4; part++) {  // 16 lines x 64 entries: lines 16 hl .. of the quarter, entries 64 kh ..
+        const int kh = part >> 1, hl = part & 1;
+        uint32_t lo[16], hi[16];
+        if (tl >= 0) {
+          uint32_t w[16];  // entry pairs, as fragments
+          if (rowdot) {
+            const uint32_t ad = raw + row_base + 16384 * kh + 16 * 128 * hl;
 #pragma unroll
-            for (int g = 0; g < 4; g++) ldmatrix4<false>(a + (((2 * g + lk) ^ l7) << 4), w + 4 * g);
+            for (int g = 0; g < 4; g++) ldmatrix4<false>(ad + (((2 * g + lk) ^ l7) << 4), w + 4 * g);
           } else {
-            const uint32_t a = raw + col_base + (((4 * (quarter & 1) + 2 * hl + lm) ^ l7) << 4);
+            const uint32_t ad = raw + col_base + 64 * 128 * kh + (((4 * (quarter & 1) + 2 * hl + lm) ^ l7) << 4);
 #pragma unroll
-            for (int g = 0; g < 4; g++) ldmatrix4<true>(a + 16 * 128 * g, w + 4 * g);
+            for (int g = 0; g < 4; g++) ldmatrix4<true>(ad + 16 * 128 * g, w + 4 * g);
           }
-          uint32_t lo[16], hi[16];
 #pragma unroll
           for (int i = 0; i < 16; i++) {
             lo[i] = w[i] & 0x00ff00ffu;  // p = x + 2^15, per entry: the sign bit flips
             hi[i] = __byte_perm(w[i], 0, 0x4341) ^ 0x00800080u;
           }
-          const uint32_t dst = tq + ((uint32_t)(16 * hl) << 16) + 128 * c;
+        }
+        if (part == 0 && s >= TC_NC && !warp_wait(bars.done(s - TC_NC), done_parity(s - TC_NC), wait_ns)) {
+          ok = false;
+          mark_timeout(proofs, tiles, tl);
+          break;
+        }
+        if (tl >= 0) {
+          const uint32_t dst = tq + ((uint32_t)(16 * hl) << 16) + 128 * c + 32 * kh;
           tmem_st_frag(dst, lo);
           tmem_st_frag(dst + 64, hi);
         }
+      }
+      if (!ok) break;
+      if (tl >= 0) {
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bars.raw_empty(slot));
         tmem_wait_st();
       }
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) {
-        mbar_arrive(bars.conv_full(c));
-        if (tl >= 0) mbar_arrive(bars.raw_empty(slot));
-      }
-      if (tl < 0 && ++ends == 2) break;
+      if (lane == 0) mbar_arrive(bars.conv_full(c));
+      if (tl < 0) break;  // one end marker for each issuer pair: the groups' stages
     }
   } else {
     // ---------------------------------------------------------------- drainers
