@@ -149,13 +149,16 @@ typedef struct vl_batch_opts {
                             a wait that runs out sets the proof's status to
                             VL_ETIMEOUT and its CTA returns                  */
   int32_t rounds_variant; /* rounds kernel: CTAs per SM, 7, 6, 5, 4, 3 or 2
-                            (0: 7); 7 to 4 set the register budget, 3 and 2 also
+                            (0: 7, or, with rounds_threads 0 too, by the number
+                            of proofs: while each finds SMs to itself a cluster
+                            of 8, 4 or 2 CTAs or 512 or 256 threads per proof,
+                            else 4); 7 to 4 set the register budget, 3 and 2 also
                             cap residency (fewer proofs share an SM); 8:
                             batched rounds, one launch per round for the
                             vector work of all proofs and one for their
                             transcript steps (one-group phase launches) */
-  int32_t rounds_threads; /* rounds kernel threads per proof: 128, 192 or 256
-                            (0: 128)                                         */
+  int32_t rounds_threads; /* rounds kernel threads per proof: 128, 192, 256 or
+                            512 (0: 128, or see rounds_variant)              */
   int32_t tc_seg;        /* tensor-core fold: reduced entries per tile, a
                             multiple of 128 up to 32768 (0: 16384); shorter
                             segments spread narrow operands over more SMs */

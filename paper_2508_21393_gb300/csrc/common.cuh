@@ -109,7 +109,8 @@ struct StepItem {
 };
 // Dynamic shared memory of the prologue and rounds block functions.
 static constexpr int PRO_SMEM = 18816;
-static constexpr int RND_SMEM = 21760;
+static constexpr int RND_SMEM = 20736;         // rounds on one CTA per proof
+static constexpr int RND_SMEM_LOOK = 25600;    // with look-ahead or clusters (rounds_dev.cuh)
 // Prologue items run this many proofs ahead of their fold tiles in the queue.
 static constexpr int STEP_LOOKAHEAD = 256;
 

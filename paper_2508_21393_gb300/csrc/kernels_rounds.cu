@@ -10,7 +10,7 @@ __global__ void __launch_bounds__(THREADS, MINB) rounds_kernel(const DevProof* _
                                                                vl_proof* __restrict__ out) {
   extern __shared__ __align__(128) uint8_t rnd_smem[];
   const DevProof& P = proofs[blockIdx.x];
-  rounds_block(P, out + P.job, rnd_smem);
+  rounds_block<(THREADS >= LOOK_THREADS)>(P, out + P.job, rnd_smem);
 }
 
 // A cluster of CTAs per proof, its first rounds over the cluster.
@@ -18,7 +18,7 @@ __global__ void __launch_bounds__(512, 1) rounds_cluster_kernel(const DevProof* 
                                                                 vl_proof* __restrict__ out) {
   extern __shared__ __align__(128) uint8_t rnd_smem[];
   const DevProof& P = proofs[blockIdx.x / cluster_size()];
-  rounds_block(P, out + P.job, rnd_smem, 1, true);
+  rounds_block<true>(P, out + P.job, rnd_smem, 1, true);
 }
 
 // variant: CTAs per SM.  7, 6, 5 and 4 set the register allocation (7: one
@@ -45,17 +45,17 @@ cudaError_t launch_rounds(const DevProof* proofs, int nproofs, vl_proof* out, in
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
     const int ctas = cluster_rounds(max_d1) > 0 ? cluster_ctas(nproofs, sms) : 1;
-    if (ctas > 1) return launch_clusters(rounds_cluster_kernel, nproofs, ctas, 512, RND_SMEM, st, proofs, out);
+    if (ctas > 1) return launch_clusters(rounds_cluster_kernel, nproofs, ctas, 512, RND_SMEM_LOOK, st, proofs, out);
     if (nproofs <= sms) threads = 512;
     else if (nproofs <= 2 * sms) threads = 256;
     else variant = 4;
   }
   if (threads == 512) {
-    rounds_kernel<1, 512><<<nproofs, 512, RND_SMEM, st>>>(proofs, out);
+    rounds_kernel<1, 512><<<nproofs, 512, RND_SMEM_LOOK, st>>>(proofs, out);
   } else if (threads == 192) {
     rounds_kernel<4, 192><<<nproofs, 192, RND_SMEM, st>>>(proofs, out);
   } else if (threads == 256) {
-    rounds_kernel<2, 256><<<nproofs, 256, RND_SMEM, st>>>(proofs, out);
+    rounds_kernel<2, 256><<<nproofs, 256, RND_SMEM_LOOK, st>>>(proofs, out);
   } else if (variant == 2 || variant == 3) {
     static std::atomic<int> set{0};  // launches come from several host threads
     const int smem = variant == 2 ? 100 * 1024 : 70 * 1024;
@@ -214,7 +214,7 @@ __global__ void __launch_bounds__(128, 4) rounds_tail_kernel(const DevProof* __r
                                                              vl_proof* __restrict__ out) {
   extern __shared__ __align__(128) uint8_t rnd_smem[];
   const DevProof& P = proofs[blockIdx.x];
-  rounds_block(P, out + P.job, rnd_smem, 1 + batched_rounds(P.d1));
+  rounds_block<false>(P, out + P.job, rnd_smem, 1 + batched_rounds(P.d1));
 }
 
 }  // namespace

@@ -25,6 +25,11 @@
 //    one term on two of them (two products on the chain instead of six);
 //    vectors of at most RND_VEC entries live in shared memory, and the last
 //    rounds run on warp 0 alone, whose last lane forms the next claim;
+//  * blocks with warps to spare have more to gain there: the next message is ready but for the challenge:
+//    g(0) and G of round i + 1 are quadratics in r_i, as are the claim and g(2), and
+//    other warps sum their coefficients from the unfolded vectors while warps 0
+//    to 2 hash.  From the challenge to the next message are two products then,
+//    and the fold with r_i runs beside the next hash (look_terms);
 //  * the transcript runs on warps 0 to 2: the rounds of each SHA-256
 //    compression on warp 0, its message schedule on warp 1 (of an absorb's
 //    second block: on warp 2); the two halves of the challenge and the
@@ -52,9 +57,12 @@ struct RndShared {
   Fr r;                            // the latest challenge (Montgomery)
   alignas(16) unsigned long long red[3 * 8 * RND_MAX_WARPS];
   Fr fa[RND_VEC], fb[RND_VEC];
-  Fr part[RND_MAX_CTAS][4];        // rounds of a cluster: each CTA's g(0), G, g(1), in the first CTA
+  // look-ahead and clusters only:
+  Fr part[RND_MAX_CTAS][4];        // each CTA's g(0), G, g(1), in the first CTA
+  Fr look[2][4][3];                // coefficients in r of the next g(0), G, claim, g(2) (canonical), two rounds
+  Fr lsum[RND_MAX_WARPS][6];       // look_terms: the warps' sums
 };
-static_assert(sizeof(RndShared) <= RND_SMEM, "shared memory of the rounds");
+static_assert(offsetof(RndShared, part) <= RND_SMEM && sizeof(RndShared) <= RND_SMEM_LOOK, "shared memory of the rounds");
 
 __device__ __forceinline__ Fr load_acc_fr(const unsigned long long* acc, int w, const Fr& corr) {
   U64x8 a;
@@ -176,8 +184,11 @@ __device__ __forceinline__ Fr challenge_of(const uint32_t (&d)[8]) {
 
 // The transcript step of round i (0-based): warps 0 to 2 of the block.  Warp 0
 // has the message in sh.g; with_claim: the claim is absorbed before it.  At the
-// end sh.r, sh.S are set (visible after the block's next barrier).
-__device__ __forceinline__ void transcript_step(RndShared& sh, int warp, bool with_claim, Fr* rch) {
+// end sh.r, sh.S are set (visible after the block's next barrier).  msg: where
+// the proof takes the message, written beside the hashes, g(1) being the claim
+// less g(0) (null: round_message wrote it).
+__device__ __forceinline__ void transcript_step(RndShared& sh, int warp, bool with_claim, Fr* rch,
+                                                vl_fr* msg = nullptr) {
   const int lane = threadIdx.x & 31;
   if (warp == 0) {
     if (with_claim) {
@@ -209,6 +220,11 @@ __device__ __forceinline__ void transcript_step(RndShared& sh, int warp, bool wi
   } else if (warp < 3) {
     if (with_claim) absorb_help(sh, warp);
     absorb_help(sh, warp);
+    if (msg && warp == 2) {
+      if (lane == 0) sh.g[1] = fr_sub(sh.claim, sh.g[0]);
+      __syncwarp();
+      if (lane < 24) msg[lane >> 3].limb[lane & 7] = sh.g[lane >> 3].v[lane & 7];
+    }
     if (warp == 1) {
       named_sync(8, 64);
       uint32_t S[8];
@@ -308,6 +324,91 @@ __device__ __forceinline__ Fr quad_block_sum(RndShared& sh, Fr p, int warp, int 
     p = from_mont_ni(p);
   }
   return p;
+}
+
+// ----------------------------------------------------------------- look-ahead
+//
+// With p = x[j], q = x[j + h] the vectors fold to p + r (q - p), so the next
+// round's g(0) = sum_j a b and G = sum_j (a' - a)(b' - b) (a' hh = h / 2 entries
+// on) are quadratics in r, fixed by their values at 0 and 1 and their leading
+// coefficients: six products per pair of the next round instead of two, off
+// the chain of hashes.  A short round of a lone proof: 8.5 -> 6.5 us (a 64 x 128 x
+// 64 product 139 -> 122 us, one 7B projection 207 -> 190); with 128 threads, where
+// many proofs share the GPU, slower (rounds of the 7B step 427 -> 437 us).
+static constexpr int LOOK_THREADS = 256;  // blocks of at least this many threads have the warps to spare
+
+// The warps that look ahead: of the schedulers 2 and 3 (warp mod 4), so that they
+// take no issue slots from the hash's rounds (warp 0) and schedule (warp 1); warp
+// 2's schedule of an absorb's second block has time.  (Warps 3 up: the first
+// compression of a round 3400 cycles instead of 2700.)
+__device__ __forceinline__ bool look_warp(int warp) { return (warp & 2) && warp != 2; }
+__device__ __forceinline__ int look_rank(int warp) { return ((warp >> 2) << 1 | (warp & 1)) - 1; }
+__device__ __forceinline__ int look_warps() { return (int)(blockDim.x >> 6) - 1; }
+
+// The look-ahead warps: the coefficients of the message after round i's, whose vectors of
+// N entries are in sh.fa, sh.fb, into sh.look[par].  Barrier 9: these warps; 10:
+// warp 0 arrives once round i's message is in sh.g.
+__device__ __forceinline__ void look_terms(RndShared& sh, int warp, int N, int par) {
+  const int lane = threadIdx.x & 31, nwk = look_warps(), wk = look_rank(warp);
+  const int h = N >> 1, hh = N >> 2, s = lane & 7, g = lane >> 3, v = s % 3;
+  named_sync(9, 32 * nwk);  // the folded vectors
+  Fr acc = fr_zero();
+  for (int b = 4 * wk; b < hh; b += 4 * nwk) {
+    const int j = b + g;
+    const bool act = j < hh && s < 6;
+    Fr z[2];
+#pragma unroll
+    for (int m = 0; m < 2; m++) {
+      const Fr* f = (m ? sh.fb : sh.fa) + (act ? j : 0);
+      Fr x = f[0], y = f[h];  // at r = 0, 1
+      if (s >= 3) x = fr_sub(f[hh], x), y = fr_sub(f[h + hh], y);
+      z[m] = v == 0 ? x : v == 1 ? y : fr_sub(y, x);
+    }
+    const Fr p = mont_mul_ni(z[0], z[1]);
+    if (act) acc = fr_add(acc, p);
+  }
+  acc = fr_add(acc, shfl_xor_fr(acc, 8));
+  acc = fr_add(acc, shfl_xor_fr(acc, 16));
+  if (lane < 6) sh.lsum[wk][lane] = acc;
+  named_sync(9, 32 * nwk);
+  if (wk != 0) return;
+  acc = fr_zero();
+  if (s < 6)
+    for (int w = g; w < nwk; w += 4) acc = fr_add(acc, sh.lsum[w][s]);
+  acc = fr_add(acc, shfl_xor_fr(acc, 8));
+  acc = fr_add(acc, shfl_xor_fr(acc, 16));
+  acc = from_mont_ni(acc);
+  // coefficient k on lane k (g(0)), 3 + k (G): 1 is the value at 1 less the others
+  const Fr lead = shfl_fr(acc, (lane + 1) & 31), low = shfl_fr(acc, (lane + 31) & 31);
+  const Fr c = v == 1 ? fr_sub(fr_sub(acc, low), lead) : acc;
+  if (lane < 6) sh.look[par][lane / 3][v] = c;
+  const Fr cg = shfl_fr(c, (lane + 3) & 31);
+  named_sync(10, 64);  // round i's message
+  if (lane < 3) {
+    const Fr g0 = sh.g[0], G = sh.g[3];
+    const Fr cl = lane == 0 ? g0 : lane == 1 ? fr_sub(fr_sub(sh.claim, fr_dbl(g0)), G) : G;
+    sh.look[par][2][lane] = cl;
+    // g(2) = 2 (claim - g(0) + G) - g(0)
+    sh.look[par][3][lane] = fr_sub(fr_dbl(fr_add(fr_sub(cl, c), cg)), c);
+  }
+}
+
+// Warp 0: round i + 1's message and claim at r_i, into sh.g and sh.claim.
+__device__ __forceinline__ void look_message(RndShared& sh, const Fr& r, int par) {
+  const int lane = threadIdx.x & 31, q = lane & 3;
+  const Fr* c = sh.look[par][q];
+  const Fr x = fr_add(c[0], mont_mul_ni(r, fr_add(c[1], mont_mul_ni(r, c[2]))));
+  if (lane < 4) (lane == 0 ? sh.g[0] : lane == 1 ? sh.g[3] : lane == 2 ? sh.claim : sh.g[2]) = x;
+  __syncwarp();
+}
+
+// The look-ahead warps: the vectors of N entries in shared memory folded with r.
+__device__ __forceinline__ void look_fold(RndShared& sh, int warp, int N, const Fr& r) {
+  const int h = N >> 1;
+  for (int i = 32 * look_rank(warp) + (threadIdx.x & 31); i < N; i += 32 * look_warps()) {
+    Fr* f = i < h ? sh.fa + i : sh.fb + (i - h);
+    f[0] = fold1(f[0], f[h], r);
+  }
 }
 
 // ------------------------------------------------------------------ clusters
@@ -449,6 +550,8 @@ static __device__ void rounds_cluster(const DevProof& P, vl_proof* pf, RndShared
 // ran batched over many proofs (kernels_rounds.cu): their messages are in the
 // proof already, the transcript state, the claim and r_(t0-1) are in the
 // scratch, and the vectors hold the round-(t0-1) values, 2^(d1-t0+2) entries each.
+// LOOK: blocks of LOOK_THREADS threads or more.
+template <bool LOOK>
 static __device__ void rounds_block(const DevProof& P, vl_proof* pf, uint8_t* smem, int t0 = 1,
                                     bool clustered = false) {
   RndShared& sh = *reinterpret_cast<RndShared*>(smem);
@@ -536,13 +639,20 @@ static __device__ void rounds_block(const DevProof& P, vl_proof* pf, uint8_t* sm
     }
   }
 
+  bool looked = false;  // the round's message is look_message's
   for (int i = ncl > 0 ? ncl - 1 : t0 - 1; i < d1; i++) {
+    const int h = K >> (i + 1);  // the vectors hold 2h entries
+    const bool look = LOOK && 2 * h <= RND_VEC && h > 1;  // prepare the next message
     if (i >= ncl) {
-      transcript_step(sh, warp, i == 0, P.rch ? P.rch + i : nullptr);
+      if (look && warp == 0) {
+        __syncwarp();
+        named_arrive(10, 64);
+      }
+      if (look && look_warp(warp)) look_terms(sh, warp, 2 * h, i & 1);
+      else transcript_step(sh, warp, i == 0, P.rch ? P.rch + i : nullptr, looked ? pf->g[i] : nullptr);
       __syncthreads();
     }
     const Fr r = sh.r;
-    const int h = K >> (i + 1);  // the vectors hold 2h entries
     const Fr* sA = 2 * h <= RND_VEC ? sh.fa : fA;
     const Fr* sB = 2 * h <= RND_VEC ? sh.fb : fB;
     if (i + 1 == d1) {
@@ -562,6 +672,12 @@ static __device__ void rounds_block(const DevProof& P, vl_proof* pf, uint8_t* sm
         absorb_help(sh, warp);
       }
       break;
+    }
+    looked = look;
+    if (look) {
+      if (warp == 0) look_message(sh, r, i & 1);
+      else if (look_warp(warp)) look_fold(sh, warp, 2 * h, r);
+      continue;
     }
     const int hh = h >> 1;
     Fr* dA = h <= RND_VEC ? sh.fa : fA;

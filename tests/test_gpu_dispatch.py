@@ -4,15 +4,17 @@ long for the oracle, the same statement proved alone.
 
 The rules: matmul rounds on clusters of 8, 4 or 2 CTAs, or on 512, 256 or 128
 threads, by the number of proofs, short rounds on four lanes per pair and vectors
-of at most 256 entries in shared memory; CUDA-core fold tiles cut by the number of products; linear reductions
-of at most 128 entries on register fragments (16-entry steps, two accumulator
-starts, 32-line tiles, blocks of 256 to 1024 lines); lookup tails on clusters, 512
-or 128 threads, each from another round on, the table kernel's entries per thread.
+of at most 256 entries in shared memory; batched claims' last rounds in one
+cluster; CUDA-core fold tiles cut by the number of products; linear reductions
+of at most 128 entries on register fragments (16-entry steps, 32-line tiles,
+blocks of 256 to 1024 lines); lookup tails on clusters, 512 or 128 threads, each
+from another round on, the table kernel's entries per thread.
 """
 import numpy as np
 import pytest
 
 import oracle
+from oracle import batch as OB
 from oracle import lookup as OL
 from paper_2508_21393_gb300 import binding as B
 
@@ -88,6 +90,19 @@ def test_cuda_core_fold_tiles_of_lone_and_many_products(m, k, n, mont):
     job = B.job(*ops, 0, 0, 9)
     assert _prove([job]) == [want]
     assert _prove([job] * 40) == [want] * 40
+
+
+@pytest.mark.parametrize("count,k", [(1, 1), (7, 1), (2, 2), (9, 5), (1, 8192), (9, 1500), (64, 128), (65, 256), (130, 70),
+                                     (512, 3), (512, 40), (513, 3), (520, 36)])
+def test_batched_claims_tails(count, k):
+    """Batches whose last rounds run in one cluster, from every kind of first round, and larger ones without."""
+    rng = np.random.default_rng(count + k)
+    jobs = [{"P": _rand(rng, (2, k)), "Q": _rand(rng, (k, 1 + i % 2)), "tp": 0, "tq": 0} for i in range(count)]
+    cj = [B.job(_dev(j["P"]), _dev(j["Q"]), 0, 0, 0) for j in jobs]
+    n = B.vl_batch_workspace_bytes(cj)
+    ws = _ws(n)
+    res = B.vl_prove_matmul_batched(cj, 11, ws.data_ptr(), n)
+    assert res.to_bytes() == OB.prove_matmul_batch(jobs, seed=11).to_bytes()
 
 
 def _linear(mats, trans, seed):
