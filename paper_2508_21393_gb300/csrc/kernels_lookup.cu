@@ -569,7 +569,8 @@ __device__ void lk_finish(LkDev* L, LkShared& sh, vl_lookup_proof* out) {
 // In a table round the first half of the warps take the A side's pairs, the
 // second half the table side's.  Short rounds spread a pair over four lanes
 // (one fold each, then one product and one product by f).  The last warp forms
-// the claims and scalars of the next round beside its share of a pass.
+// the claims and scalars of the next round, of 512 threads beside the pass of the
+// others, of 128 before its share.
 // In a cluster (CL) the rounds of at least RND_CL_PAIRS pairs are spread over its
 // CTAs as in rounds_cluster (CTA c owns the entries k with (k / 32) mod CTAs = c);
 // the first CTA makes the transcript steps and, alone, the rounds after those.
@@ -582,8 +583,9 @@ __global__ void __launch_bounds__(THREADS, MINB) lk_tail_kernel(LkDev* Ls, vl_lo
   LkDev* L = Ls + proof;
   vl_lookup_proof* out = outs + proof;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  constexpr int NW = THREADS / 32;
+  constexpr int NW = THREADS / 32, NP = THREADS >= 512 ? NW - 1 : NW;  // warps, of them in the passes
   lk_copy_run(&sh.run, &L->run);
+  if (tid < 8 && L->tail > 1) sh.r.v[tid] = L->r[L->tail - 2].v[tid];
   __syncthreads();
   if (L->tail == 1 && L->L >= 1) lk_first_step(L, sh);
   if (CL) cluster_sync();  // every CTA has started: its shared memory may be written
@@ -604,16 +606,18 @@ __global__ void __launch_bounds__(THREADS, MINB) lk_tail_kernel(LkDev* Ls, vl_lo
         lk_step_r(L, sh, t - 1);
       }
     }
-    const bool qform = t == 2 && 4 * own > THREADS / (t > L->L - L->log2_n ? 2 : 1);  // see the loop below
     const LkEq q(L, t);
-    const int na = jr ? NW / 2 : NW;  // warps of the A side
+    const Fr r = sh.r;
+    const int na = jr ? NW / 2 : NP;  // warps of the A side
     const bool sideb = warp >= na;
-    const int id = sideb ? tid - 32 * na : tid, nid = 32 * (sideb ? NW - na : na);
-    if (4 * own > nid) {
+    const int id = sideb ? tid - 32 * na : tid, nid = 32 * (sideb ? NP - na : na);
+    const bool loop = 4 * own > 32 * (jr ? NP - na : na), qform = t == 2 && loop;
+    if (loop) {
       unsigned long long a[32];
 #pragma unroll
       for (int i = 0; i < 32; i++) a[i] = 0;
-      if (!sideb) {
+      if (warp >= NP) {
+      } else if (!sideb) {
         LkSumA s;
         s.zero();
 #pragma unroll 1
@@ -621,10 +625,10 @@ __global__ void __launch_bounds__(THREADS, MINB) lk_tail_kernel(LkDev* Ls, vl_lo
           const int k = pair(l);
           Fr f = q.f_tab[k & q.f_mask];
           if (q.high) f = mont_mul_ni(f, q.hi_tab[k >> L->sE]);
-          if (t == 1) lk_pair_a<0>(L, t, k, h, f, s);
-          else if (t == 2) lk_pair_a<1>(L, t, k, h, f, s);
-          else if (t == 3) lk_pair_a<2>(L, t, k, h, f, s);
-          else lk_pair_a<3>(L, t, k, h, f, s);
+          if (t == 1) lk_pair_a<0>(L, k, h, f, r, s);
+          else if (t == 2) lk_pair_a<1>(L, k, h, f, r, s);
+          else if (t == 3) lk_pair_a<2>(L, k, h, f, r, s);
+          else lk_pair_a<3>(L, k, h, f, r, s);
         }
         unsigned long long col[3][8];
         s.columns(col);
@@ -639,19 +643,19 @@ __global__ void __launch_bounds__(THREADS, MINB) lk_tail_kernel(LkDev* Ls, vl_lo
           const int k = pair(l);
           Fr f = q.f_tab[k & q.f_mask];
           if (q.high) f = mont_mul_ni(f, q.hi_tab[k >> L->sE]);
-          lk_pair_b(L, t, tj, k, h, f, toff, s);
+          lk_pair_b(L, tj, k, h, f, r, toff, s);
         }
         unsigned long long col[4][8];
         s.columns(col);
 #pragma unroll
         for (int i = 0; i < 32; i++) a[i] = col[i / 8][i % 8];
       }
-      sh.red[32 * warp + lane] = warp_transpose_sum<32>(a);
+      if (warp < NP) sh.red[32 * warp + lane] = warp_transpose_sum<32>(a);
       __syncthreads();
       if (warp == 0) {
         unsigned long long ta = 0, tb = 0;
         for (int w = 0; w < na; w++) ta += sh.red[32 * w + lane];
-        for (int w = na; w < NW; w++) tb += sh.red[32 * w + lane];
+        for (int w = na; w < NP; w++) tb += sh.red[32 * w + lane];
         U64x8 col;
 #pragma unroll
         for (int l = 0; l < 8; l++) {
@@ -665,7 +669,9 @@ __global__ void __launch_bounds__(THREADS, MINB) lk_tail_kernel(LkDev* Ls, vl_lo
       }
     } else {
       const int j = pair(id >> 2), qd = id & 3, at = j + (qd & 1) * h;
-      const bool act = (id >> 2) < own;
+      const bool act = warp < NP && (id >> 2) < own;
+      Fr p = fr_zero();
+      if (warp < NP && ((id & ~31) >> 2) < own) {  // warps without a pair leave their slots to zeros
       Fr x = fr_zero(), x1 = fr_zero(), f = fr_zero(), u0 = fr_zero();
       bool fold = false;
       Fr* dst = nullptr;
@@ -691,7 +697,7 @@ __global__ void __launch_bounds__(THREADS, MINB) lk_tail_kernel(LkDev* Ls, vl_lo
       }
       __syncwarp();
       if (t > 1 && (!sideb || tj > 1)) {
-        const Fr fx = fr_add(x, mont_mul_ni(L->r[t - 2], fr_sub(x1, x)));
+        const Fr fx = fr_add(x, mont_mul_ni(r, fr_sub(x1, x)));
         if (fold) x = fx;
       }
       if (dst) dst[at] = x;
@@ -701,19 +707,20 @@ __global__ void __launch_bounds__(THREADS, MINB) lk_tail_kernel(LkDev* Ls, vl_lo
       const Fr a0 = w;
       if (sideb && qd == 0) w = u0;
       if (sideb && qd == 1) w = f;
-      Fr p = mont_mul_ni(z, w);
+      p = mont_mul_ni(z, w);
       const Fr pf = mont_mul_ni(p, f);
       if (sideb ? qd == 0 : qd < 2) p = pf;
       if (!sideb && qd == 2) p = a0;
       if (!act || (!sideb && qd == 3)) p = fr_zero();
 #pragma unroll
       for (int off = 4; off < 32; off <<= 1) p = fr_add(p, shfl_xor_fr(p, off));
+      }
       Fr* red = reinterpret_cast<Fr*>(sh.red);
-      if (lane < 4) red[4 * warp + lane] = p;
+      if (lane < 4 && warp < NP) red[4 * warp + lane] = p;
       __syncthreads();
       if (warp == 0) {
         Fr va = fr_zero(), vb = fr_zero();
-        for (int w2 = lane >> 2; w2 < NW; w2 += 8) {
+        for (int w2 = lane >> 2; w2 < NP; w2 += 8) {
           const Fr v = red[4 * w2 + qd];
           if (w2 < na) va = fr_add(va, v);
           else vb = fr_add(vb, v);
@@ -751,10 +758,13 @@ __global__ void __launch_bounds__(THREADS, MINB) lk_tail_kernel(LkDev* Ls, vl_lo
       lk_transcript(L, sh, warp, t);
     }
     if (spread && (h >> 1) >= RND_CL_PAIRS) {
-      // the other CTAs need T''s offset (r_t is in memory)
+      // the other CTAs need r_t and T''s offset
       if (rank == 0 && warp == 0) {
         __syncwarp();
-        for (int i = lane; i < 8 * (C - 1); i += 32) st_cluster(&sh.run.toff.v[i & 7], 1 + (i >> 3), sh.run.toff.v[i & 7]);
+        for (int i = lane; i < 8 * (C - 1); i += 32) {
+          st_cluster(&sh.r.v[i & 7], 1 + (i >> 3), sh.r.v[i & 7]);
+          st_cluster(&sh.run.toff.v[i & 7], 1 + (i >> 3), sh.run.toff.v[i & 7]);
+        }
       }
       cluster_sync();
     }

@@ -38,12 +38,13 @@ __global__ void __launch_bounds__(LK_PASS_THREADS, JR ? 3 : 4) lk_pass_kernel(Lk
   LkDev* L = Ls + it.proof;
   const int h = 1 << (L->L - t);
   const LkEq q(L, t);
+  const Fr r = t > 1 ? L->r[t - 2] : fr_zero();
   const Fr* hf = q.high ? q.hi_tab + (it.k0 >> L->sE) : nullptr;
   {
     LkSumA s;
     s.zero();
 #pragma unroll 1
-    for (int k = it.k0 + lane; k < it.k1; k += 32) lk_pair_a<MODE>(L, t, k, h, q.f_tab[k & q.f_mask], s);
+    for (int k = it.k0 + lane; k < it.k1; k += 32) lk_pair_a<MODE>(L, k, h, q.f_tab[k & q.f_mask], r, s);
     unsigned long long col[3][8];
     s.columns(col);
     const Fr x = lk_warp_sum<3>(col, 2, hf);
@@ -55,7 +56,7 @@ __global__ void __launch_bounds__(LK_PASS_THREADS, JR ? 3 : 4) lk_pass_kernel(Lk
     LkSumB s;
     s.zero();
 #pragma unroll 1
-    for (int k = it.k0 + lane; k < it.k1; k += 32) lk_pair_b(L, t, tj, k, h, q.f_tab[k & q.f_mask], toff, s);
+    for (int k = it.k0 + lane; k < it.k1; k += 32) lk_pair_b(L, tj, k, h, q.f_tab[k & q.f_mask], r, toff, s);
     unsigned long long col[4][8];
     s.columns(col);
     const Fr x = lk_warp_sum<4>(col, 2, hf);

@@ -97,12 +97,12 @@ struct LkSumB {
   }
 };
 
-// One pair (k, k + h) of round t, A side.  MODE 0: round 1, from the unfolded
+// One pair (k, k + h) of round t, r = r_(t-1), A side.  MODE 0: round 1, from the unfolded
 // cube; 1: round 2, A folded on the fly and written, t0 summing Q = f (a' - a)(j'
 // - j) (T(0) = 1 - r (1 - r) Q); 2: round 3, A folded in place, S' formed and
 // written; 3: later rounds, both folded in place.
 template <int MODE>
-__device__ __forceinline__ void lk_pair_a(LkDev* L, int t, int k, int h, const Fr& f, LkSumA& s) {
+__device__ __forceinline__ void lk_pair_a(LkDev* L, int k, int h, const Fr& f, const Fr& r, LkSumA& s) {
   if constexpr (MODE == 0) {
     const int j0 = lk_table_index(*L, k), j1 = lk_table_index(*L, k + h), d = j1 - j0;
     const Fr a0 = L->Binv[j0], a1 = L->Binv[j1];
@@ -110,7 +110,6 @@ __device__ __forceinline__ void lk_pair_a(LkDev* L, int t, int k, int h, const F
     // (a1 - a0)(s1 - s0) = (a1 - a0)(j1 - j0), both signs flipped for j1 < j0
     wide_mac_small(s.ti, f, d < 0 ? fr_sub(a0, a1) : fr_sub(a1, a0), (uint32_t)(d < 0 ? -d : d));
   } else if constexpr (MODE == 1) {
-    const Fr r = L->r[0];
     const int j0 = lk_table_index(*L, k), j1 = lk_table_index(*L, k + h);
     const int j2 = lk_table_index(*L, k + 2 * h), j3 = lk_table_index(*L, k + 3 * h);
     const Fr b0 = L->Binv[j0], b2 = L->Binv[j2];
@@ -130,7 +129,6 @@ __device__ __forceinline__ void lk_pair_a(LkDev* L, int t, int k, int h, const F
     const Fr ds = fr_add(lk_times(fr_r1(), j1 - j0), lk_times(r, (j3 - j2) - (j1 - j0)));
     wide_mac(s.ti, f, mont_mul_ni(fr_sub(a1, a0), ds));
   } else {
-    const Fr r = L->r[t - 2];
     const Fr a0 = lk_fold(L->VA[k], L->VA[k + 2 * h], r);
     const Fr a1 = lk_fold(L->VA[k + h], L->VA[k + 3 * h], r);
     Fr s0, s1;
@@ -152,14 +150,13 @@ __device__ __forceinline__ void lk_pair_a(LkDev* L, int t, int k, int h, const F
 // One pair of a table round (round tj of the last log2 N; eq(u_low, .) folded
 // by the bound table variables is the A side's factor f times a scalar of the
 // transcript step): B and m are folded in place after the first table round.
-__device__ __forceinline__ void lk_pair_b(LkDev* L, int t, int tj, int k, int h, const Fr& f, const Fr& toff,
+__device__ __forceinline__ void lk_pair_b(LkDev* L, int tj, int k, int h, const Fr& f, const Fr& r, const Fr& toff,
                                           LkSumB& s) {
   Fr b0, b1, m0, m1;
   if (tj == 1) {
     b0 = L->WB[k], b1 = L->WB[k + h];
     m0 = L->WM[k], m1 = L->WM[k + h];
   } else {
-    const Fr r = L->r[t - 2];
     b0 = lk_fold(L->WB[k], L->WB[k + 2 * h], r);
     b1 = lk_fold(L->WB[k + h], L->WB[k + 3 * h], r);
     m0 = lk_fold(L->WM[k], L->WM[k + 2 * h], r);
