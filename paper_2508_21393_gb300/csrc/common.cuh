@@ -395,12 +395,24 @@ struct BtState {
   vl_fr* b_out;
   vl_batch_proof* out;
 };
+// Batches of up to BT_TAIL_PRODUCTS products run the rounds of at most
+// BT_TAIL_PAIRS pairs (over all products) in one cluster launch (bt_tail_kernel).
+static constexpr int BT_TAIL_PRODUCTS = 512;
+static constexpr int BT_TAIL_PAIRS = 1024;
+// The tail's first round (2 .. d1 + 1; with no rounds 1), 0 without a tail.
+inline int batch_tail(int K, int d1) {
+  if (K > BT_TAIL_PRODUCTS) return 0;
+  if (d1 == 0) return 1;
+  int t = d1 + 1;
+  while (t > 2 && ((int64_t)K << (d1 - t + 1)) <= BT_TAIL_PAIRS) t--;
+  return t;
+}
 // Claims (one CTA per product), then the batch start with round 1.
 cudaError_t launch_batch_claims(const DevProof* dp, int np, BtState* B, cudaStream_t st);
 // Round t >= 2.
 cudaError_t launch_batch_round(const DevProof* dp, BtState* B, int t, const LkItem* items, int nitems,
                                cudaStream_t st);
-cudaError_t launch_batch_finish(const DevProof* dp, int np, BtState* B, int k, cudaStream_t st);
+cudaError_t launch_batch_finish(const DevProof* dp, int np, BtState* B, int k, int tail, cudaStream_t st);
 
 // Host helpers of the engine shared with the linear prover.
 bool encode_tc_operand(const void* base, int64_t rows, int64_t cols, int64_t ld, int32_t mode, void* map);

@@ -1444,9 +1444,10 @@ int batch_layout(const vl_job* jobs, int32_t njobs, BatchLayout* L) {
   while (L->P2 < njobs) L->P2 <<= 1;
   // round items: each proof's pairs in chunks, round by round (slots = item index)
   L->roff.assign(L->d1 + 2, 0);
+  const int tail = batch_tail(njobs, L->d1);
   for (int t = 1; t <= L->d1; t++) {
     L->roff[t] = (int)L->items.size();
-    if (t == 1) continue;  // round 1 is evaluated with the claims
+    if (t == 1 || (tail && t >= tail)) continue;  // with the claims; in the tail
     const int h = 1 << (L->d1 - t);
     for (int s = 0; s < njobs; s++)
       for (int k0 = 0; k0 < h; k0 += BT_PAIRS)
@@ -1581,9 +1582,10 @@ extern "C" int32_t vl_claims_plan_run(vl_claims_plan* C, void* workspace, size_t
   if (ce == cudaSuccess) ce = launch_fold_tc(dc, (int)p->tc_tiles.size(), dp, wait_ns(p), st);
   if (ce == cudaSuccess) ce = launch_fold(dt, dl, (int)p->tiles.size(), dp, p->fold_smem, wait_ns(p), st);
   if (ce == cudaSuccess) ce = launch_batch_claims(dp, np, dS, st);
-  for (int t = 2; t <= L.d1 && ce == cudaSuccess; t++)
+  const int tail = batch_tail(K, L.d1);
+  for (int t = 2; t <= (tail ? tail - 1 : L.d1) && ce == cudaSuccess; t++)
     ce = launch_batch_round(dp, dS, t, di + L.roff[t], L.roff[t + 1] - L.roff[t], st);
-  if (ce == cudaSuccess) ce = launch_batch_finish(dp, np, dS, L.k, st);
+  if (ce == cudaSuccess) ce = launch_batch_finish(dp, np, dS, L.k, tail, st);
   const cudaMemcpyKind kind = out_space == VL_HOST ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice;
   if (ce == cudaSuccess) ce = cudaMemcpyAsync(out, ws + L.off_proof, sizeof(vl_batch_proof), kind, st);
   if (ce == cudaSuccess) ce = cudaMemcpyAsync(claims, ws + L.off_cout, sizeof(vl_fr) * K, kind, st);

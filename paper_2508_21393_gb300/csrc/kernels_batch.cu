@@ -13,8 +13,10 @@
 //           previous challenge, then rho^i-weighted sums of g(0) and the leading
 //           coefficient, see rounds_dev.cuh); the CTA that finishes last runs
 //           the transcript step (g(1) = claim - g(0));
-//   finish  (one CTA per product) a_i, b_i and their leaves; (one CTA) the
-//           root, absorb 'f', the proof.
+//   tail    (one cluster) of up to BT_TAIL_PRODUCTS products the rounds of at most
+//           BT_TAIL_PAIRS pairs, then a_i, b_i and their leaves (of more products:
+//           one CTA per product);
+//   close   (one CTA) the root, absorb 'f', the proof.
 #include "prologue_dev.cuh"
 #include "rounds_dev.cuh"
 
@@ -23,6 +25,7 @@ namespace vl {
 namespace {
 
 constexpr int BT_THREADS = 256;
+constexpr int BT_TAIL_THREADS = 512;
 constexpr uint8_t LBL_P = 'p';
 
 // f_A[w] (side 0) or f_B[w] (side 1) of the unfolded vectors; 0 past k.
@@ -111,6 +114,20 @@ __device__ void bt_tree(BtState* B) {
   }
 }
 
+// Warp 0: round t's message from g(0) and G, into sh.g and the proof.
+__device__ __forceinline__ void bt_message(BtState* B, RndShared& sh, int t, const Fr& g0, const Fr& G) {
+  const int lane = threadIdx.x & 31;
+  const Fr g1 = fr_sub(sh.claim, g0), g2 = fr_sub(fr_dbl(fr_add(g1, G)), g0);
+  if (lane == 0) {
+    sh.g[0] = g0;
+    sh.g[1] = g1;
+    sh.g[2] = g2;
+    sh.g[3] = G;
+  }
+  __syncwarp();
+  if (lane < 24) B->out->g[t - 1][lane >> 3].limb[lane & 7] = sh.g[lane >> 3].v[lane & 7];
+}
+
 // Round t's transcript step by the whole block (at least 4 warps) from g(0)
 // and the leading coefficient G (canonical, valid in warp 0): message, absorb,
 // squeeze r_t, the next claim.
@@ -119,17 +136,7 @@ __device__ void bt_step(BtState* B, RndShared& sh, int t, const Fr& g0, const Fr
   if (tid < 8) sh.S[tid] = B->St[tid];
   if (tid == 0) sh.claim = B->claim;
   __syncthreads();
-  if (warp == 0) {
-    const Fr g1 = fr_sub(sh.claim, g0), g2 = fr_sub(fr_dbl(fr_add(g1, G)), g0);
-    if (tid == 0) {
-      sh.g[0] = g0;
-      sh.g[1] = g1;
-      sh.g[2] = g2;
-      sh.g[3] = G;
-    }
-    __syncwarp();
-    if (tid < 24) B->out->g[t - 1][tid >> 3].limb[tid & 7] = sh.g[tid >> 3].v[tid & 7];
-  }
+  if (warp == 0) bt_message(B, sh, t, g0, G);
   transcript_step(sh, warp, false, &B->r[t - 1]);
   __syncthreads();
   if (tid < 8) B->St[tid] = sh.S[tid];
@@ -254,15 +261,14 @@ __global__ void __launch_bounds__(BT_THREADS) bt_round_kernel(const DevProof* dp
   bt_step(B, sh, t, acc[0], acc[1]);
 }
 
-// One warp per product: a_i (lane 0) and b_i (lane 1), the last pair folded with
+// One warp: a_i (lane 0) and b_i (lane 1) of a product, the last pair folded with
 // r_d1, their canonical outputs and Merkle leaf.
-__global__ void __launch_bounds__(32) bt_final_kernel(const DevProof* dp, BtState* B) {
-  const DevProof& P = dp[blockIdx.x];
-  const int i = P.member1 - 1, d1 = B->d1, lane = threadIdx.x;
+__device__ __forceinline__ void bt_final(const DevProof& P, BtState* B, const Fr& r) {
+  const int i = P.member1 - 1, d1 = B->d1, lane = threadIdx.x & 31;
   Fr x = fr_zero();
   if (lane < 2) {
     const Fr* f = lane == 0 ? P.fA : P.fB;
-    x = d1 == 0 ? f[0] : fold1(f[0], f[1], B->r[d1 - 1]);
+    x = d1 == 0 ? f[0] : fold1(f[0], f[1], r);
     x = from_mont_ni(x);
     store_fr(lane == 0 ? &B->a_out[i] : &B->b_out[i], x);
   }
@@ -274,6 +280,78 @@ __global__ void __launch_bounds__(32) bt_final_kernel(const DevProof* dp, BtStat
   bt_words(Y, 9, bc);
   dev_hash_tagged<17>(0u, Y, node);
   if (lane == 0) store_digest_bytes(B->tree + (size_t)(B->P2 + i) * 32, node);
+}
+
+__global__ void __launch_bounds__(32) bt_final_kernel(const DevProof* dp, BtState* B) {
+  bt_final(dp[blockIdx.x], B, B->d1 > 0 ? B->r[B->d1 - 1] : fr_zero());
+}
+
+// Rounds t0 .. d1 and the final values by one cluster: CTA c takes the products
+// i = c (mod CTAs), four lanes per pair, so no vector entry changes hands; the
+// sums go to the first CTA, which makes the transcript step, and the challenge
+// comes back (as in rounds_cluster).  A round this short is latency, about 16 us as
+// a launch of its own: 256 products of a 7B model 773 -> 762 us (from 8192 pairs
+// on, with twice the products per pair of bt_round_kernel's loop, 794).
+__global__ void __launch_bounds__(BT_TAIL_THREADS, 1) bt_tail_kernel(const DevProof* dp, BtState* B, int t0) {
+  __shared__ RndShared sh;
+  const int rank = (int)cluster_rank(), C = (int)cluster_size();
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, q = tid & 3, last = BT_TAIL_THREADS / 32 - 1;
+  const int d1 = B->d1, np = (B->K - rank + C - 1) / C;  // this CTA's products
+  if (tid < 8) {
+    sh.S[tid] = B->St[tid];
+    sh.claim.v[tid] = B->claim.v[tid];
+    sh.r.v[tid] = d1 > 0 ? B->r[t0 - 2].v[tid] : 0u;
+  }
+  cluster_sync();
+  for (int t = t0; t <= d1; t++) {
+    const int lg = d1 - t, hh = 1 << lg, h = 2 * hh;
+    const Fr r = sh.r;
+    if (rank == 0 && t > t0 && warp == last && lane == 0) next_claim(sh);
+    Fr acc = fr_zero();
+    for (int b = 0; b < np << lg; b += BT_TAIL_THREADS / 4) {
+      const int e = b + (tid >> 2);
+      const bool act = e < np << lg;
+      Fr x = fr_zero(), d = fr_zero(), w = fr_zero();
+      Fr* f = nullptr;
+      if (act) {
+        const DevProof& P = dp[rank + C * (e >> lg)];
+        f = (q < 2 ? P.fA : P.fB) + (e & (hh - 1)) + (q & 1) * hh;
+        x = f[0];
+        d = fr_sub(f[h], x);
+        w = B->w[P.member1 - 1];
+      }
+      __syncwarp();
+      const Fr p = mont_mul_ni(quad_terms(x, d, r, false), w);
+      if (act) {
+        f[0] = x;
+        acc = fr_add(acc, p);
+      }
+    }
+#pragma unroll
+    for (int off = 4; off < 32; off <<= 1) acc = fr_add(acc, shfl_xor_fr(acc, off));
+    const Fr s = quad_block_sum(sh, acc, warp, last);
+    if (warp == 0 && lane < 2) {
+#pragma unroll
+      for (int l = 0; l < 8; l++) st_cluster(&sh.part[rank][lane].v[l], 0, s.v[l]);
+    }
+    cluster_sync();
+    if (rank == 0) {
+      if (warp == 0) {
+        Fr v = (lane >> 2) < C && q < 2 ? sh.part[lane >> 2][q] : fr_zero();
+#pragma unroll
+        for (int off = 4; off < 32; off <<= 1) v = fr_add(v, shfl_xor_fr(v, off));
+        bt_message(B, sh, t, shfl_fr(v, 0), shfl_fr(v, 1));
+      }
+      transcript_step(sh, warp, false, &B->r[t - 1]);
+      if (warp == 0) {
+        __syncwarp();
+        for (int i = lane; i < 8 * (C - 1); i += 32) st_cluster(&sh.r.v[i & 7], 1 + (i >> 3), sh.r.v[i & 7]);
+      }
+    }
+    cluster_sync();
+  }
+  for (int i = warp; i < np; i += BT_TAIL_THREADS / 32) bt_final(dp[rank + C * i], B, sh.r);
+  if (rank == 0 && tid < 8) B->St[tid] = sh.S[tid];
 }
 
 // One block: the root of the final values, absorb 'f', the proof.
@@ -308,8 +386,14 @@ cudaError_t launch_batch_round(const DevProof* dp, BtState* B, int t, const LkIt
   return cudaGetLastError();
 }
 
-cudaError_t launch_batch_finish(const DevProof* dp, int np, BtState* B, int k, cudaStream_t st) {
-  bt_final_kernel<<<np, 32, 0, st>>>(dp, B);
+// tail: the first round of the tail, 0 without one.
+cudaError_t launch_batch_finish(const DevProof* dp, int np, BtState* B, int k, int tail, cudaStream_t st) {
+  if (tail) {
+    const cudaError_t e = launch_clusters(bt_tail_kernel, 1, RND_MAX_CTAS, BT_TAIL_THREADS, 0, st, dp, B, tail);
+    if (e != cudaSuccess) return e;
+  } else {
+    bt_final_kernel<<<np, 32, 0, st>>>(dp, B);
+  }
   bt_close_kernel<<<1, BT_THREADS, 0, st>>>(B, k);
   return cudaGetLastError();
 }
