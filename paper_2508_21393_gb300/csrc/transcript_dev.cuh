@@ -27,28 +27,42 @@ struct ShaBlock {
   uint32_t w[16];
 };
 
-// One SHA-256 compression, fully unrolled with the round constants as
-// immediates, kept out of line (one copy per kernel module): the transcript
-// is a serial chain of compressions, and an inlined copy at every call site
-// makes the latency-bound kernels larger than the instruction cache.  h + K +
-// W is formed off the e-chain, Ch and Maj use their two-operation forms.
+// Word i + 16 of the message schedule from the latest 16 (word i among them).
+__device__ __forceinline__ uint32_t sha_next(const ShaBlock& m, int i) {
+  const uint32_t x = m.w[(i + 1) & 15], y = m.w[(i + 14) & 15];
+  return m.w[i & 15] + (rotr_dev(x, 7) ^ rotr_dev(x, 18) ^ (x >> 3)) + m.w[(i + 9) & 15] +
+         (rotr_dev(y, 17) ^ rotr_dev(y, 19) ^ (y >> 10));
+}
+
+// The round constants for indices that are not known at compile time.
+static __constant__ uint32_t sha_kc[64] = {VL_SHA_K};
+
+// One SHA-256 compression, kept out of line (one copy per kernel module) and as
+// loops over 16 rounds: the transcript is a serial chain of compressions, and
+// straight-line code for 64 rounds (or a copy at every call site) does not stay in
+// the instruction cache.  h + K + W is formed off the e-chain, Ch and Maj use their
+// two-operation forms.
 static __device__ __noinline__ ShaState sha256_block_ni(ShaState st, ShaBlock m) {
   uint32_t a = st.h[0], b = st.h[1], c = st.h[2], d = st.h[3], e = st.h[4], f = st.h[5], g = st.h[6],
            h = st.h[7];
-#pragma unroll
-  for (int i = 0; i < 64; i++) {
-    if (i >= 16) {
-      const uint32_t x = m.w[(i - 15) & 15], y = m.w[(i - 2) & 15];
-      m.w[i & 15] += (rotr_dev(x, 7) ^ rotr_dev(x, 18) ^ (x >> 3)) + m.w[(i - 7) & 15] +
-                     (rotr_dev(y, 17) ^ rotr_dev(y, 19) ^ (y >> 10));
-    }
-    const uint32_t hkw = h + (sha_k(i) + m.w[i & 15]);
+  auto round = [&](uint32_t kw) {
+    const uint32_t hkw = h + kw;
     const uint32_t s1 = rotr_dev(e, 6) ^ rotr_dev(e, 11) ^ rotr_dev(e, 25);
     const uint32_t ch = g ^ (e & (f ^ g));
     const uint32_t t1 = hkw + ch + s1;
     const uint32_t s0 = rotr_dev(a, 2) ^ rotr_dev(a, 13) ^ rotr_dev(a, 22);
     const uint32_t mj = (a & b) | (c & (a | b));
     h = g; g = f; f = e; e = d + t1; d = c; c = b; b = a; a = t1 + (s0 + mj);
+  };
+#pragma unroll
+  for (int i = 0; i < 16; i++) round(sha_k(i) + m.w[i]);
+#pragma unroll 1
+  for (int q = 16; q < 64; q += 16) {
+#pragma unroll
+    for (int i = 0; i < 16; i++) {
+      m.w[i] = sha_next(m, i);
+      round(sha_kc[q + i] + m.w[i]);
+    }
   }
   st.h[0] += a; st.h[1] += b; st.h[2] += c; st.h[3] += d;
   st.h[4] += e; st.h[5] += f; st.h[6] += g; st.h[7] += h;
@@ -74,16 +88,17 @@ __device__ __forceinline__ void named_arrive(int id, int threads) {
   asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(threads) : "memory");
 }
 static __device__ __noinline__ void sha_sched_ni(ShaBlock m, uint32_t* wk, int bar) {
+#pragma unroll 1
+  for (int q = 16; q < 64; q += 16) {
 #pragma unroll
-  for (int i = 16; i < 64; i++) {
-    const uint32_t x = m.w[(i - 15) & 15], y = m.w[(i - 2) & 15];
-    m.w[i & 15] += (rotr_dev(x, 7) ^ rotr_dev(x, 18) ^ (x >> 3)) + m.w[(i - 7) & 15] +
-                   (rotr_dev(y, 17) ^ rotr_dev(y, 19) ^ (y >> 10));
-    if ((i & 3) == 3)
-      *reinterpret_cast<uint4*>(wk + i - 3) =
-          make_uint4(m.w[(i - 3) & 15] + sha_k(i - 3), m.w[(i - 2) & 15] + sha_k(i - 2),
-                     m.w[(i - 1) & 15] + sha_k(i - 1), m.w[i & 15] + sha_k(i));
-    if ((i & 15) == 15) named_arrive(bar + (i >> 4) - 1, 64);
+    for (int i = 0; i < 16; i++) {
+      m.w[i] = sha_next(m, i);
+      if ((i & 3) == 3)
+        *reinterpret_cast<uint4*>(wk + q + i - 3) =
+            make_uint4(m.w[i - 3] + sha_kc[q + i - 3], m.w[i - 2] + sha_kc[q + i - 2],
+                       m.w[i - 1] + sha_kc[q + i - 1], m.w[i] + sha_kc[q + i]);
+    }
+    named_arrive(bar + (q >> 4) - 1, 64);
   }
 }
 // The rounds as a loop over 16: its body fits the instruction cache beside what
