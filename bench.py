@@ -230,22 +230,23 @@ def oracle_cores_baseline(kind, seed):
                       f"(the slowest worker's proving time)"}
 
 
-# Rounds of one matmul proof with d1 variables: round 1 evaluates g(0), g(1),
-# g(2) on 2^(d1-1) pairs (three field products each); every later round t
-# folds four values and evaluates three products on 2^(d1-t) pairs; the last
-# fold is two products.
+# Rounds of one matmul proof with d1 variables: round 1 sums g(0), g(1) and the
+# leading coefficient on 2^(d1-1) pairs (three unreduced products each, half a
+# Montgomery product); every later round t folds four values and sums two
+# unreduced products on 2^(d1-t) pairs; the last fold is two products.
 def rounds_products(d1):
     if d1 == 0:
         return 1
-    return 3 * (1 << (d1 - 1)) + 7 * ((1 << (d1 - 1)) - 1) + 2
+    return 3 * (1 << (d1 - 1)) // 2 + 5 * ((1 << (d1 - 1)) - 1) + 2
 
 
 # One round's transcript step on the GPU (absorb g(0) || g(2): two SHA-256
-# compressions; squeeze r: one more; the 512-bit reduction): a serial chain
-# of 12.3 K cycles for one warp alone (clock64 over 200 dependent steps on the
-# box, at 2.07 GHz 5.9 us).  The derived field-product peak: 152 SMs x 32
-# IMAD.WIDE per clock x 2.07 GHz / 128 IMAD.WIDE per Montgomery product.
-ROUND_HASH_CYCLES = 12300
+# compressions; squeeze r: one more; its reduction): a serial chain of 8.4 K
+# cycles (clock64 in a lone proof's rounds: three compressions 2050 to 2450, the
+# challenge 1400, message words and barriers 500; at 2.07 GHz 4.1 us).  The
+# derived field-product peak: 152 SMs x 32 IMAD.WIDE per clock x 2.07 GHz / 128
+# IMAD.WIDE per Montgomery product.
+ROUND_HASH_CYCLES = 8400
 PRODUCTS_PEAK = SMS * MADWIDE_PER_SM_CLK * SM_MAX_MHZ * 1e6 / 128
 
 
@@ -261,7 +262,7 @@ def rounds_bound(jobs, rounds_ms):
     return {"field_products": prods, "throughput_bound_us": thr_us, "latency_bound_us": lat_us,
             "bound_us": bound_us, "measured_us": 1e3 * rounds_ms, "frac": bound_us / (1e3 * rounds_ms),
             "note": "products at the derived ALU peak (152 SMs x 32 IMAD.WIDE/clk x 2070 MHz / 128 per product); "
-                    "latency = max d1 x 12.3 K-cycle transcript step (measured single-warp chain)"}
+                    "latency = max d1 x 8.4 K-cycle transcript step (measured chain)"}
 
 
 def pinned_h2d_gbs(stream, nbytes=1 << 30, reps=3):
@@ -581,22 +582,20 @@ def update_main(args, rank, world, local, cpu):
         pass
     hbm_peak, hbm_note = (peaks["hbm_gbs"], "measured") if "hbm_gbs" in peaks else (6800.0, "fallback")
     hbm_gbs = 2 * entries / (fold_ms / 1e3) / 1e9
-    # The LoRA factors reduce over the rank (at most 64 entries): the fold runs
-    # on CUDA cores (lin_short_kernel), one thread per line: eight 32 x 32 ->
-    # 64-bit multiply-adds per entry and one REDC (64 more) per line.  Bound:
-    # those multiply-adds at the derived ALU peak; the 2 B per entry of HBM
-    # traffic would take a fifth of that time.
+    # The LoRA factors reduce over the rank (at most 64 entries): lin_short_kernel
+    # multiplies the entries' bytes on mma.sync and spends 72 wide multiply-adds
+    # per line on line sum x eq weight.  Bound: the 2 B per entry of HBM traffic;
+    # the multiply-adds at the derived ALU peak take about as long.
     lines = sum(len(st["mats"]) * max(st["mats"][0].shape) for st in stmts)
-    madw = 8 * entries + 64 * lines
+    madw = 72 * lines
     alu_peak = SMS * MADWIDE_PER_SM_CLK * SM_MAX_MHZ * 1e6
-    roof = {"bound": "alu", "kernel": "lin_short_kernel", "achieved": madw / (fold_ms / 1e3) / 1e12,
-            "peak": alu_peak / 1e12, "unit": "T mad.wide/s", "frac": madw / (fold_ms / 1e3) / alu_peak,
-            "traffic": None,
-            "peak_note": f"derived: {SMS} SMs x {MADWIDE_PER_SM_CLK} IMAD.WIDE/clk x {SM_MAX_MHZ} MHz",
-            "algorithmic_madwide_per_launch": madw,
-            "hbm": {"achieved_gbs": hbm_gbs, "peak_gbs": hbm_peak, "frac": hbm_gbs / hbm_peak,
-                    "algorithmic_bytes_per_launch": 2 * entries,
-                    "peak_note": f"{hbm_note} copy bandwidth (MEASURED_PEAKS.json hbm_gbs)"}}
+    roof = {"bound": "hbm", "kernel": "lin_short_kernel", "achieved": hbm_gbs, "peak": hbm_peak, "unit": "GB/s",
+            "frac": hbm_gbs / hbm_peak, "traffic": None,
+            "peak_note": f"{hbm_note} copy bandwidth (MEASURED_PEAKS.json hbm_gbs)",
+            "algorithmic_bytes_per_launch": 2 * entries,
+            "alu": {"achieved": madw / (fold_ms / 1e3) / 1e12, "peak": alu_peak / 1e12, "unit": "T mad.wide/s",
+                    "frac": madw / (fold_ms / 1e3) / alu_peak, "algorithmic_madwide_per_launch": madw,
+                    "peak_note": f"derived: {SMS} SMs x {MADWIDE_PER_SM_CLK} IMAD.WIDE/clk x {SM_MAX_MHZ} MHz"}}
     # End to end: pinned host operands in (staged by the library), host proofs out.
     host = [[torch.from_numpy(m).pin_memory() for m in st["mats"]] for st in stmts]
     hjobs = [B.lin_job([B.mat(t) for t in h], list(st["coeffs"]), st["seed"]) for h, st in zip(host, stmts)]
@@ -726,15 +725,17 @@ def lookups_main(args, rank, world, local, cpu):
     value = job_value(entries, world, ms_max / 1e3)
     # the sumcheck rounds: batched passes plus each proof's tail rounds
     rounds_ms = statistics.mean(p[1] + p[2] for p in phases)
-    # algorithmic field products of the rounds: per round and pair, 3 folds +
-    # 3 evaluation points x 2 products (9 per pair; sum over rounds 9 D), plus
-    # the eq(u, .) entry (1 per cube entry): 10 per cube entry
-    achieved = 10 * cube / (rounds_ms / 1e3)
+    # field products of the rounds per cube entry (a wide multiply-add sum counts
+    # half a product, a multiply by a 16-bit integer an eighth): round 1 0.4 on 1/2
+    # pair per entry, round 2 2.3 on 1/4, round 3 5.5 on 1/8, the later ones 7 on
+    # 1/8 together (the table side is left out)
+    products = (0.4 / 2 + 2.3 / 4 + 5.5 / 8 + 7 / 8) * cube
+    achieved = products / (rounds_ms / 1e3)
     roof = {"bound": "alu", "kernel": "lk_pass_kernel + lk_round_kernel + lk_tail_kernel (all rounds)",
             "achieved": achieved / 1e9,
             "peak": MONT_PEAK / 1e9, "unit": "G Montgomery products/s", "frac": achieved / MONT_PEAK,
             "traffic": None, "peak_note": "derived: 152 SMs x 32 IMAD.WIDE/clk x 2070 MHz / 128 per product",
-            "algorithmic_products_per_step": 10 * cube}
+            "algorithmic_products_per_step": products}
     host = [torch.from_numpy(np.ascontiguousarray(x["S"])).pin_memory() for x in looks]
     hjobs = [B.lookup_job(B.mat(h), x["t0"], x["log2_n"], x["seed"]) for h, x in zip(host, looks)]
     hplan = B.LookupPlan(hjobs)
