@@ -171,7 +171,7 @@ __global__ void __launch_bounds__(CH_EVAL_THREADS) chain_eval_kernel(ChainDev* c
   claim_point(C, q, &x, &y);
   const int16_t* rho = C.rho[q >> 1];
   const int64_t ld = C.rho_ld[q >> 1];
-  eq_factors(x, C.ln, C.n, false, y, C.lr, C.r, true, fac, sub);
+  eq_factors(x, C.ln, C.n, false, y, C.lr, C.r, true, fac, sub, (int)blockDim.x);
   if (tid < 32) {
     const Fr s = eq_prefix_sum(y, C.lr, C.r);
     const Fr c = mont_mul_ni(s, to_mont_ni(fr_small(1u << 15)));

@@ -150,7 +150,6 @@ __device__ void bt_step(BtState* B, RndShared& sh, int t, const Fr& g0, const Fr
 __global__ void __launch_bounds__(BT_THREADS) bt_start_kernel(BtState* B) {
   __shared__ RndShared sh;
   __shared__ uint32_t S0[8], S1[8];
-  __shared__ uint32_t dig[3][8];
   __shared__ Fr ch[1];
   __shared__ Fr red[3 * (BT_THREADS / 32)];
   bt_tree(B);
@@ -166,7 +165,7 @@ __global__ void __launch_bounds__(BT_THREADS) bt_start_kernel(BtState* B) {
     store_digest(S0, d);
   }
   __syncthreads();
-  squeeze_dev(S0, LBL_P, 1, ch, S1, dig);
+  squeeze_dev(S0, LBL_P, 1, ch, S1);
   const Fr rho = ch[0];
   Fr acc[3] = {fr_zero(), fr_zero(), fr_zero()};  // claim, g(0), G
   for (int i = threadIdx.x; i < B->K; i += blockDim.x) {

@@ -157,21 +157,6 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[32]) {
       : TC_R8(OFF), TC_R8(OFF + 8)
       : "r"(taddr));
 }
-// 32 columns into r[0 .. 31].
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
-      "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
-      : TC_R8(0), TC_R8(8), TC_R8(16), TC_R8(24)
-      : "r"(taddr));
-}
-// 8 columns into r[OFF .. OFF + 7].
-template <int OFF>
-__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&r)[32]) {
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-               : TC_R8(OFF)
-               : "r"(taddr));
-}
 #undef TC_R8
 // 1 column into r[OFF].
 template <int OFF>
@@ -248,10 +233,6 @@ __device__ __forceinline__ bool tc_wait(uint32_t bar, uint32_t parity, unsigned 
 // so the warp never splits before a .sync.aligned instruction.
 __device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity, unsigned long long wait_ns) {
   return __all_sync(0xffffffffu, tc_wait(bar, parity, wait_ns));
-}
-
-__device__ __forceinline__ uint32_t fbits_add(uint32_t a, uint32_t b) {
-  return __float_as_uint(__fadd_rn(__uint_as_float(a), __uint_as_float(b)));
 }
 
 // One pipeline stage as every role sees it (written by the producer).

@@ -29,8 +29,7 @@ constexpr int LIN_THREADS = 256;
 // One block per proof.
 __global__ void __launch_bounds__(LIN_THREADS) lin_start_kernel(LinDev* Ls) {
   LinDev* L = Ls + blockIdx.x;
-  __shared__ uint32_t S0[8], S1[8], S2[8];
-  __shared__ uint32_t dig[2 * MAX_VARS + 1][8];
+  __shared__ uint32_t S0[8], S2[8];
   __shared__ Fr xs[MAX_VARS], ys[MAX_VARS];
   __shared__ __align__(16) Fr sub[128];  // factor tables; before them the statement's message (at most 17 blocks)
   static_assert(sizeof(sub) >= 64 * ((23 + 20 + 64 * VL_LIN_MAX + 9 + 63) / 64), "message buffer");
@@ -49,11 +48,10 @@ __global__ void __launch_bounds__(LIN_THREADS) lin_start_kernel(LinDev* Ls) {
     store_digest(S0, d);
   }
   __syncthreads();
-  squeeze_dev(S0, LBL_X, L->d0, xs, S1, dig);
-  squeeze_dev(S1, LBL_Y, L->d1, ys, S2, dig);
+  squeeze2_dev(S0, LBL_X, L->d0, xs, LBL_Y, L->d1, ys, S2);
   if (tid < 8) L->S[tid] = S2[tid];
   const bool rr = L->red_rows != 0;
-  eq_factors(xs, L->d0, L->rows, rr, ys, L->d1, L->cols, !rr, L->fac, sub);
+  eq_factors(xs, L->d0, L->rows, rr, ys, L->d1, L->cols, !rr, L->fac, sub, LIN_THREADS);
   if (tid < 32) {
     const Fr sx = eq_prefix_sum(xs, L->d0, L->rows), sy = eq_prefix_sum(ys, L->d1, L->cols);
     const Fr corr = mont_mul_ni(rr ? sx : sy, to_mont_ni(fr_small(1u << 15)));

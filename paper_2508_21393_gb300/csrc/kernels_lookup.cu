@@ -56,13 +56,13 @@ __global__ void __launch_bounds__(LK_THREADS) lk_start_kernel(LkDev* Ls) {
     store_digest(S0, d);
   }
   __syncthreads();
-  squeeze_dev(S0, LBL_BETA, 1, ch, S1, dig);
+  squeeze_dev(S0, LBL_BETA, 1, ch, S1);
   if (tid == 0) beta_sh = ch[0];
   __syncthreads();
-  squeeze_dev(S1, LBL_ALPHA, 1, ch, S2, dig);
+  squeeze_dev(S1, LBL_ALPHA, 1, ch, S2);
   if (tid == 0) alpha_sh = ch[0];
   __syncthreads();
-  squeeze_dev(S2, LBL_U, L->L, ch, S3, dig);
+  squeeze_dev(S2, LBL_U, L->L, ch, S3);
   if (tid < L->L) L->u[tid] = ch[tid];
   if (tid < 8) L->run.St[tid] = S3[tid];
   if (tid == 0) {
@@ -571,8 +571,8 @@ __device__ void lk_finish(LkDev* L, LkShared& sh, vl_lookup_proof* out) {
 // (one fold each, then one product and one product by f).  The last warp forms
 // the claims and scalars of the next round, of 512 threads beside the pass of the
 // others, of 128 before its share.
-// In a cluster (CL) the rounds of at least RND_CL_PAIRS pairs are spread over its
-// CTAs as in rounds_cluster (CTA c owns the entries k with (k / 32) mod CTAs = c);
+// In a cluster (CL) the rounds of at least LK_CL_PAIRS pairs are spread over its
+// CTAs as in rounds_cluster (CTA c owns the entries k with (k / 8) mod CTAs = c);
 // the first CTA makes the transcript steps and, alone, the rounds after those.
 template <int THREADS, int MINB, bool CL>
 __global__ void __launch_bounds__(THREADS, MINB) lk_tail_kernel(LkDev* Ls, vl_lookup_proof* outs) {
@@ -591,10 +591,10 @@ __global__ void __launch_bounds__(THREADS, MINB) lk_tail_kernel(LkDev* Ls, vl_lo
   if (CL) cluster_sync();  // every CTA has started: its shared memory may be written
   for (int t = L->tail; t <= L->L; t++) {
     const int h = 1 << (L->L - t);
-    const bool spread = CL && h >= RND_CL_PAIRS;
+    const bool spread = CL && h >= LK_CL_PAIRS;
     if (CL && !spread && rank > 0) return;
     const int own = spread ? h / C : h;  // this CTA's pairs
-    auto pair = [&](int l) { return spread ? ((l >> 5) * C + rank) * 32 + (l & 31) : l; };
+    auto pair = [&](int l) { return spread ? ((l >> 3) * C + rank) * 8 + (l & 7) : l; };
     const int tj = t - (L->L - L->log2_n);
     const bool jr = tj > 0;
     if (t > L->tail) {
@@ -757,7 +757,7 @@ __global__ void __launch_bounds__(THREADS, MINB) lk_tail_kernel(LkDev* Ls, vl_lo
       if (warp == 0) lk_step_g(L, sh, t, tj, qform, out);
       lk_transcript(L, sh, warp, t);
     }
-    if (spread && (h >> 1) >= RND_CL_PAIRS) {
+    if (spread && (h >> 1) >= LK_CL_PAIRS) {
       // the other CTAs need r_t and T''s offset
       if (rank == 0 && warp == 0) {
         __syncwarp();

@@ -35,6 +35,7 @@ namespace {
 constexpr uint8_t LBL_BETA = 'b', LBL_ALPHA = 'a';
 constexpr int LK_STEP_THREADS = 128;  // transcript step: its message schedules take warps 1 to 3
 constexpr int LK_MAX_WARPS = 16;
+constexpr int LK_CL_PAIRS = 8 * RND_MAX_CTAS;  // pairs of a round spread over a cluster, at least
 
 __device__ __forceinline__ int lk_table_index(const LkDev& L, int k) {
   if (k >= L.n) return 0;  // padding entries hold t0

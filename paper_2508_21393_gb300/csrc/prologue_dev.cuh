@@ -92,57 +92,78 @@ __device__ static Fr build_eq(const Fr* x, int d, int size, int tabs, Fr* out, u
   return mont_mul_ni(sum[0], fr_small(1u << 15));
 }
 
+// The challenge halves of a squeeze: thread i of n = 2 count (whole warps from a
+// multiple of 32 on; lanes past n may take part) holds half i & 1 of challenge
+// i >> 1 as a digest; even threads write the challenges (Montgomery) to x:
+// challenge i = (lo + hi . 2^256) mod r in Montgomery form = REDC(lo . R^2) +
+// REDC(hi . R^3) by two lanes at once, then one addition.
+__device__ __forceinline__ void squeeze_store(const uint32_t (&d)[8], int i, int n, Fr* x) {
+  const Fr part = mont_mul_ni(digest_le(d), (i & 1) ? fr_r3() : fr_r2());
+  const Fr other = shfl_xor_fr(part, 1);
+  if (i < n && !(i & 1)) x[i >> 1] = fr_add(part, other);
+}
+
 // Squeeze `count` challenges with `label` from the state Sw (big-endian
 // words): thread 2t + h hashes half h of challenge t, thread 2 count the
 // closing update.  Writes the challenges (Montgomery) to x and the new state
-// to Sn.  Block-wide (two barriers).
-__device__ static void squeeze_dev(const uint32_t* Sw, uint32_t label, int count, Fr* x, uint32_t* Sn,
-                                   uint32_t (*dig)[8]) {
+// to Sn.  Block-wide (one barrier).
+__device__ static void squeeze_dev(const uint32_t* Sw, uint32_t label, int count, Fr* x, uint32_t* Sn) {
   const int tid = threadIdx.x;
-  if (tid <= 2 * count) {
+  if ((tid & ~31) <= 2 * count) {
     uint32_t st[8], d[8];
 #pragma unroll
     for (int i = 0; i < 8; i++) st[i] = Sw[i];
-    if (tid < 2 * count) {
-      dev_squeeze_block(st, label, (uint32_t)(tid >> 1), tid & 1, d);
-#pragma unroll
-      for (int i = 0; i < 8; i++) dig[tid][i] = d[i];
-    } else {
-      dev_squeeze_block(st, label, (uint32_t)count, 2, d);
+    const bool half = tid < 2 * count;
+    dev_squeeze_block(st, label, (uint32_t)(half ? tid >> 1 : count), half ? tid & 1 : 2, d);
+    if (tid == 2 * count) {
 #pragma unroll
       for (int i = 0; i < 8; i++) Sn[i] = d[i];
     }
+    squeeze_store(d, tid, 2 * count, x);
   }
   __syncthreads();
-  // challenge i = (lo + hi . 2^256) mod r in Montgomery form (lo = digest 2i,
-  // hi = digest 2i + 1) = lo . R + hi . R^2: REDC(lo . R^2) and REDC(hi . R^3)
-  // by two threads at once, then one addition
-  Fr part;
-  if (tid < 2 * count) part = mont_mul_ni(digest_le(dig[tid]), (tid & 1) ? fr_r3() : fr_r2());
-  __syncthreads();
-  if (tid < 2 * count) {
+}
+
+// Two squeezes in a row, na challenges x with label la, then nb challenges y with
+// lb (at most 31 each): the threads of the second, from thread 64 on, each form
+// the state between the two for themselves, so the chain is two compressions
+// and one product.  Block-wide (at least 128 threads, one barrier).
+__device__ static void squeeze2_dev(const uint32_t* Sw, uint32_t la, int na, Fr* x, uint32_t lb, int nb, Fr* y,
+                                    uint32_t* Sn) {
+  const int tid = threadIdx.x, i = tid & 63;
+  const bool second = tid >= 64;
+  if (tid < 128 && (i & ~31) <= 2 * (second ? nb : na)) {
+    uint32_t st[8], d[8];
 #pragma unroll
-    for (int i = 0; i < 8; i++) dig[tid][i] = part.v[i];
-  }
-  __syncthreads();
-  if (tid < count) {
-    Fr lo, hi;
+    for (int q = 0; q < 8; q++) st[q] = Sw[q];
+    if (second) {
+      dev_squeeze_block(st, la, (uint32_t)na, 2, d);
 #pragma unroll
-    for (int i = 0; i < 8; i++) {
-      lo.v[i] = dig[2 * tid][i];
-      hi.v[i] = dig[2 * tid + 1][i];
+      for (int q = 0; q < 8; q++) st[q] = d[q];
     }
-    x[tid] = fr_add(lo, hi);
+    const int n = second ? nb : na;
+    const bool half = i < 2 * n;
+    dev_squeeze_block(st, second ? lb : la, (uint32_t)(half ? i >> 1 : n), half ? i & 1 : 2, d);
+    if (second && i == 2 * n) {
+#pragma unroll
+      for (int q = 0; q < 8; q++) Sn[q] = d[q];
+    }
+    squeeze_store(d, i, 2 * n, second ? y : x);
   }
   __syncthreads();
 }
 
 // Transcript start and the squeezes of u, v into shared memory, or, for a
 // proof with a given point, the given start state and point; the state after
-// them goes to P.scr->state.  Block-wide.
-// msg: 192 bytes of scratch.
-__device__ static void start_or_given(const DevProof& P, uint32_t* S0, uint32_t* S1, uint32_t* S2,
-                                      uint32_t (*dig)[8], Fr* u, Fr* v, void* msg) {
+// them goes to P.scr->state.  Block-wide (at least 128 threads); S0: 24 words;
+// msg: START_SCRATCH bytes of scratch.  JOIN, the shorter chain for a block with
+// an SM's issue slots to itself: warp 0 runs the rounds of the start's three
+// blocks, warps 1 to 3 a schedule each, and both squeezes run at once.  Else
+// the fewer instructions: one warp hashes, one squeeze after the other.
+static constexpr int START_SCRATCH = 192 + 3 * 68 * 4;
+template <bool JOIN>
+__device__ static void start_or_given(const DevProof& P, uint32_t* S0, Fr* u, Fr* v, void* msg) {
+  uint32_t* S2 = S0 + 16;
   const int tid = threadIdx.x;
   if (P.given) {
     for (int i = tid; i < P.d0 + P.d2; i += blockDim.x) {
@@ -153,7 +174,9 @@ __device__ static void start_or_given(const DevProof& P, uint32_t* S0, uint32_t*
     __syncthreads();
     return;
   }
-  if (tid < 32) {
+  const int warp = tid >> 5;
+  uint32_t(*wk)[68] = reinterpret_cast<uint32_t(*)[68]>(static_cast<uint8_t*>(msg) + 192);
+  if (warp == 0) {
     // the message of ts_start (a product of a batch: of ts_start_member)
     WarpMsg h(msg);
     if (P.member1 > 0) h.bytes("verilora-gb300/zkbatch/v1/member", 32);
@@ -169,13 +192,30 @@ __device__ static void start_or_given(const DevProof& P, uint32_t* S0, uint32_t*
     h.byte((uint32_t)(P.tp & 1));
     h.byte((uint32_t)(P.tq & 1));
     h.bytes(P.binds, 96);
-    uint32_t d[8];
-    h.hash(d);
-    store_digest(S0, d);
+    if (JOIN) {
+      h.pad();  // 141 or 158 bytes: three blocks
+      named_sync(10, 128);
+      ShaState st = sha_iv_state();
+#pragma unroll 1
+      for (int b = 0; b < 3; b++) st = sha_rounds_ni(st, h.block(b), wk[b], 1 + 3 * b);
+      store_digest(S0, st.h);
+    } else {
+      uint32_t d[8];
+      h.hash(d);
+      store_digest(S0, d);
+    }
+  } else if (JOIN && warp < 4) {
+    named_sync(10, 128);
+    WarpMsg h(msg);
+    sha_sched_ni(h.block(warp - 1), wk[warp - 1], 1 + 3 * (warp - 1));
   }
   __syncthreads();
-  squeeze_dev(S0, LBL_U, P.d0, u, S1, dig);
-  squeeze_dev(S1, LBL_V, P.d2, v, S2, dig);
+  if (JOIN) {
+    squeeze2_dev(S0, LBL_U, P.d0, u, LBL_V, P.d2, v, S2);
+  } else {
+    squeeze_dev(S0, LBL_U, P.d0, u, S0 + 8);
+    squeeze_dev(S0 + 8, LBL_V, P.d2, v, S2);
+  }
   if (tid < 32) P.scr->state[tid] = (uint8_t)(S2[tid >> 2] >> (24 - 8 * (tid & 3)));
 }
 
@@ -183,12 +223,9 @@ __device__ static void start_or_given(const DevProof& P, uint32_t* S0, uint32_t*
 static_assert(PRO_SMEM == 128 + 2 * MAX_VARS * 32 + 2 * MAX_VARS * 32 + 2 * MAX_HALF * 32 + 8 * 32, "layout");
 
 // Prologue of one proof by the whole block (any multiple of 32 threads, at
-// least 64): transcript start, squeezes of u and v, eq tables, corrections.
+// least 128): transcript start, squeezes of u and v, eq tables, corrections.
 static __device__ void prologue_block(const DevProof& P, uint8_t* smem) {
   uint32_t* S0 = reinterpret_cast<uint32_t*>(smem);
-  uint32_t* S1 = S0 + 8;
-  uint32_t* S2 = S0 + 16;
-  uint32_t(*dig)[8] = reinterpret_cast<uint32_t(*)[8]>(smem + 128);
   Fr* u = reinterpret_cast<Fr*>(smem + 128 + 2 * MAX_VARS * 32);
   Fr* v = u + MAX_VARS;
   Fr* lo = v + MAX_VARS;
@@ -196,7 +233,7 @@ static __device__ void prologue_block(const DevProof& P, uint8_t* smem) {
   Fr* red = hi + MAX_HALF;
   const int tid = threadIdx.x;
 
-  start_or_given(P, S0, S1, S2, dig, u, v, v + MAX_VARS);
+  start_or_given<true>(P, S0, u, v, v + MAX_VARS);
 
   Fr ca = build_eq(u, P.d0, P.m, P.tabA, P.eqA, P.eqA_soa, P.soa_pitchA, P.w8A, lo, hi, red);
   __syncthreads();
@@ -218,11 +255,12 @@ static __device__ void prologue_block(const DevProof& P, uint8_t* smem) {
 // once more into two of at most 4: 8 small tables of at most 16 entries, one
 // entry per thread (four products on a thread's chain), then one product per
 // factor entry, instead of one chain of up to eight products per entry.
-// sub: 128 entries of shared memory.
+// sub: 128 entries of shared memory.  By the block's first n threads (whole warps;
+// barrier 11).
 __device__ static void eq_factors(const Fr* x, int dx, int sizex, bool dblx, const Fr* y, int dy, int sizey, bool dbly,
-                                  Fr* fac, Fr* sub) {
+                                  Fr* fac, Fr* sub, int n_threads) {
   const int tid = threadIdx.x;
-  for (int e = tid; e < 128; e += blockDim.x) {
+  for (int e = tid; e < 128; e += n_threads) {
     const int q = e >> 4, j = e & 15;  // q: side, hi block, low half
     const bool second = q & 4;
     const int d = second ? dy : dx, s = (d + 1) >> 1;
@@ -241,10 +279,10 @@ __device__ static void eq_factors(const Fr* x, int dx, int sizex, bool dblx, con
       sub[e] = acc;
     }
   }
-  __syncthreads();
+  named_sync(11, n_threads);
   const int sx = (dx + 1) >> 1, sy = (dy + 1) >> 1;
   const int lx = 1 << sx, hx = (sizex + lx - 1) >> sx, ly = 1 << sy, hy = (sizey + ly - 1) >> sy;
-  for (int e = tid; e < lx + hx + ly + hy; e += blockDim.x) {
+  for (int e = tid; e < lx + hx + ly + hy; e += n_threads) {
     const bool second = e >= lx + hx;
     const int e2 = second ? e - (lx + hx) : e, nlo = second ? ly : lx;
     const bool hi = e2 >= nlo;
@@ -284,32 +322,35 @@ __device__ static Fr eq_prefix_sum(const Fr* x, int d, int size) {
   return warp_sum_fr(one ? term : fr_zero());
 }
 
-// First launch of the prologue, one proof per block (any multiple of 32
-// threads, at least 64): transcript start, squeezes of u and v, the factor
-// tables of both eq tables (to P.fac) and the offset corrections
-// 2^15 . sum_i E[i] (Montgomery).
+// Offset correction 2^15 . sum_i E[i] (Montgomery) of one side, by one warp.
+__device__ static void prologue_corr(const DevProof& P, const Fr* u, const Fr* v, bool a) {
+  const Fr c = to_mont_ni(fr_small(1u << 15));
+  // sum . R times 2^15 . R, reduced once: 2^15 . sum (Montgomery)
+  const Fr corr = mont_mul_ni(a ? eq_prefix_sum(u, P.d0, P.m) : eq_prefix_sum(v, P.d2, P.n), c);
+  if ((threadIdx.x & 31) == 0) {
+    const bool i16 = (a ? P.dtypeA : P.dtypeB) == VL_I16;
+    (a ? P.scr->corrA : P.scr->corrB) = i16 ? corr : fr_zero();
+  }
+}
+
+// First launch of the prologue, one proof per block of THREADS (128 or 192):
+// transcript start, squeezes of u and v, then the factor tables of both eq tables
+// (to P.fac; four warps) and the offset corrections (one warp each; of 192
+// threads beside the factors).  A chain: three and two compressions, the factors'
+// five products or the corrections' seven.
+template <int THREADS>
 static __device__ void transcript_block(const DevProof& P, uint8_t* smem) {
   uint32_t* S0 = reinterpret_cast<uint32_t*>(smem);
-  uint32_t* S1 = S0 + 8;
-  uint32_t* S2 = S0 + 16;
-  uint32_t(*dig)[8] = reinterpret_cast<uint32_t(*)[8]>(smem + 128);
   Fr* u = reinterpret_cast<Fr*>(smem + 128 + 2 * MAX_VARS * 32);
   Fr* v = u + MAX_VARS;
-  const int tid = threadIdx.x;
-  start_or_given(P, S0, S1, S2, dig, u, v, v + MAX_VARS);
-  eq_factors(u, P.d0, P.m, true, v, P.d2, P.n, true, P.fac, v + MAX_VARS);
-  if (tid < 64) {
-    const bool a = tid < 32;
-    const Fr sum = a ? eq_prefix_sum(u, P.d0, P.m) : eq_prefix_sum(v, P.d2, P.n);
-    if ((tid & 31) == 0) {
-      // sum . R times 2^15 . R, reduced once: 2^15 . sum (Montgomery)
-      const Fr corr = mont_mul_ni(sum, to_mont_ni(fr_small(1u << 15)));
-      const bool i16 = (a ? P.dtypeA : P.dtypeB) == VL_I16;
-      (a ? P.scr->corrA : P.scr->corrB) = i16 ? corr : fr_zero();
-    }
+  const int warp = threadIdx.x >> 5;
+  constexpr int CORR = THREADS >= 192 ? 4 : 0;  // first of the two warps of the corrections
+  start_or_given<(THREADS >= 192)>(P, S0, u, v, v + MAX_VARS);
+  if (warp < 4) {
+    eq_factors(u, P.d0, P.m, true, v, P.d2, P.n, true, P.fac, v + MAX_VARS, 128);
+    if (threadIdx.x == 0) P.scr->status = VL_OK;
   }
-  if (tid == 0) P.scr->status = VL_OK;
-  __syncthreads();
+  if (warp == CORR || warp == CORR + 1) prologue_corr(P, u, v, warp == CORR);
 }
 
 // Second launch: entries [i0, i1) of one eq table, E[i] = hi[i >> s] . lo[i

@@ -322,21 +322,31 @@ struct WarpMsg {
     buf[len + lane] = (uint8_t)(S[lane >> 2] >> (24 - 8 * (lane & 3)));
     len += 32;
   }
-  // The digest (big-endian words); the buffer may be reused afterwards.
-  __device__ void hash(uint32_t (&out)[8]) {
+  // Padding and length; the number of bytes then (whole blocks).
+  __device__ int pad() {
     const int end = (len + 9 + 63) / 64 * 64;
     for (int i = len + (int)(threadIdx.x & 31); i < end; i += 32)
       buf[i] = i == len ? 0x80 : i >= end - 4 ? (uint8_t)((uint32_t)(len * 8) >> (8 * (end - 1 - i))) : 0;
     __syncwarp();
-    sha256_iv(out);
-    for (int b = 0; b < end; b += 64) {
-      uint32_t m[16];
+    return end;
+  }
+  // Block b of the padded message.
+  __device__ ShaBlock block(int b) const {
+    ShaBlock m;
 #pragma unroll
-      for (int q = 0; q < 4; q++) {
-        const uint4 v = reinterpret_cast<const uint4*>(buf + b)[q];
-        m[4 * q] = bswap32(v.x), m[4 * q + 1] = bswap32(v.y), m[4 * q + 2] = bswap32(v.z), m[4 * q + 3] = bswap32(v.w);
-      }
-      sha256_block(out, m);
+    for (int q = 0; q < 4; q++) {
+      const uint4 v = reinterpret_cast<const uint4*>(buf + 64 * b)[q];
+      m.w[4 * q] = bswap32(v.x), m.w[4 * q + 1] = bswap32(v.y), m.w[4 * q + 2] = bswap32(v.z), m.w[4 * q + 3] = bswap32(v.w);
+    }
+    return m;
+  }
+  // The digest (big-endian words); the buffer may be reused afterwards.
+  __device__ void hash(uint32_t (&out)[8]) {
+    const int n = pad() / 64;
+    sha256_iv(out);
+    for (int b = 0; b < n; b++) {
+      const ShaBlock m = block(b);
+      sha256_block(out, m.w);
     }
     __syncwarp();
   }

@@ -56,7 +56,7 @@ def test_rounds_at_every_vector_length(k):
         assert _prove([job], o) == [want], (variant, threads)
 
 
-@pytest.mark.parametrize("count", [19, 20, 38, 39, 76, 77, 152, 153, 304, 305])
+@pytest.mark.parametrize("count", [19, 20, 38, 39, 76, 77, 152, 153, 304, 305, 608, 609])
 def test_rounds_threads_by_number_of_proofs(count):
     rng = np.random.default_rng(count)
     ks = [1, 2, 7, 16, 40, 129, 300, 600, 5000]
