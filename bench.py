@@ -1214,22 +1214,24 @@ def main():
                 "frac": achieved / peak, "traffic": None, "hbm_gbs_algorithmic": hbm_gbs,
                 "peak_note": "152 SMs x 32 IMAD.WIDE/clk x 2070 MHz (derived)"}
     else:
-        # Tensor-core fold: streams every operand entry once from HBM.
+        # Tensor-core fold: every operand matrix must come from HBM once; several
+        # products of a projection fold the same matrix, and their further reads
+        # (2 B per fold entry in all) go through L2.
         kernel, phase_ms = "fold_tc_kernel", {"clear+prologue": pro_ms, "fold": fold_ms, "rounds": rnd_ms}
         # 64 fp16 MACs per entry (two bytes x 32 weight bytes) plus the two
         # constant MMAs of each 128-entry stage (2 x 128 x 32 x 16 MACs per
         # 128 x 128 entries: 8 per entry)
         tflops = 2 * (64 + 8) * entries / (fold_ms / 1e3) / 1e12
         # DRAM traffic per launch: ncu capture of the same kernel on the first
-        # two layers (profiles/fold_tc_kernel_7b_2layers.md), 444.4 MB for 750 MB
-        # algorithmic, scaled by entries (the tile mix repeats per projection).
-        traffic = 0.5926 * 2 * entries if args.workload == "7b-step" else None
-        roof = {"bound": "hbm", "kernel": kernel, "achieved": hbm_gbs, "peak": hbm_peak, "unit": "GB/s",
-                "frac": hbm_gbs / hbm_peak, "traffic": traffic,
+        # two layers (profiles/fold_tc_kernel_7b_2layers.md), 442 MB for 750 MB of
+        # operand reads, scaled by entries (the tile mix repeats per projection).
+        traffic = 0.589 * 2 * entries if args.workload == "7b-step" else None
+        unique_gbs = in_bytes / (fold_ms / 1e3) / 1e9
+        roof = {"bound": "hbm", "kernel": kernel, "achieved": unique_gbs, "peak": hbm_peak, "unit": "GB/s",
+                "frac": unique_gbs / hbm_peak, "traffic": traffic,
                 "peak_note": f"{hbm_note} copy bandwidth (MEASURED_PEAKS.json hbm_gbs)",
-                "algorithmic_bytes_per_launch": 2 * entries,
-                "unique_input_bytes": in_bytes,
-                "frac_of_unique_bytes": in_bytes / (fold_ms / 1e3) / 1e9 / hbm_peak,
+                "algorithmic_bytes_per_launch": in_bytes,
+                "operand_reads": {"bytes_per_launch": 2 * entries, "gbs": hbm_gbs},
                 "tensor_tflops_fp16": tflops}
     rounds_roof = rounds_bound(jobs, rnd_ms)
 

@@ -289,7 +289,7 @@ __global__ void __launch_bounds__(32) bt_final_kernel(const DevProof* dp, BtStat
 // i = c (mod CTAs), four lanes per pair, so no vector entry changes hands; the
 // sums go to the first CTA, which makes the transcript step, and the challenge
 // comes back (as in rounds_cluster).  A round this short is latency, about 16 us as
-// a launch of its own: 256 products of a 7B model 773 -> 762 us (from 8192 pairs
+// a launch of its own: 128 products of a 7B model 773 -> 762 us (from 8192 pairs
 // on, with twice the products per pair of bt_round_kernel's loop, 794).
 __global__ void __launch_bounds__(BT_TAIL_THREADS, 1) bt_tail_kernel(const DevProof* dp, BtState* B, int t0) {
   __shared__ RndShared sh;

@@ -103,7 +103,7 @@ static __device__ __noinline__ void sha_sched_ni(ShaBlock m, uint32_t* wk, int b
 }
 // The rounds as a loop over 16: its body fits the instruction cache beside what
 // the other warps run (unrolled over 64, the first compression after other code
-// took 2700 to 3400 cycles against 2050 for the next: 7B step 2.03 -> 2.00 ms, 256
+// took 2700 to 3400 cycles against 2050 for the next: 7B step 2.03 -> 2.00 ms, 128
 // batched claims 762 -> 742 us).
 static __device__ __noinline__ ShaState sha_rounds_ni(ShaState st, ShaBlock m, const uint32_t* wk, int bar) {
   uint32_t a = st.h[0], b = st.h[1], c = st.h[2], d = st.h[3], e = st.h[4], f = st.h[5], g = st.h[6], h = st.h[7];
