@@ -334,6 +334,7 @@ struct LkDev {
   Fr* Tb;                          // beta + t0 + j, N (gather source)
   Fr* WB; Fr* WM;                  // table side: B, m (folded in place)
   Fr* UB; Fr* VB;                  // (1 - r_1) B, r_1 B, N each (round2)
+  uint16_t* idx;                   // table index of every cube entry (padding: 0)
   Fr* VA; Fr* VS;                  // folded A and S + beta, D/2 each
   uint32_t* counts;                // N multiplicities
   Fr* part;                        // partial sums (LK_PART per slot)

@@ -103,44 +103,47 @@ __global__ void __launch_bounds__(LK_THREADS) lk_start_kernel(LkDev* Ls) {
   }
 }
 
-// Multiplicities of entries [k0, k1) of S; a value outside the table marks
-// the proof VL_ELOOKUP.  Tables up to 4096 entries count in shared memory.
+// Multiplicities and table indices of cube entries [k0, k1): S's entries, then the
+// padding (index 0, counted by lk_start_kernel).  A value outside the table marks
+// the proof VL_ELOOKUP (its index is clamped).  Tables up to 4096 entries count in
+// shared memory.
 __global__ void __launch_bounds__(LK_THREADS) lk_hist_kernel(LkDev* Ls, const LkItem* items) {
   __shared__ uint32_t h[4096];
   const LkItem it = items[blockIdx.x];
   LkDev* L = Ls + it.proof;
-  const int N = 1 << L->log2_n;
+  const int N = 1 << L->log2_n, end = min(it.k1, L->n);
   const bool local = N <= 4096;
+  uint16_t* idx = L->idx;
   if (local)
     for (int j = threadIdx.x; j < N; j += blockDim.x) h[j] = 0;
   __syncthreads();
   bool bad = false;
-  auto count = [&](int64_t v) {
+  auto count = [&](int k, int64_t v) {
     const int64_t j = v - L->t0;
-    if (j < 0 || j >= N) {
-      bad = true;
-      return;
-    }
-    if (local) atomicAdd(&h[j], 1u);
+    const bool in = j >= 0 && j < N;
+    idx[k] = (uint16_t)(in ? j : j < 0 ? 0 : N - 1);
+    if (!in) bad = true;
+    else if (local) atomicAdd(&h[j], 1u);
     else atomicAdd(&L->counts[j], 1u);
   };
+  int k = it.k0 + threadIdx.x;
   if (L->dense) {
     const int16_t* S = L->S;
-    int k = it.k0 + threadIdx.x;
-    for (; k + 3 * (int)blockDim.x < it.k1; k += 4 * blockDim.x) {  // four loads in flight
+    for (; k + 3 * (int)blockDim.x < end; k += 4 * blockDim.x) {  // four loads in flight
       int16_t v[4];
 #pragma unroll
       for (int i = 0; i < 4; i++) v[i] = S[k + i * (int)blockDim.x];
 #pragma unroll
-      for (int i = 0; i < 4; i++) count(v[i]);
+      for (int i = 0; i < 4; i++) count(k + i * (int)blockDim.x, v[i]);
     }
-    for (; k < it.k1; k += blockDim.x) count(S[k]);
+    for (; k < end; k += blockDim.x) count(k, S[k]);
   } else {
-    for (int k = it.k0 + threadIdx.x; k < it.k1; k += blockDim.x) {
+    for (; k < end; k += blockDim.x) {
       const int row = k / (int)L->cols, col = k - row * (int)L->cols;
-      count(L->S[(int64_t)row * L->ld + col]);
+      count(k, L->S[(int64_t)row * L->ld + col]);
     }
   }
+  for (; k < it.k1; k += blockDim.x) idx[k] = 0;
   if (bad) atomicExch(&L->scr->status, VL_ELOOKUP);
   __syncthreads();
   if (local)
@@ -216,7 +219,7 @@ __global__ void __launch_bounds__(LK_THREADS, 2) lk_table_kernel(LkDev* Ls, cons
 
 // The tables of round 2 (entries of a table item): UB = (1 - r_1) B, VB = r_1 B.
 // One product per entry (51 us for the 512 lookups of a 7B step) against two per
-// pair: with S' left to round 3, round 2's pass took 1068 us, now 892.
+// pair: with S' left to round 3, round 2's pass went from 1068 us to 892.
 __global__ void __launch_bounds__(LK_THREADS) lk_tables2_kernel(LkDev* Ls, const LkItem* items) {
   const LkItem it = items[blockIdx.x];
   LkDev* L = Ls + it.proof;
@@ -799,7 +802,7 @@ cudaError_t launch_lookup_round(LkDev* Ls, int np, int t, const LkItem* items, i
 // A proof's tail is a chain of rounds: with SMs to spare it runs on a cluster of 8,
 // 4 or 2 CTAs (one lookup of 512 x 16 remainders 423 -> 355 us, its tail now from
 // 2^LK_TAIL_LOG_FEW pairs), with an SM for every proof on 512 threads, else on 128, four proofs per SM (one lookup of 512 x 16 remainders
-// 0.98 -> 0.42 ms, the 512 of a 7B step 8.86 -> 4.13 ms with the other changes
+// 0.98 -> 0.42 ms, the 512 of a 7B step 8.86 -> 3.69 ms with the other changes
 // described in lookup_dev.cuh).
 cudaError_t launch_lookup_finish(LkDev* Ls, int np, vl_lookup_proof* out, cudaStream_t st) {
   int dev = 0, sms = 0;

@@ -45,7 +45,7 @@ int check_job(const vl_lookup_job& J) {
 }
 
 struct LkBufs {
-  size_t lop = 0, hip = 0, binv = 0, tb = 0, wb = 0, wm = 0, ub = 0, vb = 0, va = 0, vs = 0, counts = 0, stage = 0;
+  size_t lop = 0, hip = 0, binv = 0, tb = 0, wb = 0, wm = 0, ub = 0, vb = 0, idx = 0, va = 0, vs = 0, counts = 0, stage = 0;
 };
 
 int cuda_fail(const char* where, cudaError_t e) {
@@ -117,7 +117,8 @@ int lk_build(vl_lookup_plan* P, const vl_lookup_job* jobs, int32_t njobs) {
     P->tables2 = P->tables2 || L.round2;
     P->maxL = std::max(P->maxL, L.L);
     const int N = 1 << L.log2_n;
-    for (int k0 = 0; k0 < L.n; k0 += LK_HIST) P->hist.push_back(LkItem{i, k0, std::min(L.n, k0 + LK_HIST), 0});
+    const int D = 1 << L.L;
+    for (int k0 = 0; k0 < D; k0 += LK_HIST) P->hist.push_back(LkItem{i, k0, std::min(D, k0 + LK_HIST), 0});
     L.xbeg = slot;
     for (int k0 = 0; k0 < N; k0 += LK_ENTRIES) P->tab.push_back(LkItem{i, k0, std::min(N, k0 + LK_ENTRIES), slot++});
     L.xend = slot;
@@ -189,6 +190,7 @@ int lk_build(vl_lookup_plan* P, const vl_lookup_job* jobs, int32_t njobs) {
       b.ub = take(sizeof(Fr) * N);
       b.vb = take(sizeof(Fr) * N);
     }
+    b.idx = take(sizeof(uint16_t) << L.L);
     b.va = take(sizeof(Fr) * half);
     b.vs = take(sizeof(Fr) * half);
     if (jobs[i].S.space == VL_HOST) b.stage = take(sizeof(int16_t) * (size_t)L.n);
@@ -212,6 +214,7 @@ int lk_bind(vl_lookup_plan* P, uint8_t* ws, cudaStream_t st) {
     L.WM = reinterpret_cast<Fr*>(ws + b.wm);
     L.UB = L.round2 ? reinterpret_cast<Fr*>(ws + b.ub) : nullptr;
     L.VB = L.round2 ? reinterpret_cast<Fr*>(ws + b.vb) : nullptr;
+    L.idx = reinterpret_cast<uint16_t*>(ws + b.idx);
     L.VA = reinterpret_cast<Fr*>(ws + b.va);
     L.VS = reinterpret_cast<Fr*>(ws + b.vs);
     L.counts = reinterpret_cast<uint32_t*>(ws + P->off_counts + b.counts);
