@@ -137,11 +137,11 @@ __device__ void bt_step(BtState* B, RndShared& sh, int t, const Fr& g0, const Fr
   if (tid == 0) sh.claim = B->claim;
   __syncthreads();
   if (warp == 0) bt_message(B, sh, t, g0, G);
-  transcript_step(sh, warp, false, &B->r[t - 1]);
+  transcript_step(sh, warp, t, false, &B->r[t - 1]);
   __syncthreads();
   if (tid < 8) B->St[tid] = sh.S[tid];
   if (tid == 0) {
-    next_claim(sh);
+    next_claim(sh, t);
     B->claim = sh.claim;
   }
 }
@@ -299,13 +299,13 @@ __global__ void __launch_bounds__(BT_TAIL_THREADS, 1) bt_tail_kernel(const DevPr
   if (tid < 8) {
     sh.S[tid] = B->St[tid];
     sh.claim.v[tid] = B->claim.v[tid];
-    sh.r.v[tid] = d1 > 0 ? B->r[t0 - 2].v[tid] : 0u;
+    sh.r[(t0 - 1) & 1].v[tid] = d1 > 0 ? B->r[t0 - 2].v[tid] : 0u;
   }
   cluster_sync();
   for (int t = t0; t <= d1; t++) {
     const int lg = d1 - t, hh = 1 << lg, h = 2 * hh;
-    const Fr r = sh.r;
-    if (rank == 0 && t > t0 && warp == last && lane == 0) next_claim(sh);
+    const Fr r = sh.r[(t - 1) & 1];
+    if (rank == 0 && t > t0 && warp == last && lane == 0) next_claim(sh, t - 1);
     Fr acc = fr_zero();
     for (int b = 0; b < np << lg; b += BT_TAIL_THREADS / 4) {
       const int e = b + (tid >> 2);
@@ -341,15 +341,16 @@ __global__ void __launch_bounds__(BT_TAIL_THREADS, 1) bt_tail_kernel(const DevPr
         for (int off = 4; off < 32; off <<= 1) v = fr_add(v, shfl_xor_fr(v, off));
         bt_message(B, sh, t, shfl_fr(v, 0), shfl_fr(v, 1));
       }
-      transcript_step(sh, warp, false, &B->r[t - 1]);
+      transcript_step(sh, warp, t, false, &B->r[t - 1]);
       if (warp == 0) {
         __syncwarp();
-        for (int i = lane; i < 8 * (C - 1); i += 32) st_cluster(&sh.r.v[i & 7], 1 + (i >> 3), sh.r.v[i & 7]);
+        const Fr& rt = sh.r[t & 1];
+        for (int i = lane; i < 8 * (C - 1); i += 32) st_cluster(&rt.v[i & 7], 1 + (i >> 3), rt.v[i & 7]);
       }
     }
     cluster_sync();
   }
-  for (int i = warp; i < np; i += BT_TAIL_THREADS / 32) bt_final(dp[rank + C * i], B, sh.r);
+  for (int i = warp; i < np; i += BT_TAIL_THREADS / 32) bt_final(dp[rank + C * i], B, sh.r[d1 & 1]);
   if (rank == 0 && tid < 8) B->St[tid] = sh.S[tid];
 }
 

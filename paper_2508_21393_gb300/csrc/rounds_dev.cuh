@@ -29,7 +29,10 @@
 //    g(0) and G of round i + 1 are quadratics in r_i, as are the claim and g(2), and
 //    other warps sum their coefficients from the unfolded vectors while warps 0
 //    to 2 hash.  From the challenge to the next message are two products then,
-//    and the fold with r_i runs beside the next hash (look_terms);
+//    and the fold with r_i runs beside the next hash (look_terms).  So r_i is read
+//    while r_(i+1) is made, by warps that meet the hash's warps only at the block
+//    barrier that ends each transcript step: odd and even rounds have a slot each,
+//    and between a slot's last read and its next write lies the other slot's barrier;
 //  * the transcript runs on warps 0 to 2: the rounds of each SHA-256
 //    compression on warp 0, its message schedule on warp 1 (of an absorb's
 //    second block: on warp 2); the two halves of the challenge and the
@@ -54,7 +57,7 @@ struct RndShared {
   alignas(16) uint32_t sq[8];      // state before a squeeze
   Fr g[4];                         // g(0), g(1), g(2), G of the round (canonical)
   Fr claim;                        // the running claim (canonical)
-  Fr r;                            // the latest challenge (Montgomery)
+  Fr r[2];                         // challenge r_i (Montgomery) of round i (1-based) at i mod 2
   alignas(16) unsigned long long red[3 * 8 * RND_MAX_WARPS];
   Fr fa[RND_VEC], fb[RND_VEC];
   // look-ahead and clusters only:
@@ -182,12 +185,12 @@ __device__ __forceinline__ Fr challenge_of(const uint32_t (&d)[8]) {
   return fr_add(half, other);
 }
 
-// The transcript step of round i (0-based): warps 0 to 2 of the block.  Warp 0
+// The transcript step of round t (1-based): warps 0 to 2 of the block.  Warp 0
 // has the message in sh.g; with_claim: the claim is absorbed before it.  At the
-// end sh.r, sh.S are set (visible after the block's next barrier).  msg: where
+// end sh.r[t & 1], sh.S are set (visible after the block's next barrier).  msg: where
 // the proof takes the message, written beside the hashes, g(1) being the claim
 // less g(0) (null: round_message wrote it).
-__device__ __forceinline__ void transcript_step(RndShared& sh, int warp, bool with_claim, Fr* rch,
+__device__ __forceinline__ void transcript_step(RndShared& sh, int warp, int t, bool with_claim, Fr* rch,
                                                 vl_fr* msg = nullptr) {
   const int lane = threadIdx.x & 31;
   if (warp == 0) {
@@ -214,7 +217,7 @@ __device__ __forceinline__ void transcript_step(RndShared& sh, int warp, bool wi
     }
     const Fr r = challenge_of(st.h);
     if (lane == 0) {
-      sh.r = r;
+      sh.r[t & 1] = r;
       if (rch) *rch = r;  // chained proofs continue from this point
     }
   } else if (warp < 3) {
@@ -259,9 +262,9 @@ __device__ __forceinline__ void round_message(RndShared& sh, const Fr& g0, const
   if (lane < 24) pf->g[i][lane >> 3].limb[lane & 7] = sh.g[lane >> 3].v[lane & 7];
 }
 
-// One lane: the claim of the next round, g(r).
-__device__ __forceinline__ void next_claim(RndShared& sh) {
-  const Fr r = sh.r, b = fr_sub(fr_sub(sh.g[1], sh.g[0]), sh.g[3]);
+// One lane: the claim of the next round, g(r), from round t's message and challenge.
+__device__ __forceinline__ void next_claim(RndShared& sh, int t) {
+  const Fr r = sh.r[t & 1], b = fr_sub(fr_sub(sh.g[1], sh.g[0]), sh.g[3]);
   sh.claim = fr_add(sh.g[0], mont_mul_ni(r, fr_add(b, mont_mul_ni(r, sh.g[3]))));
 }
 
@@ -470,7 +473,7 @@ __device__ __forceinline__ void st_cluster(const void* p, uint32_t rank, uint32_
 }
 
 // Rounds 1 to n = cluster_rounds(d1) >= 1 of the proof, the fold with r_n left
-// out.  The first CTA returns with sh.r = r_n and the vectors in memory as round
+// out.  The first CTA returns with r_n in its slot and the vectors in memory as round
 // n saw them (rounds_block goes on from there); the others may leave.
 static __device__ void rounds_cluster(const DevProof& P, vl_proof* pf, RndShared& sh, int n) {
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, nthr = blockDim.x, last = (nthr >> 5) - 1;
@@ -502,9 +505,9 @@ static __device__ void rounds_cluster(const DevProof& P, vl_proof* pf, RndShared
       wide_redc(w1, col[2]);
       s = block_sum_columns<3>(col, sh.red);
     } else {
-      const Fr r = sh.r;
+      const Fr r = sh.r[(t - 1) & 1];
       const int h = 2 * hh;
-      if (rank == 0 && warp == last && lane == 0) next_claim(sh);
+      if (rank == 0 && warp == last && lane == 0) next_claim(sh, t - 1);
       if (4 * own <= nthr) {
         const int l = tid >> 2;
         s = quad_pass(sh, fA, fB, fA, fB, pair(l), l < own, h, r, false);
@@ -533,10 +536,11 @@ static __device__ void rounds_cluster(const DevProof& P, vl_proof* pf, RndShared
         const Fr g1 = shfl_fr(v, 2);
         round_message(sh, shfl_fr(v, 0), shfl_fr(v, 1), t == 1 ? &g1 : nullptr, pf, t - 1);
       }
-      transcript_step(sh, warp, t == 1, P.rch ? P.rch + (t - 1) : nullptr);
+      transcript_step(sh, warp, t, t == 1, P.rch ? P.rch + (t - 1) : nullptr);
       if (warp == 0 && t < n) {
         __syncwarp();
-        for (int i = lane; i < 8 * (C - 1); i += 32) st_cluster(&sh.r.v[i & 7], 1 + (i >> 3), sh.r.v[i & 7]);
+        const Fr& r = sh.r[t & 1];
+        for (int i = lane; i < 8 * (C - 1); i += 32) st_cluster(&r.v[i & 7], 1 + (i >> 3), r.v[i & 7]);
       }
     }
     if (t < n) cluster_sync();
@@ -649,10 +653,10 @@ static __device__ void rounds_block(const DevProof& P, vl_proof* pf, uint8_t* sm
         named_arrive(10, 64);
       }
       if (look && look_warp(warp)) look_terms(sh, warp, 2 * h, i & 1);
-      else transcript_step(sh, warp, i == 0, P.rch ? P.rch + i : nullptr, looked ? pf->g[i] : nullptr);
+      else transcript_step(sh, warp, i + 1, i == 0, P.rch ? P.rch + i : nullptr, looked ? pf->g[i] : nullptr);
       __syncthreads();
     }
-    const Fr r = sh.r;
+    const Fr r = sh.r[(i + 1) & 1];
     const Fr* sA = 2 * h <= RND_VEC ? sh.fa : fA;
     const Fr* sB = 2 * h <= RND_VEC ? sh.fb : fB;
     if (i + 1 == d1) {
@@ -684,7 +688,7 @@ static __device__ void rounds_block(const DevProof& P, vl_proof* pf, uint8_t* sm
     Fr* dB = h <= RND_VEC ? sh.fb : fB;
     if (4 * hh > nthr) {
       // Fold with r_i and evaluate round i + 2 (1-based; pairs j, j + hh) in one pass.
-      if (warp == last && lane == 0) next_claim(sh);
+      if (warp == last && lane == 0) next_claim(sh, i + 1);
       uint32_t w0[17], wi[17];
       wide_zero(w0), wide_zero(wi);
       for (int j = tid; j < hh; j += nthr) fold_pair(sA, sB, dA, dB, j, h, r, w0, wi);
@@ -701,7 +705,7 @@ static __device__ void rounds_block(const DevProof& P, vl_proof* pf, uint8_t* sm
     const bool alone = hh <= 4;
     if (alone && warp != 0) continue;
     const int j = tid >> 2;
-    if (!alone && warp == last && lane == 0) next_claim(sh);
+    if (!alone && warp == last && lane == 0) next_claim(sh, i + 1);
     Fr p = quad_pass(sh, sA, sB, dA, dB, j, j < hh, h, r, alone && j >= hh && lane == 31);
     p = alone ? from_mont_ni(p) : quad_block_sum(sh, p, warp, last);
     if (warp == 0) round_message(sh, shfl_fr(p, 0), shfl_fr(p, 1), nullptr, pf, i + 1);
