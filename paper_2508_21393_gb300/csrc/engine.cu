@@ -1142,6 +1142,22 @@ int make_plan(const vl_job* jobs, int32_t njobs, const vl_batch_opts* opts, vl_p
   return VL_OK;
 }
 
+// A plan made for one call: given up when the call ends, by an exception too (a
+// failed allocation).  Unless the call went well, it waits for the stream first:
+// table copies may still be reading the plan's memory.
+struct OneCallPlan {
+  vl_plan* p = nullptr;
+  cudaStream_t st;
+  bool ok = false;
+  explicit OneCallPlan(void* stream) : st(static_cast<cudaStream_t>(stream)) {}
+  OneCallPlan(const OneCallPlan&) = delete;
+  ~OneCallPlan() {
+    if (!p) return;
+    if (!ok) (void)cudaStreamSynchronize(st);
+    vl_plan_destroy(p);
+  }
+};
+
 }  // namespace
 
 namespace vl {
@@ -1261,15 +1277,14 @@ void vl_plan_destroy(vl_plan* plan) {
 int32_t vl_prove_batch(const vl_job* jobs, int32_t njobs, void* workspace, size_t workspace_bytes, vl_proof* out,
                        int32_t out_space, void* stream, const vl_batch_opts* opts) {
   VL_ABI_TRY
-  vl_plan* p = nullptr;
-  int e = make_plan(jobs, njobs, opts, &p);
+  OneCallPlan one(stream);
+  int e = make_plan(jobs, njobs, opts, &one.p);
   if (e != VL_OK) return e;
   // With device output the descriptor tables are uploaded synchronously, so the
   // host plan can go while device work is still queued; with host output the
   // call ends with a wait for the stream.
-  e = run_plan(p, workspace, workspace_bytes, out, out_space, static_cast<cudaStream_t>(stream), false, false, false);
-  if (e != VL_OK) (void)cudaStreamSynchronize(static_cast<cudaStream_t>(stream));  // uploads of a failed call
-  vl_plan_destroy(p);
+  e = run_plan(one.p, workspace, workspace_bytes, out, out_space, one.st, false, false, false);
+  one.ok = e == VL_OK;
   return e;
   VL_ABI_CATCH(VL_ENOMEM)
 }
@@ -1339,24 +1354,27 @@ extern "C" int32_t vl_prove_matmul_noalloc(const vl_mat* P, const vl_mat* Q, con
   j.P = *P;
   j.Q = *Q;
   j.fs = *fs;
-  vl_plan* p = nullptr;
+  std::unique_lock<std::mutex> lk(g_noalloc_mu, std::defer_lock);  // given back last, after the plan's wait
+  OneCallPlan one(stream);
   vl_batch_opts o{};
   o.persistent = 2;
   o.fold_engine = 1;  // the launches below run the CUDA-core fold
-  int e = make_plan(&j, 1, &o, &p);
+  int e = make_plan(&j, 1, &o, &one.p);
   if (e != VL_OK) return e;
+  vl_plan* const p = one.p;
+  one.ok = true;  // nothing is on the stream yet
   if (p->total > VL_NOALLOC_SCRATCH_BYTES) {
     snprintf(g_last_error, sizeof(g_last_error),
              "vl_prove_matmul_noalloc: job needs %zu bytes of scratch, the fixed array holds %u", p->total,
              (unsigned)VL_NOALLOC_SCRATCH_BYTES);
-    vl_plan_destroy(p);
     return VL_ENOMEM;
   }
-  cudaStream_t st = static_cast<cudaStream_t>(stream);
-  std::lock_guard<std::mutex> lk(g_noalloc_mu);
+  cudaStream_t st = one.st;
+  lk.lock();
   void* ptr = nullptr;
   e = noalloc_scratch_ptr(&ptr);
   uint8_t* ws = static_cast<uint8_t*>(ptr);
+  one.ok = false;
   if (e == VL_OK) e = bind_workspace(p, ws, st);  // descriptor tables into the array (synchronous)
   if (e == VL_OK) {
     const DevProof* dp = reinterpret_cast<const DevProof*>(ws + p->off_proofs);
@@ -1372,12 +1390,11 @@ extern "C" int32_t vl_prove_matmul_noalloc(const vl_mat* P, const vl_mat* Q, con
     if (ce == cudaSuccess) ce = cudaMemcpyAsync(out, dout, sizeof(vl_proof), cudaMemcpyDeviceToHost, st);
     if (ce == cudaSuccess) ce = cudaStreamSynchronize(st);
     // A failed enqueue may leave earlier kernels of this call running on the
-    // array: let them finish before the lock lets the next call rebind it.
-    if (ce != cudaSuccess) (void)cudaStreamSynchronize(st);
+    // array: they finish (~OneCallPlan) before the lock lets the next call rebind it.
+    one.ok = ce == cudaSuccess;
     e = cuda_status(ce, "vl_prove_matmul_noalloc");
     if (e == VL_OK && out->status != VL_OK) e = out->status;
   }
-  vl_plan_destroy(p);
   return e;
   VL_ABI_CATCH(VL_ENOMEM)
 }
