@@ -172,7 +172,7 @@ struct vl_plan {
   std::vector<int> r_item0, r_nitem, r_ib0, r_np;  // per round t (index t): first item, items, ibase start, proofs
   size_t off_ritems = 0, off_ibase = 0, off_ritems_end = 0, off_partials = 0;
   size_t off_tables_end = 0;
-  std::vector<uint8_t> upload;      // the packed tables while their copy may be running
+  std::vector<uint8_t> upload;      // the packed tables while their copy may be running, else empty
   struct PerProof {
     size_t eqA, eqB, soaA, soaB, w8A, w8B, accA, accB, fA, fB, fac;
   };
@@ -1123,6 +1123,7 @@ int run_plan(vl_plan* p, void* workspace, size_t ws_bytes, vl_proof* out, int32_
     if ((ce = cudaMemcpyAsync(out, dout, bytes, cudaMemcpyDeviceToHost, st)) != cudaSuccess)
       return cuda_status(ce, "proof copy-out");
     if ((ce = cudaStreamSynchronize(st)) != cudaSuccess) return cuda_status(ce, "cudaStreamSynchronize");
+    std::vector<uint8_t>().swap(p->upload);  // the copies are done
     for (size_t i = 0; i < p->jobs.size(); i++)
       if (out[i].status != VL_OK) return out[i].status;
   }
@@ -1143,17 +1144,18 @@ int make_plan(const vl_job* jobs, int32_t njobs, const vl_batch_opts* opts, vl_p
 }
 
 // A plan made for one call: given up when the call ends, by an exception too (a
-// failed allocation).  Unless the call went well, it waits for the stream first:
-// table copies may still be reading the plan's memory.
+// failed allocation).  It waits for the stream first while table copies may still
+// be reading the plan's memory, and only then: a call that is refused (a workspace
+// too small or out of alignment) has put nothing on the stream, which may hold
+// other work or be under capture.
 struct OneCallPlan {
   vl_plan* p = nullptr;
   cudaStream_t st;
-  bool ok = false;
   explicit OneCallPlan(void* stream) : st(static_cast<cudaStream_t>(stream)) {}
   OneCallPlan(const OneCallPlan&) = delete;
   ~OneCallPlan() {
     if (!p) return;
-    if (!ok) (void)cudaStreamSynchronize(st);
+    if (!p->upload.empty()) (void)cudaStreamSynchronize(st);
     vl_plan_destroy(p);
   }
 };
@@ -1283,9 +1285,7 @@ int32_t vl_prove_batch(const vl_job* jobs, int32_t njobs, void* workspace, size_
   // With device output the descriptor tables are uploaded synchronously, so the
   // host plan can go while device work is still queued; with host output the
   // call ends with a wait for the stream.
-  e = run_plan(one.p, workspace, workspace_bytes, out, out_space, one.st, false, false, false);
-  one.ok = e == VL_OK;
-  return e;
+  return run_plan(one.p, workspace, workspace_bytes, out, out_space, one.st, false, false, false);
   VL_ABI_CATCH(VL_ENOMEM)
 }
 
@@ -1362,7 +1362,6 @@ extern "C" int32_t vl_prove_matmul_noalloc(const vl_mat* P, const vl_mat* Q, con
   int e = make_plan(&j, 1, &o, &one.p);
   if (e != VL_OK) return e;
   vl_plan* const p = one.p;
-  one.ok = true;  // nothing is on the stream yet
   if (p->total > VL_NOALLOC_SCRATCH_BYTES) {
     snprintf(g_last_error, sizeof(g_last_error),
              "vl_prove_matmul_noalloc: job needs %zu bytes of scratch, the fixed array holds %u", p->total,
@@ -1374,7 +1373,6 @@ extern "C" int32_t vl_prove_matmul_noalloc(const vl_mat* P, const vl_mat* Q, con
   void* ptr = nullptr;
   e = noalloc_scratch_ptr(&ptr);
   uint8_t* ws = static_cast<uint8_t*>(ptr);
-  one.ok = false;
   if (e == VL_OK) e = bind_workspace(p, ws, st);  // descriptor tables into the array (synchronous)
   if (e == VL_OK) {
     const DevProof* dp = reinterpret_cast<const DevProof*>(ws + p->off_proofs);
@@ -1390,8 +1388,8 @@ extern "C" int32_t vl_prove_matmul_noalloc(const vl_mat* P, const vl_mat* Q, con
     if (ce == cudaSuccess) ce = cudaMemcpyAsync(out, dout, sizeof(vl_proof), cudaMemcpyDeviceToHost, st);
     if (ce == cudaSuccess) ce = cudaStreamSynchronize(st);
     // A failed enqueue may leave earlier kernels of this call running on the
-    // array: they finish (~OneCallPlan) before the lock lets the next call rebind it.
-    one.ok = ce == cudaSuccess;
+    // array: let them finish before the lock lets the next call rebind it.
+    if (ce != cudaSuccess) (void)cudaStreamSynchronize(st);
     e = cuda_status(ce, "vl_prove_matmul_noalloc");
     if (e == VL_OK && out->status != VL_OK) e = out->status;
   }
