@@ -209,6 +209,13 @@ bool tc_eligible(const vl_plan* p, const vl_mat& M) {
   return M.space == VL_HOST || (reinterpret_cast<uintptr_t>(M.data) & 15) == 0;
 }
 
+// Row lanes of a column-sum tile of `cols` columns, `per` columns to a thread.
+int colsum_lanes(int64_t cols, int per) {
+  int groups = 1;
+  while ((int64_t)groups * per < cols) groups <<= 1;
+  return FOLD_THREADS / groups;
+}
+
 void add_fold_task(vl_plan* p, const vl_mat& M, int32_t mode, int proof, int side) {
   FoldTask t{};
   t.mat = nullptr;  // bound at run time
@@ -264,16 +271,27 @@ void add_fold_task(vl_plan* p, const vl_mat& M, int32_t mode, int proof, int sid
   // Tiles are cut smaller while the batch would leave SMs without work: two
   // tiles per SM over all tasks, down to 32 rows (16 of a Montgomery column
   // sum), then to 256 columns.  A lone 601 x 2057 x 1033 product with odd rows has
-  // 43 full-size tiles (435 us, 407 in 350 small ones), one of 512 x 2048 x 256
-  // Montgomery operands 32 (563 and 378 us).
+  // 43 full-size tiles (435 us, 407 in 366 small ones; later 231, and 222 in 252,
+  // with the bound on column sums below), one of 512 x 2048 x 256 Montgomery
+  // operands 32 (563 and 378 us).
   const int64_t want = std::max<int64_t>(1, FOLD_TILE_TARGET / (2 * (int64_t)p->jobs.size()));
   auto count = [&](int tr, int tc) { return (((int64_t)t.rows + tr - 1) / tr) * (((int64_t)t.cols + tc - 1) / tc); };
   if (mode == MODE_COLSUM) {
     int tc = fr ? FR_COLSUM_TILE_COLS : COLSUM_TILE_COLS;
     int tr = p->opts.colsum_rows > 0 ? p->opts.colsum_rows : 256;
+    // A tile's row lanes each add their sums to the accumulators, so with l rows to
+    // a lane an accumulator takes rows / l additions, one after the other (0.02 to
+    // 0.03 us each), and all of them 8 rows cols / l (about 47 per ns), while a lane's
+    // chain is l rows (0.24 to 0.36 us each).  The best l is about sqrt(rows max(1,
+    // cols / 176)) / 4: no cut goes below it.  (Cut to 32 rows all the same, the
+    // fold of 4096 x 16 took 506 us, in tiles of 256 rows 35.)
+    auto cut_pays = [&](int tr, int tc) {
+      const int64_t l = std::min<int64_t>(tr, t.rows) / colsum_lanes(std::min<int64_t>(tc, t.cols), fr ? 1 : COLSUM_VEC);
+      return 16 * 176 * l * l >= t.rows * std::max<int64_t>(176, t.cols);
+    };
     if (p->opts.colsum_rows <= 0) {
-      while (tr > (fr ? 16 : 32) && count(tr, tc) < want) tr /= 2;
-      while (tc > 256 && count(tr, tc) < want) tc /= 2;
+      while (tr > (fr ? 16 : 32) && count(tr, tc) < want && cut_pays(tr / 2, tc)) tr /= 2;
+      while (tc > 256 && count(tr, tc) < want && cut_pays(tr, tc / 2)) tc /= 2;
     }
     for (int c0 = 0; c0 < t.cols; c0 += tc)
       for (int r0 = 0; r0 < t.rows; r0 += tr) {
