@@ -129,12 +129,6 @@ __device__ __forceinline__ uint4 lds_u4(uint32_t addr) {
   return r;
 }
 
-__device__ __forceinline__ uint2 lds_u2(uint32_t addr) {
-  uint2 r;
-  asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(r.x), "=r"(r.y) : "r"(addr));
-  return r;
-}
-
 // Offset int16 -> [0, 2^16).
 __device__ __forceinline__ uint32_t off16(int16_t x) { return (uint32_t)(uint16_t)x ^ 0x8000u; }
 

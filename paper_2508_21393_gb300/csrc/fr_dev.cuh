@@ -18,13 +18,4 @@ static __device__ __noinline__ Fr redc_columns_ni(U64x8 acc) { return redc_colum
 __device__ __forceinline__ Fr to_mont_ni(const Fr& a) { return mont_mul_ni(a, fr_r2()); }
 static __device__ __noinline__ Fr from_mont_ni(Fr a) { return from_mont(a); }  // the reduction rows alone
 
-// (lo + hi . 2^256) mod r, canonical (hi . 2^256 = mont_mul(hi, R^2)).
-__device__ __forceinline__ Fr reduce_512_ni(const Fr& lo, const Fr& hi) {
-  const Fr h = mont_mul_ni(hi, fr_r2());
-  Fr l = lo;
-  cond_sub_r(l.v, 0);
-  cond_sub_r(l.v, 0);
-  return fr_add(l, h);
-}
-
 }  // namespace vl

@@ -38,12 +38,12 @@ namespace {
 __global__ void __launch_bounds__(LK_THREADS) lk_start_kernel(LkDev* Ls) {
   LkDev* L = Ls + blockIdx.x;
   __shared__ uint32_t S0[8], S1[8], S2[8], S3[8];
-  __shared__ __align__(16) uint32_t dig[2 * LK_MAX_L + 1][8];
+  __shared__ __align__(16) uint8_t msg[128];
   __shared__ Fr ch[LK_MAX_L];
   __shared__ Fr beta_sh, alpha_sh;
   const int tid = threadIdx.x;
   if (tid < 32) {
-    WarpMsg h(dig);  // the message of ts_start_lookup
+    WarpMsg h(msg);  // the message of ts_start_lookup (86 bytes)
     h.bytes("verilora-gb300/zklookup/v1", 26);
     h.u64le(L->seed);
     h.u32le((uint32_t)L->n);
