@@ -440,9 +440,9 @@ cudaError_t launch_step(const StepItem* items, int nitems, const FoldTask* tasks
                         unsigned long long wait_ns, int never_ready, cudaStream_t st);
 // Batched rounds: round t (1-based, t <= batched_rounds(d1)) of every such
 // proof.  Pass: fold with r_(t-1) (for t = 1 the fold's output is reduced)
-// and evaluate the round over `nitems` items, one canonical partial triple
-// per item; transcript: one warp per proof of [0, nproofs) sums its items'
-// partials (items ibase[p] .. ibase[p + 1]), writes and absorbs the round
+// and sum the round's terms over `nitems` items, three canonical slots per
+// item: g(0), the leading coefficient and, in round 1 only, g(1); transcript:
+// one warp per proof of [0, nproofs) sums its items' partials (items ibase[p] .. ibase[p + 1]), writes and absorbs the round
 // message and squeezes r_t.  Tail: one CTA per proof runs its remaining
 // rounds and writes the proof.
 cudaError_t launch_rounds_pass(const DevProof* proofs, const RoundItem* items, int nitems, Fr* partials, int t,

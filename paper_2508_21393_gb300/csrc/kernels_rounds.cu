@@ -36,6 +36,9 @@ __global__ void __launch_bounds__(512, 1) rounds_cluster_kernel(const DevProof* 
 // host memory 750 -> 578, the 7B step (1024 proofs) 2.60 -> 2.48 ms; with the
 // clusters: the 7B projection 230 -> 207 us (rounds 154 -> 131), the 13B one 460 ->
 // 411, a lone product of 2057 terms 294 -> 250.
+// Batches of a server's four streams, one beside the other, gain too: 1,000 requests of 8
+// proofs a second have a median latency of 0.40 ms, on one CTA of 512 threads per
+// proof 0.45, of 128 threads 0.52; at 10,000 and 20,000 the throughput is the same.
 cudaError_t launch_rounds(const DevProof* proofs, int nproofs, vl_proof* out, int variant, int threads, int max_d1,
                           cudaStream_t st) {
   if (nproofs <= 0) return cudaSuccess;
@@ -84,10 +87,11 @@ cudaError_t launch_rounds(const DevProof* proofs, int nproofs, vl_proof* out, in
 //
 // The same claim and rounds as rounds_block, with the heavy first rounds
 // organised by round instead of by proof: while a proof's round has more
-// than RB_TAIL pairs, the round's vector work (fold with the previous
-// challenge, evaluation of g(0), g(1), g(2)) for all such proofs is one launch
-// of many CTAs, each on a range of one proof's pairs, and the round's
-// transcript step is one launch with one warp per proof.  The first rounds'
+// than 2^RB_TAIL_LOG pairs, the round's vector work (fold with the previous
+// challenge, the sums of g(0) and the leading coefficient, in round 1 of g(1)
+// too) for all such proofs is one launch of many CTAs, each on a range of one
+// proof's pairs, and the round's transcript step is one launch with one warp
+// per proof.  The first rounds'
 // vector work (three quarters of a proof's) then spreads over the whole GPU
 // instead of one CTA per proof; the rounds after that, short vector passes
 // between serial hashes, run as before, one CTA per proof (rounds_block from

@@ -1,8 +1,10 @@
 // Host engine and C ABI of the lookup-argument prover (Protocol 1, Eq.
 // eq:lookup-sumcheck) for range tables, batched: one plan holds the
 // statements, the workspace layout and the work-item tables; a run enqueues
-// the host-operand copies, the multiplicity clear and 6 + 3 per round
-// launches on the caller's stream (see kernels_lookup.cu).
+// the host-operand copies, the multiplicity clear and the launches on the
+// caller's stream (see kernels_lookup.cu): start, histogram, table; per round
+// before the tails at most two passes and a transcript step, before the second
+// round its tables; the tails.
 #include <cuda_runtime.h>
 
 #include <algorithm>
